@@ -215,14 +215,11 @@ def _route_inputs(case, inp, x):
         state["b1"] = inp.normal((MLP_HIDDEN,), 0.1, torch.float32)
         state["W2"] = inp.normal((MLP_HIDDEN, C), MLP_HIDDEN ** -0.5, torch.float32)
         state["b2"] = inp.normal((C,), 0.1, torch.float32)
-        state["image"] = molora.molora_route_mlp_prepare(x.dtype, state["W1"], C)
-    if case["router"] == "gate" and case["layers"] > 1:
-        # a decode loop lays the gate's weights out once
-        state["image"] = molora.molora_route_gate_prepare(x.dtype, state["G"])
     return state
 
 
-def prepare(case, seed):
+def _draw_inputs(case, seed):
+    """Activations, what the router reads, base projections and the adapter stacks of every layer."""
     inp = _Inputs(seed)
     n, C, r = case["tokens"], case["adapters"], case["rank"]
     dtype = torch.float32 if case["dtype"] == "f32" else torch.bfloat16
@@ -237,6 +234,19 @@ def prepare(case, seed):
     state["y"] = y
     weights = [[(inp.normal((C, d_in, r), d_in ** -0.5, dtype), inp.normal((C, r, d_out), 0.1, dtype))
                 for _, d_in, d_out in projs] for _ in range(case["layers"])]
+    return state, weights
+
+
+def prepare(case, seed):
+    n, C = case["tokens"], case["adapters"]
+    projs = _projections(case)
+    state, weights = _draw_inputs(case, seed)
+    x, y = state["x"], state["y"]
+    if case["router"] == "mlp":
+        state["image"] = molora.molora_route_mlp_prepare(x["attn"].dtype, state["W1"], C)
+    if case["router"] == "gate" and case["layers"] > 1:
+        # a decode loop lays the gate's weights out once
+        state["image"] = molora.molora_route_gate_prepare(x["attn"].dtype, state["G"])
     if case["call"] == "host":
         host = {buf: t.cpu().pin_memory() for buf, t in x.items()}
         state["y"] = [t.cpu().pin_memory() for t in y]
@@ -303,3 +313,47 @@ def run(state):
         molora.molora_forward_host(molora.ROUTE_GATE, state["projs"], state["arena"], G=state["G"])
         return {"y": state["y"]}
     return _step(state)
+
+
+# ------------------------------------------------------------------------------------------------ 64 bits
+def _exact_targets(state):
+    """(idx [top, n], weight [top, n]) of every token in 64-bit arithmetic."""
+    case, x = state["case"], state["x"]["attn"].double()
+    if case["router"] == "given":
+        return state["r"].long()[None], None
+    if case["router"] in ("vocab", "composite"):
+        r = torch.bucketize(state["ids"], state["breaks"], right=True) - 1
+        if case["router"] == "composite":
+            r = state["request"].long() * MODALITIES + r
+        return r[None], None
+    if case["router"] == "gate":
+        logits = x @ state["G"].double()
+    else:
+        hidden = torch.nn.functional.gelu(x @ state["W1"].double() + state["b1"].double())
+        logits = hidden @ state["W2"].double() + state["b2"].double()
+    best, idx = logits.topk(case["top"], dim=1)
+    return idx.T, torch.softmax(best, dim=1).T if case["top"] > 1 else None
+
+
+def exact(case, seed):
+    """What the first `run` returns, in 64 bits: y (and the routing weights); whole numbers have no rounding to measure."""
+    state, weights = _draw_inputs(case, seed)
+    idx, weight = _exact_targets(state)
+    ys = []
+    for p, (buf, _, _) in enumerate(_projections(case)):
+        x, y = state["x"][buf].double(), state["y"][p].double()
+        for layer in weights:
+            A, B = layer[p]
+            for slot in range(len(idx)):
+                for c in range(case["adapters"]):
+                    rows = (idx[slot] == c).nonzero()[:, 0]
+                    if len(rows):
+                        delta = x[rows] @ A[c].double() @ B[c].double()
+                        y[rows] += delta if weight is None else weight[slot, rows, None] * delta
+        ys.append(y)
+    if case["call"] == "host":
+        return {"y": [y.cpu() for y in ys]}
+    if case["top"] > 1:
+        return {"r": None, "idx": None, "weight": weight, "y": ys}
+    out = {"counts": None, "offsets": None, "perm": None, "y": ys}
+    return out if case["layers"] > 1 and case["router"] == "given" else dict(out, r=None)
