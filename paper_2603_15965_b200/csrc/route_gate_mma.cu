@@ -218,6 +218,133 @@ __global__ void __launch_bounds__(WARPS * 32) route_gate_mma_kernel(const __nv_b
     }
 }
 
+// The same product for calls of a few hundred tokens.  A warp that walks all of d for its 16 tokens is a chain of d / KC
+// dependent memory round trips (32 of them at d = 4096, ~1 us each), and 64 tokens per CTA leave most SMs without
+// one.  Here 16 tokens belong to a cluster of S CTAs whose 8 S warps take one k chunk each (every 8 S-th if there are
+// more): all operands go from global memory straight into registers in one round trip, the partial logits are summed in
+// warp order in shared memory and in rank order through distributed shared memory.  Bound by one load round trip and the
+// launch.  Measured (us, before -> after): 93 tokens x 4096, C = 16: 34.4 -> 5.7; 777 x 2048, C = 8: 12.0 -> 4.7.
+// Every 16 tokens read the whole weight image (L2), so calls of more than 1023 tokens, which fill the SMs with 64 tokens
+// per CTA (or run on the tcgen05 gate), keep the kernel above.
+constexpr int kGateSplitWarps = 8;
+constexpr int64_t kGateSplitMaxTokens = 1024;
+template <int NT, int KC>
+__global__ void __launch_bounds__(kGateSplitWarps * 32, 2)
+    route_gate_split_kernel(const __nv_bfloat16* __restrict__ x, int64_t N, int d, int64_t ldx,
+                            const __nv_bfloat16* __restrict__ img, const float* __restrict__ bias, int C,
+                            int32_t* __restrict__ r_out, float* __restrict__ logits_out)
+{
+    using Img = GateImage<NT, KC>;
+    constexpr int CP = Img::CP, ROW = Img::ROW, NB = KC / 32;
+    __shared__ __align__(16) float part_s[kGateSplitWarps][16][CP + 4];
+    __shared__ __align__(16) float sum_s[16][CP];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
+    const int S = (int)ptx::cluster_nctarank(), crank = (int)ptx::cluster_ctarank();
+    const int64_t tok0 = (int64_t)(blockIdx.x / S) * 16;
+    const int64_t rowA = tok0 + g < N ? tok0 + g : N - 1;             // tail rows recompute the last token
+    const int64_t rowB = tok0 + g + 8 < N ? tok0 + g + 8 : N - 1;
+    const __nv_bfloat16* xa = x + rowA * ldx + q * 8;
+    const __nv_bfloat16* xb = x + rowB * ldx + q * 8;
+    float acc[NT][3][4];
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int t = 0; t < 3; ++t)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[n][t][i] = 0.f;
+    const int chunks = (d + KC - 1) / KC;
+    bool waited = false;
+    for (int ch = crank * kGateSplitWarps + warp; ch < chunks; ch += S * kGateSplitWarps) {
+        uint4 va[NB], vb[NB];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            const int k = ch * KC + b * 32;
+            const bool in = k + q * 8 < d;
+            va[b] = in ? ldg128_stream(xa + k) : make_uint4(0, 0, 0, 0);
+            vb[b] = in ? ldg128_stream(xb + k) : make_uint4(0, 0, 0, 0);
+        }
+        if (!waited) ptx::grid_dependency_sync();                     // the weight images come from gate_split_kernel
+        waited = true;
+        const __nv_bfloat16* gi = img + (int64_t)ch * Img::kElems + g * ROW + q * 4;
+        constexpr int BB = NT == 1 ? 4 : NT == 2 ? 2 : 1;             // blocks whose weights are in flight at once
+        static_assert(NB % BB == 0, "whole batches");
+#pragma unroll
+        for (int b0 = 0; b0 < NB; b0 += BB) {
+            uint32_t w[BB][2][NT][3][2];
+            // (volatile: the compiler must not move these above the wait for the kernel that writes the image)
+#pragma unroll
+            for (int b = 0; b < BB; ++b)
+#pragma unroll
+                for (int s = 0; s < 2; ++s)
+#pragma unroll
+                    for (int n = 0; n < NT; ++n)
+#pragma unroll
+                        for (int t = 0; t < 3; ++t)
+                            asm volatile("ld.global.v2.u32 {%0,%1}, [%2];"
+                                         : "=r"(w[b][s][n][t][0]), "=r"(w[b][s][n][t][1])
+                                         : "l"(gi + (t * CP + n * 8) * ROW + (b0 + b) * 32 + s * 16)
+                                         : "memory");
+#pragma unroll
+            for (int b = 0; b < BB; ++b)
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const uint4 u = va[b0 + b], v = vb[b0 + b];
+                    const uint32_t a[4] = {s ? u.z : u.x, s ? v.z : v.x, s ? u.w : u.y, s ? v.w : v.y};
+#pragma unroll
+                    for (int n = 0; n < NT; ++n)
+#pragma unroll
+                        for (int t = 0; t < 3; ++t) mma_bf16_16816(acc[n][t], a, w[b][s][n][t][0], w[b][s][n][t][1]);
+                }
+        }
+    }
+    if (!waited) ptx::grid_dependency_sync();
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            part_s[warp][g + 8 * (i >> 1)][n * 8 + 2 * q + (i & 1)] = (acc[n][2][i] + acc[n][1][i]) + acc[n][0][i];
+    __syncthreads();
+    for (int e = tid; e < 16 * CP; e += kGateSplitWarps * 32) {
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < kGateSplitWarps; ++w) v += part_s[w][e / CP][e % CP];
+        sum_s[e / CP][e % CP] = v;
+    }
+    __syncthreads();
+    if (S > 1) ptx::cluster_sync_all();
+    if (crank == 0) {
+        // 16 threads per token, CP / 16 (or one) logits each; ties go to the lowest adapter
+        const int row = tid >> 4, l16 = tid & 15;
+        const int64_t i = tok0 + row;
+        float best = 0.f;
+        int arg = INT32_MAX;
+#pragma unroll
+        for (int j = 0; j < (CP + 15) / 16; ++j) {
+            const int c = l16 + 16 * j;
+            if (c < C) {
+                float z = 0.f;
+                const uint32_t at = ptx::smem_u32(&sum_s[row][c]);
+                for (int k = 0; k < S; ++k) {
+                    float u;
+                    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(u) : "r"(ptx::map_to_cta(at, k)) : "memory");
+                    z += u;
+                }
+                if (bias != nullptr) z += __ldg(bias + c);
+                if (logits_out != nullptr && i < N) logits_out[i * C + c] = z;
+                if (arg == INT32_MAX || z > best) { best = z; arg = c; }
+            }
+        }
+#pragma unroll
+        for (int off = 1; off <= 8; off <<= 1) {
+            const float ob = __shfl_xor_sync(0xFFFFFFFFu, best, off);
+            const int oa = __shfl_xor_sync(0xFFFFFFFFu, arg, off);
+            if (oa != INT32_MAX && (arg == INT32_MAX || ob > best || (ob == best && oa < arg))) { best = ob; arg = oa; }
+        }
+        if (l16 == 0 && i < N) r_out[i] = arg;
+    }
+    if (S > 1) ptx::cluster_sync_all();                              // rank 0 has read this CTA's sums
+}
+
 template <int NT, int WARPS, int KC>
 static molora_status_t gate_mma_launch(const void* x, int64_t N, int d, int64_t ldx, const float* G, const float* bias,
                                        int C, int32_t* r_out, float* logits_out, void* ws, cudaStream_t s, int image)
@@ -233,6 +360,13 @@ static molora_status_t gate_mma_launch(const void* x, int64_t N, int d, int64_t 
             return MOLORA_ERR_CUDA;
     }
     if (image == kImageBuildOnly) return MOLORA_OK;
+    if (N < kGateSplitMaxTokens) {
+        int S = 1;
+        while (S < 8 && S * kGateSplitWarps < chunks) S *= 2;
+        return cuda_ok(launch_kernel(route_gate_split_kernel<NT, KC>, dim3((unsigned)(ceil_div64(N, 16) * S)), dim3(kGateSplitWarps * 32), 0,
+                                     s, (unsigned)S, image == kImageBuildAndUse, static_cast<const __nv_bfloat16*>(x), N, d, ldx, img, bias,
+                                     C, r_out, logits_out));
+    }
     const int64_t blocks = ceil_div64(N, 16 * WARPS);
     return cuda_ok(launch_kernel(route_gate_mma_kernel<NT, WARPS, KC>, dim3((unsigned)blocks), dim3(WARPS * 32), 0, s, 1,
                                  image == kImageBuildAndUse,
