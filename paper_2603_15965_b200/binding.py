@@ -198,7 +198,7 @@ def molora_launch_count() -> int:
 
 
 TUNING_NAMES = ("umma_min_tokens", "small_path", "stream_tile", "umma_split", "umma_tile_rows", "group_split",
-                "chained_launch_off", "jobs_launch")
+                "chained_launch_off", "stream_split", "jobs_launch")
 
 
 def molora_debug_set(name: str, value: int) -> None:

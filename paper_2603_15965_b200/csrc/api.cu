@@ -16,7 +16,7 @@ std::atomic<int64_t> g_tune[kTuneCount];
 std::atomic<uint64_t> g_launches{0};
 std::once_flag g_tune_once;
 const char* const kTuneNames[kTuneCount] = {"umma_min_tokens", "small_path", "stream_tile", "umma_split",
-                                            "umma_tile_rows", "group_split", "chained_launch_off", "jobs_launch"};
+                                            "umma_tile_rows", "group_split", "chained_launch_off", "stream_split", "jobs_launch"};
 void tune_from_environment()
 {
     auto num = [](const char* name) {
@@ -32,6 +32,7 @@ void tune_from_environment()
     g_tune[kTuneGroupSplit] = num("MOLORA_GROUP_SPLIT");
     const char* ch = std::getenv("MOLORA_CHAINED_LAUNCH");
     g_tune[kTuneChainedLaunchOff] = ch != nullptr && std::strcmp(ch, "0") == 0 ? 1 : 0;
+    g_tune[kTuneStreamSplit] = num("MOLORA_STREAM_SPLIT");
     g_tune[kTuneJobsLaunch] = num("MOLORA_JOBS_LAUNCH");
 }
 }  // namespace
@@ -642,10 +643,10 @@ molora_status_t molora_apply_topk(const molora_proj_desc_t* projs, int32_t P, mo
             return launch_apply_umma(pass, P, N, n_sets, offsets, perm, dev_status, 1, s, nullptr, nullptr, k, C, table);
         }
         if (group_apply_stream_eligible(N))         // the CTAs of the apply group the sets themselves
-            return launch_group_apply_stream_sets(sets, pass, P, N, n_sets, k, table, counts, offsets, perm, dev_status, s);
+            return launch_group_apply_stream_sets(sets, pass, P, N, n_sets, k, C, table, counts, offsets, perm, dev_status, s);
         st = molora_group(sets, N, n_sets, counts, offsets, perm, nullptr, 0, dev_status, stream);
         if (st != MOLORA_OK) return st;
-        return launch_apply_stream_sets(pass, P, N, n_sets, k, table, offsets, perm, dev_status, s);
+        return launch_apply_stream_sets(pass, P, N, n_sets, k, C, table, offsets, perm, dev_status, s);
     }
     for (int32_t j = 0; j < k; ++j) {               // one (group, apply) pass per kept adapter slot
         for (int i = 0; i < P; ++i) {

@@ -304,10 +304,10 @@ molora_status_t launch_apply_stream(const molora_proj_desc_t* projs, int32_t P, 
 // j-th adapter of the set), the projections carry the stacked rank parts x r and row_scale = weights [parts][N].
 bool stream_eligible(const molora_proj_desc_t& p, molora_dtype_t dt);
 molora_status_t launch_apply_stream_sets(const molora_proj_desc_t* projs, int32_t P, int64_t N, int32_t n_sets, int32_t parts,
-                                         const uint8_t* set_table, const int32_t* offsets, const int32_t* perm,
+                                         int32_t n_adapters, const uint8_t* set_table, const int32_t* offsets, const int32_t* perm,
                                          uint32_t* dev_status, cudaStream_t s);
 molora_status_t launch_group_apply_stream_sets(const int32_t* sets, const molora_proj_desc_t* projs, int32_t P, int64_t N,
-                                               int32_t n_sets, int32_t parts, const uint8_t* set_table, int32_t* counts,
+                                               int32_t n_sets, int32_t parts, int32_t n_adapters, const uint8_t* set_table, int32_t* counts,
                                                int32_t* offsets, int32_t* perm, uint32_t* dev_status, cudaStream_t s);
 // The same kernel started from the routing decisions r: grouping (counts, offsets, perm as molora_group writes them)
 // and apply in one launch; all projections of one rank, at most 4096 tokens.
@@ -361,11 +361,12 @@ bool chained_launch_enabled();   // false when the "chained_launch_off" override
 enum TuneKey {
     kTuneUmmaMinTokens = 0,   // tcgen05 apply from this many tokens
     kTuneSmallPath,           // kernel below the tcgen05 crossover: 1 streaming, 2 two-launch, 3 job-list decode kernel
-    kTuneStreamTile,          // rank-16 streaming tile: 16 or 32 rows
+    kTuneStreamTile,          // streaming tile: 16 or 32 rows
     kTuneUmmaSplit,           // cluster size of the tcgen05 apply
     kTuneUmmaTileRows,        // rows per tile of the tcgen05 apply
     kTuneGroupSplit,          // cluster size of the grouping kernel
     kTuneChainedLaunchOff,    // 1: no programmatic dependent launches
+    kTuneStreamSplit,         // cluster size of the streaming kernel: 1, 2, 4 or 8
     kTuneJobsLaunch,          // job-list kernel: 0 cooperative launch, 1 plain, 2 programmatic (measurements only)
     kTuneCount
 };

@@ -38,4 +38,19 @@ static inline bool make_tensor_map_bf16_2d(CUtensorMap* m, const void* ptr, uint
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Row blocks of a bf16 matrix [rows, cols] of pitch `cols` for loads of many columns at once: dimensions (block columns, rows,
+// cols / block), so that one box of all blocks lands as one [rows][block] tile per block.  `block` divides cols.
+static inline bool make_tensor_map_bf16_blocks(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint32_t block,
+                                               uint32_t box_rows, uint32_t box_blocks, CUtensorMapSwizzle swz)
+{
+    EncodeTiledFn fn = tensor_map_encode_fn();
+    if (fn == nullptr) return false;
+    const cuuint64_t dims[3] = {block, rows, cols / block};
+    const cuuint64_t strides[2] = {cols * 2, (cuuint64_t)block * 2};
+    const cuuint32_t box[3] = {block, box_rows, box_blocks};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace molora
