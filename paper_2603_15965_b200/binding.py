@@ -1,4 +1,5 @@
-"""ctypes binding of the C ABI in include/molora.h.  Argument marshalling only.
+"""Binding of the C ABI in include/molora.h.  Argument marshalling only: the entry points of a serving step in the
+compiled extension ``_marshal`` (csrc/marshal.cpp), the others with ctypes.
 
 Each ``molora_*`` function mirrors the C entry point of the same name: torch tensors stand for the
 device pointers (``data_ptr()``), sizes and pitches are read from their shapes and strides, and the
@@ -17,13 +18,14 @@ from typing import List, Optional, Sequence, Tuple
 
 import torch
 
-from .build import LIB_PATH, ROOT
+from .build import LIB_PATH, MARSHAL_PATH, ROOT
 
 F32, BF16 = 0, 1
 MAX_ADAPTERS = 256
 MAX_PROJECTIONS = 8
 
 _lib = None
+_marshal = None
 
 
 class MoloraError(RuntimeError):
@@ -150,6 +152,18 @@ def load_library():
     return lib
 
 
+def _load_marshal():
+    """Import the in-tree extension beside the library (both built by ``paper_2603_15965_b200.build``)."""
+    global _marshal
+    load_library()
+    if not os.path.exists(MARSHAL_PATH):
+        raise ImportError(f"{MARSHAL_PATH} is missing: run `python -m paper_2603_15965_b200.build` (there is no fallback)")
+    from . import _marshal as extension
+    extension.bind(_check)
+    _marshal = extension
+    return extension
+
+
 # ----------------------------------------------------------------------------- helpers
 def _check(fn: str, status: int) -> None:
     if status != 0:
@@ -213,31 +227,14 @@ def molora_status_string(status: int) -> str:
 def molora_route_vocab(ids: torch.Tensor, breaks: torch.Tensor, r_out: Optional[torch.Tensor] = None,
                        dev_status: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """r_out[i] = m with breaks[m] <= ids[i] < breaks[m+1] (Definition 3.1, 0-based); -1 if unrouted."""
-    lib = load_library()
-    _i32_dev(ids, "ids"), _i32_dev(breaks, "breaks")
-    N, M = ids.numel(), breaks.numel() - 1
-    if r_out is None:
-        r_out = torch.empty(N, dtype=torch.int32, device=ids.device)
-    _check("molora_route_vocab", lib.molora_route_vocab(_ptr(ids), N, _ptr(breaks), M, _ptr(_i32_dev(r_out, "r_out")),
-                                                        _ptr(dev_status), _stream(stream)))
-    return r_out
+    return (_marshal or _load_marshal()).route_vocab(ids, breaks, r_out, dev_status, stream)
 
 
 def molora_route_composite(ids: torch.Tensor, adapter: torch.Tensor, breaks: torch.Tensor, n_adapters: int,
                            r_out: Optional[torch.Tensor] = None, dev_status: Optional[torch.Tensor] = None,
                            stream=None) -> torch.Tensor:
     """r_out[i] = adapter[i] * M + m(ids[i]) (Definition 3.2 / Algorithm 1); -1 if the token is unrouted."""
-    lib = load_library()
-    _i32_dev(ids, "ids"), _i32_dev(adapter, "adapter"), _i32_dev(breaks, "breaks")
-    N, M = ids.numel(), breaks.numel() - 1
-    if adapter.numel() != N:
-        raise ValueError("adapter must hold one index per token")
-    if r_out is None:
-        r_out = torch.empty(N, dtype=torch.int32, device=ids.device)
-    _check("molora_route_composite", lib.molora_route_composite(_ptr(ids), _ptr(adapter), N, _ptr(breaks), M,
-                                                                int(n_adapters), _ptr(_i32_dev(r_out, "r_out")),
-                                                                _ptr(dev_status), _stream(stream)))
-    return r_out
+    return (_marshal or _load_marshal()).route_composite(ids, adapter, breaks, n_adapters, r_out, dev_status, stream)
 
 
 def molora_route_mlp_workspace_bytes(xdt: int, d: int, H: int, C: int) -> int:
@@ -250,28 +247,7 @@ def molora_route_mlp(x: torch.Tensor, W1: torch.Tensor, b1: Optional[torch.Tenso
                      dev_status: Optional[torch.Tensor] = None, stream=None, prepared: Optional[torch.Tensor] = None) -> torch.Tensor:
     """r_out[i] = argmax_c (W2 GELU(W1 x_i + b1) + b2)[c] (Eq. 9, top-1); W1 [d, H], W2 [H, C] fp32.
     ``prepared``: the workspace molora_route_mlp_prepare returned for this W1 (saves the preparation launch)."""
-    lib = load_library()
-    N, d, ldx = _matrix(x, "x")
-    if W1.dtype != torch.float32 or W2.dtype != torch.float32 or not W1.is_contiguous() or not W2.is_contiguous():
-        raise ValueError("W1 [d, H] and W2 [H, C] must be dense fp32 tensors")
-    H, C = W2.shape
-    if tuple(W1.shape) != (d, H):
-        raise ValueError("W1 must be [d, H]")
-    if r_out is None:
-        r_out = torch.empty(N, dtype=torch.int32, device=x.device)
-    need = molora_route_mlp_workspace_bytes(_dtype_code(x), d, H, C)
-    if ws is None and need > 0:
-        ws = torch.zeros(need, dtype=torch.uint8, device=x.device)
-    ws_bytes = 0 if ws is None else ws.numel() * ws.element_size()
-    if prepared is not None:
-        _check("molora_route_mlp_prepared", lib.molora_route_mlp_prepared(
-            _ptr(x), _dtype_code(x), N, d, ldx, _ptr(W1), _ptr(b1), H, _ptr(W2), _ptr(b2), C, _ptr(_i32_dev(r_out, "r_out")),
-            _ptr(logits_out), _ptr(prepared), prepared.numel(), _ptr(dev_status), _stream(stream)))
-        return r_out
-    _check("molora_route_mlp", lib.molora_route_mlp(_ptr(x), _dtype_code(x), N, d, ldx, _ptr(W1), _ptr(b1), H, _ptr(W2),
-                                                    _ptr(b2), C, _ptr(_i32_dev(r_out, "r_out")), _ptr(logits_out),
-                                                    _ptr(ws), ws_bytes, _ptr(dev_status), _stream(stream)))
-    return r_out
+    return (_marshal or _load_marshal()).route_mlp(x, W1, b1, W2, b2, r_out, logits_out, ws, dev_status, stream, prepared)
 
 
 def molora_route_gate_workspace_bytes(xdt: int, d: int, C: int) -> int:
@@ -284,31 +260,7 @@ def molora_route_gate(x: torch.Tensor, G: torch.Tensor, bias: Optional[torch.Ten
                       stream=None, prepared: Optional[torch.Tensor] = None) -> torch.Tensor:
     """r_out[i] = argmax_c sum_k x[i,k] G[k,c] (+ bias[c]) (Eq. 8, k = 1); lowest index on ties.
     ``prepared``: the workspace molora_route_gate_prepare returned for this G (saves the preparation launch)."""
-    lib = load_library()
-    N, d, ldx = _matrix(x, "x")
-    if G.dtype != torch.float32 or not G.is_cuda or not G.is_contiguous() or G.dim() != 2 or G.shape[0] != d:
-        raise ValueError("G: expected a contiguous fp32 CUDA tensor of shape [d, C]")
-    C = G.shape[1]
-    if bias is not None and (bias.dtype != torch.float32 or bias.numel() != C or not bias.is_contiguous()):
-        raise ValueError("bias: expected contiguous fp32 [C]")
-    if r_out is None:
-        r_out = torch.empty(N, dtype=torch.int32, device=x.device)
-    if logits_out is not None and (logits_out.dtype != torch.float32 or logits_out.shape != (N, C)
-                                   or not logits_out.is_contiguous()):
-        raise ValueError("logits_out: expected contiguous fp32 [N, C]")
-    if prepared is not None:
-        _check("molora_route_gate_prepared", lib.molora_route_gate_prepared(
-            _ptr(x), _dtype_code(x), N, d, ldx, _ptr(G), _ptr(bias), C, _ptr(_i32_dev(r_out, "r_out")), _ptr(logits_out),
-            _ptr(prepared), prepared.numel(), _ptr(dev_status), _stream(stream)))
-        return r_out
-    need = molora_route_gate_workspace_bytes(_dtype_code(x), d, C)
-    if ws is None and need > 0:
-        ws = torch.zeros(need, dtype=torch.uint8, device=x.device)
-    ws_bytes = 0 if ws is None else ws.numel() * ws.element_size()
-    _check("molora_route_gate", lib.molora_route_gate(_ptr(x), _dtype_code(x), N, d, ldx, _ptr(G), _ptr(bias), C,
-                                                      _ptr(_i32_dev(r_out, "r_out")), _ptr(logits_out), _ptr(ws),
-                                                      ws_bytes, _ptr(dev_status), _stream(stream)))
-    return r_out
+    return (_marshal or _load_marshal()).route_gate(x, G, bias, r_out, logits_out, ws, dev_status, stream, prepared)
 
 
 def molora_route_gate_prepare(x_dtype: torch.dtype, G: torch.Tensor, ws: Optional[torch.Tensor] = None, stream=None):
@@ -383,20 +335,7 @@ def molora_group(r: torch.Tensor, C: int, counts: Optional[torch.Tensor] = None,
                  ws: Optional[torch.Tensor] = None, dev_status: Optional[torch.Tensor] = None,
                  stream=None) -> Tuple[torch.Tensor, torch.Tensor, torch.Tensor]:
     """(counts [C], offsets [C+1], perm [N]) of Section 3.3; perm is stable, its first offsets[C] entries valid."""
-    lib = load_library()
-    _i32_dev(r, "r")
-    N = r.numel()
-    dev = r.device
-    counts = torch.empty(C, dtype=torch.int32, device=dev) if counts is None else _i32_dev(counts, "counts")
-    offsets = torch.empty(C + 1, dtype=torch.int32, device=dev) if offsets is None else _i32_dev(offsets, "offsets")
-    perm = torch.empty(max(N, 1), dtype=torch.int32, device=dev) if perm is None else _i32_dev(perm, "perm")
-    need = molora_group_workspace_bytes(N, C)
-    if ws is None and need > 0:
-        ws = torch.zeros(need, dtype=torch.uint8, device=dev)
-    ws_bytes = 0 if ws is None else ws.numel() * ws.element_size()
-    _check("molora_group", lib.molora_group(_ptr(r), N, C, _ptr(counts), _ptr(offsets), _ptr(perm), _ptr(ws), ws_bytes,
-                                            _ptr(dev_status), _stream(stream)))
-    return counts, offsets, perm
+    return (_marshal or _load_marshal()).group(r, C, counts, offsets, perm, ws, dev_status, stream)
 
 
 def molora_apply_workspace_bytes(N: int, C: int, d_in: int, d_out: int, rank: int) -> int:
@@ -474,15 +413,7 @@ def molora_apply_batched_workspace_bytes(arr, N: int, C: int) -> int:
 def molora_apply_batched(projs, offsets: torch.Tensor, perm: torch.Tensor, ws: Optional[torch.Tensor] = None,
                          dev_status: Optional[torch.Tensor] = None, stream=None, packed=None) -> None:
     """One launch for the projections of a layer (shared N, C, offsets, perm).  ``projs``: ProjDesc list."""
-    lib = load_library()
-    arr, N, C, dt = packed if packed is not None else pack_proj_descs(projs)
-    if ws is None:
-        need = molora_apply_batched_workspace_bytes(arr, N, C)
-        if need > 0:
-            ws = torch.zeros(need, dtype=torch.uint8, device=offsets.device)
-    ws_bytes = 0 if ws is None else ws.numel() * ws.element_size()
-    _check("molora_apply_batched", lib.molora_apply_batched(arr, len(arr), dt, N, C, _ptr(offsets), _ptr(perm),
-                                                            _ptr(ws), ws_bytes, _ptr(dev_status), _stream(stream)))
+    (_marshal or _load_marshal()).apply_batched(projs, offsets, perm, ws, dev_status, stream, packed)
 
 
 def molora_group_apply_batched(r: torch.Tensor, projs, C: Optional[int] = None, counts: Optional[torch.Tensor] = None,
@@ -491,55 +422,19 @@ def molora_group_apply_batched(r: torch.Tensor, projs, C: Optional[int] = None, 
                                packed=None) -> Tuple[torch.Tensor, torch.Tensor, torch.Tensor]:
     """molora_group followed by molora_apply_batched as one call (one launch where the library can fuse them).
     Returns (counts, offsets, perm) as molora_group does."""
-    lib = load_library()
-    _i32_dev(r, "r")
-    arr, N, C_, dt = packed if packed is not None else pack_proj_descs(projs)
-    C = C_ if C is None else C
-    if r.numel() != N or C != C_:
-        raise ValueError("r must hold one routing decision per token of the projections")
-    dev = r.device
-    counts = torch.empty(C, dtype=torch.int32, device=dev) if counts is None else _i32_dev(counts, "counts")
-    offsets = torch.empty(C + 1, dtype=torch.int32, device=dev) if offsets is None else _i32_dev(offsets, "offsets")
-    perm = torch.empty(max(N, 1), dtype=torch.int32, device=dev) if perm is None else _i32_dev(perm, "perm")
-    if ws is None:
-        need = molora_apply_batched_workspace_bytes(arr, N, C)
-        if need > 0:
-            ws = torch.zeros(need, dtype=torch.uint8, device=dev)
-    ws_bytes = 0 if ws is None else ws.numel() * ws.element_size()
-    _check("molora_group_apply_batched",
-           lib.molora_group_apply_batched(_ptr(r), N, C, _ptr(counts), _ptr(offsets), _ptr(perm), arr, len(arr), dt, _ptr(ws),
-                                          ws_bytes, _ptr(dev_status), _stream(stream)))
-    return counts, offsets, perm
+    return (_marshal or _load_marshal()).group_apply_batched(r, projs, C, counts, offsets, perm, ws, dev_status, stream, packed)
 
 
 def molora_topk_softmax(logits: torch.Tensor, k: int, stream=None):
     """Eq. 8: the k largest logits per token (ties: lowest index first) and the softmax over them.
     Returns (idx int32 [k, N], w fp32 [k, N]), slot 0 = the largest logit."""
-    lib = load_library()
-    if logits.dtype != torch.float32 or logits.dim() != 2 or not logits.is_contiguous():
-        raise ValueError("logits must be a dense fp32 [N, C] tensor")
-    N, C = logits.shape
-    idx = torch.empty(k, N, dtype=torch.int32, device=logits.device)
-    w = torch.empty(k, N, dtype=torch.float32, device=logits.device)
-    _check("molora_topk_softmax", lib.molora_topk_softmax(_ptr(logits), N, C, int(k), _ptr(idx), _ptr(w), _stream(stream)))
-    return idx, w
+    return (_marshal or _load_marshal()).topk_softmax(logits, k, stream)
 
 
 def molora_apply_topk(projs, idx: torch.Tensor, w: torch.Tensor, C: int, ws: Optional[torch.Tensor] = None,
                       dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
     """Eq. 8: y_i += sum_j w[j, i] * scale * (x_i A[idx[j, i]]) B[idx[j, i]] as k passes of (group, apply)."""
-    lib = load_library()
-    arr, N, C_, dt = pack_proj_descs(projs)
-    if C_ != C or idx.dtype != torch.int32 or w.dtype != torch.float32 or tuple(idx.shape) != tuple(w.shape) or idx.shape[1] != N:
-        raise ValueError("idx int32 [k, N] and w fp32 [k, N] must match the projections")
-    k = idx.shape[0]
-    need = int(lib.molora_apply_topk_workspace_bytes(arr, len(arr), N, C))
-    if ws is None:
-        ws = torch.zeros(need + 256, dtype=torch.uint8, device=idx.device)
-    off = (-ws.data_ptr()) % 256
-    _check("molora_apply_topk", lib.molora_apply_topk(arr, len(arr), dt, N, C, k, _ptr(idx.contiguous()), _ptr(w.contiguous()),
-                                                      ctypes.c_void_p(ws.data_ptr() + off), ws.numel() - off,
-                                                      _ptr(dev_status), _stream(stream)))
+    (_marshal or _load_marshal()).apply_topk(projs, idx, w, C, ws, dev_status, stream)
 
 
 ROUTE_VOCAB, ROUTE_GATE, ROUTE_GIVEN = 0, 1, 2

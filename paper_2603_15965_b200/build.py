@@ -1,15 +1,18 @@
-"""In-tree build of the CUDA library (nvcc, sm_100a only).  `python -m paper_2603_15965_b200.build`."""
+"""In-tree build of the CUDA library (nvcc, sm_100a only) and of the extension that marshals its arguments (g++ against
+torch's headers).  `python -m paper_2603_15965_b200.build`."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libmolora.so")
+MARSHAL_PATH = os.path.join(PKG_DIR, "_marshal.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--threads", "0", "-I", os.path.join(ROOT, "include")]
@@ -27,9 +30,33 @@ def _stale() -> bool:
     return any(os.path.getmtime(p) > built for p in deps)
 
 
+def build_marshal(force: bool = False) -> str:
+    """Compile csrc/marshal.cpp into _marshal.so beside the library it links to (no GPU, no nvcc)."""
+    src = os.path.join(CSRC, "marshal.cpp")
+    deps = [src] + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    if not force and os.path.exists(MARSHAL_PATH) and all(os.path.getmtime(p) <= os.path.getmtime(MARSHAL_PATH) for p in deps):
+        return MARSHAL_PATH
+    import torch
+    torch_dir = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = MARSHAL_PATH + f".{os.getpid()}.tmp"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++20", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(ROOT, "include"), "-isystem", os.path.join(torch_dir, "include"),
+           "-isystem", os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+           "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), src, "-o", tmp,
+           "-L", os.path.join(torch_dir, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-L", PKG_DIR, "-l:libmolora.so",
+           "-Wl,-rpath,$ORIGIN"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed:\n" + res.stdout + res.stderr)
+    os.replace(tmp, MARSHAL_PATH)
+    return MARSHAL_PATH
+
+
 def build_library(force: bool = False, verbose: bool = False) -> str:
     """Compile csrc/*.cu into libmolora.so next to this file (cross-compiles without a GPU)."""
     if not force and not _stale():
+        build_marshal()
         return LIB_PATH
     nvcc = os.environ.get("NVCC", "nvcc")
     tmp = LIB_PATH + f".{os.getpid()}.tmp"
@@ -40,6 +67,7 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
     if verbose:
         sys.stderr.write(res.stderr)
     os.replace(tmp, LIB_PATH)
+    build_marshal(force)
     return LIB_PATH
 
 

@@ -1,0 +1,441 @@
+// Argument marshalling of the hot entry points, as a CPython extension over the C ABI in include/molora.h.
+//
+// What a small call costs is mostly this: reading the shapes, strides, types and pointers of up to 33 tensors, three output
+// allocations and the current stream.  Done attribute by attribute from Python it took 35 - 60 us per step, several times
+// what the kernels take (one decode layer of seven projections: 58 us per call against 11 us of GPU time); here it is a few
+// microseconds.  Every call does all of it again: nothing is kept between calls.
+//
+// Checks, messages and results are those documented in binding.py, which keeps the public signatures and calls the
+// functions below with positional arguments.  A refused call raises MoloraError through `raise_status`.
+#include <Python.h>
+
+#include <ATen/ATen.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <algorithm>
+#include <string>
+#include <vector>
+
+#include "molora.h"
+
+namespace {
+
+PyObject* g_raise_status = nullptr;      // binding._check(function name, status)
+PyObject *s_x, *s_y, *s_A, *s_B, *s_scale, *s_row_scale, *s_cuda_stream;
+
+struct PyRaised {};                      // a Python exception is set
+[[noreturn]] void raise(PyObject* type, const std::string& text)
+{
+    PyErr_SetString(type, text.c_str());
+    throw PyRaised{};
+}
+struct Ref {                             // owned reference
+    PyObject* p;
+    explicit Ref(PyObject* q) : p(q)
+    {
+        if (p == nullptr) throw PyRaised{};
+    }
+    ~Ref() { Py_XDECREF(p); }
+    Ref(const Ref&) = delete;
+    Ref& operator=(const Ref&) = delete;
+};
+
+void check(const char* fn, molora_status_t status)
+{
+    if (status == MOLORA_OK) return;
+    Ref r(PyObject_CallFunction(g_raise_status, "si", fn, (int)status));
+    raise(PyExc_RuntimeError, std::string(fn) + " was refused");      // (not reached: the callable raises)
+}
+
+const at::Tensor& tensor(PyObject* o, const char* name)
+{
+    if (!THPVariable_Check(o)) raise(PyExc_TypeError, std::string(name) + ": expected a tensor");
+    return THPVariable_Unpack(o);
+}
+void* ptr(PyObject* o, const char* name) { return o == Py_None ? nullptr : tensor(o, name).data_ptr(); }
+PyObject* wrap(const at::Tensor& t)
+{
+    PyObject* o = THPVariable_Wrap(t);
+    if (o == nullptr) throw PyRaised{};
+    return o;
+}
+int64_t integer(PyObject* o)
+{
+    const long long v = PyLong_AsLongLong(o);
+    if (v == -1 && PyErr_Occurred()) throw PyRaised{};
+    return v;
+}
+void* stream_of(PyObject* o)
+{
+    if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+    Ref v(PyObject_HasAttr(o, s_cuda_stream) ? PyObject_GetAttr(o, s_cuda_stream) : PyNumber_Long(o));
+    void* p = PyLong_AsVoidPtr(v.p);
+    if (p == nullptr && PyErr_Occurred()) throw PyRaised{};
+    return p;
+}
+const at::Tensor& i32_dev(PyObject* o, const char* name)
+{
+    const at::Tensor& t = tensor(o, name);
+    if (!t.is_cuda() || t.scalar_type() != at::kInt || !t.is_contiguous())
+        raise(PyExc_ValueError, std::string(name) + ": expected a contiguous int32 CUDA tensor");
+    return t;
+}
+at::Tensor i32_out(PyObject* o, const char* name, int64_t n, const at::Device& dev)
+{
+    if (o != Py_None) return i32_dev(o, name);
+    return at::empty({n}, at::TensorOptions().dtype(at::kInt).device(dev));
+}
+molora_dtype_t dtype_code(const at::Tensor& t)
+{
+    if (t.scalar_type() == at::kFloat) return MOLORA_F32;
+    if (t.scalar_type() == at::kBFloat16) return MOLORA_BF16;
+    raise(PyExc_TypeError, std::string("unsupported element type ") + c10::toString(t.scalar_type()) + ": fp32 or bf16 only");
+}
+struct Matrix {
+    int64_t rows, cols, pitch;
+};
+Matrix matrix(const at::Tensor& t, const char* name)
+{
+    if (!t.is_cuda() || t.dim() != 2 || (t.size(1) > 1 && t.stride(1) != 1))
+        raise(PyExc_ValueError, std::string(name) + ": expected a 2-D row-major CUDA tensor");
+    const int64_t rows = t.size(0), cols = t.size(1);
+    return {rows, cols, rows > 1 ? t.stride(0) : std::max<int64_t>(t.stride(0), cols)};
+}
+// the caller's workspace, or one of `need` bytes
+struct Workspace {
+    at::Tensor t;
+    void* p = nullptr;
+    size_t n = 0;
+    Workspace(PyObject* o, size_t need, const at::Device& dev, bool zero)
+    {
+        const auto opt = at::TensorOptions().dtype(at::kByte).device(dev);
+        if (o != Py_None) t = tensor(o, "ws");
+        else if (need > 0) t = zero ? at::zeros({(int64_t)need}, opt) : at::empty({(int64_t)need}, opt);
+        else return;
+        p = t.data_ptr();
+        n = (size_t)t.numel() * t.element_size();
+    }
+};
+
+// ---- descriptors of a batched apply: from ProjDesc objects, or the array that pack_proj_descs returned
+struct Projs {
+    std::vector<molora_proj_desc_t> own;
+    Py_buffer view{};
+    const molora_proj_desc_t* d = nullptr;
+    int32_t P = 0;
+    int64_t N = 0, C = 0;
+    molora_dtype_t dt = MOLORA_F32;
+
+    Projs(PyObject* projs, PyObject* packed)
+    {
+        if (packed != Py_None) {
+            Ref arr(PySequence_GetItem(packed, 0)), n(PySequence_GetItem(packed, 1)), c(PySequence_GetItem(packed, 2)),
+                t(PySequence_GetItem(packed, 3));
+            N = integer(n.p), C = integer(c.p), dt = (molora_dtype_t)integer(t.p);
+            if (PyObject_GetBuffer(arr.p, &view, PyBUF_SIMPLE) != 0) throw PyRaised{};
+            d = static_cast<const molora_proj_desc_t*>(view.buf);
+            P = (int32_t)(view.len / (Py_ssize_t)sizeof(molora_proj_desc_t));
+            return;
+        }
+        Ref seq(PySequence_Fast(projs, "projs: expected a sequence of ProjDesc"));
+        P = (int32_t)PySequence_Fast_GET_SIZE(seq.p);
+        own.resize((size_t)P);
+        for (int32_t i = 0; i < P; ++i) fill(PySequence_Fast_GET_ITEM(seq.p, i), own[(size_t)i], i == 0);
+        d = own.data();
+    }
+    ~Projs()
+    {
+        if (view.obj != nullptr) PyBuffer_Release(&view);
+    }
+    Projs(const Projs&) = delete;
+    Projs& operator=(const Projs&) = delete;
+
+    size_t apply_bytes() const
+    {
+        size_t need = 0;
+        for (int32_t i = 0; i < P; ++i) need += molora_apply_workspace_bytes(N, (int32_t)C, d[i].d_in, d[i].d_out, d[i].rank);
+        return need;
+    }
+
+private:
+    void fill(PyObject* o, molora_proj_desc_t& out, bool first)
+    {
+        Ref ox(PyObject_GetAttr(o, s_x)), oy(PyObject_GetAttr(o, s_y)), oA(PyObject_GetAttr(o, s_A)), oB(PyObject_GetAttr(o, s_B)),
+            osc(PyObject_GetAttr(o, s_scale));
+        const at::Tensor &x = tensor(ox.p, "x"), &y = tensor(oy.p, "y"), &A = tensor(oA.p, "A"), &B = tensor(oB.p, "B");
+        const Matrix mx = matrix(x, "x"), my = matrix(y, "y");
+        const auto st = x.scalar_type();
+        if (my.rows != mx.rows || y.scalar_type() != st || A.scalar_type() != st || B.scalar_type() != st)
+            raise(PyExc_ValueError, "x, y, A, B must share the token count and the element type");
+        if (A.dim() < 3) raise(PyExc_IndexError, "A: expected 3 dimensions");
+        const int64_t c = A.size(0), rank = A.size(2);
+        if (!A.is_contiguous() || !B.is_contiguous() || A.size(1) != mx.cols || B.dim() != 3 || B.size(0) != c || B.size(1) != rank ||
+            B.size(2) != my.cols)
+            raise(PyExc_ValueError, "A / B shapes do not match x / y");
+        const molora_dtype_t code = dtype_code(x);
+        if (first) {
+            N = mx.rows;
+            C = c;
+            dt = code;
+        } else if (N != mx.rows || C != c || dt != code) {
+            raise(PyExc_ValueError, "all projections of a batched apply share N, C and the element type");
+        }
+        out.row_scale = nullptr;
+        PyObject* rs = PyObject_GetAttr(o, s_row_scale);
+        if (rs == nullptr) {
+            if (!PyErr_ExceptionMatches(PyExc_AttributeError)) throw PyRaised{};
+            PyErr_Clear();
+        } else {
+            Ref hold(rs);
+            if (rs != Py_None) {
+                const at::Tensor& t = tensor(rs, "row_scale");
+                if (t.scalar_type() != at::kFloat || t.numel() != mx.rows || !t.is_contiguous())
+                    raise(PyExc_ValueError, "row_scale must be a dense fp32 tensor with one factor per token");
+                out.row_scale = static_cast<const float*>(t.data_ptr());
+            }
+        }
+        const double scale = PyFloat_AsDouble(osc.p);
+        if (scale == -1.0 && PyErr_Occurred()) throw PyRaised{};
+        out.x = x.data_ptr();
+        out.ldx = mx.pitch;
+        out.y = y.data_ptr();
+        out.ldy = my.pitch;
+        out.A = A.data_ptr();
+        out.B = B.data_ptr();
+        out.d_in = (int32_t)mx.cols;
+        out.d_out = (int32_t)my.cols;
+        out.rank = (int32_t)rank;
+        out.scale = (float)scale;
+    }
+};
+
+int32_t* i32(const at::Tensor& t) { return static_cast<int32_t*>(t.data_ptr()); }
+float* f32(PyObject* o, const char* name) { return static_cast<float*>(ptr(o, name)); }
+uint32_t* status_word(PyObject* o) { return static_cast<uint32_t*>(ptr(o, "dev_status")); }
+
+// ---- (ids, breaks, r_out, dev_status, stream)
+PyObject* route_vocab(PyObject* const* a)
+{
+    const at::Tensor &ids = i32_dev(a[0], "ids"), &breaks = i32_dev(a[1], "breaks");
+    at::Tensor r = i32_out(a[2], "r_out", ids.numel(), ids.device());
+    check("molora_route_vocab", molora_route_vocab(i32(ids), ids.numel(), i32(breaks), (int32_t)breaks.numel() - 1, i32(r),
+                                                   status_word(a[3]), stream_of(a[4])));
+    return wrap(r);
+}
+
+// ---- (ids, adapter, breaks, n_adapters, r_out, dev_status, stream)
+PyObject* route_composite(PyObject* const* a)
+{
+    const at::Tensor &ids = i32_dev(a[0], "ids"), &adapter = i32_dev(a[1], "adapter"), &breaks = i32_dev(a[2], "breaks");
+    if (adapter.numel() != ids.numel()) raise(PyExc_ValueError, "adapter must hold one index per token");
+    Ref n(PyNumber_Long(a[3]));
+    at::Tensor r = i32_out(a[4], "r_out", ids.numel(), ids.device());
+    check("molora_route_composite",
+          molora_route_composite(i32(ids), i32(adapter), ids.numel(), i32(breaks), (int32_t)breaks.numel() - 1, (int32_t)integer(n.p), i32(r),
+                                 status_word(a[5]), stream_of(a[6])));
+    return wrap(r);
+}
+
+// ---- (x, G, bias, r_out, logits_out, ws, dev_status, stream, prepared)
+PyObject* route_gate(PyObject* const* a)
+{
+    const at::Tensor &x = tensor(a[0], "x"), &G = tensor(a[1], "G");
+    const Matrix m = matrix(x, "x");
+    if (G.scalar_type() != at::kFloat || !G.is_cuda() || !G.is_contiguous() || G.dim() != 2 || G.size(0) != m.cols)
+        raise(PyExc_ValueError, "G: expected a contiguous fp32 CUDA tensor of shape [d, C]");
+    const int32_t C = (int32_t)G.size(1), d = (int32_t)m.cols;
+    if (a[2] != Py_None) {
+        const at::Tensor& b = tensor(a[2], "bias");
+        if (b.scalar_type() != at::kFloat || b.numel() != C || !b.is_contiguous())
+            raise(PyExc_ValueError, "bias: expected contiguous fp32 [C]");
+    }
+    if (a[4] != Py_None) {
+        const at::Tensor& z = tensor(a[4], "logits_out");
+        if (z.scalar_type() != at::kFloat || z.dim() != 2 || z.size(0) != m.rows || z.size(1) != C || !z.is_contiguous())
+            raise(PyExc_ValueError, "logits_out: expected contiguous fp32 [N, C]");
+    }
+    const molora_dtype_t dt = dtype_code(x);
+    at::Tensor r = i32_out(a[3], "r_out", m.rows, x.device());
+    const float *g = f32(a[1], "G"), *bias = f32(a[2], "bias");
+    float* logits = f32(a[4], "logits_out");
+    if (a[8] != Py_None) {
+        const at::Tensor& prepared = tensor(a[8], "prepared");
+        check("molora_route_gate_prepared",
+              molora_route_gate_prepared(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, i32(r), logits, prepared.data_ptr(),
+                                         (size_t)prepared.numel(), status_word(a[6]), stream_of(a[7])));
+        return wrap(r);
+    }
+    // (the weight images are written before they are read: the scratch need not be cleared)
+    const Workspace ws(a[5], molora_route_gate_workspace_bytes(dt, d, C), x.device(), false);
+    check("molora_route_gate", molora_route_gate(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, i32(r), logits, ws.p, ws.n,
+                                                 status_word(a[6]), stream_of(a[7])));
+    return wrap(r);
+}
+
+// ---- (x, W1, b1, W2, b2, r_out, logits_out, ws, dev_status, stream, prepared)
+PyObject* route_mlp(PyObject* const* a)
+{
+    const at::Tensor &x = tensor(a[0], "x"), &W1 = tensor(a[1], "W1"), &W2 = tensor(a[3], "W2");
+    const Matrix m = matrix(x, "x");
+    if (W1.scalar_type() != at::kFloat || W2.scalar_type() != at::kFloat || !W1.is_contiguous() || !W2.is_contiguous())
+        raise(PyExc_ValueError, "W1 [d, H] and W2 [H, C] must be dense fp32 tensors");
+    if (W2.dim() != 2) raise(PyExc_ValueError, "W2 must be [H, C]");
+    const int32_t H = (int32_t)W2.size(0), C = (int32_t)W2.size(1), d = (int32_t)m.cols;
+    if (W1.dim() != 2 || W1.size(0) != d || W1.size(1) != H) raise(PyExc_ValueError, "W1 must be [d, H]");
+    const molora_dtype_t dt = dtype_code(x);
+    at::Tensor r = i32_out(a[5], "r_out", m.rows, x.device());
+    const float *w1 = f32(a[1], "W1"), *b1 = f32(a[2], "b1"), *w2 = f32(a[3], "W2"), *b2 = f32(a[4], "b2");
+    float* logits = f32(a[6], "logits_out");
+    if (a[10] != Py_None) {
+        const at::Tensor& prepared = tensor(a[10], "prepared");
+        check("molora_route_mlp_prepared",
+              molora_route_mlp_prepared(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, i32(r), logits, prepared.data_ptr(),
+                                        (size_t)prepared.numel(), status_word(a[8]), stream_of(a[9])));
+        return wrap(r);
+    }
+    const Workspace ws(a[7], molora_route_mlp_workspace_bytes(dt, d, H, C), x.device(), false);
+    check("molora_route_mlp", molora_route_mlp(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, i32(r), logits, ws.p, ws.n,
+                                               status_word(a[8]), stream_of(a[9])));
+    return wrap(r);
+}
+
+PyObject* tuple_of(std::initializer_list<at::Tensor> ts)
+{
+    PyObject* t = PyTuple_New((Py_ssize_t)ts.size());
+    if (t == nullptr) throw PyRaised{};
+    Py_ssize_t i = 0;
+    for (const at::Tensor& x : ts) {
+        PyObject* o = THPVariable_Wrap(x);
+        if (o == nullptr) {
+            Py_DECREF(t);
+            throw PyRaised{};
+        }
+        PyTuple_SET_ITEM(t, i++, o);
+    }
+    return t;
+}
+
+// ---- (r, C, counts, offsets, perm, ws, dev_status, stream)
+PyObject* group(PyObject* const* a)
+{
+    const at::Tensor& r = i32_dev(a[0], "r");
+    const int64_t N = r.numel(), C = integer(a[1]);
+    const at::Device dev = r.device();
+    at::Tensor counts = i32_out(a[2], "counts", C, dev), offsets = i32_out(a[3], "offsets", C + 1, dev),
+               perm = i32_out(a[4], "perm", std::max<int64_t>(N, 1), dev);
+    const Workspace ws(a[5], molora_group_workspace_bytes(N, (int32_t)C), dev, true);
+    check("molora_group", molora_group(i32(r), N, (int32_t)C, i32(counts), i32(offsets), i32(perm), ws.p, ws.n, status_word(a[6]),
+                                       stream_of(a[7])));
+    return tuple_of({counts, offsets, perm});
+}
+
+// ---- (projs, offsets, perm, ws, dev_status, stream, packed)
+PyObject* apply_batched(PyObject* const* a)
+{
+    const Projs pr(a[0], a[6]);
+    const at::Tensor &offsets = tensor(a[1], "offsets"), &perm = tensor(a[2], "perm");
+    const Workspace ws(a[3], a[3] == Py_None ? pr.apply_bytes() : 0, offsets.device(), true);
+    check("molora_apply_batched", molora_apply_batched(pr.d, pr.P, pr.dt, pr.N, (int32_t)pr.C, i32(offsets), i32(perm), ws.p, ws.n,
+                                                       status_word(a[4]), stream_of(a[5])));
+    Py_RETURN_NONE;
+}
+
+// ---- (r, projs, C, counts, offsets, perm, ws, dev_status, stream, packed)
+PyObject* group_apply_batched(PyObject* const* a)
+{
+    const at::Tensor& r = i32_dev(a[0], "r");
+    const Projs pr(a[1], a[9]);
+    const int64_t C = a[2] == Py_None ? pr.C : integer(a[2]);
+    if (r.numel() != pr.N || C != pr.C) raise(PyExc_ValueError, "r must hold one routing decision per token of the projections");
+    const at::Device dev = r.device();
+    at::Tensor counts = i32_out(a[3], "counts", C, dev), offsets = i32_out(a[4], "offsets", C + 1, dev),
+               perm = i32_out(a[5], "perm", std::max<int64_t>(pr.N, 1), dev);
+    const Workspace ws(a[6], a[6] == Py_None ? pr.apply_bytes() : 0, dev, true);
+    check("molora_group_apply_batched",
+          molora_group_apply_batched(i32(r), pr.N, (int32_t)C, i32(counts), i32(offsets), i32(perm), pr.d, pr.P, pr.dt, ws.p, ws.n,
+                                     status_word(a[7]), stream_of(a[8])));
+    return tuple_of({counts, offsets, perm});
+}
+
+// ---- (logits, k, stream)
+PyObject* topk_softmax(PyObject* const* a)
+{
+    const at::Tensor& z = tensor(a[0], "logits");
+    if (z.scalar_type() != at::kFloat || z.dim() != 2 || !z.is_contiguous()) raise(PyExc_ValueError, "logits must be a dense fp32 [N, C] tensor");
+    Ref kk(PyNumber_Long(a[1]));
+    const int64_t k = integer(kk.p), N = z.size(0);
+    at::Tensor idx = at::empty({k, N}, at::TensorOptions().dtype(at::kInt).device(z.device())),
+               w = at::empty({k, N}, at::TensorOptions().dtype(at::kFloat).device(z.device()));
+    check("molora_topk_softmax", molora_topk_softmax(static_cast<const float*>(z.data_ptr()), N, (int32_t)z.size(1), (int32_t)k, i32(idx),
+                                                     static_cast<float*>(w.data_ptr()), stream_of(a[2])));
+    return tuple_of({idx, w});
+}
+
+// ---- (projs, idx, w, C, ws, dev_status, stream)
+PyObject* apply_topk(PyObject* const* a)
+{
+    const Projs pr(a[0], Py_None);
+    const at::Tensor &idx0 = tensor(a[1], "idx"), &w0 = tensor(a[2], "w");
+    const int64_t C = integer(a[3]);
+    if (pr.C != C || idx0.scalar_type() != at::kInt || w0.scalar_type() != at::kFloat || idx0.dim() != 2 || idx0.sizes() != w0.sizes() ||
+        idx0.size(1) != pr.N)
+        raise(PyExc_ValueError, "idx int32 [k, N] and w fp32 [k, N] must match the projections");
+    const at::Tensor idx = idx0.contiguous(), w = w0.contiguous();
+    // only the apply part of the scratch has to start cleared, and only where a kernel keeps control words in it
+    const Workspace ws(a[4], a[4] == Py_None ? molora_apply_topk_workspace_bytes(pr.d, pr.P, pr.N, (int32_t)C) + 256 : 0, idx.device(),
+                       a[4] == Py_None && pr.apply_bytes() > 0);
+    const size_t off = (size_t)(-(intptr_t)ws.p) % 256;
+    check("molora_apply_topk",
+          molora_apply_topk(pr.d, pr.P, pr.dt, pr.N, (int32_t)C, (int32_t)idx.size(0), i32(idx), static_cast<const float*>(w.data_ptr()),
+                            static_cast<char*>(ws.p) + off, ws.n - off, status_word(a[5]), stream_of(a[6])));
+    Py_RETURN_NONE;
+}
+
+// ---- (raise_status)
+PyObject* bind(PyObject* const* a)
+{
+    Py_INCREF(a[0]);
+    Py_XDECREF(g_raise_status);
+    g_raise_status = a[0];
+    Py_RETURN_NONE;
+}
+
+// fixed number of positional arguments; C++ exceptions end here
+template <PyObject* (*F)(PyObject* const*), int ARGS>
+PyObject* entry(PyObject*, PyObject* const* args, Py_ssize_t n)
+{
+    if (n != ARGS) {
+        PyErr_Format(PyExc_TypeError, "expected %d arguments, got %zd", ARGS, n);
+        return nullptr;
+    }
+    try {
+        return F(args);
+    } catch (const PyRaised&) {
+    } catch (const std::exception& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+    } catch (...) {
+        PyErr_SetString(PyExc_RuntimeError, "unknown C++ exception");
+    }
+    return nullptr;
+}
+
+#define ENTRY(name, n) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(entry<name, n>)), METH_FASTCALL, nullptr}
+PyMethodDef methods[] = {ENTRY(route_vocab, 5), ENTRY(route_composite, 7), ENTRY(route_gate, 9), ENTRY(route_mlp, 11), ENTRY(group, 8),
+                         ENTRY(apply_batched, 7), ENTRY(group_apply_batched, 10), ENTRY(topk_softmax, 3), ENTRY(apply_topk, 7), ENTRY(bind, 1),
+                         {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__marshal()
+{
+    s_x = PyUnicode_InternFromString("x");
+    s_y = PyUnicode_InternFromString("y");
+    s_A = PyUnicode_InternFromString("A");
+    s_B = PyUnicode_InternFromString("B");
+    s_scale = PyUnicode_InternFromString("scale");
+    s_row_scale = PyUnicode_InternFromString("row_scale");
+    s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
+    return PyModule_Create(&module);
+}
