@@ -49,38 +49,45 @@ namespace {
 
 // ---- path selection (bf16, ranks 16 / 32 / 64; everything else runs on the CUDA-core row-tile kernel)
 // Three kernels cover the bf16 calls: the tcgen05 kernel (128-row tiles, clusters), the single-launch streaming
-// kernel (32-row tiles, one CTA per item) and the two-launch small-tile kernels.  Measured on B200 (2048- and
-// 4096-wide projections, 4-128 adapters, 1-7 projections per call):
-//   rank 16  streaming wins until the projections of the call move ~150 MB (x once, y twice), tcgen05 above;
-//   rank 32  streaming until ~60 MB, tcgen05 above (below 1024 tokens the two-launch pair ties for one projection
-//            and loses by a third for a layer's worth of them);
-//   rank 64  tcgen05 (tiles split over clusters of up to 8 CTAs) once the projections of the call move ~12 MB with at
-//            least 256 tokens and segments of 32 rows on average (one 4096-wide projection: from 512 tokens, 21.0 us
-//            against 24.3; two: 23.2 against 38.9 at 512 tokens; a layer of seven: 89.7 against 134.9), and from 1280
-//            tokens in any case; below, the two-launch pair for one or two projections and the streaming kernel for
-//            more (the streaming kernel has only two stages at this rank).
+// kernel (16- and 32-row tiles, clusters) and the two-launch small-tile kernels.  The tcgen05 kernel is at its best with full
+// tiles, i.e. many tokens per adapter.  Measured on B200 (us, tcgen05 / streaming; layers of seven 2048-wide projections
+// unless said otherwise):
+//   rank 16  only calls of one projection that move 150 MB (x once, y twice) with 128 tokens per adapter: 4096-wide, 8000
+//            tokens, 4 adapters 43.6 / 47.2, 16 adapters 46.8 / 48.1.  Two projections, 16384 tokens 127 / 119; layers: 1500
+//            tokens, 8 adapters 47.6 / 44.8, 16 adapters 60.6 / 46.4; 4000 tokens, 4 adapters 91.8 / 86.5; 8192, 16: 180 / 172
+//   rank 32  from 60 MB with 128 tokens per adapter: 1500 tokens, 8 adapters 48.9 / 55.1, 3000 tokens, 16 adapters 85.5 /
+//            90.0; below: 1500 tokens, 16 adapters 63.1 / 57.3, the attention projections at 1900 tokens 35.2 / 25.7
+//   rank 64  one or two projections (the two-launch pair below): once they move ~12 MB with at least 256 tokens and segments
+//            of 32 rows on average (one 4096-wide projection: from 512 tokens, 21.0 against 24.3; two: 23.2 against 38.9 at
+//            512 tokens).  More: from 576 tokens with 64 per adapter: 650 tokens, 8 adapters 44.7 / 51.3, 512: 44.0 / 41.6,
+//            260: 39.2 / 29.3; 777 tokens, 16 adapters 65.2 / 61.4.  From 1280 tokens in any case (1250 tokens, 16 adapters
+//            67 / 88), unless more than 64 adapters share fewer than 64 tokens each.
+//   more than 64 adapters   four projections, 3001 tokens, 256 adapters: rank 32 271 (both kernels, each its segments) / 59,
+//            rank 64 304 / 88
 // The overrides "umma_min_tokens" (tcgen05 from n tokens) and "small_path" (the kernel used below it) of
 // molora_debug_set force a choice, for measurements and for tests that target one kernel.
 int64_t forced_umma_min_tokens() { return std::max<int64_t>(0, tune(kTuneUmmaMinTokens)); }
 constexpr double kUmmaMinBytesR16 = 150e6, kUmmaMinBytesR32 = 60e6;
-constexpr int64_t kUmmaMinTokensR64 = 1280, kUmmaMinTokensR64Wide = 256;
+constexpr int64_t kUmmaMinTokensR64 = 1280, kUmmaMinTokensR64Wide = 256, kUmmaMinTokensR64Layer = 576;
 constexpr double kUmmaMinBytesR64 = 12e6;
 
 double proj_bytes(int64_t N, int32_t d_in, int32_t d_out) { return (double)N * ((double)d_in + 2.0 * d_out) * 2.0; }
 
-// group_bytes: bytes moved by all projections of this rank in the call
-// rank 64: group_bytes may be a lower bound (one projection's own bytes when the others are not known)
-bool use_umma_r64(int64_t N, int32_t C, double group_bytes)
+// group_bytes: bytes moved by all projections of this rank in the call, same_rank: how many they are
+// rank 64: group_bytes may be a lower bound and same_rank 1 (one projection when the others are not known)
+bool use_umma_r64(int64_t N, int32_t C, double group_bytes, int same_rank)
 {
+    if (C > kUmmaAllSegmentsMaxC && N < (int64_t)C * 64) return false;
     if (N >= kUmmaMinTokensR64) return true;
+    if (same_rank > 2) return N >= kUmmaMinTokensR64Layer && N >= (int64_t)C * 64;
     return N >= kUmmaMinTokensR64Wide && N >= (int64_t)C * kUmmaMinRows && group_bytes >= kUmmaMinBytesR64;
 }
-bool use_umma(int32_t rank, int64_t N, int32_t C, double group_bytes)
+bool use_umma(int32_t rank, int64_t N, int32_t C, double group_bytes, int same_rank)
 {
     if (const int64_t forced = forced_umma_min_tokens()) return N >= forced;
-    if (rank == 64) return use_umma_r64(N, C, group_bytes);
-    if (N < kUmmaMinTokens) return false;
-    if (rank == 16) return group_bytes >= kUmmaMinBytesR16;
+    if (rank == 64) return use_umma_r64(N, C, group_bytes, same_rank);
+    if (N < kUmmaMinTokens || N < (int64_t)C * 128) return false;
+    if (rank == 16) return group_bytes >= kUmmaMinBytesR16 && same_rank == 1;
     return group_bytes >= kUmmaMinBytesR32;
 }
 // the kernel for what the tcgen05 kernel does not take; same_rank: projections of this rank in the call (0: unknown)
@@ -100,14 +107,15 @@ bool small_path_is_stream(int32_t rank, int64_t N, int same_rank)
 // Its jobs cost more than the streaming kernel's chunks (a partial exchange through L2 per shrink chunk), so it only pays
 // where the streaming kernel's longest items dominate: measured on B200 (seven 2048 / 6144-wide rank-16 projections,
 // 8 adapters, graph replay, us, streaming / job list): 32 tokens 10.4 / 11.7, 128: 12.0 / 13.9, 256: 14.9 / 16.6,
-// 512: 26.4 / 21.7, 1024: 36.3 / 34.1; one projection, ranks 32 and 64: the streaming or the two-launch kernels win at
-// every size.  Hence: rank 16, at least four projections of that rank in the call, more than 256 and at most 1024 tokens.
+// 300: 18.8 / 15.9, 512: 20.4 / 19.8, 777: 25.7 / 25.7, 1000: 30.3 / 31.4; one projection, ranks 32 and 64: the streaming or
+// the two-launch kernels win at every size.  Hence: rank 16, at least four projections of that rank in the call, more than
+// 256 and fewer than 1024 tokens.
 bool use_jobs(const molora_proj_desc_t& p, molora_dtype_t dt, int64_t N, int32_t C, int same_rank)
 {
     (void)C;
     if (!jobs_eligible(p, dt, N)) return false;
     if (const int64_t forced = tune(kTuneSmallPath)) return forced == 3;
-    return p.rank == 16 && same_rank >= 4 && N > 256;
+    return p.rank == 16 && same_rank >= 4 && N > 256 && N < kUmmaMinTokens;
 }
 
 bool rank_supported(int r) { return r == 8 || r == 16 || r == 32 || r == 64; }
@@ -313,7 +321,7 @@ size_t molora_apply_workspace_bytes(int64_t N, int32_t C, int32_t d_in, int32_t 
     // two-launch kernels: needed unless the tcgen05 kernel is certain to take every segment (for ranks 16 and 32 that
     // depends on the other projections of the call, which are not known here)
     const int64_t forced = forced_umma_min_tokens();
-    const bool umma_certain = forced > 0 ? N >= forced : (rank == 64 && use_umma_r64(N, C, proj_bytes(N, d_in, d_out)));
+    const bool umma_certain = forced > 0 ? N >= forced : (rank == 64 && use_umma_r64(N, C, proj_bytes(N, d_in, d_out), 1));
     if (umma_certain && C <= kUmmaAllSegmentsMaxC && (d_in % 64) == 0 && (d_out % 64) == 0) return need;
     return need + decode_workspace_bytes(N, d_in, rank);
 }
@@ -357,7 +365,7 @@ molora_status_t plan_apply(const molora_proj_desc_t* projs, int32_t P, molora_dt
         if (decode_eligible(projs[i], dt)) ++same_rank[group_of(projs[i].rank)];
     for (int i = 0; i < P; ++i) {
         const int32_t rank = projs[i].rank;
-        if (umma_eligible(projs[i], dt) && use_umma(rank, N, C, group_bytes[group_of(rank)])) pl.tc[pl.n_tc++] = projs[i];
+        if (umma_eligible(projs[i], dt) && use_umma(rank, N, C, group_bytes[group_of(rank)], same_rank[group_of(rank)])) pl.tc[pl.n_tc++] = projs[i];
         else if (use_jobs(projs[i], dt, N, C, same_rank[group_of(rank)])) pl.jc[group_of(rank)][pl.n_jc[group_of(rank)]++] = projs[i];
         else if (decode_eligible(projs[i], dt)) {
             if (small_path_is_stream(rank, N, same_rank[group_of(rank)])) pl.sc[pl.n_sc++] = projs[i];
@@ -448,7 +456,7 @@ static int group_apply_mode(const molora_proj_desc_t* projs, int32_t P, molora_d
         umma = umma && umma_eligible(projs[i], dt);
         if (umma_eligible(projs[i], dt)) bytes += proj_bytes(N, projs[i].d_in, projs[i].d_out);
     }
-    if (use_umma(projs[0].rank, N, C, bytes)) return umma && group_apply_umma_eligible(N, C) ? 4 : 0;
+    if (use_umma(projs[0].rank, N, C, bytes, P)) return umma && group_apply_umma_eligible(N, C) ? 4 : 0;
     if (jobs) return 3;
     if (stream && group_apply_stream_eligible(N)) return 1;
     if (twophase && group_apply_decode_eligible(N)) return 2;
@@ -591,11 +599,19 @@ int topk_single_pass(const molora_proj_desc_t* projs, int32_t P, molora_dtype_t 
         umma_ok = umma_ok && umma_eligible(projs[i], dt);
         bytes += proj_bytes(N, projs[i].d_in, projs[i].d_out);
     }
-    // (with many sets every 128-row tile is a partial one: 64 sets at 8192 tokens lost to two passes, 113 against 106 us)
-    if (umma_ok && (sets <= 16 || N >= sets * 256) && use_umma(projs[0].rank * k, N, (int32_t)sets, bytes)) return 2;
+    // The tcgen05 kernel's 128-row tiles want full sets: with many sets for the tokens every tile is a partial one, and the
+    // streaming kernel's 16- and 32-row tiles are faster even for calls that would take the tcgen05 kernel pass by pass.
+    // Measured (us, two passes / one on tcgen05 / one on the streaming kernel), a layer of 2048, k = 2, 36 sets:
+    // rank 16, 2048 tokens 115 / 106 / 78, 4000 tokens 189 / 168 / 123; 10 sets, 2048 tokens - / 67 / 74; stacked rank
+    // 64 (rank 32), whose streaming chunks are half as wide: 2048 tokens 121 / 112 / 140, but one projection 25 streaming, 33
+    // tcgen05.  Beyond 8192 tokens the two passes are kept (not measured).
+    const int stacked = projs[0].rank * k;
+    const bool dense_sets = sets <= 16 || N >= sets * 256;
+    if (umma_ok && (dense_sets || (stacked == 64 && bytes >= 100e6)) && use_umma(stacked, N, (int32_t)sets, bytes, P)) return 2;
     const int64_t small = tune(kTuneSmallPath);
     if (small != 0 && small != 1) return 0;                         // a test or a measurement asks for another kernel
-    return use_umma(projs[0].rank, N, C, bytes) ? 0 : 1;
+    if (stacked <= 32 && N <= 8192 && forced_umma_min_tokens() == 0) return 1;
+    return use_umma(projs[0].rank, N, C, bytes, P) ? 0 : 1;
 }
 }  // namespace
 
