@@ -240,10 +240,12 @@ size_t route_gate_prepared_workspace_bytes(molora_dtype_t xdt, int32_t d, int32_
 // Tensor-core (mma.sync) gate for bf16 activations; the CUDA-core kernel above serves fp32 activations.
 // Needs route_gate_mma_workspace_bytes(d, C) bytes of scratch for the split gate weights.
 size_t route_gate_mma_workspace_bytes(int32_t d, int32_t C);
+// calls that its small-call kernel (16 tokens per cluster) takes, also where the tcgen05 gate could
+bool gate_split_preferred(int64_t N, int32_t d, int32_t C);
 molora_status_t launch_route_gate_mma(const void* x, int64_t N, int32_t d, int64_t ldx, const float* G,
                                       const float* bias, int32_t C, int32_t* r_out, float* logits_out, void* ws,
                                       cudaStream_t s, int image = kImageBuildAndUse);
-// The paper's MLP router (Eq. 9).  The tensor-core path (bf16 x, d a multiple of 64, at least 128 tokens) needs
+// The paper's MLP router (Eq. 9).  The tensor-core path (bf16 x, d a multiple of 64; optional below 128 tokens) needs
 // route_mlp_workspace_bytes(...) bytes for the split first-layer weights.
 size_t route_mlp_workspace_bytes(molora_dtype_t xdt, int32_t d, int32_t H);
 molora_status_t launch_route_mlp(const void* x, molora_dtype_t xdt, int64_t N, int32_t d, int64_t ldx, const float* W1,

@@ -617,7 +617,7 @@ molora_status_t launch_route_gate(const void* x, molora_dtype_t xdt, int64_t N, 
         return launch_route_gate_mma(nullptr, 0, d, 0, G, nullptr, C, nullptr, nullptr, ws_mma, s, image);
     }
     if (N == 0) return MOLORA_OK;
-    if (xdt == MOLORA_BF16 && gate_umma_eligible(N, d, C))       // the only gate kernel with device-side waits
+    if (xdt == MOLORA_BF16 && gate_umma_eligible(N, d, C) && !gate_split_preferred(N, d, C))       // the only gate kernel with device-side waits
         return launch_route_gate_umma(x, N, d, ldx, G, bias, C, r_out, logits_out, ws, dev_status, s, image);
     if (xdt == MOLORA_BF16 && C > 4)
         return launch_route_gate_mma(x, N, d, ldx, G, bias, C, r_out, logits_out, ws_mma, s, image);

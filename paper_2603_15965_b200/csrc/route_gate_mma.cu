@@ -224,10 +224,11 @@ __global__ void __launch_bounds__(WARPS * 32) route_gate_mma_kernel(const __nv_b
 // more): all operands go from global memory straight into registers in one round trip, the partial logits are summed in
 // warp order in shared memory and in rank order through distributed shared memory.  Bound by one load round trip and the
 // launch.  Measured (us, before -> after): 93 tokens x 4096, C = 16: 34.4 -> 5.7; 777 x 2048, C = 8: 12.0 -> 4.7.
-// Every 16 tokens read the whole weight image (L2), so calls of more than 1023 tokens, which fill the SMs with 64 tokens
-// per CTA (or run on the tcgen05 gate), keep the kernel above.
+// Every 16 tokens read the whole weight image (L2), so large calls keep the tcgen05 gate or the kernel above; the line lies
+// where they meet (us, tcgen05 / here, image built before): 8 adapters 1500 x 2048 8.0 / 4.9, 2300 x 2048 8.4 / 5.1, 4000 x
+// 2048 8.8 / 9.5, 1500 x 4096 10.5 / 9.7, 2300 x 4096 10.8 / 12.5; 16 adapters 2300 x 2048 8.8 / 6.7, 1500 x 4096 10.9 /
+// 12.1; 32 adapters 1500 x 2048 11.9 / 13.5.
 constexpr int kGateSplitWarps = 8;
-constexpr int64_t kGateSplitMaxTokens = 1024;
 template <int NT, int KC>
 __global__ void __launch_bounds__(kGateSplitWarps * 32, 2)
     route_gate_split_kernel(const __nv_bfloat16* __restrict__ x, int64_t N, int d, int64_t ldx,
@@ -345,6 +346,12 @@ __global__ void __launch_bounds__(kGateSplitWarps * 32, 2)
     if (S > 1) ptx::cluster_sync_all();                              // rank 0 has read this CTA's sums
 }
 
+bool gate_split_preferred(int64_t N, int32_t d, int32_t C)
+{
+    if (N < 1024) return true;
+    return C <= 16 && N * d <= (C <= 8 ? 6500000 : 5000000);
+}
+
 template <int NT, int WARPS, int KC>
 static molora_status_t gate_mma_launch(const void* x, int64_t N, int d, int64_t ldx, const float* G, const float* bias,
                                        int C, int32_t* r_out, float* logits_out, void* ws, cudaStream_t s, int image)
@@ -360,7 +367,7 @@ static molora_status_t gate_mma_launch(const void* x, int64_t N, int d, int64_t 
             return MOLORA_ERR_CUDA;
     }
     if (image == kImageBuildOnly) return MOLORA_OK;
-    if (N < kGateSplitMaxTokens) {
+    if (gate_split_preferred(N, d, C)) {
         int S = 1;
         while (S < 8 && S * kGateSplitWarps < chunks) S *= 2;
         return cuda_ok(launch_kernel(route_gate_split_kernel<NT, KC>, dim3((unsigned)(ceil_div64(N, 16) * S)), dim3(kGateSplitWarps * 32), 0,

@@ -1,5 +1,5 @@
 // Linear gate with top-1 argmax (Eq. 8, k = 1) on the 5th-generation tensor cores, for bf16 activations,
-// more than four adapters and calls of at least 1024 tokens.
+// more than four adapters and calls of at least 1024 tokens that gate_split_preferred leaves to it.
 //
 // z = x G is a [N, d] x [d, C] product with a tiny C: its cost is streaming x once.  One CTA owns 128
 // consecutive tokens (rows of x are contiguous, so an x chunk [128, 64] is ONE 2-D TMA load into the

@@ -10,8 +10,9 @@
 // fp32 FMA chain.  The epilogue (one thread per token) walks the hidden units in slices of 16 TMEM columns: bias,
 // exact GELU 0.5 t (1 + erf(t / sqrt 2)), and the second layer as FMAs against W2 held in shared memory; then the
 // output bias and the argmax.  The hidden activations never leave the SM.  Calls with few tiles split the input
-// dimension of a tile over a cluster of 2 or 4 CTAs (see SPLIT below): measured on B200, graph replay, both launches,
-// 4096 tokens 2048 -> 64 -> 4: 25.8 -> 17.8 us; 2560 -> 128 -> 4: 47.6 -> 29.8 us; 256 tokens: 23.5 -> 16.0 us.
+// dimension of a tile over a cluster of 2, 4 or 8 CTAs (see SPLIT below): measured on B200, graph replay, both launches,
+// 4096 tokens 2048 -> 64 -> 4: 25.8 -> 17.8 us; 2560 -> 128 -> 4: 47.6 -> 29.8 us; 256 tokens: 23.5 -> 16.0 us.  Calls
+// below 128 tokens are one partial tile: 64 tokens x 2048 took 294 us on the CUDA cores (a warp walks d alone).
 //
 // Other inputs (fp32 activations, d not a multiple of 64, H not a multiple of 16) take a CUDA-core kernel: one warp
 // per token, lanes split d, HP partial pre-activations per lane, butterfly sums, GELU and the second layer in lanes.
@@ -56,7 +57,7 @@ struct MlpCtrl {
 __device__ __forceinline__ float gelu_exact(float t) { return 0.5f * t * (1.f + erff(t * 0.70710678118654752f)); }
 
 // HP: padded hidden width, 64 or 128.
-// SPLIT: the input dimension of a 128-token tile is split over a cluster of S = 2 or 4 CTAs (calls with so few tiles that
+// SPLIT: the input dimension of a 128-token tile is split over a cluster of S = 2, 4 or 8 CTAs (calls with so few tiles that
 // the chunks a CTA walks, ~0.7 us each, set the time).  Every CTA accumulates its slice of d, turns the three terms into
 // partial pre-activations (lo + mid) + hi, and sends the rows [128 o / S, 128 (o + 1) / S) to CTA o (asynchronous stores
 // that count their bytes on o's barrier; its own rows go into its own slot); CTA o sums the S partials in rank order and
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(128) route_mlp_simple_kernel(const T* __restri
 // ------------------------------------------------------------------------------------------------ host side
 static bool mlp_umma_eligible(molora_dtype_t xdt, int64_t N, int32_t d, int32_t H)
 {
-    return xdt == MOLORA_BF16 && (d % 64) == 0 && H >= 1 && H <= 128 && N >= 128;
+    return xdt == MOLORA_BF16 && (d % 64) == 0 && H >= 1 && H <= 128 && N >= 1;
 }
 
 size_t route_mlp_workspace_bytes(molora_dtype_t xdt, int32_t d, int32_t H)
@@ -392,7 +393,10 @@ static molora_status_t mlp_umma_launch(const void* x, int64_t N, int d, int64_t 
     // CTAs per 128-token tile (split along d) while the tiles alone leave most SMs idle; at least four chunks each
     const int64_t tiles = ceil_div64(N, 128);
     unsigned split = 1;
-    if (tiles * 4 <= 148 && d / 64 / 4 >= 4) split = 4;
+    // (1000 tokens x 4096: 16.4 us with four, 12.0 with eight; more clusters of eight than the GPCs hold at once run in two
+    // waves: 2300 tokens, 18 tiles, 14.1 us with four, 20.6 with eight)
+    if (tiles <= 14 && d / 64 / 8 >= 4) split = 8;
+    else if (tiles * 4 <= 148 && d / 64 / 4 >= 4) split = 4;
     else if (tiles * 2 <= 148 && d / 64 / 2 >= 4) split = 2;
     __nv_bfloat16* img = static_cast<__nv_bfloat16*>(ws);
     {
@@ -444,7 +448,9 @@ molora_status_t launch_route_mlp(const void* x, molora_dtype_t xdt, int64_t N, i
                                  float* logits_out, void* ws, size_t ws_bytes, uint32_t* dev_status, cudaStream_t s, int image)
 {
     if (N == 0 && image != kImageBuildOnly) return MOLORA_OK;
-    if (mlp_umma_eligible(xdt, image == kImageBuildOnly ? 128 : N, d, H)) {
+    const bool room = ws != nullptr && ws_bytes >= route_mlp_workspace_bytes(xdt, d, H) && aligned16(ws);
+    // (below 128 tokens the images are optional: without room for them the call runs on the CUDA cores)
+    if (mlp_umma_eligible(xdt, image == kImageBuildOnly ? 128 : N, d, H) && (room || image == kImageBuildOnly || N >= 128)) {
         if (ws == nullptr || ws_bytes < route_mlp_workspace_bytes(xdt, d, H) || !aligned16(ws)) return MOLORA_ERR_WORKSPACE;
         return H <= 64 ? mlp_umma_launch<64>(x, N, d, ldx, W1, b1, H, W2, b2, C, r_out, logits_out, ws, dev_status, s, image)
                        : mlp_umma_launch<128>(x, N, d, ldx, W1, b1, H, W2, b2, C, r_out, logits_out, ws, dev_status, s, image);

@@ -35,3 +35,32 @@ def test_small_call_gate_matches_oracle(N, d, C):
     # equal logits go to the lowest adapter
     flat = M.molora_route_gate(xd, torch.ones(d, C, device="cuda"))
     assert not flat.any()
+
+
+@pytest.mark.parametrize("N,d,C", [(1024, 2048, 8), (3173, 2048, 8), (3174, 2048, 8), (2441, 2048, 16), (2442, 2048, 16), (1500, 64, 17)])
+def test_both_sides_of_the_small_call_rule(N, d, C):
+    rng = np.random.default_rng(N + C)
+    x = W.round_to_bf16(rng.standard_normal((N, d), dtype=np.float32))
+    G = (rng.standard_normal((d, C)) * d ** -0.5).astype(np.float32)
+    z = torch.empty(N, C, dtype=torch.float32, device="cuda")
+    r = M.molora_route_gate(dev_tensor(x, "bf16"), dev_tensor(G, "f32"), logits_out=z)
+    r_ref, z_ref, margin = oracle.route_gate(x, G)
+    np.testing.assert_allclose(z.cpu().numpy(), z_ref, rtol=0, atol=4e-6 * max(1.0, np.abs(z_ref).max()))
+    assert np.array_equal(r.cpu().numpy()[margin >= 1e-3], r_ref[margin >= 1e-3])
+
+
+@pytest.mark.parametrize("N", [1, 63, 127, 128, 1000, 1792, 1793])
+@pytest.mark.parametrize("d,H", [(64, 64), (2048, 64), (4096, 128)])
+def test_mlp_router_of_small_calls(N, d, H):
+    C = 5
+    rng = np.random.default_rng(N + d)
+    x = W.round_to_bf16(rng.standard_normal((N, d), dtype=np.float32))
+    W1 = (rng.standard_normal((d, H)) * d ** -0.5).astype(np.float32)
+    W2 = (rng.standard_normal((H, C)) * H ** -0.5).astype(np.float32)
+    b1, b2 = (rng.standard_normal(H) * 0.1).astype(np.float32), (rng.standard_normal(C) * 0.1).astype(np.float32)
+    xd, W1d, b1d, W2d, b2d = (dev_tensor(v, "bf16" if v is x else "f32") for v in (x, W1, b1, W2, b2))
+    z = torch.empty(N, C, dtype=torch.float32, device="cuda")
+    r = M.molora_route_mlp(xd, W1d, b1d, W2d, b2d, logits_out=z)
+    r_ref, z_ref, margin = oracle.route_mlp(x, W1, b1, W2, b2)
+    np.testing.assert_allclose(z.cpu().numpy(), z_ref, rtol=0, atol=1e-5 * max(1.0, np.abs(z_ref).max()))
+    assert np.array_equal(r.cpu().numpy()[margin >= 1e-3], r_ref[margin >= 1e-3])
