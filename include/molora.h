@@ -74,7 +74,7 @@ const char *molora_status_string(molora_status_t status);
  * molora_debug_set: overrides one of the library's own choices, for measurements and for tests that target one
  *   kernel; value 0 restores the default.  Names: "umma_min_tokens" (tcgen05 apply from that many tokens),
  *   "small_path" (kernel below it: 1 streaming, 2 two-launch, 3 job-list decode kernel), "stream_tile" (16 | 32),
- *   "umma_split", "umma_tile_rows", "group_split" (cluster sizes / tile height), "chained_launch_off" (1: plain stream
+ *   "umma_split", "umma_tile_rows", "group_split", "stream_split" (cluster sizes / tile height), "chained_launch_off" (1: plain stream
  *   order), "jobs_launch" (job-list kernel: 0 cooperative, 1 plain, 2 programmatic launch).  The start values are read once from the environment variables MOLORA_<NAME>.  Unknown name:
  *   MOLORA_ERR_INVALID_ARG.  Not meant to be changed while calls are in flight on other threads. */
 uint64_t molora_launch_count(void);
@@ -232,7 +232,7 @@ molora_status_t molora_group(const int32_t *r, int64_t N, int32_t C, int32_t *co
  * dev_status      device uint32 or NULL; MOLORA_DEV_TIMEOUT is OR-ed in if a bounded wait inside a kernel gave
  *                 up (the kernel then returns without hanging; y is incomplete)
  * The kernel variant is chosen per call on the host from rank, token count and bytes (tcgen05 tiles of 128 rows
- * for large calls, a single-launch streaming kernel with 32-row tiles below that, a job-list kernel with 16-row
+ * for large calls, a single-launch streaming kernel with 16- and 32-row tiles below that, a job-list kernel with 16-row
  * tiles whose CTAs share chunk-sized shrink and expand jobs for decode-sized calls, CUDA cores for fp32 storage,
  * rank 8 and odd widths) and per segment on the device from the segment sizes; the paper picks its tile shape
  * from the histogram too (Eq. 12-13). */
