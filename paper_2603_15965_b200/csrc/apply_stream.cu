@@ -37,11 +37,11 @@
 // takes ~1 us on an SM, against 0.8 us at the rate of the copy bandwidth); layers of a few hundred tokens the uneven
 // numbers of chunk jobs per SM.  Measured with one CTA per item, linear weights and full-width rank-64 chunks (before) and
 // as it is (after), us per layer of seven projections, grouping included:
-//   rank 64, hidden 4096, 16 adapters, 20 / 93 / 250 tokens   84 / 91 / 92 -> 31 / 49 / 58
-//   rank 64, hidden 2048,  8 adapters,  8 / 60 tokens         42 / 49 -> 15.5 / 21
-//   rank 32, hidden 2048,  8 adapters,  8 / 256 / 777 tokens  21.7 / 25.8 / 43 -> 12.3 / 20.1 / 36
+//   rank 64, hidden 4096, 16 adapters, 20 / 93 / 250 tokens   84 / 91 / 92 -> 29 / 43 / 52
+//   rank 64, hidden 2048,  8 adapters,  8 / 60 tokens         42 / 49 -> 15.5 / 20.5
+//   rank 32, hidden 2048,  8 adapters,  8 / 256 / 777 tokens  21.7 / 25.8 / 43 -> 12.3 / 20.1 / 28
 //   rank 16, hidden 2048,  8 adapters,  8 / 256 tokens        11.0 / 14.8 -> 10.9 / 14.1;  hidden 4096, 256: 24.5 -> 22.5
-//   rank 16, four projections, 256 adapters, 3001 tokens      48.6 -> 38.2
+//   rank 16, four projections, 256 adapters, 3001 tokens      48.6 -> 37.0
 //
 // mma.sync is the legacy tensor path on sm_100a; a 32-row tile is far below the 128-row tcgen05 tile, and this path
 // is bound by the bytes it moves, not by its flops.  Every wait is bounded; after a time-out the CTA stops issuing
@@ -261,7 +261,13 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
     __syncthreads();
     const int T = tstart_s[prm.C];
     const int nitems = T * prm.ustart[prm.P];
-    const int mine = nitems > cid ? (nitems - cid + ncl - 1) / ncl : 0;       // items of my cluster: cid, cid + ncl, ...
+    // Items of my cluster: one of every ncl consecutive ones, from the front and from the back in turn.  Items are numbered
+    // heaviest projection first, so the clusters that took the heaviest of one round take the lightest of the next, or none.
+    // (Always from the front, the clusters with a gate or up projection also got the second item: 93 tokens of a wide rank-64
+    // layer 48.7 us, so 42.7; rank 32, 777 tokens 36.0 / 28.3; rank 16, 1500 tokens 44.6 / 39.3.)
+    auto item_of = [&](int i) { return i * ncl + ((i & 1) ? ncl - 1 - cid : cid); };
+    const int rounds = nitems / ncl;
+    const int mine = rounds + (item_of(rounds) < nitems ? 1 : 0);
     const uint32_t stage0 = smem_u32(dsm);
     if (S > 1) cluster_sync_all();             // every peer's barriers are initialised
 
@@ -370,7 +376,7 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
             cur = next;
             ctok = ntok;
             if (i + 1 < mine) {
-                next = fs_item(prm, offs_s, tstart_s, T, cid + (i + 1) * ncl, Cfg::CH, Cfg::ROWS);
+                next = fs_item(prm, offs_s, tstart_s, T, item_of(i + 1), Cfg::CH, Cfg::ROWS);
                 ntok = token_of(next);
                 issue_shrink(next, ntok);
                 if (abort_s) break;
@@ -644,7 +650,7 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
         for (int i = -1; i < mine; ++i) {
             cur = next;
             if (i + 1 < mine) {
-                next = fs_item(prm, offs_s, tstart_s, T, cid + (i + 1) * ncl, Cfg::CH, Cfg::ROWS);
+                next = fs_item(prm, offs_s, tstart_s, T, item_of(i + 1), Cfg::CH, Cfg::ROWS);
                 shrink(next, i + 1);
             }
             if (i >= 0) expand(cur, i);
