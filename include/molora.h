@@ -232,8 +232,7 @@ molora_status_t molora_group(const int32_t *r, int64_t N, int32_t C, int32_t *co
  * dev_status      device uint32 or NULL; MOLORA_DEV_TIMEOUT is OR-ed in if a bounded wait inside a kernel gave
  *                 up (the kernel then returns without hanging; y is incomplete)
  * The kernel variant is chosen per call on the host from rank, token count and bytes (tcgen05 tiles of 128 rows
- * for large calls, a single-launch streaming kernel with 16- and 32-row tiles below that, a job-list kernel with 16-row
- * tiles whose CTAs share chunk-sized shrink and expand jobs for decode-sized calls, CUDA cores for fp32 storage,
+ * for large calls with full segments, a single-launch streaming kernel with 16- and 32-row tiles otherwise, CUDA cores for fp32 storage,
  * rank 8 and odd widths) and per segment on the device from the segment sizes; the paper picks its tile shape
  * from the histogram too (Eq. 12-13). */
 size_t molora_apply_workspace_bytes(int64_t N, int32_t C, int32_t d_in, int32_t d_out, int32_t rank);

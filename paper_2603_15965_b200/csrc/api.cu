@@ -53,22 +53,23 @@ namespace {
 // tiles, i.e. many tokens per adapter.  Measured on B200 (us, tcgen05 / streaming; layers of seven 2048-wide projections
 // unless said otherwise):
 //   rank 16  only calls of one projection that move 150 MB (x once, y twice) with 128 tokens per adapter: 4096-wide, 8000
-//            tokens, 4 adapters 43.6 / 47.2, 16 adapters 46.8 / 48.1.  Two projections, 16384 tokens 127 / 119; layers: 1500
-//            tokens, 8 adapters 47.6 / 44.8, 16 adapters 60.6 / 46.4; 4000 tokens, 4 adapters 91.8 / 86.5; 8192, 16: 180 / 172
-//   rank 32  from 60 MB with 128 tokens per adapter: 1500 tokens, 8 adapters 48.9 / 55.1, 3000 tokens, 16 adapters 85.5 /
-//            90.0; below: 1500 tokens, 16 adapters 63.1 / 57.3, the attention projections at 1900 tokens 35.2 / 25.7
+//            tokens, 4 adapters 44.5 / 47.3.  Two projections, 16384 tokens 127 / 119; layers: 1500 tokens, 8 adapters 47.1 /
+//            38.5; 4000 tokens, 16 adapters 95.7 / 87.1; a 4096-wide layer, 8192 tokens, 16 adapters 329 / 312
+//   rank 32  with 160 tokens per adapter, one projection from 60 MB (8000 tokens, 98 MB, 26.8 / 30.9), more from 170 MB: 1050
+//            tokens, 8 adapters 39.4 / 36.5, 1500 48.9 / 49.0, 1990 57.1 / 64.1; two projections, 3000 tokens, 4 adapters
+//            (123 MB) 34.2 / 28.4, 16384 tokens 127 / 141
 //   rank 64  one or two projections (the two-launch pair below): once they move ~12 MB with at least 256 tokens and segments
 //            of 32 rows on average (one 4096-wide projection: from 512 tokens, 21.0 against 24.3; two: 23.2 against 38.9 at
-//            512 tokens).  More: from 576 tokens with 64 per adapter: 650 tokens, 8 adapters 44.7 / 51.3, 512: 44.0 / 41.6,
-//            260: 39.2 / 29.3; 777 tokens, 16 adapters 65.2 / 61.4.  From 1280 tokens in any case (1250 tokens, 16 adapters
-//            67 / 88), unless more than 64 adapters share fewer than 64 tokens each.
+//            512 tokens).  More: from 680 tokens with 60 per adapter: 600 tokens, 8 adapters 44.8 / 39.6, 777: 44.6 / 51.3;
+//            1000 tokens, 16 adapters 66.2 / 70.4.  From 1280 tokens in any case, unless more than 64 adapters share fewer
+//            than 64 tokens each.
 //   more than 64 adapters   four projections, 3001 tokens, 256 adapters: rank 32 271 (both kernels, each its segments) / 59,
 //            rank 64 304 / 88
 // The overrides "umma_min_tokens" (tcgen05 from n tokens) and "small_path" (the kernel used below it) of
 // molora_debug_set force a choice, for measurements and for tests that target one kernel.
 int64_t forced_umma_min_tokens() { return std::max<int64_t>(0, tune(kTuneUmmaMinTokens)); }
-constexpr double kUmmaMinBytesR16 = 150e6, kUmmaMinBytesR32 = 60e6;
-constexpr int64_t kUmmaMinTokensR64 = 1280, kUmmaMinTokensR64Wide = 256, kUmmaMinTokensR64Layer = 576;
+constexpr double kUmmaMinBytesR16 = 150e6, kUmmaMinBytesR32 = 60e6, kUmmaMinBytesR32More = 170e6;
+constexpr int64_t kUmmaMinTokensR64 = 1280, kUmmaMinTokensR64Wide = 256, kUmmaMinTokensR64Layer = 680;
 constexpr double kUmmaMinBytesR64 = 12e6;
 
 double proj_bytes(int64_t N, int32_t d_in, int32_t d_out) { return (double)N * ((double)d_in + 2.0 * d_out) * 2.0; }
@@ -79,16 +80,16 @@ bool use_umma_r64(int64_t N, int32_t C, double group_bytes, int same_rank)
 {
     if (C > kUmmaAllSegmentsMaxC && N < (int64_t)C * 64) return false;
     if (N >= kUmmaMinTokensR64) return true;
-    if (same_rank > 2) return N >= kUmmaMinTokensR64Layer && N >= (int64_t)C * 64;
+    if (same_rank > 2) return N >= kUmmaMinTokensR64Layer && N >= (int64_t)C * 60;
     return N >= kUmmaMinTokensR64Wide && N >= (int64_t)C * kUmmaMinRows && group_bytes >= kUmmaMinBytesR64;
 }
 bool use_umma(int32_t rank, int64_t N, int32_t C, double group_bytes, int same_rank)
 {
     if (const int64_t forced = forced_umma_min_tokens()) return N >= forced;
     if (rank == 64) return use_umma_r64(N, C, group_bytes, same_rank);
-    if (N < kUmmaMinTokens || N < (int64_t)C * 128) return false;
-    if (rank == 16) return group_bytes >= kUmmaMinBytesR16 && same_rank == 1;
-    return group_bytes >= kUmmaMinBytesR32;
+    if (N < kUmmaMinTokens) return false;
+    if (rank == 16) return group_bytes >= kUmmaMinBytesR16 && same_rank == 1 && N >= (int64_t)C * 128;
+    return group_bytes >= (same_rank == 1 ? kUmmaMinBytesR32 : kUmmaMinBytesR32More) && N >= (int64_t)C * 160;
 }
 // the kernel for what the tcgen05 kernel does not take; same_rank: projections of this rank in the call (0: unknown)
 bool small_path_is_stream(int32_t rank, int64_t N, int same_rank)
@@ -103,19 +104,16 @@ bool small_path_is_stream(int32_t rank, int64_t N, int same_rank)
     return rank == 16 || rank == 32 || same_rank > 2;
 }
 
-// The job-list kernel shares chunk-sized jobs between all CTAs instead of giving every (tile, projection) pair to one CTA.
-// Its jobs cost more than the streaming kernel's chunks (a partial exchange through L2 per shrink chunk), so it only pays
-// where the streaming kernel's longest items dominate: measured on B200 (seven 2048 / 6144-wide rank-16 projections,
-// 8 adapters, graph replay, us, streaming / job list): 32 tokens 10.4 / 11.7, 128: 12.0 / 13.9, 256: 14.9 / 16.6,
-// 300: 18.8 / 15.9, 512: 20.4 / 19.8, 777: 25.7 / 25.7, 1000: 30.3 / 31.4; one projection, ranks 32 and 64: the streaming or
-// the two-launch kernels win at every size.  Hence: rank 16, at least four projections of that rank in the call, more than
-// 256 and fewer than 1024 tokens.
+// The job-list kernel shares chunk-sized jobs between all CTAs instead of giving every (tile, projection) pair to one cluster.
+// Its jobs cost more than the streaming kernel's chunks (a partial exchange through L2 per shrink chunk), and since the
+// streaming kernel deals its items evenly it is the faster one at every size: seven 2048 / 6144-wide rank-16 projections, 8
+// adapters, us, streaming / job list: 256 tokens 14.0 / 15.3, 300: 14.4 / 15.7, 512: 17.5 / 19.6, 777: 22.7 / 25.7, 1000: 28.5 /
+// 31.9; rank 64, 4096 wide, 93 tokens 43 / 61.  It runs where "small_path" asks for it.
 bool use_jobs(const molora_proj_desc_t& p, molora_dtype_t dt, int64_t N, int32_t C, int same_rank)
 {
     (void)C;
-    if (!jobs_eligible(p, dt, N)) return false;
-    if (const int64_t forced = tune(kTuneSmallPath)) return forced == 3;
-    return p.rank == 16 && same_rank >= 4 && N > 256 && N < kUmmaMinTokens;
+    (void)same_rank;
+    return tune(kTuneSmallPath) == 3 && jobs_eligible(p, dt, N);
 }
 
 bool rank_supported(int r) { return r == 8 || r == 16 || r == 32 || r == 64; }
@@ -313,7 +311,7 @@ size_t molora_apply_workspace_bytes(int64_t N, int32_t C, int32_t d_in, int32_t 
     probe.d_out = d_out;
     probe.rank = rank;
     const int64_t small = tune(kTuneSmallPath);
-    // (by default the job-list kernel only takes rank 16 above 256 tokens, see use_jobs)
+    // (the size covers what the job-list kernel once took by default as well: callers keep it across calls)
     if (jobs_eligible(probe, MOLORA_BF16, N) && (small == 3 || (small == 0 && rank == 16 && N > 256)))
         need += jobs_control_bytes() + jobs_partial_bytes(N, C, d_in, rank);
     if (small == 3 && need > 0) return need;
