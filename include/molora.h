@@ -219,7 +219,7 @@ molora_status_t molora_group(const int32_t *r, int64_t N, int32_t C, int32_t *co
  * A   device [C, d_in, rank] of type dt, dense;  B  device [C, rank, d_out] of type dt, dense
  * offsets, perm   device outputs of molora_group for the same N, C (read on the device only)
  * ws, ws_bytes    device scratch of at least molora_apply_workspace_bytes(...) bytes, 16-byte aligned (NULL if
- *                 that is 0).  Two kernels use it.  The job-list kernel (bf16, at most 1024 tokens, few tiles per SM:
+ *                 that is 0).  Two kernels use it.  The job-list kernel (only where "small_path" asks for it; bf16, at most 1024 tokens:
  *                 decode-sized calls) keeps two control words and the fp32 partial shrink results there, the latter as
  *                 64-bit records {value, tag of the launch}: ALL of ws must be ZERO-FILLED before its first use (never
  *                 clear only a part of it later); after that the same ws can be passed to any number of calls, of any
