@@ -475,6 +475,10 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
                             *reinterpret_cast<float2*>(&tpart[(mt * 16 + g4) * R + c]) = make_float2(acc[mt][n][0], acc[mt][n][1]);
                             *reinterpret_cast<float2*>(&tpart[(mt * 16 + g4 + 8) * R + c]) = make_float2(acc[mt][n][2], acc[mt][n][3]);
                         }
+                    // My slot still feeds the copies of item i - 2 to the peers until every peer has read what arrived; no warp
+                    // writes to it before that (the barrier orders them behind warp 0's wait).
+                    if (S > 1 && warp == 0 && i >= 2)
+                        wait_bar_cluster(smem_u32(&tfree_s[i & 1]), (uint32_t)((i >> 1) - 1) & 1u, &abort_s, prm.dev_status);
                     fs_compute_sync();
                     float* out = slot_of(i, crank);
                     for (int e4 = tid; e4 < Cfg::TFLOATS / 4; e4 += kFsWarps * 32) {
@@ -492,8 +496,7 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
                     fence_proxy_async_smem();          // my writes are ordered before the copies that refill the stage or read the slot
                     fs_compute_sync();                 // the partial is complete; the stage is free
                     if (lane == 0) mbar_arrive(smem_u32(&done_s[s]));
-                    if (S > 1 && warp == 0) {          // push it to the peers, once they have read what the slot held before
-                        if (i >= 2) wait_bar_cluster(smem_u32(&tfree_s[i & 1]), (uint32_t)((i >> 1) - 1) & 1u, &abort_s, prm.dev_status);
+                    if (S > 1 && warp == 0) {          // push it to the peers, who have read what their slots held before (waited for above)
                         if (lane == 0) mbar_arrive_expect_tx(smem_u32(&tfull_s[i & 1]), (uint32_t)(S - 1) * Cfg::TFLOATS * 4u);
                         if (lane < S && lane != crank && !abort_s)
                             bulk_copy_to_peer(map_to_cta(smem_u32(out), lane), smem_u32(out), Cfg::TFLOATS * 4u,

@@ -56,3 +56,18 @@ def test_grouping_inside_and_many_items(N, C, rank, split):
     total = int(offsets[-1])
     assert torch.equal(got[0], counts) and torch.equal(got[1], offsets) and torch.equal(got[2][:total], perm[:total])
     assert torch.equal(ya, yb)
+
+
+@pytest.mark.parametrize("rank,split,d_in", [(32, 2, 1024), (32, 8, 4096), (64, 2, 512), (64, 4, 1024)])
+def test_many_items_of_one_chunk_a_cta(rank, split, d_in):
+    """The shortest items a cluster can have -- one shrink chunk a CTA and, for all but one CTA, no expand chunk -- and many of them,
+    so that a slot of the exchange is reused as early as it can be."""
+    force_stream(split, 16)
+    w = W.random_problem(rank + split, 4000, 7, d_in, 32, rank, "bf16")
+    run_and_check(w)
+    p = w.projections[0]
+    x, y, A, B = dev_tensor(w.inputs["x"], "bf16"), dev_tensor(p.y, "bf16"), dev_tensor(p.A, "bf16"), dev_tensor(p.B, "bf16")
+    _, offsets, perm = M.molora_group(dev_tensor(w.r, "i"), 7)
+    first = M.molora_apply(x, y.clone(), A, B, offsets, perm)
+    for _ in range(30):
+        assert torch.equal(M.molora_apply(x, y.clone(), A, B, offsets, perm), first)
