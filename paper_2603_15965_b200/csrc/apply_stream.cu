@@ -466,6 +466,11 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
                     // last chunk: sum the per-warp partials in warp order through this stage, then release it
                     float* tparts = reinterpret_cast<float*>(dsm + s * Cfg::STAGE);
                     float* tpart = tparts + kw * Cfg::TFLOATS + n0;
+                    // My slot still feeds the copies of item i - 2 to the peers until every peer has read what arrived; no warp
+                    // writes to it before that (the barriers order them behind warp 0's wait; waiting after the sums have been laid
+                    // out instead costs the layer of a wide rank-64 model at 93 tokens 48 us, not 41).
+                    if (S > 1 && warp == 0 && i >= 2)
+                        wait_bar_cluster(smem_u32(&tfree_s[i & 1]), (uint32_t)((i >> 1) - 1) & 1u, &abort_s, prm.dev_status);
                     fs_compute_sync();                 // every warp has finished reading the stage
 #pragma unroll
                     for (int mt = 0; mt < MT; ++mt)
@@ -475,10 +480,6 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
                             *reinterpret_cast<float2*>(&tpart[(mt * 16 + g4) * R + c]) = make_float2(acc[mt][n][0], acc[mt][n][1]);
                             *reinterpret_cast<float2*>(&tpart[(mt * 16 + g4 + 8) * R + c]) = make_float2(acc[mt][n][2], acc[mt][n][3]);
                         }
-                    // My slot still feeds the copies of item i - 2 to the peers until every peer has read what arrived; no warp
-                    // writes to it before that (the barrier orders them behind warp 0's wait).
-                    if (S > 1 && warp == 0 && i >= 2)
-                        wait_bar_cluster(smem_u32(&tfree_s[i & 1]), (uint32_t)((i >> 1) - 1) & 1u, &abort_s, prm.dev_status);
                     fs_compute_sync();
                     float* out = slot_of(i, crank);
                     for (int e4 = tid; e4 < Cfg::TFLOATS / 4; e4 += kFsWarps * 32) {
