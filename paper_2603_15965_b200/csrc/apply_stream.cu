@@ -554,12 +554,13 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
             // DIRECT: finished y leaves through the warp that computed it: 16-byte pieces, 64 bytes of eight rows per store
             char* yrow[MT][2];
             if constexpr (Cfg::DIRECT) {
+                const bool live = *static_cast<volatile int*>(&abort_s) == 0;      // no wait has run out: t is what it should be
 #pragma unroll
                 for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const int row = mt * 16 + h * 8 + (lane & 7);
-                        yrow[mt][h] = row < it.rows ? static_cast<char*>(pd.y) + (int64_t)fs_token(prm, perm_s, it.row0 + row) * pd.ldy * 2 : nullptr;
+                        yrow[mt][h] = live && row < it.rows ? static_cast<char*>(pd.y) + (int64_t)fs_token(prm, perm_s, it.row0 + row) * pd.ldy * 2 : nullptr;
                     }
             }
 
@@ -572,7 +573,8 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
                 const uint32_t s = g % NS;
                 const uint32_t bs = stage0 + s * Cfg::STAGE;
                 unsigned char* ysp = dsm + s * Cfg::STAGE + Cfg::WBYTES;
-                wait_bar(smem_u32(&full_s[s]), (g / NS) & 1u, &abort_s, prm.dev_status);
+                const bool arrived = wait_bar(smem_u32(&full_s[s]), (g / NS) & 1u, &abort_s, prm.dev_status);
+                if (Cfg::DIRECT && !arrived) break;        // a wait ran out: the stage may hold anything, y keeps what it has
                 const int ngroups = min(Cfg::CH, pd.d_out - it.col0 - j * Cfg::CH) / 32;
                 // my 32-column groups: y words first, then the MMAs, then add, round once and write back.
                 // Rows past the tile hold stale shared memory; they are updated like the others and never stored.

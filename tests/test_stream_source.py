@@ -26,3 +26,17 @@ def test_slot_is_written_only_after_the_peers_have_read_the_copies_made_from_it(
     push = shrink.index("bulk_copy_to_peer(")
     assert wait < barrier < write < push
     assert shrink.count("tfree_s") == 1
+
+
+def test_nothing_is_stored_to_y_after_a_time_out(code):
+    """Every wait falls through once one has run out; what the stages and t hold from then on must not reach y."""
+    expand = code[code.index("auto expand = "):code.index("shrink(next, i + 1)")]
+    # rank 64, where the compute warps store: t is checked once an item, the stage once a chunk
+    live = expand.index("live = *static_cast<volatile int*>(&abort_s) == 0")
+    leave = expand.index("if (Cfg::DIRECT && !arrived) break;")
+    assert expand.index("tfull_s[i & 1]") < live < expand.index("arrived = wait_bar(smem_u32(&full_s[s])") < leave < expand.index("stg128(")
+    assert re.search(r"yrow\[mt\]\[h\] = live && row < it.rows \?", expand) and re.search(r"if \(yrow\[mt\]\[h\] != nullptr\)\s*stg128\(", expand)
+    assert expand.count("stg128(") == code.count("stg128(") == 1
+    # ranks 16 and 32, where the copy warps do
+    retire = code[code.index("auto retire = "):code.index("auto token_of = ")]
+    assert re.search(r"nb != 0 && !abort_s", retire) and code.count("bulk_store(") == retire.count("bulk_store(") == 1
