@@ -65,6 +65,7 @@ using namespace ptx;
 constexpr int kFsWarps = 8;               // compute warps
 constexpr int kFsCopyWarps = 4;           // each moves a quarter of the rows of the tile
 constexpr int kFsThreads = (kFsWarps + kFsCopyWarps) * 32;
+constexpr long long kFsLandingCycles = 1000000;    // ~0.5 ms; a copy between CTAs takes ~1 us
 constexpr int kFsPermCache = 4096;        // calls with at most this many tokens keep perm in shared memory
 
 // Weight boxes of the launch's projections (the kernels that use none are launched without them).
@@ -662,10 +663,21 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
             if (i >= 0) expand(cur, i);
         }
     }
-    // No CTA leaves while a peer may still write into its shared memory.  Every wait above is bounded, so all get here.
+    // No CTA leaves while a peer may still write into its shared memory or read from it.  Every wait above is bounded, so all get here.
     if (S > 1) {
+        // After a time-out copies between the CTAs may be in flight that nobody has waited for: all of them learn of it, stop
+        // issuing (the first barrier) and give the copies, of a few KB each, a bounded time to land.
+        volatile int* aborted = &abort_s;
+        if (*aborted && lane < S) st_cluster_u32(map_to_cta(smem_u32(&abort_s), lane), 1u);
         __syncwarp();
         cluster_sync_all();
+        if (*aborted) {
+            const long long t0 = clock64();
+            while (clock64() - t0 < kFsLandingCycles) {
+            }
+            __syncwarp();
+            cluster_sync_all();
+        }
     }
 }
 

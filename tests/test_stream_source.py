@@ -40,3 +40,15 @@ def test_nothing_is_stored_to_y_after_a_time_out(code):
     # ranks 16 and 32, where the copy warps do
     retire = code[code.index("auto retire = "):code.index("auto token_of = ")]
     assert re.search(r"nb != 0 && !abort_s", retire) and code.count("bulk_store(") == retire.count("bulk_store(") == 1
+
+
+def test_no_cta_leaves_after_a_time_out_while_copies_between_ctas_may_be_in_flight(code):
+    """A CTA that has given up waits for nothing, so the copies to and from it are not known to be done when it reaches the end: the
+    whole cluster learns of the time-out, stops at a barrier, lets them land and leaves together."""
+    end = code[code.index("expand(cur, i)"):code.index("bool stream_eligible(")]
+    tell = end.index("st_cluster_u32(map_to_cta(smem_u32(&abort_s), lane), 1u)")
+    stop = end.index("cluster_sync_all()")
+    land = end.index("kFsLandingCycles")
+    leave = end.index("cluster_sync_all()", land)
+    assert tell < stop < land < leave
+    assert re.search(r"if \(\*aborted\) \{[^{}]*kFsLandingCycles\) \{\s*\}[^{}]*cluster_sync_all\(\);\s*\}", end)
