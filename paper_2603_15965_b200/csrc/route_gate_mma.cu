@@ -332,7 +332,9 @@ __global__ void __launch_bounds__(kGateSplitWarps * 32, 2)
                 }
                 if (bias != nullptr) z += __ldg(bias + c);
                 if (logits_out != nullptr && i < N) logits_out[i * C + c] = z;
-                if (arg == INT32_MAX || z > best) { best = z; arg = c; }
+                // as a scan from adapter 0 with '>' decides: a NaN there stays the best, one anywhere else never is
+                if (c == 0 && z != z) { best = INFINITY; arg = 0; }
+                else if (z == z && (arg == INT32_MAX || z > best)) { best = z; arg = c; }
             }
         }
 #pragma unroll

@@ -49,6 +49,32 @@ def test_both_sides_of_the_small_call_rule(N, d, C):
     assert np.array_equal(r.cpu().numpy()[margin >= 1e-3], r_ref[margin >= 1e-3])
 
 
+@pytest.mark.parametrize("N", [40, 1500])
+@pytest.mark.parametrize("C", [7, 16, 31])
+def test_nan_and_infinite_logits_decide_as_a_scan_does(N, C):
+    """Logits of NaN (an adapter whose gate column or bias is damaged) and of -inf (one that is masked): the winner is that of a scan
+    from adapter 0 that replaces the best by what is greater."""
+    rng = np.random.default_rng(C)
+    d = 2048
+    x = W.round_to_bf16(rng.standard_normal((N, d), dtype=np.float32))
+    G = (rng.standard_normal((d, C)) * d ** -0.5).astype(np.float32)
+    z64 = x.astype(np.float64) @ G.astype(np.float64)
+    for bad in ([1], [2, 5], [0], [0, 3], list(range(C)), list(range(1, C))):
+        for value in (np.nan, -np.inf, np.inf):
+            bias = np.zeros(C, np.float32)
+            bias[bad] = value
+            r = M.molora_route_gate(dev_tensor(x, "bf16"), dev_tensor(G, "f32"), dev_tensor(bias, "f32")).cpu().numpy()
+            z = z64 + bias
+            want = np.zeros(N, np.int64)
+            best = z[:, 0].copy()
+            for c in range(1, C):
+                more = z[:, c] > best
+                want[more], best[more] = c, z[more, c]
+            order = np.sort(np.where(np.isfinite(z), z, -1e30), axis=1)
+            clear = order[:, -1] - order[:, -2] >= 1e-3
+            assert np.array_equal(r[clear], want[clear]), (bad, value)
+
+
 @pytest.mark.parametrize("N", [1, 63, 127, 128, 1000, 1792, 1793])
 @pytest.mark.parametrize("d,H", [(64, 64), (2048, 64), (4096, 128)])
 def test_mlp_router_of_small_calls(N, d, H):
