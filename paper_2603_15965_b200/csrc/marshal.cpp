@@ -22,7 +22,7 @@
 namespace {
 
 PyObject* g_raise_status = nullptr;      // binding._check(function name, status)
-PyObject *s_x, *s_y, *s_A, *s_B, *s_scale, *s_row_scale, *s_cuda_stream;
+PyObject *s_x, *s_y, *s_A, *s_B, *s_scale, *s_row_scale, *s_cuda_stream, *s_data_ptr;
 
 struct PyRaised {};                      // a Python exception is set
 [[noreturn]] void raise(PyObject* type, const std::string& text)
@@ -53,7 +53,16 @@ const at::Tensor& tensor(PyObject* o, const char* name)
     if (!THPVariable_Check(o)) raise(PyExc_TypeError, std::string(name) + ": expected a tensor");
     return THPVariable_Unpack(o);
 }
-void* ptr(PyObject* o, const char* name) { return o == Py_None ? nullptr : tensor(o, name).data_ptr(); }
+// device pointer of a tensor, or of anything else that has data_ptr(); None is a null pointer, which the library judges
+void* ptr(PyObject* o)
+{
+    if (o == Py_None) return nullptr;
+    if (THPVariable_Check(o)) return THPVariable_Unpack(o).data_ptr();
+    Ref v(PyObject_CallMethodNoArgs(o, s_data_ptr));
+    void* p = PyLong_AsVoidPtr(v.p);
+    if (p == nullptr && PyErr_Occurred()) throw PyRaised{};
+    return p;
+}
 PyObject* wrap(const at::Tensor& t)
 {
     PyObject* o = THPVariable_Wrap(t);
@@ -211,8 +220,8 @@ private:
 };
 
 int32_t* i32(const at::Tensor& t) { return static_cast<int32_t*>(t.data_ptr()); }
-float* f32(PyObject* o, const char* name) { return static_cast<float*>(ptr(o, name)); }
-uint32_t* status_word(PyObject* o) { return static_cast<uint32_t*>(ptr(o, "dev_status")); }
+float* f32(PyObject* o) { return static_cast<float*>(ptr(o)); }
+uint32_t* status_word(PyObject* o) { return static_cast<uint32_t*>(ptr(o)); }
 
 // ---- (ids, breaks, r_out, dev_status, stream)
 PyObject* route_vocab(PyObject* const* a)
@@ -257,8 +266,8 @@ PyObject* route_gate(PyObject* const* a)
     }
     const molora_dtype_t dt = dtype_code(x);
     at::Tensor r = i32_out(a[3], "r_out", m.rows, x.device());
-    const float *g = f32(a[1], "G"), *bias = f32(a[2], "bias");
-    float* logits = f32(a[4], "logits_out");
+    const float *g = f32(a[1]), *bias = f32(a[2]);
+    float* logits = f32(a[4]);
     if (a[8] != Py_None) {
         const at::Tensor& prepared = tensor(a[8], "prepared");
         check("molora_route_gate_prepared",
@@ -285,8 +294,8 @@ PyObject* route_mlp(PyObject* const* a)
     if (W1.dim() != 2 || W1.size(0) != d || W1.size(1) != H) raise(PyExc_ValueError, "W1 must be [d, H]");
     const molora_dtype_t dt = dtype_code(x);
     at::Tensor r = i32_out(a[5], "r_out", m.rows, x.device());
-    const float *w1 = f32(a[1], "W1"), *b1 = f32(a[2], "b1"), *w2 = f32(a[3], "W2"), *b2 = f32(a[4], "b2");
-    float* logits = f32(a[6], "logits_out");
+    const float *w1 = f32(a[1]), *b1 = f32(a[2]), *w2 = f32(a[3]), *b2 = f32(a[4]);
+    float* logits = f32(a[6]);
     if (a[10] != Py_None) {
         const at::Tensor& prepared = tensor(a[10], "prepared");
         check("molora_route_mlp_prepared",
@@ -334,10 +343,11 @@ PyObject* group(PyObject* const* a)
 PyObject* apply_batched(PyObject* const* a)
 {
     const Projs pr(a[0], a[6]);
-    const at::Tensor &offsets = tensor(a[1], "offsets"), &perm = tensor(a[2], "perm");
-    const Workspace ws(a[3], a[3] == Py_None ? pr.apply_bytes() : 0, offsets.device(), true);
-    check("molora_apply_batched", molora_apply_batched(pr.d, pr.P, pr.dt, pr.N, (int32_t)pr.C, i32(offsets), i32(perm), ws.p, ws.n,
-                                                       status_word(a[4]), stream_of(a[5])));
+    const auto *offsets = static_cast<const int32_t*>(ptr(a[1])), *perm = static_cast<const int32_t*>(ptr(a[2]));
+    const size_t need = a[3] == Py_None ? pr.apply_bytes() : 0;
+    const Workspace ws(a[3], need, need > 0 ? tensor(a[1], "offsets").device() : at::Device(at::kCUDA), true);
+    check("molora_apply_batched", molora_apply_batched(pr.d, pr.P, pr.dt, pr.N, (int32_t)pr.C, offsets, perm, ws.p, ws.n, status_word(a[4]),
+                                                       stream_of(a[5])));
     Py_RETURN_NONE;
 }
 
@@ -437,5 +447,6 @@ PyMODINIT_FUNC PyInit__marshal()
     s_scale = PyUnicode_InternFromString("scale");
     s_row_scale = PyUnicode_InternFromString("row_scale");
     s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
+    s_data_ptr = PyUnicode_InternFromString("data_ptr");
     return PyModule_Create(&module);
 }
