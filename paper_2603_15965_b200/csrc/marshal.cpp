@@ -11,6 +11,7 @@
 
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <algorithm>
@@ -422,10 +423,8 @@ PyObject* entry(PyObject*, PyObject* const* args, Py_ssize_t n)
     try {
         return F(args);
     } catch (const PyRaised&) {
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
     } catch (...) {
-        PyErr_SetString(PyExc_RuntimeError, "unknown C++ exception");
+        torch::translate_exception_to_python(std::current_exception());      // (out of memory is torch.OutOfMemoryError, as from torch itself)
     }
     return nullptr;
 }
