@@ -396,7 +396,7 @@ PyObject* apply_topk(PyObject* const* a)
     // only the apply part of the scratch has to start cleared, and only where a kernel keeps control words in it
     const Workspace ws(a[4], a[4] == Py_None ? molora_apply_topk_workspace_bytes(pr.d, pr.P, pr.N, (int32_t)C) + 256 : 0, idx.device(),
                        a[4] == Py_None && pr.apply_bytes() > 0);
-    const size_t off = (size_t)(-(intptr_t)ws.p) % 256;
+    const size_t off = std::min((size_t)(-(intptr_t)ws.p) % 256, ws.n);      // (a shorter workspace is refused as too small)
     check("molora_apply_topk",
           molora_apply_topk(pr.d, pr.P, pr.dt, pr.N, (int32_t)C, (int32_t)idx.size(0), i32(idx), static_cast<const float*>(w.data_ptr()),
                             static_cast<char*>(ws.p) + off, ws.n - off, status_word(a[5]), stream_of(a[6])));

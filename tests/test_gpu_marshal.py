@@ -17,3 +17,16 @@ def test_out_of_memory_is_torchs_own_error():
     finally:
         torch.cuda.set_per_process_memory_fraction(1.0)
     assert not M.molora_route_vocab(ids, breaks).any()
+
+
+@pytest.mark.parametrize("offset,size", [(1, 20), (1, 255), (1, 256), (0, 255), (256, 0)])
+def test_topk_workspace_shorter_than_its_alignment_is_refused(offset, size):
+    """(the workspace starts at its first 256-byte boundary, which may lie past its end)"""
+    N, C = 40, 4
+    x, y = torch.randn(N, 64, device="cuda").bfloat16(), torch.zeros(N, 64, dtype=torch.bfloat16, device="cuda")
+    A, B = torch.randn(C, 64, 16, device="cuda").bfloat16(), torch.randn(C, 16, 64, device="cuda").bfloat16()
+    idx, w = M.molora_topk_softmax(torch.randn(N, C, device="cuda"), 2)
+    buffer = torch.zeros(4096, dtype=torch.uint8, device="cuda")
+    with pytest.raises(M.MoloraError, match="workspace"):
+        M.molora_apply_topk([M.ProjDesc(x, y, A, B)], idx, w, C, ws=buffer[offset:offset + size])
+    assert not y.any() and not buffer.any()
