@@ -42,6 +42,13 @@ struct Ref {                             // owned reference
     Ref& operator=(const Ref&) = delete;
 };
 
+// Other Python threads run while a call allocates and enqueues: either may block (an allocation that goes to the driver, a launch
+// into a full queue).
+struct NoGil {
+    PyThreadState* state = PyEval_SaveThread();
+    ~NoGil() { PyEval_RestoreThread(state); }
+};
+
 void check(const char* fn, molora_status_t status)
 {
     if (status == MOLORA_OK) return;
@@ -91,11 +98,21 @@ const at::Tensor& i32_dev(PyObject* o, const char* name)
         raise(PyExc_ValueError, std::string(name) + ": expected a contiguous int32 CUDA tensor");
     return t;
 }
-at::Tensor i32_out(PyObject* o, const char* name, int64_t n, const at::Device& dev)
-{
-    if (o != Py_None) return i32_dev(o, name);
-    return at::empty({n}, at::TensorOptions().dtype(at::kInt).device(dev));
-}
+// an output: the caller's tensor, or n words allocated on first use
+struct Out {
+    at::Tensor t;
+    at::Device dev;
+    int64_t n;
+    Out(PyObject* o, const char* name, int64_t n_, const at::Device& dev_) : dev(dev_), n(n_)
+    {
+        if (o != Py_None) t = i32_dev(o, name);
+    }
+    int32_t* get()
+    {
+        if (!t.defined()) t = at::empty({n}, at::TensorOptions().dtype(at::kInt).device(dev));
+        return static_cast<int32_t*>(t.data_ptr());
+    }
+};
 molora_dtype_t dtype_code(const at::Tensor& t)
 {
     if (t.scalar_type() == at::kFloat) return MOLORA_F32;
@@ -112,22 +129,25 @@ Matrix matrix(const at::Tensor& t, const char* name)
     const int64_t rows = t.size(0), cols = t.size(1);
     return {rows, cols, rows > 1 ? t.stride(0) : std::max<int64_t>(t.stride(0), cols)};
 }
-// the caller's workspace, or one of `need` bytes
+// the caller's workspace, or one of `need` bytes allocated by make()
 struct Workspace {
     at::Tensor t;
     void* p = nullptr;
-    size_t n = 0;
-    Workspace(PyObject* o, size_t need, const at::Device& dev, bool zero)
+    size_t n = 0, need = 0;
+    Workspace(PyObject* o, size_t need_)
+    {
+        if (o != Py_None) t = tensor(o, "ws");
+        else need = need_;
+    }
+    void make(const at::Device& dev, bool zero)
     {
         const auto opt = at::TensorOptions().dtype(at::kByte).device(dev);
-        if (o != Py_None) t = tensor(o, "ws");
-        else if (need > 0) t = zero ? at::zeros({(int64_t)need}, opt) : at::empty({(int64_t)need}, opt);
-        else return;
+        if (need > 0) t = zero ? at::zeros({(int64_t)need}, opt) : at::empty({(int64_t)need}, opt);
+        if (!t.defined()) return;
         p = t.data_ptr();
         n = (size_t)t.numel() * t.element_size();
     }
 };
-
 // ---- descriptors of a batched apply: from ProjDesc objects, or the array that pack_proj_descs returned
 struct Projs {
     std::vector<molora_proj_desc_t> own;
@@ -222,29 +242,46 @@ private:
 
 int32_t* i32(const at::Tensor& t) { return static_cast<int32_t*>(t.data_ptr()); }
 float* f32(PyObject* o) { return static_cast<float*>(ptr(o)); }
+// one call of the library: f() allocates what it needs, enqueues and returns the status
+template <class F>
+void call(const char* fn, F f)
+{
+    molora_status_t status;
+    {
+        const NoGil others;
+        status = f();
+    }
+    check(fn, status);
+}
 uint32_t* status_word(PyObject* o) { return static_cast<uint32_t*>(ptr(o)); }
 
 // ---- (ids, breaks, r_out, dev_status, stream)
 PyObject* route_vocab(PyObject* const* a)
 {
     const at::Tensor &ids = i32_dev(a[0], "ids"), &breaks = i32_dev(a[1], "breaks");
-    at::Tensor r = i32_out(a[2], "r_out", ids.numel(), ids.device());
-    check("molora_route_vocab", molora_route_vocab(i32(ids), ids.numel(), i32(breaks), (int32_t)breaks.numel() - 1, i32(r),
-                                                   status_word(a[3]), stream_of(a[4])));
-    return wrap(r);
+    const int64_t N = ids.numel();
+    Out r(a[2], "r_out", N, ids.device());
+    uint32_t* status = status_word(a[3]);
+    void* stream = stream_of(a[4]);
+    call("molora_route_vocab", [&] { return molora_route_vocab(i32(ids), N, i32(breaks), (int32_t)breaks.numel() - 1, r.get(), status, stream); });
+    return wrap(r.t);
 }
 
 // ---- (ids, adapter, breaks, n_adapters, r_out, dev_status, stream)
 PyObject* route_composite(PyObject* const* a)
 {
     const at::Tensor &ids = i32_dev(a[0], "ids"), &adapter = i32_dev(a[1], "adapter"), &breaks = i32_dev(a[2], "breaks");
-    if (adapter.numel() != ids.numel()) raise(PyExc_ValueError, "adapter must hold one index per token");
+    const int64_t N = ids.numel();
+    if (adapter.numel() != N) raise(PyExc_ValueError, "adapter must hold one index per token");
     Ref n(PyNumber_Long(a[3]));
-    at::Tensor r = i32_out(a[4], "r_out", ids.numel(), ids.device());
-    check("molora_route_composite",
-          molora_route_composite(i32(ids), i32(adapter), ids.numel(), i32(breaks), (int32_t)breaks.numel() - 1, (int32_t)integer(n.p), i32(r),
-                                 status_word(a[5]), stream_of(a[6])));
-    return wrap(r);
+    const int32_t n_adapters = (int32_t)integer(n.p);
+    Out r(a[4], "r_out", N, ids.device());
+    uint32_t* status = status_word(a[5]);
+    void* stream = stream_of(a[6]);
+    call("molora_route_composite", [&] {
+        return molora_route_composite(i32(ids), i32(adapter), N, i32(breaks), (int32_t)breaks.numel() - 1, n_adapters, r.get(), status, stream);
+    });
+    return wrap(r.t);
 }
 
 // ---- (x, G, bias, r_out, logits_out, ws, dev_status, stream, prepared)
@@ -266,21 +303,25 @@ PyObject* route_gate(PyObject* const* a)
             raise(PyExc_ValueError, "logits_out: expected contiguous fp32 [N, C]");
     }
     const molora_dtype_t dt = dtype_code(x);
-    at::Tensor r = i32_out(a[3], "r_out", m.rows, x.device());
+    Out r(a[3], "r_out", m.rows, x.device());
     const float *g = f32(a[1]), *bias = f32(a[2]);
     float* logits = f32(a[4]);
+    uint32_t* status = status_word(a[6]);
+    void* stream = stream_of(a[7]);
     if (a[8] != Py_None) {
         const at::Tensor& prepared = tensor(a[8], "prepared");
-        check("molora_route_gate_prepared",
-              molora_route_gate_prepared(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, i32(r), logits, prepared.data_ptr(),
-                                         (size_t)prepared.numel(), status_word(a[6]), stream_of(a[7])));
-        return wrap(r);
+        call("molora_route_gate_prepared", [&] {
+            return molora_route_gate_prepared(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, r.get(), logits, prepared.data_ptr(),
+                                              (size_t)prepared.numel(), status, stream);
+        });
+        return wrap(r.t);
     }
-    // (the weight images are written before they are read: the scratch need not be cleared)
-    const Workspace ws(a[5], molora_route_gate_workspace_bytes(dt, d, C), x.device(), false);
-    check("molora_route_gate", molora_route_gate(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, i32(r), logits, ws.p, ws.n,
-                                                 status_word(a[6]), stream_of(a[7])));
-    return wrap(r);
+    Workspace ws(a[5], molora_route_gate_workspace_bytes(dt, d, C));
+    call("molora_route_gate", [&] {
+        ws.make(x.device(), false);        // (the weight images are written before they are read: the scratch need not be cleared)
+        return molora_route_gate(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, r.get(), logits, ws.p, ws.n, status, stream);
+    });
+    return wrap(r.t);
 }
 
 // ---- (x, W1, b1, W2, b2, r_out, logits_out, ws, dev_status, stream, prepared)
@@ -294,20 +335,25 @@ PyObject* route_mlp(PyObject* const* a)
     const int32_t H = (int32_t)W2.size(0), C = (int32_t)W2.size(1), d = (int32_t)m.cols;
     if (W1.dim() != 2 || W1.size(0) != d || W1.size(1) != H) raise(PyExc_ValueError, "W1 must be [d, H]");
     const molora_dtype_t dt = dtype_code(x);
-    at::Tensor r = i32_out(a[5], "r_out", m.rows, x.device());
+    Out r(a[5], "r_out", m.rows, x.device());
     const float *w1 = f32(a[1]), *b1 = f32(a[2]), *w2 = f32(a[3]), *b2 = f32(a[4]);
     float* logits = f32(a[6]);
+    uint32_t* status = status_word(a[8]);
+    void* stream = stream_of(a[9]);
     if (a[10] != Py_None) {
         const at::Tensor& prepared = tensor(a[10], "prepared");
-        check("molora_route_mlp_prepared",
-              molora_route_mlp_prepared(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, i32(r), logits, prepared.data_ptr(),
-                                        (size_t)prepared.numel(), status_word(a[8]), stream_of(a[9])));
-        return wrap(r);
+        call("molora_route_mlp_prepared", [&] {
+            return molora_route_mlp_prepared(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, r.get(), logits, prepared.data_ptr(),
+                                             (size_t)prepared.numel(), status, stream);
+        });
+        return wrap(r.t);
     }
-    const Workspace ws(a[7], molora_route_mlp_workspace_bytes(dt, d, H, C), x.device(), false);
-    check("molora_route_mlp", molora_route_mlp(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, i32(r), logits, ws.p, ws.n,
-                                               status_word(a[8]), stream_of(a[9])));
-    return wrap(r);
+    Workspace ws(a[7], molora_route_mlp_workspace_bytes(dt, d, H, C));
+    call("molora_route_mlp", [&] {
+        ws.make(x.device(), false);
+        return molora_route_mlp(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, r.get(), logits, ws.p, ws.n, status, stream);
+    });
+    return wrap(r.t);
 }
 
 PyObject* tuple_of(std::initializer_list<at::Tensor> ts)
@@ -332,12 +378,16 @@ PyObject* group(PyObject* const* a)
     const at::Tensor& r = i32_dev(a[0], "r");
     const int64_t N = r.numel(), C = integer(a[1]);
     const at::Device dev = r.device();
-    at::Tensor counts = i32_out(a[2], "counts", C, dev), offsets = i32_out(a[3], "offsets", C + 1, dev),
-               perm = i32_out(a[4], "perm", std::max<int64_t>(N, 1), dev);
-    const Workspace ws(a[5], molora_group_workspace_bytes(N, (int32_t)C), dev, true);
-    check("molora_group", molora_group(i32(r), N, (int32_t)C, i32(counts), i32(offsets), i32(perm), ws.p, ws.n, status_word(a[6]),
-                                       stream_of(a[7])));
-    return tuple_of({counts, offsets, perm});
+    Out counts(a[2], "counts", C, dev), offsets(a[3], "offsets", C + 1, dev), perm(a[4], "perm", std::max<int64_t>(N, 1), dev);
+    Workspace ws(a[5], molora_group_workspace_bytes(N, (int32_t)C));
+    uint32_t* status = status_word(a[6]);
+    void* stream = stream_of(a[7]);
+    call("molora_group", [&] {
+        int32_t *c = counts.get(), *o = offsets.get(), *p = perm.get();
+        ws.make(dev, true);
+        return molora_group(i32(r), N, (int32_t)C, c, o, p, ws.p, ws.n, status, stream);
+    });
+    return tuple_of({counts.t, offsets.t, perm.t});
 }
 
 // ---- (projs, offsets, perm, ws, dev_status, stream, packed)
@@ -345,10 +395,14 @@ PyObject* apply_batched(PyObject* const* a)
 {
     const Projs pr(a[0], a[6]);
     const auto *offsets = static_cast<const int32_t*>(ptr(a[1])), *perm = static_cast<const int32_t*>(ptr(a[2]));
-    const size_t need = a[3] == Py_None ? pr.apply_bytes() : 0;
-    const Workspace ws(a[3], need, need > 0 ? tensor(a[1], "offsets").device() : at::Device(at::kCUDA), true);
-    check("molora_apply_batched", molora_apply_batched(pr.d, pr.P, pr.dt, pr.N, (int32_t)pr.C, offsets, perm, ws.p, ws.n, status_word(a[4]),
-                                                       stream_of(a[5])));
+    Workspace ws(a[3], a[3] == Py_None ? pr.apply_bytes() : 0);
+    const at::Device dev = ws.need > 0 ? tensor(a[1], "offsets").device() : at::Device(at::kCUDA);
+    uint32_t* status = status_word(a[4]);
+    void* stream = stream_of(a[5]);
+    call("molora_apply_batched", [&] {
+        ws.make(dev, true);
+        return molora_apply_batched(pr.d, pr.P, pr.dt, pr.N, (int32_t)pr.C, offsets, perm, ws.p, ws.n, status, stream);
+    });
     Py_RETURN_NONE;
 }
 
@@ -360,13 +414,16 @@ PyObject* group_apply_batched(PyObject* const* a)
     const int64_t C = a[2] == Py_None ? pr.C : integer(a[2]);
     if (r.numel() != pr.N || C != pr.C) raise(PyExc_ValueError, "r must hold one routing decision per token of the projections");
     const at::Device dev = r.device();
-    at::Tensor counts = i32_out(a[3], "counts", C, dev), offsets = i32_out(a[4], "offsets", C + 1, dev),
-               perm = i32_out(a[5], "perm", std::max<int64_t>(pr.N, 1), dev);
-    const Workspace ws(a[6], a[6] == Py_None ? pr.apply_bytes() : 0, dev, true);
-    check("molora_group_apply_batched",
-          molora_group_apply_batched(i32(r), pr.N, (int32_t)C, i32(counts), i32(offsets), i32(perm), pr.d, pr.P, pr.dt, ws.p, ws.n,
-                                     status_word(a[7]), stream_of(a[8])));
-    return tuple_of({counts, offsets, perm});
+    Out counts(a[3], "counts", C, dev), offsets(a[4], "offsets", C + 1, dev), perm(a[5], "perm", std::max<int64_t>(pr.N, 1), dev);
+    Workspace ws(a[6], a[6] == Py_None ? pr.apply_bytes() : 0);
+    uint32_t* status = status_word(a[7]);
+    void* stream = stream_of(a[8]);
+    call("molora_group_apply_batched", [&] {
+        int32_t *c = counts.get(), *o = offsets.get(), *p = perm.get();
+        ws.make(dev, true);
+        return molora_group_apply_batched(i32(r), pr.N, (int32_t)C, c, o, p, pr.d, pr.P, pr.dt, ws.p, ws.n, status, stream);
+    });
+    return tuple_of({counts.t, offsets.t, perm.t});
 }
 
 // ---- (logits, k, stream)
@@ -376,10 +433,14 @@ PyObject* topk_softmax(PyObject* const* a)
     if (z.scalar_type() != at::kFloat || z.dim() != 2 || !z.is_contiguous()) raise(PyExc_ValueError, "logits must be a dense fp32 [N, C] tensor");
     Ref kk(PyNumber_Long(a[1]));
     const int64_t k = integer(kk.p), N = z.size(0);
-    at::Tensor idx = at::empty({k, N}, at::TensorOptions().dtype(at::kInt).device(z.device())),
-               w = at::empty({k, N}, at::TensorOptions().dtype(at::kFloat).device(z.device()));
-    check("molora_topk_softmax", molora_topk_softmax(static_cast<const float*>(z.data_ptr()), N, (int32_t)z.size(1), (int32_t)k, i32(idx),
-                                                     static_cast<float*>(w.data_ptr()), stream_of(a[2])));
+    void* stream = stream_of(a[2]);
+    at::Tensor idx, w;
+    call("molora_topk_softmax", [&] {
+        idx = at::empty({k, N}, at::TensorOptions().dtype(at::kInt).device(z.device()));
+        w = at::empty({k, N}, at::TensorOptions().dtype(at::kFloat).device(z.device()));
+        return molora_topk_softmax(static_cast<const float*>(z.data_ptr()), N, (int32_t)z.size(1), (int32_t)k, i32(idx),
+                                   static_cast<float*>(w.data_ptr()), stream);
+    });
     return tuple_of({idx, w});
 }
 
@@ -392,14 +453,19 @@ PyObject* apply_topk(PyObject* const* a)
     if (pr.C != C || idx0.scalar_type() != at::kInt || w0.scalar_type() != at::kFloat || idx0.dim() != 2 || idx0.sizes() != w0.sizes() ||
         idx0.size(1) != pr.N)
         raise(PyExc_ValueError, "idx int32 [k, N] and w fp32 [k, N] must match the projections");
-    const at::Tensor idx = idx0.contiguous(), w = w0.contiguous();
-    // only the apply part of the scratch has to start cleared, and only where a kernel keeps control words in it
-    const Workspace ws(a[4], a[4] == Py_None ? molora_apply_topk_workspace_bytes(pr.d, pr.P, pr.N, (int32_t)C) + 256 : 0, idx.device(),
-                       a[4] == Py_None && pr.apply_bytes() > 0);
-    const size_t off = std::min((size_t)(-(intptr_t)ws.p) % 256, ws.n);      // (a shorter workspace is refused as too small)
-    check("molora_apply_topk",
-          molora_apply_topk(pr.d, pr.P, pr.dt, pr.N, (int32_t)C, (int32_t)idx.size(0), i32(idx), static_cast<const float*>(w.data_ptr()),
-                            static_cast<char*>(ws.p) + off, ws.n - off, status_word(a[5]), stream_of(a[6])));
+    const bool zero = pr.apply_bytes() > 0;
+    Workspace ws(a[4], a[4] == Py_None ? molora_apply_topk_workspace_bytes(pr.d, pr.P, pr.N, (int32_t)C) + 256 : 0);
+    uint32_t* status = status_word(a[5]);
+    void* stream = stream_of(a[6]);
+    at::Tensor idx, w;
+    call("molora_apply_topk", [&] {
+        idx = idx0.contiguous();
+        w = w0.contiguous();
+        ws.make(idx.device(), zero);        // (only the apply part has to start cleared, and only where a kernel keeps control words in it)
+        const size_t off = std::min((size_t)(-(intptr_t)ws.p) % 256, ws.n);      // (a shorter workspace is refused as too small)
+        return molora_apply_topk(pr.d, pr.P, pr.dt, pr.N, (int32_t)C, (int32_t)idx.size(0), i32(idx), static_cast<const float*>(w.data_ptr()),
+                                 static_cast<char*>(ws.p) + off, ws.n - off, status, stream);
+    });
     Py_RETURN_NONE;
 }
 

@@ -1,4 +1,7 @@
 """The compiled marshalling on a GPU: what a caller passes is what is used, and errors keep their types."""
+import threading
+import time
+
 import pytest
 import torch
 
@@ -30,3 +33,27 @@ def test_topk_workspace_shorter_than_its_alignment_is_refused(offset, size):
     with pytest.raises(M.MoloraError, match="workspace"):
         M.molora_apply_topk([M.ProjDesc(x, y, A, B)], idx, w, C, ws=buffer[offset:offset + size])
     assert not y.any() and not buffer.any()
+
+
+def test_other_threads_run_while_a_call_waits_for_the_launch_queue():
+    ids, breaks = torch.zeros(64, dtype=torch.int32, device="cuda"), torch.tensor([0, 5], dtype=torch.int32, device="cuda")
+    r = M.molora_route_vocab(ids, breaks)
+    torch.cuda.synchronize()
+
+    def launches():
+        for _ in range(4000):                        # more than the queue holds: some call blocks until the kernel ahead ends
+            M.molora_route_vocab(ids, breaks, r_out=r)
+
+    torch.cuda._sleep(1_500_000_000)                 # ~0.8 s
+    worker = threading.Thread(target=launches)
+    start = last = time.perf_counter()
+    longest = 0.0
+    worker.start()
+    while worker.is_alive():
+        time.sleep(0.001)
+        now = time.perf_counter()
+        longest, last = max(longest, now - last), now
+    worker.join()
+    torch.cuda.synchronize()
+    assert last - start > 0.3, "the queue never filled"
+    assert longest < 0.15
