@@ -10,6 +10,7 @@
 #include <Python.h>
 
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -98,6 +99,17 @@ const at::Tensor& i32_dev(PyObject* o, const char* name)
         raise(PyExc_ValueError, std::string(name) + ": expected a contiguous int32 CUDA tensor");
     return t;
 }
+// What a call allocates belongs to the stream that it runs on: memory that the current stream's allocator hands out may still be in
+// use there, and is handed out again there as soon as the call has returned.
+template <class F>
+at::Tensor allocate(void* stream, F f)
+{
+    c10::cuda::OptionalCUDAStreamGuard on;
+    // (odd values are not addresses but the runtime's names of its default streams)
+    if (stream != c10::cuda::getCurrentCUDAStream().stream() && ((uintptr_t)stream & 1u) == 0)
+        on.reset_stream(c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream), c10::cuda::current_device()));
+    return f();
+}
 // an output: the caller's tensor, or n words allocated on first use
 struct Out {
     at::Tensor t;
@@ -107,9 +119,9 @@ struct Out {
     {
         if (o != Py_None) t = i32_dev(o, name);
     }
-    int32_t* get()
+    int32_t* get(void* stream)
     {
-        if (!t.defined()) t = at::empty({n}, at::TensorOptions().dtype(at::kInt).device(dev));
+        if (!t.defined()) t = allocate(stream, [&] { return at::empty({n}, at::TensorOptions().dtype(at::kInt).device(dev)); });
         return static_cast<int32_t*>(t.data_ptr());
     }
 };
@@ -139,10 +151,10 @@ struct Workspace {
         if (o != Py_None) t = tensor(o, "ws");
         else need = need_;
     }
-    void make(const at::Device& dev, bool zero)
+    void make(const at::Device& dev, bool zero, void* stream)
     {
         const auto opt = at::TensorOptions().dtype(at::kByte).device(dev);
-        if (need > 0) t = zero ? at::zeros({(int64_t)need}, opt) : at::empty({(int64_t)need}, opt);
+        if (need > 0) t = allocate(stream, [&] { return zero ? at::zeros({(int64_t)need}, opt) : at::empty({(int64_t)need}, opt); });
         if (!t.defined()) return;
         p = t.data_ptr();
         n = (size_t)t.numel() * t.element_size();
@@ -263,7 +275,7 @@ PyObject* route_vocab(PyObject* const* a)
     Out r(a[2], "r_out", N, ids.device());
     uint32_t* status = status_word(a[3]);
     void* stream = stream_of(a[4]);
-    call("molora_route_vocab", [&] { return molora_route_vocab(i32(ids), N, i32(breaks), (int32_t)breaks.numel() - 1, r.get(), status, stream); });
+    call("molora_route_vocab", [&] { return molora_route_vocab(i32(ids), N, i32(breaks), (int32_t)breaks.numel() - 1, r.get(stream), status, stream); });
     return wrap(r.t);
 }
 
@@ -279,7 +291,7 @@ PyObject* route_composite(PyObject* const* a)
     uint32_t* status = status_word(a[5]);
     void* stream = stream_of(a[6]);
     call("molora_route_composite", [&] {
-        return molora_route_composite(i32(ids), i32(adapter), N, i32(breaks), (int32_t)breaks.numel() - 1, n_adapters, r.get(), status, stream);
+        return molora_route_composite(i32(ids), i32(adapter), N, i32(breaks), (int32_t)breaks.numel() - 1, n_adapters, r.get(stream), status, stream);
     });
     return wrap(r.t);
 }
@@ -311,15 +323,15 @@ PyObject* route_gate(PyObject* const* a)
     if (a[8] != Py_None) {
         const at::Tensor& prepared = tensor(a[8], "prepared");
         call("molora_route_gate_prepared", [&] {
-            return molora_route_gate_prepared(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, r.get(), logits, prepared.data_ptr(),
+            return molora_route_gate_prepared(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, r.get(stream), logits, prepared.data_ptr(),
                                               (size_t)prepared.numel(), status, stream);
         });
         return wrap(r.t);
     }
     Workspace ws(a[5], molora_route_gate_workspace_bytes(dt, d, C));
     call("molora_route_gate", [&] {
-        ws.make(x.device(), false);        // (the weight images are written before they are read: the scratch need not be cleared)
-        return molora_route_gate(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, r.get(), logits, ws.p, ws.n, status, stream);
+        ws.make(x.device(), false, stream);        // (the weight images are written before they are read: the scratch need not be cleared)
+        return molora_route_gate(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, r.get(stream), logits, ws.p, ws.n, status, stream);
     });
     return wrap(r.t);
 }
@@ -343,15 +355,15 @@ PyObject* route_mlp(PyObject* const* a)
     if (a[10] != Py_None) {
         const at::Tensor& prepared = tensor(a[10], "prepared");
         call("molora_route_mlp_prepared", [&] {
-            return molora_route_mlp_prepared(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, r.get(), logits, prepared.data_ptr(),
+            return molora_route_mlp_prepared(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, r.get(stream), logits, prepared.data_ptr(),
                                              (size_t)prepared.numel(), status, stream);
         });
         return wrap(r.t);
     }
     Workspace ws(a[7], molora_route_mlp_workspace_bytes(dt, d, H, C));
     call("molora_route_mlp", [&] {
-        ws.make(x.device(), false);
-        return molora_route_mlp(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, r.get(), logits, ws.p, ws.n, status, stream);
+        ws.make(x.device(), false, stream);
+        return molora_route_mlp(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, r.get(stream), logits, ws.p, ws.n, status, stream);
     });
     return wrap(r.t);
 }
@@ -383,8 +395,8 @@ PyObject* group(PyObject* const* a)
     uint32_t* status = status_word(a[6]);
     void* stream = stream_of(a[7]);
     call("molora_group", [&] {
-        int32_t *c = counts.get(), *o = offsets.get(), *p = perm.get();
-        ws.make(dev, true);
+        int32_t *c = counts.get(stream), *o = offsets.get(stream), *p = perm.get(stream);
+        ws.make(dev, true, stream);
         return molora_group(i32(r), N, (int32_t)C, c, o, p, ws.p, ws.n, status, stream);
     });
     return tuple_of({counts.t, offsets.t, perm.t});
@@ -400,7 +412,7 @@ PyObject* apply_batched(PyObject* const* a)
     uint32_t* status = status_word(a[4]);
     void* stream = stream_of(a[5]);
     call("molora_apply_batched", [&] {
-        ws.make(dev, true);
+        ws.make(dev, true, stream);
         return molora_apply_batched(pr.d, pr.P, pr.dt, pr.N, (int32_t)pr.C, offsets, perm, ws.p, ws.n, status, stream);
     });
     Py_RETURN_NONE;
@@ -419,8 +431,8 @@ PyObject* group_apply_batched(PyObject* const* a)
     uint32_t* status = status_word(a[7]);
     void* stream = stream_of(a[8]);
     call("molora_group_apply_batched", [&] {
-        int32_t *c = counts.get(), *o = offsets.get(), *p = perm.get();
-        ws.make(dev, true);
+        int32_t *c = counts.get(stream), *o = offsets.get(stream), *p = perm.get(stream);
+        ws.make(dev, true, stream);
         return molora_group_apply_batched(i32(r), pr.N, (int32_t)C, c, o, p, pr.d, pr.P, pr.dt, ws.p, ws.n, status, stream);
     });
     return tuple_of({counts.t, offsets.t, perm.t});
@@ -436,8 +448,8 @@ PyObject* topk_softmax(PyObject* const* a)
     void* stream = stream_of(a[2]);
     at::Tensor idx, w;
     call("molora_topk_softmax", [&] {
-        idx = at::empty({k, N}, at::TensorOptions().dtype(at::kInt).device(z.device()));
-        w = at::empty({k, N}, at::TensorOptions().dtype(at::kFloat).device(z.device()));
+        idx = allocate(stream, [&] { return at::empty({k, N}, at::TensorOptions().dtype(at::kInt).device(z.device())); });
+        w = allocate(stream, [&] { return at::empty({k, N}, at::TensorOptions().dtype(at::kFloat).device(z.device())); });
         return molora_topk_softmax(static_cast<const float*>(z.data_ptr()), N, (int32_t)z.size(1), (int32_t)k, i32(idx),
                                    static_cast<float*>(w.data_ptr()), stream);
     });
@@ -459,9 +471,9 @@ PyObject* apply_topk(PyObject* const* a)
     void* stream = stream_of(a[6]);
     at::Tensor idx, w;
     call("molora_apply_topk", [&] {
-        idx = idx0.contiguous();
-        w = w0.contiguous();
-        ws.make(idx.device(), zero);        // (only the apply part has to start cleared, and only where a kernel keeps control words in it)
+        idx = allocate(stream, [&] { return idx0.contiguous(); });
+        w = allocate(stream, [&] { return w0.contiguous(); });
+        ws.make(idx.device(), zero, stream);        // (only the apply part has to start cleared, and only where a kernel keeps control words in it)
         const size_t off = std::min((size_t)(-(intptr_t)ws.p) % 256, ws.n);      // (a shorter workspace is refused as too small)
         return molora_apply_topk(pr.d, pr.P, pr.dt, pr.N, (int32_t)C, (int32_t)idx.size(0), i32(idx), static_cast<const float*>(w.data_ptr()),
                                  static_cast<char*>(ws.p) + off, ws.n - off, status, stream);

@@ -57,3 +57,50 @@ def test_other_threads_run_while_a_call_waits_for_the_launch_queue():
     torch.cuda.synchronize()
     assert last - start > 0.3, "the queue never filled"
     assert longest < 0.15
+
+
+@pytest.mark.parametrize("raw", [False, True])
+def test_what_a_call_allocates_belongs_to_its_stream(raw):
+    """Memory freed on the current stream is still read there when a call on another stream asks for an output of that size."""
+    N = 1 << 20
+    ids, breaks = torch.zeros(N, dtype=torch.int32, device="cuda"), torch.tensor([0, 5], dtype=torch.int32, device="cuda")
+    side = torch.cuda.Stream()
+    freed = torch.full((N,), 7, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    torch.cuda._sleep(200_000_000)
+    copy = freed.clone()
+    del freed
+    r = M.molora_route_vocab(ids, breaks, stream=side.cuda_stream if raw else side)
+    side.synchronize()
+    assert not r.any()
+    assert (copy == 7).all()
+
+
+def test_callers_outputs_stream_and_workspace_are_used():
+    N, C = 300, 5
+    r = torch.randint(0, C, (N,), dtype=torch.int32, device="cuda")
+    x, y = torch.randn(N, 512, device="cuda").bfloat16(), torch.randn(N, 256, device="cuda").bfloat16()
+    A, B = torch.randn(C, 512, 64, device="cuda").bfloat16() * 0.05, torch.randn(C, 64, 256, device="cuda").bfloat16() * 0.1
+    want = y.clone()
+    M.molora_group_apply_batched(r, [M.ProjDesc(x, want, A, B)])
+    counts, offsets, perm = (torch.full((n,), -9, dtype=torch.int32, device="cuda") for n in (C, C + 1, N))
+    need = M.molora_apply_workspace_bytes(N, C, 512, 256, 64)
+    assert need > 0
+    ws = torch.full((need,), 255, dtype=torch.uint8, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(100_000_000)
+    got = M.molora_group_apply_batched(r, [M.ProjDesc(x, y, A, B)], counts=counts, offsets=offsets, perm=perm, ws=ws, stream=side)
+    assert got[0] is counts and got[1] is offsets and got[2] is perm
+    assert not side.query() and bool((counts == -9).all())         # it waits for what is ahead of it on that stream
+    side.synchronize()
+    assert torch.equal(y, want) and torch.equal(counts, torch.bincount(r, minlength=C).int()) and not bool((ws == 255).all())
+    with pytest.raises(M.MoloraError, match="workspace"):
+        M.molora_group_apply_batched(r, [M.ProjDesc(x, y, A, B)], ws=ws[:need - 16])
+    ids, breaks = torch.arange(N, dtype=torch.int32, device="cuda"), torch.tensor([0, 100, 300], dtype=torch.int32, device="cuda")
+    out = torch.full((N,), -9, dtype=torch.int32, device="cuda")
+    assert M.molora_route_vocab(ids, breaks, r_out=out) is out and int(out.sum()) == 200
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    M.molora_route_vocab(ids + 1, breaks, r_out=out, dev_status=status)
+    assert int(status) == 1 and int(out[-1]) == -1
