@@ -88,9 +88,10 @@ def test_callers_outputs_stream_and_workspace_are_used():
     assert need > 0
     ws = torch.full((need,), 255, dtype=torch.uint8, device="cuda")
     side = torch.cuda.Stream()
+    assert bool((counts == -9).all())                              # (its kernels are loaded before the time counts)
     torch.cuda.synchronize()
     with torch.cuda.stream(side):
-        torch.cuda._sleep(100_000_000)
+        torch.cuda._sleep(400_000_000)
     got = M.molora_group_apply_batched(r, [M.ProjDesc(x, y, A, B)], counts=counts, offsets=offsets, perm=perm, ws=ws, stream=side)
     assert got[0] is counts and got[1] is offsets and got[2] is perm
     assert not side.query() and bool((counts == -9).all())         # it waits for what is ahead of it on that stream
