@@ -18,7 +18,7 @@ from typing import List, Optional, Sequence, Tuple
 
 import torch
 
-from .build import LIB_PATH, MARSHAL_PATH, ROOT
+from .build import LIB_PATH, MARSHAL_PATH, ROOT, marshal_abi, marshal_built_for
 
 F32, BF16 = 0, 1
 MAX_ADAPTERS = 256
@@ -158,6 +158,9 @@ def _load_marshal():
     load_library()
     if not os.path.exists(MARSHAL_PATH):
         raise ImportError(f"{MARSHAL_PATH} is missing: run `python -m paper_2603_15965_b200.build` (there is no fallback)")
+    built_for = marshal_built_for()
+    if built_for and built_for != marshal_abi():
+        raise ImportError(f"{MARSHAL_PATH} was built for {built_for}, this is {marshal_abi()}: run `python -m paper_2603_15965_b200.build`")
     from . import _marshal as extension
     extension.bind(_check)
     _marshal = extension

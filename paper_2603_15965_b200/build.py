@@ -13,6 +13,7 @@ ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libmolora.so")
 MARSHAL_PATH = os.path.join(PKG_DIR, "_marshal.so")
+MARSHAL_ABI_PATH = os.path.join(PKG_DIR, "_marshal.abi")      # what the extension was built for, written beside it
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--threads", "0", "-I", os.path.join(ROOT, "include")]
@@ -30,11 +31,26 @@ def _stale() -> bool:
     return any(os.path.getmtime(p) > built for p in deps)
 
 
+def marshal_abi() -> str:
+    """The interpreter and the torch whose C++ interfaces the extension is compiled against."""
+    import torch
+    return f"{sys.implementation.cache_tag} torch {torch.__version__} cxx11abi {int(torch._C._GLIBCXX_USE_CXX11_ABI)}"
+
+
+def marshal_built_for() -> str:
+    """What marshal_abi() was when the extension was built; empty if that is not known."""
+    if not os.path.exists(MARSHAL_ABI_PATH):
+        return ""
+    with open(MARSHAL_ABI_PATH) as f:
+        return f.read().strip()
+
+
 def build_marshal(force: bool = False) -> str:
     """Compile csrc/marshal.cpp into _marshal.so beside the library it links to (no GPU, no nvcc)."""
     src = os.path.join(CSRC, "marshal.cpp")
     deps = [src] + glob.glob(os.path.join(ROOT, "include", "*.h"))
-    if not force and os.path.exists(MARSHAL_PATH) and all(os.path.getmtime(p) <= os.path.getmtime(MARSHAL_PATH) for p in deps):
+    if (not force and os.path.exists(MARSHAL_PATH) and marshal_built_for() == marshal_abi()
+            and all(os.path.getmtime(p) <= os.path.getmtime(MARSHAL_PATH) for p in deps)):
         return MARSHAL_PATH
     import torch
     torch_dir = os.path.dirname(torch.__file__)
@@ -50,6 +66,8 @@ def build_marshal(force: bool = False) -> str:
     if res.returncode != 0:
         raise RuntimeError("g++ failed:\n" + res.stdout + res.stderr)
     os.replace(tmp, MARSHAL_PATH)
+    with open(MARSHAL_ABI_PATH, "w") as f:
+        f.write(marshal_abi() + "\n")
     return MARSHAL_PATH
 
 
