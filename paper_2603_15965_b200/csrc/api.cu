@@ -319,7 +319,10 @@ size_t molora_apply_workspace_bytes(int64_t N, int32_t C, int32_t d_in, int32_t 
     // two-launch kernels: needed unless the tcgen05 kernel is certain to take every segment (for ranks 16 and 32 that
     // depends on the other projections of the call, which are not known here)
     const int64_t forced = forced_umma_min_tokens();
-    const bool umma_certain = forced > 0 ? N >= forced : (rank == 64 && use_umma_r64(N, C, proj_bytes(N, d_in, d_out), 1));
+    // (of more than two projections fewer go to the tcgen05 kernel; by default the others stream and need nothing, but "small_path"
+    // may send them to the two-launch kernels)
+    const double own = proj_bytes(N, d_in, d_out);
+    const bool umma_certain = forced > 0 ? N >= forced : (rank == 64 && use_umma_r64(N, C, own, 1) && (small != 2 || use_umma_r64(N, C, own, 3)));
     if (umma_certain && C <= kUmmaAllSegmentsMaxC && (d_in % 64) == 0 && (d_out % 64) == 0) return need;
     return need + decode_workspace_bytes(N, d_in, rank);
 }
