@@ -449,8 +449,11 @@ molora_status_t launch_route_mlp(const void* x, molora_dtype_t xdt, int64_t N, i
 {
     if (N == 0 && image != kImageBuildOnly) return MOLORA_OK;
     const bool room = ws != nullptr && ws_bytes >= route_mlp_workspace_bytes(xdt, d, H) && aligned16(ws);
-    // (below 128 tokens the images are optional: without room for them the call runs on the CUDA cores)
-    if (mlp_umma_eligible(xdt, image == kImageBuildOnly ? 128 : N, d, H) && (room || image == kImageBuildOnly || N >= 128)) {
+    // Below 128 tokens the images are optional: without room for them the call runs on the CUDA cores, as do routers so small that
+    // building the images costs more than it saves (us, CUDA cores / both launches: 64 -> 16 hidden units, 16 tokens 6.9 / 7.9; 128 -> 16:
+    // 8.4 / 8.2; 64 -> 64: 25 / 12; with images built before 6.9 / 6.4).
+    const bool tiny = image == kImageBuildAndUse && N < 128 && (int64_t)std::max(H, 16) * d <= 1024;
+    if (mlp_umma_eligible(xdt, image == kImageBuildOnly ? 128 : N, d, H) && !tiny && (room || image == kImageBuildOnly || N >= 128)) {
         if (ws == nullptr || ws_bytes < route_mlp_workspace_bytes(xdt, d, H) || !aligned16(ws)) return MOLORA_ERR_WORKSPACE;
         return H <= 64 ? mlp_umma_launch<64>(x, N, d, ldx, W1, b1, H, W2, b2, C, r_out, logits_out, ws, dev_status, s, image)
                        : mlp_umma_launch<128>(x, N, d, ldx, W1, b1, H, W2, b2, C, r_out, logits_out, ws, dev_status, s, image);

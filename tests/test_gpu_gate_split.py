@@ -90,3 +90,23 @@ def test_mlp_router_of_small_calls(N, d, H):
     r_ref, z_ref, margin = oracle.route_mlp(x, W1, b1, W2, b2)
     np.testing.assert_allclose(z.cpu().numpy(), z_ref, rtol=0, atol=1e-5 * max(1.0, np.abs(z_ref).max()))
     assert np.array_equal(r.cpu().numpy()[margin >= 1e-3], r_ref[margin >= 1e-3])
+
+
+@pytest.mark.parametrize("N,d,H,launches", [(1, 64, 16, 1), (127, 64, 16, 1), (128, 64, 16, 2), (127, 64, 17, 2), (127, 128, 16, 2), (127, 128, 8, 2), (127, 64, 8, 1)])
+def test_mlp_router_on_both_sides_of_the_tiny_rule(N, d, H, launches):
+    C = 4
+    rng = np.random.default_rng(N + H)
+    x = W.round_to_bf16(rng.standard_normal((N, d), dtype=np.float32))
+    W1 = (rng.standard_normal((d, H)) * d ** -0.5).astype(np.float32)
+    W2 = (rng.standard_normal((H, C)) * H ** -0.5).astype(np.float32)
+    xd, W1d, W2d = dev_tensor(x, "bf16"), dev_tensor(W1, "f32"), dev_tensor(W2, "f32")
+    z = torch.empty(N, C, dtype=torch.float32, device="cuda")
+    before = M.molora_launch_count()
+    r = M.molora_route_mlp(xd, W1d, None, W2d, None, logits_out=z)
+    assert M.molora_launch_count() - before == launches
+    r_ref, z_ref, margin = oracle.route_mlp(x, W1, None, W2, None)
+    np.testing.assert_allclose(z.cpu().numpy(), z_ref, rtol=0, atol=1e-5 * max(1.0, np.abs(z_ref).max()))
+    assert np.array_equal(r.cpu().numpy()[margin >= 1e-3], r_ref[margin >= 1e-3])
+    prepared = M.molora_route_mlp_prepare(xd.dtype, W1d, C)
+    assert torch.equal(M.molora_route_mlp(xd, W1d, None, W2d, None, prepared=prepared)[torch.from_numpy(margin >= 1e-3).cuda()],
+                       r[torch.from_numpy(margin >= 1e-3).cuda()])
