@@ -224,10 +224,8 @@ __global__ void __launch_bounds__(WARPS * 32) route_gate_mma_kernel(const __nv_b
 // more): all operands go from global memory straight into registers in one round trip, the partial logits are summed in
 // warp order in shared memory and in rank order through distributed shared memory.  Bound by one load round trip and the
 // launch.  Measured (us, before -> after): 93 tokens x 4096, C = 16: 34.4 -> 5.7; 777 x 2048, C = 8: 12.0 -> 4.7.
-// Every 16 tokens read the whole weight image (L2), so large calls keep the tcgen05 gate or the kernel above; the line lies
-// where they meet (us, tcgen05 / here, image built before): 8 adapters 1500 x 2048 8.0 / 4.9, 2300 x 2048 8.4 / 5.1, 4000 x
-// 2048 8.8 / 9.5, 1500 x 4096 10.5 / 9.7, 2300 x 4096 10.8 / 12.5; 16 adapters 2300 x 2048 8.8 / 6.7, 1500 x 4096 10.9 /
-// 12.1; 32 adapters 1500 x 2048 11.9 / 13.5.
+// Every 16 tokens read the whole weight image (L2), and a second wave of CTAs costs as much as the first; gate_split_preferred says
+// which of the larger calls it still takes.
 constexpr int kGateSplitWarps = 8;
 template <int NT, int KC>
 __global__ void __launch_bounds__(kGateSplitWarps * 32, 2)
@@ -348,10 +346,25 @@ __global__ void __launch_bounds__(kGateSplitWarps * 32, 2)
     if (S > 1) ptx::cluster_sync_all();                              // rank 0 has read this CTA's sums
 }
 
+// CTAs of a cluster: one k chunk per warp, as far as that goes
+static int gate_split_ctas(int chunks)
+{
+    int S = 1;
+    while (S < 8 && S * kGateSplitWarps < chunks) S *= 2;
+    return S;
+}
+
+// From 1024 tokens on the tcgen05 gate can take the call.  With up to 16 adapters this kernel is the faster one while its CTAs, two
+// to an SM, are resident at once, which ends at 4736 tokens for d <= 1024, 2368 for d <= 2048, 1184 for d <= 4096 (us here / tcgen05,
+// image built before, 8 adapters: d = 64, 4500 tokens 3.6 / 4.1, 5000 4.6 / 4.1; d = 1024, 4500 5.1 / 7.7; d = 2048, 2200 5.7 / 8.7,
+// 2600 9.3 / 8.7; d = 3072, 1800 10.6 / 9.8; 16 adapters, d = 4096: 1024 8.4 / 11.3, 1400 12.7 / 11.3).  With up to 8 adapters a
+// second wave still pays for some widths: d = 1024, 5000 tokens 6.7 / 7.7, 6000 7.2 / 7.7; d = 4096, 1400 10.3 / 11.3.
 bool gate_split_preferred(int64_t N, int32_t d, int32_t C)
 {
     if (N < 1024) return true;
-    return C <= 16 && N * d <= (C <= 8 ? 6500000 : 5000000);
+    if (C > 16) return false;
+    if (ceil_div64(N, 16) * gate_split_ctas((d + 127) / 128) <= 2 * sm_count()) return true;
+    return C <= 8 && N <= 6000 && N * d <= 6500000 && ((d >= 512 && d <= 1024) || d >= 4096);
 }
 
 template <int NT, int WARPS, int KC>
@@ -370,8 +383,7 @@ static molora_status_t gate_mma_launch(const void* x, int64_t N, int d, int64_t 
     }
     if (image == kImageBuildOnly) return MOLORA_OK;
     if (gate_split_preferred(N, d, C)) {
-        int S = 1;
-        while (S < 8 && S * kGateSplitWarps < chunks) S *= 2;
+        const int S = gate_split_ctas(chunks);
         return cuda_ok(launch_kernel(route_gate_split_kernel<NT, KC>, dim3((unsigned)(ceil_div64(N, 16) * S)), dim3(kGateSplitWarps * 32), 0,
                                      s, (unsigned)S, image == kImageBuildAndUse, static_cast<const __nv_bfloat16*>(x), N, d, ldx, img, bias,
                                      C, r_out, logits_out));
