@@ -358,13 +358,13 @@ static int gate_split_ctas(int chunks)
 // to an SM, are resident at once, which ends at 4736 tokens for d <= 1024, 2368 for d <= 2048, 1184 for d <= 4096 (us here / tcgen05,
 // image built before, 8 adapters: d = 64, 4500 tokens 3.6 / 4.1, 5000 4.6 / 4.1; d = 1024, 4500 5.1 / 7.7; d = 2048, 2200 5.7 / 8.7,
 // 2600 9.3 / 8.7; d = 3072, 1800 10.6 / 9.8; 16 adapters, d = 4096: 1024 8.4 / 11.3, 1400 12.7 / 11.3).  With up to 8 adapters a
-// second wave still pays for some widths: d = 1024, 5000 tokens 6.7 / 7.7, 6000 7.2 / 7.7; d = 4096, 1400 10.3 / 11.3.
+// second wave still pays for some widths: d = 768, 8000 tokens 6.7 / 7.7; d = 1024, 5000 6.7 / 7.7; d = 4096, 1400 10.3 / 11.3.
 bool gate_split_preferred(int64_t N, int32_t d, int32_t C)
 {
     if (N < 1024) return true;
     if (C > 16) return false;
     if (ceil_div64(N, 16) * gate_split_ctas((d + 127) / 128) <= 2 * sm_count()) return true;
-    return C <= 8 && N <= 6000 && N * d <= 6500000 && ((d >= 512 && d <= 1024) || d >= 4096);
+    return C <= 8 && N <= 8000 && N * d <= 6500000 && ((d >= 512 && d <= 1024) || d >= 4096);
 }
 
 template <int NT, int WARPS, int KC>

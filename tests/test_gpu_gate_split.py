@@ -40,7 +40,7 @@ def test_small_call_gate_matches_oracle(N, d, C):
 @pytest.mark.parametrize("N,d,C", [(1024, 2048, 8), (3173, 2048, 8), (3174, 2048, 8), (2441, 2048, 16), (2442, 2048, 16), (1500, 64, 17),
                                    # one wave of clusters of 1, 2 and 4 CTAs, the second wave of up to 8 adapters, and what lies past either
                                    (4736, 64, 8), (4737, 64, 8), (4736, 64, 16), (4737, 192, 16), (2368, 2048, 8), (2369, 2048, 8), (1184, 4096, 16),
-                                   (1185, 4096, 16), (1185, 4096, 8), (6000, 512, 8), (6001, 512, 8), (16000, 64, 5)])
+                                   (1185, 4096, 16), (1185, 4096, 8), (8000, 512, 8), (8001, 512, 8), (16000, 64, 5)])
 def test_both_sides_of_the_small_call_rule(N, d, C):
     rng = np.random.default_rng(N + C)
     x = W.round_to_bf16(rng.standard_normal((N, d), dtype=np.float32))
