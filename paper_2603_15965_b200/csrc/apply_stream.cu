@@ -50,6 +50,7 @@
 #include <stdlib.h>
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "common.cuh"
@@ -687,6 +688,30 @@ bool stream_eligible(const molora_proj_desc_t& p, molora_dtype_t dt)
     return dt == MOLORA_BF16 && (p.rank == 16 || p.rank == 32 || p.rank == 64) && (p.d_in % 32) == 0 && (p.d_out % 32) == 0;
 }
 
+// Output slices: one item per (projection, tile) to start with; while `most` units (items per tile) allow it, the widest is split once
+// more (a second round of items costs more than the imbalance it removes).  Returns the number of units.
+static int slice_outputs(const StreamParams& prm, int CH, int64_t most, int32_t* och, int32_t* ustart)
+{
+    int slices[MOLORA_MAX_PROJECTIONS], chunks[MOLORA_MAX_PROJECTIONS], total = prm.P;
+    for (int i = 0; i < prm.P; ++i) {
+        och[i] = chunks[i] = ceil_div(prm.p[i].d_out, CH);
+        slices[i] = 1;
+    }
+    for (; total + 1 <= most; ++total) {
+        int widest = 0;
+        for (int i = 1; i < prm.P; ++i)
+            if (och[i] > och[widest]) widest = i;
+        if (och[widest] <= 1) break;
+        och[widest] = ceil_div(chunks[widest], ++slices[widest]);
+    }
+    ustart[0] = 0;
+    for (int i = 0; i < prm.P; ++i) ustart[i + 1] = ustart[i] + ceil_div(chunks[i], och[i]);
+    return ustart[prm.P];
+}
+
+// most tiles that `rows` rows in C segments can give (every segment that has rows adds at most one partial tile)
+static int64_t tiles_bound(int64_t rows, int64_t C, int tile_rows) { return std::min(rows, ceil_div64(rows, tile_rows) + std::min(C, rows)); }
+
 template <int R, bool GROUP, bool SHORT, int V>
 static cudaError_t stream_launch(StreamParams prm, [[maybe_unused]] const StreamMaps& maps, int64_t tiles_max, int S, cudaStream_t s)
 {
@@ -711,29 +736,7 @@ static cudaError_t stream_launch(StreamParams prm, [[maybe_unused]] const Stream
         if (e != cudaSuccess) return e;
         clusters = std::max(1, n);
     }
-    // Output slices (S = 1): start with one item per (projection, tile); while the items certainly fit into one wave, split
-    // the widest once more.  A second round of items costs more than the imbalance it removes.
-    int slices[MOLORA_MAX_PROJECTIONS], chunks[MOLORA_MAX_PROJECTIONS], total = prm.P;
-    for (int i = 0; i < prm.P; ++i) {
-        chunks[i] = ceil_div(prm.p[i].d_out, Cfg::CH);
-        slices[i] = 1;
-    }
-    while (S == 1) {
-        int widest = -1, width = 1;
-        for (int i = 0; i < prm.P; ++i)
-            if (ceil_div(chunks[i], slices[i]) > width) {
-                width = ceil_div(chunks[i], slices[i]);
-                widest = i;
-            }
-        if (widest < 0 || tiles_max * (total + 1) > clusters) break;
-        ++slices[widest];
-        ++total;
-    }
-    prm.ustart[0] = 0;
-    for (int i = 0; i < prm.P; ++i) {
-        prm.och[i] = ceil_div(chunks[i], slices[i]);
-        prm.ustart[i + 1] = prm.ustart[i] + ceil_div(chunks[i], prm.och[i]);
-    }
+    prm.ustart[prm.P] = slice_outputs(prm, Cfg::CH, S == 1 ? clusters / tiles_max : 0, prm.och, prm.ustart);
     const unsigned grid = (unsigned)(std::max<int64_t>(1, std::min<int64_t>(tiles_max * prm.ustart[prm.P], clusters)) * S);
     FsArgs<R, SHORT, V> args;
     static_cast<StreamParams&>(args) = prm;
@@ -742,16 +745,25 @@ static cudaError_t stream_launch(StreamParams prm, [[maybe_unused]] const Stream
 }
 
 // Estimated time of a launch (us, without its fixed part) and the CTAs per item that give it.  A launch lasts as long as its
-// busiest cluster: `tiles` items per projection, each of nks + ne chunk jobs spread over S CTAs, on sms / S clusters (a few
-// SMs are lost to S = 4 and 8: clusters do not straddle a GPC).  The exchange of t costs an item about 1.25 jobs.  A chunk job
-// costs 1.42 us with 16 x 1024 and 1.19 us with 32 x 512 elements of x or y (rank 16), 1.17 / 1.72 us (rank 32, 512 columns),
-// 1.02 / 1.67 us (rank 64, 256 columns), fitted to one projection of 300 - 8000 tokens and layers of 8 - 1000 tokens.
+// busiest cluster: `tiles` items per projection (and slice), each of nks + ne chunk jobs spread over S CTAs, on sms / S clusters (a few
+// SMs are lost to S = 4 and 8: clusters do not straddle a GPC).  The exchange of t costs an item about 2.25 jobs.  A chunk job
+// costs 1.30 us with 16 x 1024 and 1.19 us with 32 x 512 elements of x or y (rank 16), 1.17 / 1.72 us (rank 32, 512 columns),
+// 0.90 / 1.67 us (rank 64, 256 columns), fitted to one projection of 300 - 8000 tokens and layers of 8 - 1000 tokens; a third of it
+// does not depend on the chunk's width.  Against an estimate that knew neither slices nor partial chunks and counted half a tile
+// for every segment, us: rank 16, 512 wide, 200 tokens, four projections 8.2 -> 7.2; rank 32, 1536 wide, 1 token, two projections
+// 13.6 -> 11.0; rank 32, 2048 wide, 2500 tokens, one projection 19.5 -> 17.0.
 template <int R, bool SHORT>
 static double stream_estimate(const StreamParams& prm, int64_t rows, int& split)
 {
     using Cfg = FsCfg<R, SHORT, (SHORT && R >= 32 ? kFsCluster : kFsOne)>;
-    const double job_us = R == 16 ? (SHORT ? 1.42 : 1.19) : R == 32 ? (SHORT ? 1.17 : 1.72) : (SHORT ? 1.02 : 1.67);
-    const double tiles = (double)(ceil_div64(rows, Cfg::ROWS) + std::min<int64_t>(prm.C, rows) / 2);    // half a tile lost per segment
+    const double job_us = R == 16 ? (SHORT ? 1.30 : 1.19) : R == 32 ? (SHORT ? 1.17 : 1.72) : (SHORT ? 0.90 : 1.67);
+    // tiles of segments of about equal size: one each while that is well below a tile's height, half a tile lost per segment from there on
+    const double segments = (double)std::min<int64_t>(prm.C, rows), fill = (double)rows / segments / Cfg::ROWS;
+    const double tiles = segments * (fill <= 0.75 ? 1.0 : fill <= 1.0 ? 1.0 + 2.0 * (fill - 0.75) : fill + 0.5);
+    auto jobs = [](int width) {            // jobs that `width` columns cost
+        const int full = width / Cfg::CH, rest = width % Cfg::CH;
+        return full + (rest > 0 ? 0.35 + 0.65 * rest / Cfg::CH : 0.0);
+    };
     int most = Cfg::MAXS;
     for (int i = 0; i < prm.P; ++i) most = std::min(most, ceil_div(prm.p[i].d_in, Cfg::CH));      // every CTA shrinks something
     const int64_t forced = tune(kTuneStreamSplit);
@@ -759,15 +771,21 @@ static double stream_estimate(const StreamParams& prm, int64_t rows, int& split)
     double best = 1e30;
     for (int S = 1; S <= most; S *= 2) {
         const double clusters = S <= 2 ? sms / S : S == 4 ? sms * 0.9 / 4 : sms * 0.86 / 8;
+        int32_t och[MOLORA_MAX_PROJECTIONS], ustart[MOLORA_MAX_PROJECTIONS + 1];
+        const int units = slice_outputs(prm, Cfg::CH, S == 1 ? sms / tiles_bound(rows, prm.C, Cfg::ROWS) : 0, och, ustart);
         double sum = 0.0, longest = 0.0;
         for (int i = 0; i < prm.P; ++i) {
-            const double jobs = ceil_div(ceil_div(prm.p[i].d_in, Cfg::CH), S) + ceil_div(ceil_div(prm.p[i].d_out, Cfg::CH), S) + (S > 1 ? 1.25 : 0.0);
-            sum += jobs;
-            longest = std::max(longest, jobs);
+            // (the CTAs of a cluster take whole chunks: the first one has the most)
+            const int in = S == 1 ? prm.p[i].d_in : std::min(prm.p[i].d_in, ceil_div(ceil_div(prm.p[i].d_in, Cfg::CH), S) * Cfg::CH);
+            const int out = std::min(prm.p[i].d_out, ceil_div(och[i], S) * Cfg::CH);
+            const double each = jobs(in) + jobs(out) + (S > 1 ? 2.25 : 0.0);
+            sum += each * (ustart[i + 1] - ustart[i]);
+            longest = std::max(longest, each);
         }
         double t = longest;
-        if (tiles * prm.P > clusters) t = std::max(longest, sum * tiles / clusters + 0.5 * sum / prm.P);
-        t += S == 1 ? 0.0 : S == 2 ? 1.0 : S == 4 ? 1.5 : 2.0;
+        if (units == 1) t = longest * std::ceil(tiles / clusters);        // equal items, dealt in whole rounds
+        else if (tiles * units > clusters) t = std::max(longest, sum * tiles / clusters + 0.15 * sum / units);
+        t += S == 1 ? 0.0 : S == 2 ? 1.5 : S == 4 ? 2.25 : 3.0;
         if (forced > 0 ? S <= forced : t < best) {
             best = t;
             split = S;
@@ -813,7 +831,7 @@ static cudaError_t stream_rank(const molora_proj_desc_t* projs, int32_t P, int64
             return cudaErrorInvalidValue;
     }
     const int rows = small ? 16 : 32;
-    const int64_t tiles_max = ceil_div64(cap_rows, rows) + prm.C;
+    const int64_t tiles_max = tiles_bound(cap_rows, prm.C, rows);
     const int S = small ? split16 : split32;
     auto launch = [&](auto tile, auto variant) {
         constexpr bool SHORT = decltype(tile)::value;

@@ -1,0 +1,32 @@
+"""Calls on both sides of the rules that choose kernel, tile and cluster from the sizes, against the CPU oracle: the library's own
+choice throughout, several projections in one call, tokens spread evenly over the adapters."""
+import numpy as np
+import pytest
+
+from paper_2603_15965_b200 import workloads as W
+
+from _harness import run_and_check
+
+pytestmark = pytest.mark.gpu
+
+
+def check(N, C, shapes, rank, rows=150):
+    rng = np.random.default_rng(N + C + rank)
+    r = rng.permutation(N).astype(np.int32) % C
+    parts = [W.random_problem(N + C + i, N, C, a, b, rank, "bf16", r=r) for i, (a, b) in enumerate(shapes)]
+    w = parts[0]
+    for i, p in enumerate(parts):
+        p.projections[0].x_key, p.projections[0].name = f"x{i}", f"proj{i}"
+    w = W.Workload(name=f"choice-{N}-{C}-{rank}", N=N, C=C, dtype="bf16", router="given", inputs={f"x{i}": p.inputs["x"] for i, p in enumerate(parts)},
+                   projections=[p.projections[0] for p in parts], r=r)
+    run_and_check(w, rows=None if N <= rows else rng.choice(N, rows, replace=False), batched=True)
+
+
+@pytest.mark.parametrize("N,C,shapes,rank", [
+    # streaming kernel: output slices of one projection and of several, 16- and 32-row tiles, chunks that are partly empty
+    (1, 1, [(1536, 1536), (1536, 4608)], 32), (1, 16, [(512, 512)], 16), (32, 4, [(512, 512), (512, 128)], 16),
+    (200, 4, [(512, 512), (512, 128), (512, 512)], 16), (2500, 8, [(1024, 1024)], 32), (1500, 1, [(1024, 1024), (1024, 3072)], 16),
+    (6000, 256, [(512, 512), (512, 256)], 16), (1500, 64, [(1536, 384), (1536, 1536)], 16),
+])
+def test_tiles_slices_and_clusters(N, C, shapes, rank):
+    check(N, C, shapes, rank)
