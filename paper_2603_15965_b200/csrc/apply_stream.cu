@@ -108,7 +108,7 @@ __device__ __forceinline__ int fs_part_adapter(const StreamParams& prm, const ui
 // the launches of ~10 us about 0.6 us.
 enum FsVariant : int {
     kFsOne = 0,        // one CTA per item
-    kFsLinear = 1,     // ... and no tensor maps, whose first use costs ~0.5 us (rank 16, short tiles, short items)
+    kFsLinear = 1,     // ... and no tensor maps, whose first use costs ~0.5 us (rank 16, short tiles, items of at most seven jobs)
     kFsCluster = 2,    // 2 to 8 CTAs per item (ranks 32 and 64, short tiles)
 };
 template <int R, bool SHORT, int V>
@@ -815,11 +815,12 @@ static cudaError_t stream_rank(const molora_proj_desc_t* projs, int32_t P, int64
     using Short = FsCfg<R, true, kFsOne>;
     const int pr = R / prm.parts, ch = small ? Short::CH : FsCfg<R, false, kFsOne>::CH;
     StreamMaps maps;
-    // linear weights while no item has more than four chunk jobs (256 tokens, 8 adapters, a layer: hidden 512 (3 jobs) 7.8 us
-    // linear / 8.4 boxes; 2048 (8 jobs) 14.9 / 14.4; 4096 (16 jobs) 24.5 / 22.4)
+    // linear weights while no item has more than seven chunk jobs (us, linear / boxes; 256 tokens, 8 adapters, a layer: hidden 512 (3 jobs)
+    // 7.8 / 8.4, 2048 (8 jobs) 14.9 / 14.4, 4096 (16 jobs) 24.5 / 22.4; 1536 wide, two projections (7 jobs) 7.2 / 7.7 at 1 token, 8.2 / 8.7
+    // at 200)
     int jobs = 0;
     for (int i = 0; i < n; ++i) jobs = std::max(jobs, ceil_div(prm.p[i].d_in, ch) + ceil_div(prm.p[i].d_out, ch));
-    const bool box = !(R == 16 && small && jobs <= 4);
+    const bool box = !(R == 16 && small && jobs <= 7);
     for (int i = 0; i < n && box; ++i) {
         if (!make_tensor_map_bf16_2d(&maps.tm_a[i], prm.p[i].A, 64, (uint64_t)prm.n_adapters * prm.p[i].d_in * pr / 64, 64, 64,
                                      (uint32_t)(ch * pr / 64), CU_TENSOR_MAP_SWIZZLE_128B))

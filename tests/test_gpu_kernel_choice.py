@@ -30,3 +30,9 @@ def check(N, C, shapes, rank, rows=150):
 ])
 def test_tiles_slices_and_clusters(N, C, shapes, rank):
     check(N, C, shapes, rank)
+
+
+@pytest.mark.parametrize("d_in,d_out", [(1536, 5120), (2080, 4096), (1056, 5152), (2048, 6144)])
+def test_linear_and_boxed_weights(d_in, d_out):
+    """rank 16, short tiles: seven chunk jobs an item and eight, whole and ragged chunks"""
+    check(60, 5, [(d_in, d_out)], 16)
