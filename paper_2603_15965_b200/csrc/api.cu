@@ -92,16 +92,17 @@ bool use_umma(int32_t rank, int64_t N, int32_t C, double group_bytes, int same_r
     return group_bytes >= (same_rank == 1 ? kUmmaMinBytesR32 : kUmmaMinBytesR32More) && N >= (int64_t)C * 160;
 }
 // the kernel for what the tcgen05 kernel does not take; same_rank: projections of this rank in the call (0: unknown)
-bool small_path_is_stream(int32_t rank, int64_t N, int same_rank)
+bool small_path_is_stream(int32_t rank, int64_t N, int32_t C, int same_rank)
 {
     if (const int64_t forced = tune(kTuneSmallPath)) {
         if (forced == 1) return true;
         if (forced == 2) return false;
     }
-    (void)N;
     // rank 64: the two-launch pair for one or two projections (its split of the reduction over CTAs pays there);
-    // with a layer's worth of them its items no longer fit a wave and the streaming kernel is faster
-    return rank == 16 || rank == 32 || same_rank > 2;
+    // with a layer's worth of them its items no longer fit a wave and the streaming kernel is faster, as it is for calls of more than
+    // 64 adapters with 24 to 64 tokens each, where the pair sends every row's partials through the workspace (us, pair / streaming:
+    // 256 adapters, 16000 tokens, 4096 wide, one projection 393 / 199, two 1143 / 570; 8000 tokens, 2048 wide 119 / 77)
+    return rank == 16 || rank == 32 || same_rank > 2 || (same_rank > 0 && C > kUmmaAllSegmentsMaxC && N >= (int64_t)C * 24);
 }
 
 // The job-list kernel shares chunk-sized jobs between all CTAs instead of giving every (tile, projection) pair to one cluster.
@@ -315,7 +316,7 @@ size_t molora_apply_workspace_bytes(int64_t N, int32_t C, int32_t d_in, int32_t 
     if (jobs_eligible(probe, MOLORA_BF16, N) && (small == 3 || (small == 0 && rank == 16 && N > 256)))
         need += jobs_control_bytes() + jobs_partial_bytes(N, C, d_in, rank);
     if (small == 3 && need > 0) return need;
-    if (small_path_is_stream(rank, N, 0)) return need;
+    if (small_path_is_stream(rank, N, C, 0)) return need;
     // two-launch kernels: needed unless the tcgen05 kernel is certain to take every segment (for ranks 16 and 32 that
     // depends on the other projections of the call, which are not known here)
     const int64_t forced = forced_umma_min_tokens();
@@ -369,7 +370,7 @@ molora_status_t plan_apply(const molora_proj_desc_t* projs, int32_t P, molora_dt
         if (umma_eligible(projs[i], dt) && use_umma(rank, N, C, group_bytes[group_of(rank)], same_rank[group_of(rank)])) pl.tc[pl.n_tc++] = projs[i];
         else if (use_jobs(projs[i], dt, N, C, same_rank[group_of(rank)])) pl.jc[group_of(rank)][pl.n_jc[group_of(rank)]++] = projs[i];
         else if (decode_eligible(projs[i], dt)) {
-            if (small_path_is_stream(rank, N, same_rank[group_of(rank)])) pl.sc[pl.n_sc++] = projs[i];
+            if (small_path_is_stream(rank, N, C, same_rank[group_of(rank)])) pl.sc[pl.n_sc++] = projs[i];
             else pl.dc[pl.n_dc++] = projs[i];
         } else pl.cc[pl.n_cc++] = projs[i];
     }
@@ -380,7 +381,8 @@ molora_status_t plan_apply(const molora_proj_desc_t* projs, int32_t P, molora_dt
     if (pl.n_tc > 0 && pl.min_rows > 1)
         for (int i = 0; i < pl.n_tc; ++i) {
             if (!decode_eligible(pl.tc[i], dt)) pl.small_cc[pl.n_small_cc++] = pl.tc[i];
-            else if (small_path_is_stream(pl.tc[i].rank, N, same_rank[group_of(pl.tc[i].rank)])) pl.small_sc[pl.n_small_sc++] = pl.tc[i];
+            // (0 adapters: it gets short segments only, and the rule for whole calls of many adapters does not apply)
+            else if (small_path_is_stream(pl.tc[i].rank, N, 0, same_rank[group_of(pl.tc[i].rank)])) pl.small_sc[pl.n_small_sc++] = pl.tc[i];
             else pl.small_dc[pl.n_small_dc++] = pl.tc[i];
         }
     size_t need_dc = 0, need_small = 0;
@@ -450,7 +452,7 @@ static int group_apply_mode(const molora_proj_desc_t* projs, int32_t P, molora_d
         same = same && projs[i].rank == projs[0].rank && decode_eligible(projs[i], dt);
         if (!same) return 0;
         const bool jb = use_jobs(projs[i], dt, N, C, P);
-        const bool st = small_path_is_stream(projs[i].rank, N, P);
+        const bool st = small_path_is_stream(projs[i].rank, N, C, P);
         jobs = jobs && jb;
         stream = stream && !jb && st;
         twophase = twophase && !jb && !st;

@@ -15,6 +15,8 @@ from paper_2603_15965_b200.binding import _ProjDescC
     (4096, 64, [(2048, 2048, 64)] * 4, 1),
     # one rank-64 projection with few tokens per adapter: the two-launch kernels behind a grouping launch
     (3001, 256, [(2048, 2048, 64)], 0),
+    # ... from 24 tokens per adapter the streaming kernel, up to 64 adapters the tcgen05 kernel as before
+    (2399, 100, [(2048, 2048, 64)], 0), (2400, 100, [(2048, 2048, 64)], 1), (4096, 128, [(2048, 2048, 64)] * 2, 1), (4160, 65, [(2048, 2048, 64)], 0),
 ])
 def test_one_launch(N, C, shapes, expected):
     lib = M.load_library()

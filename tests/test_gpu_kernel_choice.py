@@ -36,3 +36,12 @@ def test_tiles_slices_and_clusters(N, C, shapes, rank):
 def test_linear_and_boxed_weights(d_in, d_out):
     """rank 16, short tiles: seven chunk jobs an item and eight, whole and ragged chunks"""
     check(60, 5, [(d_in, d_out)], 16)
+
+
+@pytest.mark.parametrize("N,C,shapes,rank", [
+    # rank 64, more than 64 adapters, one and two projections: two-launch, streaming and tcgen05 kernel
+    (2399, 100, [(512, 320)], 64), (2400, 100, [(512, 320)], 64), (2400, 100, [(512, 320), (512, 96)], 64), (6399, 100, [(512, 320)], 64),
+    (6400, 100, [(512, 320)], 64),
+])
+def test_many_adapters_of_rank_64(N, C, shapes, rank):
+    check(N, C, shapes, rank)
