@@ -61,14 +61,16 @@ namespace {
 //   rank 64  one or two projections (the two-launch pair below): once they move ~12 MB with at least 256 tokens and segments
 //            of 32 rows on average (one 4096-wide projection: from 512 tokens, 21.0 against 24.3; two: 23.2 against 38.9 at
 //            512 tokens).  More: from 680 tokens with 60 per adapter: 600 tokens, 8 adapters 44.8 / 39.6, 777: 44.6 / 51.3;
-//            1000 tokens, 16 adapters 66.2 / 70.4.  From 1280 tokens in any case, unless more than 64 adapters share fewer
-//            than 64 tokens each.
+//            1000 tokens, 16 adapters 66.2 / 70.4; below that from 256 tokens where segments are long or the call is large: 120 per
+//            adapter and 12 MB (4096 wide, 400 tokens, 4 adapters, four projections 23 / 30, a layer 45 / 53) or 60 and 60 MB
+//            (4096 wide, 512 tokens, 8 adapters, a layer 58 / 67).  From 1280 tokens in any case, unless more than 64 adapters share
+//            fewer than 64 tokens each.
 //   more than 64 adapters   four projections, 3001 tokens, 256 adapters: rank 32 271 (both kernels, each its segments) / 59,
 //            rank 64 304 / 88
 // The overrides "umma_min_tokens" (tcgen05 from n tokens) and "small_path" (the kernel used below it) of
 // molora_debug_set force a choice, for measurements and for tests that target one kernel.
 int64_t forced_umma_min_tokens() { return std::max<int64_t>(0, tune(kTuneUmmaMinTokens)); }
-constexpr double kUmmaMinBytesR16 = 150e6, kUmmaMinBytesR32 = 60e6, kUmmaMinBytesR32More = 170e6;
+constexpr double kUmmaMinBytesR16 = 150e6, kUmmaMinBytesR32 = 60e6, kUmmaMinBytesR32More = 170e6, kUmmaMinBytesR64More = 60e6;
 constexpr int64_t kUmmaMinTokensR64 = 1280, kUmmaMinTokensR64Wide = 256, kUmmaMinTokensR64Layer = 680;
 constexpr double kUmmaMinBytesR64 = 12e6;
 
@@ -80,8 +82,11 @@ bool use_umma_r64(int64_t N, int32_t C, double group_bytes, int same_rank)
 {
     if (C > kUmmaAllSegmentsMaxC && N < (int64_t)C * 64) return false;
     if (N >= kUmmaMinTokensR64) return true;
-    if (same_rank > 2) return N >= kUmmaMinTokensR64Layer && N >= (int64_t)C * 60;
-    return N >= kUmmaMinTokensR64Wide && N >= (int64_t)C * kUmmaMinRows && group_bytes >= kUmmaMinBytesR64;
+    if (N < kUmmaMinTokensR64Wide) return false;
+    if (same_rank > 2)
+        return (N >= (int64_t)C * 60 && (N >= kUmmaMinTokensR64Layer || group_bytes >= kUmmaMinBytesR64More)) ||
+               (N >= (int64_t)C * 120 && group_bytes >= kUmmaMinBytesR64);
+    return N >= (int64_t)C * kUmmaMinRows && group_bytes >= kUmmaMinBytesR64;
 }
 bool use_umma(int32_t rank, int64_t N, int32_t C, double group_bytes, int same_rank)
 {

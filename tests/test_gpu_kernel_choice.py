@@ -45,3 +45,12 @@ def test_linear_and_boxed_weights(d_in, d_out):
 ])
 def test_many_adapters_of_rank_64(N, C, shapes, rank):
     check(N, C, shapes, rank)
+
+
+@pytest.mark.parametrize("N,C,shapes,rank", [
+    # rank 64, three and more projections below 680 tokens: 12 MB with 120 tokens per adapter, 60 MB with 60, and one token less
+    (359, 3, [(2048, 2048), (2048, 2048), (2048, 1024)], 64), (360, 3, [(2048, 2048), (2048, 2048), (2048, 1024)], 64), (255, 2, [(4096, 4096)] * 3, 64),
+    (256, 2, [(4096, 4096)] * 3, 64), (479, 8, [(4096, 4096)] * 6, 64), (480, 8, [(4096, 4096)] * 6, 64),
+])
+def test_mid_sized_layers_of_rank_64(N, C, shapes, rank):
+    check(N, C, shapes, rank, rows=60)
