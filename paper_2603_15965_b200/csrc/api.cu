@@ -57,7 +57,9 @@ namespace {
 //            38.5; 4000 tokens, 16 adapters 95.7 / 87.1; a 4096-wide layer, 8192 tokens, 16 adapters 329 / 312
 //   rank 32  with 160 tokens per adapter, one projection from 60 MB (8000 tokens, 98 MB, 26.8 / 30.9), more from 170 MB: 1050
 //            tokens, 8 adapters 39.4 / 36.5, 1500 48.9 / 49.0, 1990 57.1 / 64.1; two projections, 3000 tokens, 4 adapters
-//            (123 MB) 34.2 / 28.4, 16384 tokens 127 / 141
+//            (123 MB) 34.2 / 28.4, 16384 tokens 127 / 141; with 3000 tokens and 300 per adapter from 60 MB already, which is what
+//            narrow models reach: four projections 512 wide, 8000 tokens (74 MB) 25 / 36, 1024 wide, 5000 (92 MB) 29 / 37; a layer
+//            512 wide, 3500 tokens (100 MB) 24 / 35
 //   rank 64  one or two projections (the two-launch pair below): once they move ~12 MB with at least 256 tokens and segments
 //            of 32 rows on average (one 4096-wide projection: from 512 tokens, 21.0 against 24.3; two: 23.2 against 38.9 at
 //            512 tokens).  More: from 680 tokens with 60 per adapter: 600 tokens, 8 adapters 44.8 / 39.6, 777: 44.6 / 51.3;
@@ -94,7 +96,8 @@ bool use_umma(int32_t rank, int64_t N, int32_t C, double group_bytes, int same_r
     if (rank == 64) return use_umma_r64(N, C, group_bytes, same_rank);
     if (N < kUmmaMinTokens) return false;
     if (rank == 16) return group_bytes >= kUmmaMinBytesR16 && same_rank == 1 && N >= (int64_t)C * 128;
-    return group_bytes >= (same_rank == 1 ? kUmmaMinBytesR32 : kUmmaMinBytesR32More) && N >= (int64_t)C * 160;
+    if (N < (int64_t)C * 160 || group_bytes < kUmmaMinBytesR32) return false;
+    return same_rank == 1 || group_bytes >= kUmmaMinBytesR32More || (N >= 3000 && N >= (int64_t)C * 300);
 }
 // the kernel for what the tcgen05 kernel does not take; same_rank: projections of this rank in the call (0: unknown)
 bool small_path_is_stream(int32_t rank, int64_t N, int32_t C, int same_rank)

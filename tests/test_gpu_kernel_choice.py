@@ -54,3 +54,12 @@ def test_many_adapters_of_rank_64(N, C, shapes, rank):
 ])
 def test_mid_sized_layers_of_rank_64(N, C, shapes, rank):
     check(N, C, shapes, rank, rows=60)
+
+
+@pytest.mark.parametrize("N,C,shapes,rank", [
+    # rank 32, several projections from 60 MB: 3000 tokens with 300 per adapter, and one less of either
+    (2999, 4, [(1024, 1024), (1024, 3072)], 32), (3000, 10, [(1024, 1024), (1024, 3072)], 32), (3000, 11, [(1024, 1024), (1024, 3072)], 32),
+    (8000, 8, [(512, 512), (512, 128), (512, 128), (512, 512)], 32),
+])
+def test_narrow_layers_of_rank_32(N, C, shapes, rank):
+    check(N, C, shapes, rank)
