@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) route_mlp_umma_kernel(const __
             wait_bar_cluster(bar(&ctrl->parts), 0, abort_flag, prm.dev_status);   // ... and the peers' partials of them
             // finish my RO tokens: thread (token tl2, part) takes a slice of the hidden units
             const int parts = 128 / RO, tl2 = et % RO, part = et / RO;
-            const int hp = HP / parts;                             // hidden units per thread: 16 ... 64
+            const int hp = HP / parts;                             // hidden units per thread: 8 ... 64
             for (int j4 = part * hp / 4; j4 < (part + 1) * hp / 4; ++j4) {
                 if (j4 * 4 >= nj16 * 16) break;
                 float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -451,8 +451,8 @@ molora_status_t launch_route_mlp(const void* x, molora_dtype_t xdt, int64_t N, i
     const bool room = ws != nullptr && ws_bytes >= route_mlp_workspace_bytes(xdt, d, H) && aligned16(ws);
     // Below 128 tokens the images are optional: without room for them the call runs on the CUDA cores, as do routers so small that
     // building the images costs more than it saves (us, CUDA cores / both launches: 64 -> 16 hidden units, 16 tokens 6.9 / 7.9; 128 -> 16:
-    // 8.4 / 8.2; 64 -> 64: 25 / 12; with images built before 6.9 / 6.4).
-    const bool tiny = image == kImageBuildAndUse && N < 128 && (int64_t)std::max(H, 16) * d <= 1024;
+    // 8.4 / 8.2; 64 -> 64: 25 / 12), whether the images have been built before or not (6.9 / 6.4): the results are the same bits.
+    const bool tiny = image != kImageBuildOnly && N < 128 && (int64_t)std::max(H, 16) * d <= 1024;
     if (mlp_umma_eligible(xdt, image == kImageBuildOnly ? 128 : N, d, H) && !tiny && (room || image == kImageBuildOnly || N >= 128)) {
         if (ws == nullptr || ws_bytes < route_mlp_workspace_bytes(xdt, d, H) || !aligned16(ws)) return MOLORA_ERR_WORKSPACE;
         return H <= 64 ? mlp_umma_launch<64>(x, N, d, ldx, W1, b1, H, W2, b2, C, r_out, logits_out, ws, dev_status, s, image)

@@ -110,6 +110,5 @@ def test_mlp_router_on_both_sides_of_the_tiny_rule(N, d, H, launches):
     r_ref, z_ref, margin = oracle.route_mlp(x, W1, None, W2, None)
     np.testing.assert_allclose(z.cpu().numpy(), z_ref, rtol=0, atol=1e-5 * max(1.0, np.abs(z_ref).max()))
     assert np.array_equal(r.cpu().numpy()[margin >= 1e-3], r_ref[margin >= 1e-3])
-    prepared = M.molora_route_mlp_prepare(xd.dtype, W1d, C)
-    assert torch.equal(M.molora_route_mlp(xd, W1d, None, W2d, None, prepared=prepared)[torch.from_numpy(margin >= 1e-3).cuda()],
-                       r[torch.from_numpy(margin >= 1e-3).cuda()])
+    prepared, zp = M.molora_route_mlp_prepare(xd.dtype, W1d, C), torch.empty_like(z)
+    assert torch.equal(M.molora_route_mlp(xd, W1d, None, W2d, None, logits_out=zp, prepared=prepared), r) and torch.equal(zp, z)
