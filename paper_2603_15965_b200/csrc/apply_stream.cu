@@ -758,7 +758,9 @@ static double stream_estimate(const StreamParams& prm, int64_t rows, int& split)
     using Cfg = FsCfg<R, SHORT, (SHORT && R >= 32 ? kFsCluster : kFsOne)>;
     const double job_us = R == 16 ? (SHORT ? 1.30 : 1.19) : R == 32 ? (SHORT ? 1.17 : 1.72) : (SHORT ? 0.90 : 1.67);
     // tiles of segments of about equal size: one each while that is well below a tile's height, half a tile lost per segment from there on
-    const double segments = (double)std::min<int64_t>(prm.C, rows), fill = (double)rows / segments / Cfg::ROWS;
+    // (of the adapter sets of top-k routing only those of different adapters are met; the others are there for callers that repeat one)
+    const int64_t met = prm.parts > 1 && prm.n_adapters >= prm.parts ? binom_small(prm.n_adapters, prm.parts) : prm.C;
+    const double segments = (double)std::min<int64_t>(met, rows), fill = (double)rows / segments / Cfg::ROWS;
     const double tiles = segments * (fill <= 0.75 ? 1.0 : fill <= 1.0 ? 1.0 + 2.0 * (fill - 0.75) : fill + 0.5);
     auto jobs = [](int width) {            // jobs that `width` columns cost
         const int full = width / Cfg::CH, rest = width % Cfg::CH;
@@ -783,7 +785,7 @@ static double stream_estimate(const StreamParams& prm, int64_t rows, int& split)
             longest = std::max(longest, each);
         }
         double t = longest;
-        if (units == 1) t = longest * std::ceil(tiles / clusters);        // equal items, dealt in whole rounds
+        if (units == 1) t = longest * std::ceil(1.05 * tiles / clusters);        // equal items, dealt in whole rounds (the tiles are an estimate)
         else if (tiles * units > clusters) t = std::max(longest, sum * tiles / clusters + 0.15 * sum / units);
         t += S == 1 ? 0.0 : S == 2 ? 1.5 : S == 4 ? 2.25 : 3.0;
         if (forced > 0 ? S <= forced : t < best) {
