@@ -615,13 +615,19 @@ int topk_single_pass(const molora_proj_desc_t* projs, int32_t P, molora_dtype_t 
     // Measured (us, two passes / one on tcgen05 / one on the streaming kernel), a layer of 2048, k = 2, 36 sets:
     // rank 16, 2048 tokens 115 / 106 / 78, 4000 tokens 189 / 168 / 123; 10 sets, 2048 tokens - / 67 / 74; stacked rank
     // 64 (rank 32), whose streaming chunks are half as wide: 2048 tokens 121 / 112 / 140, but one projection 25 streaming, 33
-    // tcgen05.  Beyond 8192 tokens the two passes are kept (not measured).
+    // tcgen05.  A set of two has to bring each projection work for its tiles: a layer 512 wide, 4096 tokens (0.46 MB) 68 in two passes, 84 on
+    // tcgen05; 2048 wide, 2048 tokens (0.93 MB) 113 / 106.  With more than 64 sets of rank-32 adapters the two passes are the faster
+    // ones from 1024 tokens and 60 MB: 16 adapters, a layer 512 wide, 4096 tokens 77 / - / 107, 2048 wide, 2048 tokens 145 / - / 160.
+    // Beyond 8192 tokens the two passes are kept (not measured).
     const int stacked = projs[0].rank * k;
     const bool dense_sets = sets <= 16 || N >= sets * 256;
-    if (umma_ok && (dense_sets || (stacked == 64 && bytes >= 100e6)) && use_umma(stacked, N, (int32_t)sets, bytes, P)) return 2;
+    if (umma_ok && (dense_sets || (stacked == 64 && bytes >= 100e6 && (k == 4 || bytes >= 0.7e6 * (double)sets * P))) && use_umma(stacked, N, (int32_t)sets, bytes, P)) return 2;
     const int64_t small = tune(kTuneSmallPath);
     if (small != 0 && small != 1) return 0;                         // a test or a measurement asks for another kernel
     if (stacked <= 32 && N <= 8192 && forced_umma_min_tokens() == 0) return 1;
+    if (stacked == 64 && projs[0].rank == 32 && sets > kUmmaAllSegmentsMaxC && N >= kUmmaMinTokens && bytes >= kUmmaMinBytesR32 && small == 0 &&
+        forced_umma_min_tokens() == 0)
+        return 0;
     return use_umma(projs[0].rank, N, C, bytes, P) ? 0 : 1;
 }
 }  // namespace

@@ -1,11 +1,13 @@
 """Calls on both sides of the rules that choose kernel, tile and cluster from the sizes, against the CPU oracle: the library's own
 choice throughout, several projections in one call, tokens spread evenly over the adapters."""
 import numpy as np
+import oracle
 import pytest
 
+import paper_2603_15965_b200 as M
 from paper_2603_15965_b200 import workloads as W
 
-from _harness import run_and_check
+from _harness import dev_tensor, run_and_check, to_f64
 
 pytestmark = pytest.mark.gpu
 
@@ -63,3 +65,28 @@ def test_mid_sized_layers_of_rank_64(N, C, shapes, rank):
 ])
 def test_narrow_layers_of_rank_32(N, C, shapes, rank):
     check(N, C, shapes, rank)
+
+
+@pytest.mark.parametrize("N,C,rank,k,width", [
+    # rank 32, top-2: more than 64 sets on both sides of 1024 tokens and of 60 MB, 36 sets on both sides of 100 MB
+    (1023, 16, 32, 2, 4096), (1024, 16, 32, 2, 4096), (2500, 16, 32, 2, 4096), (4096, 8, 32, 2, 4032), (4096, 8, 32, 2, 4160), (200, 4, 16, 4, 2048),
+])
+def test_topk_passes_and_kernels(N, C, rank, k, width):
+    rng = np.random.default_rng(N + C)
+    w = W.random_problem(N + width, N, C, width, width, rank, "bf16")
+    p = w.projections[0]
+    idx = np.argsort(rng.random((C, N)), axis=0)[:k].astype(np.int32)
+    weight = rng.random((k, N)).astype(np.float32)
+    weight /= weight.sum(axis=0, keepdims=True)
+    y = dev_tensor(p.y, "bf16")
+    M.molora_apply_topk([M.ProjDesc(dev_tensor(w.inputs["x"], "bf16"), y, dev_tensor(p.A, "bf16"), dev_tensor(p.B, "bf16"))],
+                        dev_tensor(idx, "i"), dev_tensor(weight, "f32"), C)
+    rows = rng.choice(N, min(N, 80), replace=False)
+    ref = oracle.apply_topk(w.inputs["x"][rows], p.y[rows], p.A, p.B, np.ascontiguousarray(idx[:, rows]), np.ascontiguousarray(weight[:, rows]))
+    # The harness bound, and what y loses where there are several passes: it is rounded to bf16 after each of them, and rounding to
+    # the nearest of 8 significant bits is off by at most 2^-8 of the value (half of a unit of 2^-7 in the last place, at a power of two).
+    bound = 1e-3 + 2e-2 * np.abs(ref)
+    for j in range(1, k):
+        bound += 2.0 ** -8 * np.abs(oracle.apply_topk(w.inputs["x"][rows], p.y[rows], p.A, p.B, np.ascontiguousarray(idx[:j, rows]),
+                                                      np.ascontiguousarray(weight[:j, rows])))
+    assert np.all(np.abs(to_f64(y)[rows] - ref) <= bound)
