@@ -785,7 +785,8 @@ static double stream_estimate(const StreamParams& prm, int64_t rows, int& split)
             longest = std::max(longest, each);
         }
         double t = longest;
-        if (units == 1) t = longest * std::ceil(1.05 * tiles / clusters);        // equal items, dealt in whole rounds (the tiles are an estimate)
+        // equal items are dealt in whole rounds (a margin where the number of resident clusters is an estimate)
+        if (units == 1) t = longest * std::ceil((S >= 4 ? 1.05 : 1.0) * tiles / clusters);
         else if (tiles * units > clusters) t = std::max(longest, sum * tiles / clusters + 0.15 * sum / units);
         t += S == 1 ? 0.0 : S == 2 ? 1.5 : S == 4 ? 2.25 : 3.0;
         if (forced > 0 ? S <= forced : t < best) {
