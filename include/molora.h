@@ -111,8 +111,8 @@ molora_status_t molora_route_composite(const int32_t *ids, const int32_t *adapte
  * r_out    device int32[N]
  * logits_out  device fp32 [N, C] or NULL (the logits as the kernel accumulated them, fp32)
  * ws, ws_bytes  device scratch of at least molora_route_gate_workspace_bytes(xdt, d, C) bytes, 16-byte aligned
- *               (NULL when that is 0).  For bf16 x and C > 4 the kernel runs on the tensor cores (tcgen05 when N >= 1024
- *               and d is a multiple of 64, mma.sync otherwise) and keeps there a three-term bf16 split of G
+ *               (NULL when that is 0).  For bf16 x and C > 4 the kernel runs on the tensor cores (tcgen05 for large
+ *               calls whose d is a multiple of 64, mma.sync otherwise) and keeps there a three-term bf16 split of G
  *               (hi + mid + lo = 24 mantissa bits), rebuilt on every call.
  * dev_status  device status word or NULL.  Only the tcgen05 kernel waits on the device (bounded): if a wait runs out,
  *             MOLORA_DEV_TIMEOUT is OR-ed in and the tokens of that 128-token tile get r_out = -1 (unrouted).
@@ -133,7 +133,8 @@ molora_status_t molora_route_gate(const void *x, molora_dtype_t xdt, int64_t N, 
  * ws, ws_bytes  device scratch of at least molora_route_mlp_workspace_bytes(xdt, d, H, C) bytes, 16-byte aligned (NULL
  *               when that is 0): for bf16 x and d a multiple of 64 the first layer runs on the tensor cores with a
  *               three-term bf16 split of W1 kept there (rebuilt on every call); MOLORA_ERR_WORKSPACE if it is
- *               needed (at least 128 tokens) and missing.
+ *               needed (at least 128 tokens) and missing.  Below 128 tokens without ws the first layer runs on the CUDA
+ *               cores, whose sums may differ from the tensor cores' in the last bits.
  * dev_status  device status word or NULL; as for molora_route_gate (the tensor-core kernel's waits are bounded:
  *             MOLORA_DEV_TIMEOUT, and r_out = -1 for the tokens of the tile whose wait ran out).
  * Products of the first layer are exact in fp32 for bf16 x; accumulation, GELU and the second layer are fp32. */
@@ -225,12 +226,12 @@ molora_status_t molora_group(const int32_t *r, int64_t N, int32_t C, int32_t *co
  *                 clear only a part of it later); after that the same ws can be passed to any number of calls, of any
  *                 shape, without clearing -- every launch counts itself in the control words and old records never
  *                 carry the current tag.  Calls that share one ws must not overlap on the GPU.  The
- *                 two-launch small-tile kernels (bf16 rank 64 below 1280 tokens with one or two rank-64 projections in
- *                 the call; with more than 64 adapters also the short segments of larger rank-64 calls) keep partial
- *                 shrink results [slice][N][rank] behind that.
+ *                 two-launch small-tile kernels (bf16 rank 64, one or two rank-64 projections in the call, and below 1280
+ *                 tokens or more than 64 adapters with fewer than 24 tokens each; with more than 64 adapters also the short
+ *                 segments of larger rank-64 calls) keep partial shrink results [slice][N][rank] behind that.
  *                 MOLORA_ERR_WORKSPACE if ws is needed and NULL, misaligned or too small.
  * dev_status      device uint32 or NULL; MOLORA_DEV_TIMEOUT is OR-ed in if a bounded wait inside a kernel gave
- *                 up (the kernel then returns without hanging; y is incomplete)
+ *                 up (the kernel then returns without hanging; y is incomplete: nothing more is stored to it)
  * The kernel variant is chosen per call on the host from rank, token count and bytes (tcgen05 tiles of 128 rows
  * for large calls with full segments, a single-launch streaming kernel with 16- and 32-row tiles otherwise, CUDA cores for fp32 storage,
  * rank 8 and odd widths) and per segment on the device from the segment sizes; the paper picks its tile shape
@@ -264,9 +265,9 @@ molora_status_t molora_apply_batched(const molora_proj_desc_t *projs, int32_t P,
 /* Grouping and grouped application of one layer in one call (Section 3.3 steps 1-4, Algorithm 2): exactly
  * molora_group(r, ...) followed by molora_apply_batched(projs, ...) on its outputs, with the arguments, results
  * (counts, offsets and perm are written, bit-equal to molora_group's), status bits and error behaviour of those two
- * calls; ws / ws_bytes as for molora_apply_batched.  When every projection of the call runs on the single-launch
- * streaming kernel or on the job-list kernel with one rank (bf16, at most 4096 / 1024 tokens, below the tcgen05
- * crossover) the whole call is ONE launch: every CTA builds the grouping in its shared memory before its first copy
+ * calls; ws / ws_bytes as for molora_apply_batched.  When every projection of the call runs, with one rank, on the
+ * single-launch streaming kernel, on the tcgen05 kernel (at most 64 adapters) or, where "small_path" asks for it, on the job-list
+ * kernel (bf16, at most 4096 tokens; 1024 for the job-list kernel) the whole call is ONE launch: every CTA builds the grouping in its shared memory before its first copy
  * request, which saves the grouping launch; the two-launch small-tile kernels do the same for at most 1024 tokens;
  * otherwise the grouping launch and the apply launches are enqueued in stream order. */
 molora_status_t molora_group_apply_batched(const int32_t *r, int64_t N, int32_t C, int32_t *counts, int32_t *offsets,

@@ -100,8 +100,8 @@ def test_apply_workspace_sizes_and_refusal_without_it(default_kernels):
     assert M.molora_apply_workspace_bytes(256, 8, 2048, 2048, 16) == ctl + 24 * 6 * 16 * 16 * 8
     assert M.molora_apply_workspace_bytes(1025, 8, 2048, 2048, 16) == 0                 # more tokens than the kernel takes
     M.molora_debug_set("small_path", 0)
-    # by default the job-list kernel takes rank 16 between 257 and 1024 tokens (with at least four projections, which is
-    # not known here); rank 64 runs on the two-launch kernels while the projection moves less than ~12 MB (x once, y
+    # the figure still covers the job-list kernel for rank 16 between 257 and 1024 tokens, although no call takes that kernel by
+    # itself; rank 64 runs on the two-launch kernels while the projection moves less than ~12 MB (x once, y
     # twice) or has fewer than 256 tokens, on the tcgen05 kernel (no scratch) above
     assert M.molora_apply_workspace_bytes(512, 8, 2048, 2048, 16) == ctl + (512 // 16 + 8) * 6 * 16 * 16 * 8
     assert M.molora_apply_workspace_bytes(256, 8, 2048, 2048, 16) == 0
@@ -143,7 +143,7 @@ def test_group_apply_one_call_launch_count_and_refusals(default_kernels):
     assert one_launch([(2048, 2048, 16)], 4096) == 1                    # c2's apply: streaming kernel
     layer = [(2048, 2048, 16)] * 4 + [(2048, 6144, 16)] * 2 + [(6144, 2048, 16)]
     assert one_launch(layer, 256) == 1                                  # a decode layer: streaming kernel
-    assert one_launch(layer, 512) == 1 and one_launch(layer, 1024) == 1 # ... job-list kernel (also one launch)
+    assert one_launch(layer, 512) == 1 and one_launch(layer, 1024) == 1 # ... also of several hundred tokens
     assert one_launch([(2048, 2048, 16)], 4097) == 0                    # more tokens than a CTA groups on its own
     assert one_launch([(2048, 2048, 32)], 2048) == 1 and one_launch([(2048, 2048, 32)], 512) == 1   # rank 32 streams too
     assert one_launch([(2048, 2048, 64)], 512) == 0                     # rank 64, one projection: two-launch kernels
