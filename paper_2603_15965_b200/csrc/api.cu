@@ -106,7 +106,8 @@ bool small_path_is_stream(int32_t rank, int64_t N, int32_t C, int same_rank)
         if (forced == 1) return true;
         if (forced == 2) return false;
     }
-    // rank 64: the two-launch pair for one or two projections (its split of the reduction over CTAs pays there);
+    // rank 64: the two-launch pair for one or two projections (chosen when only the pair split the reduction over CTAs; the streaming
+    // kernel does too now and measures a little ahead there as well: one 4096 wide, 8 adapters, 128 tokens 16.4 / 14.9, 400 18.0 / 14.9);
     // with a layer's worth of them its items no longer fit a wave and the streaming kernel is faster, as it is for calls of more than
     // 64 adapters with 24 to 64 tokens each, where the pair sends every row's partials through the workspace (us, pair / streaming:
     // 256 adapters, 16000 tokens, 4096 wide, one projection 393 / 199, two 1143 / 570; 8000 tokens, 2048 wide 119 / 77)
@@ -617,7 +618,7 @@ int topk_single_pass(const molora_proj_desc_t* projs, int32_t P, molora_dtype_t 
     // 64 (rank 32), whose streaming chunks are half as wide: 2048 tokens 121 / 112 / 140, but one projection 25 streaming, 33
     // tcgen05.  A set of two has to bring each projection work for its tiles: a layer 512 wide, 4096 tokens (0.46 MB) 68 in two passes, 84 on
     // tcgen05; 2048 wide, 2048 tokens (0.93 MB) 113 / 106.  With more than 64 sets of rank-32 adapters the two passes are the faster
-    // ones from 1024 tokens and 60 MB: 16 adapters, a layer 512 wide, 4096 tokens 77 / - / 107, 2048 wide, 2048 tokens 145 / - / 160.
+    // ones from 1024 tokens and 45 MB: 16 adapters, a layer 512 wide, 4096 tokens 77 / - / 107, 2048 wide, 2048 tokens 145 / - / 160.
     // Beyond 8192 tokens the two passes are kept (not measured).
     const int stacked = projs[0].rank * k;
     const bool dense_sets = sets <= 16 || N >= sets * 256;
@@ -625,7 +626,7 @@ int topk_single_pass(const molora_proj_desc_t* projs, int32_t P, molora_dtype_t 
     const int64_t small = tune(kTuneSmallPath);
     if (small != 0 && small != 1) return 0;                         // a test or a measurement asks for another kernel
     if (stacked <= 32 && N <= 8192 && forced_umma_min_tokens() == 0) return 1;
-    if (stacked == 64 && projs[0].rank == 32 && sets > kUmmaAllSegmentsMaxC && N >= kUmmaMinTokens && bytes >= kUmmaMinBytesR32 && small == 0 &&
+    if (stacked == 64 && projs[0].rank == 32 && sets > kUmmaAllSegmentsMaxC && N >= kUmmaMinTokens && bytes >= 45e6 && small == 0 &&
         forced_umma_min_tokens() == 0)
         return 0;
     return use_umma(projs[0].rank, N, C, bytes, P) ? 0 : 1;

@@ -68,8 +68,8 @@ def test_narrow_layers_of_rank_32(N, C, shapes, rank):
 
 
 @pytest.mark.parametrize("N,C,rank,k,width", [
-    # rank 32, top-2: more than 64 sets on both sides of 1024 tokens and of 60 MB, 36 sets on both sides of 100 MB
-    (1023, 16, 32, 2, 4096), (1024, 16, 32, 2, 4096), (2500, 16, 32, 2, 4096), (4096, 8, 32, 2, 4032), (4096, 8, 32, 2, 4160), (200, 4, 16, 4, 2048),
+    # rank 32, top-2: more than 64 sets on both sides of 1024 tokens and of 45 MB, 36 sets on both sides of 100 MB
+    (1023, 16, 32, 2, 4096), (1024, 16, 32, 2, 4096), (1831, 16, 32, 2, 4096), (1832, 16, 32, 2, 4096), (4096, 8, 32, 2, 4032), (4096, 8, 32, 2, 4160), (200, 4, 16, 4, 2048),
 ])
 def test_topk_passes_and_kernels(N, C, rank, k, width):
     rng = np.random.default_rng(N + C)
