@@ -84,14 +84,21 @@ int64_t integer(PyObject* o)
     if (v == -1 && PyErr_Occurred()) throw PyRaised{};
     return v;
 }
-void* stream_of(PyObject* o)
-{
-    if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
-    Ref v(PyObject_HasAttr(o, s_cuda_stream) ? PyObject_GetAttr(o, s_cuda_stream) : PyNumber_Long(o));
-    void* p = PyLong_AsVoidPtr(v.p);
-    if (p == nullptr && PyErr_Occurred()) throw PyRaised{};
-    return p;
-}
+// the stream of a call: the one given, or the current one
+struct Stream {
+    void* p;
+    bool given;
+    explicit Stream(PyObject* o) : p(nullptr), given(o != Py_None)
+    {
+        if (!given) {
+            p = c10::cuda::getCurrentCUDAStream().stream();
+            return;
+        }
+        Ref v(PyObject_HasAttr(o, s_cuda_stream) ? PyObject_GetAttr(o, s_cuda_stream) : PyNumber_Long(o));
+        p = PyLong_AsVoidPtr(v.p);
+        if (p == nullptr && PyErr_Occurred()) throw PyRaised{};
+    }
+};
 const at::Tensor& i32_dev(PyObject* o, const char* name)
 {
     const at::Tensor& t = tensor(o, name);
@@ -102,12 +109,13 @@ const at::Tensor& i32_dev(PyObject* o, const char* name)
 // What a call allocates belongs to the stream that it runs on: memory that the current stream's allocator hands out may still be in
 // use there, and is handed out again there as soon as the call has returned.
 template <class F>
-at::Tensor allocate(void* stream, F f)
+at::Tensor allocate(const Stream& stream, F f)
 {
+    if (!stream.given) return f();
     c10::cuda::OptionalCUDAStreamGuard on;
     // (odd values are not addresses but the runtime's names of its default streams)
-    if (stream != c10::cuda::getCurrentCUDAStream().stream() && ((uintptr_t)stream & 1u) == 0)
-        on.reset_stream(c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream), c10::cuda::current_device()));
+    if (stream.p != c10::cuda::getCurrentCUDAStream().stream() && ((uintptr_t)stream.p & 1u) == 0)
+        on.reset_stream(c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream.p), c10::cuda::current_device()));
     return f();
 }
 // an output: the caller's tensor, or n words allocated on first use
@@ -119,7 +127,7 @@ struct Out {
     {
         if (o != Py_None) t = i32_dev(o, name);
     }
-    int32_t* get(void* stream)
+    int32_t* get(const Stream& stream)
     {
         if (!t.defined()) t = allocate(stream, [&] { return at::empty({n}, at::TensorOptions().dtype(at::kInt).device(dev)); });
         return static_cast<int32_t*>(t.data_ptr());
@@ -151,7 +159,7 @@ struct Workspace {
         if (o != Py_None) t = tensor(o, "ws");
         else need = need_;
     }
-    void make(const at::Device& dev, bool zero, void* stream)
+    void make(const at::Device& dev, bool zero, const Stream& stream)
     {
         const auto opt = at::TensorOptions().dtype(at::kByte).device(dev);
         if (need > 0) t = allocate(stream, [&] { return zero ? at::zeros({(int64_t)need}, opt) : at::empty({(int64_t)need}, opt); });
@@ -267,19 +275,19 @@ void call(const char* fn, F f)
 }
 uint32_t* status_word(PyObject* o) { return static_cast<uint32_t*>(ptr(o)); }
 
-// ---- (ids, breaks, r_out, dev_status, stream)
+// ---- (ids, breaks, r_out, dev_status, stream.p)
 PyObject* route_vocab(PyObject* const* a)
 {
     const at::Tensor &ids = i32_dev(a[0], "ids"), &breaks = i32_dev(a[1], "breaks");
     const int64_t N = ids.numel();
     Out r(a[2], "r_out", N, ids.device());
     uint32_t* status = status_word(a[3]);
-    void* stream = stream_of(a[4]);
-    call("molora_route_vocab", [&] { return molora_route_vocab(i32(ids), N, i32(breaks), (int32_t)breaks.numel() - 1, r.get(stream), status, stream); });
+    const Stream stream(a[4]);
+    call("molora_route_vocab", [&] { return molora_route_vocab(i32(ids), N, i32(breaks), (int32_t)breaks.numel() - 1, r.get(stream), status, stream.p); });
     return wrap(r.t);
 }
 
-// ---- (ids, adapter, breaks, n_adapters, r_out, dev_status, stream)
+// ---- (ids, adapter, breaks, n_adapters, r_out, dev_status, stream.p)
 PyObject* route_composite(PyObject* const* a)
 {
     const at::Tensor &ids = i32_dev(a[0], "ids"), &adapter = i32_dev(a[1], "adapter"), &breaks = i32_dev(a[2], "breaks");
@@ -289,9 +297,9 @@ PyObject* route_composite(PyObject* const* a)
     const int32_t n_adapters = (int32_t)integer(n.p);
     Out r(a[4], "r_out", N, ids.device());
     uint32_t* status = status_word(a[5]);
-    void* stream = stream_of(a[6]);
+    const Stream stream(a[6]);
     call("molora_route_composite", [&] {
-        return molora_route_composite(i32(ids), i32(adapter), N, i32(breaks), (int32_t)breaks.numel() - 1, n_adapters, r.get(stream), status, stream);
+        return molora_route_composite(i32(ids), i32(adapter), N, i32(breaks), (int32_t)breaks.numel() - 1, n_adapters, r.get(stream), status, stream.p);
     });
     return wrap(r.t);
 }
@@ -319,19 +327,19 @@ PyObject* route_gate(PyObject* const* a)
     const float *g = f32(a[1]), *bias = f32(a[2]);
     float* logits = f32(a[4]);
     uint32_t* status = status_word(a[6]);
-    void* stream = stream_of(a[7]);
+    const Stream stream(a[7]);
     if (a[8] != Py_None) {
         const at::Tensor& prepared = tensor(a[8], "prepared");
         call("molora_route_gate_prepared", [&] {
             return molora_route_gate_prepared(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, r.get(stream), logits, prepared.data_ptr(),
-                                              (size_t)prepared.numel(), status, stream);
+                                              (size_t)prepared.numel(), status, stream.p);
         });
         return wrap(r.t);
     }
     Workspace ws(a[5], molora_route_gate_workspace_bytes(dt, d, C));
     call("molora_route_gate", [&] {
         ws.make(x.device(), false, stream);        // (the weight images are written before they are read: the scratch need not be cleared)
-        return molora_route_gate(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, r.get(stream), logits, ws.p, ws.n, status, stream);
+        return molora_route_gate(x.data_ptr(), dt, m.rows, d, m.pitch, g, bias, C, r.get(stream), logits, ws.p, ws.n, status, stream.p);
     });
     return wrap(r.t);
 }
@@ -351,19 +359,19 @@ PyObject* route_mlp(PyObject* const* a)
     const float *w1 = f32(a[1]), *b1 = f32(a[2]), *w2 = f32(a[3]), *b2 = f32(a[4]);
     float* logits = f32(a[6]);
     uint32_t* status = status_word(a[8]);
-    void* stream = stream_of(a[9]);
+    const Stream stream(a[9]);
     if (a[10] != Py_None) {
         const at::Tensor& prepared = tensor(a[10], "prepared");
         call("molora_route_mlp_prepared", [&] {
             return molora_route_mlp_prepared(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, r.get(stream), logits, prepared.data_ptr(),
-                                             (size_t)prepared.numel(), status, stream);
+                                             (size_t)prepared.numel(), status, stream.p);
         });
         return wrap(r.t);
     }
     Workspace ws(a[7], molora_route_mlp_workspace_bytes(dt, d, H, C));
     call("molora_route_mlp", [&] {
         ws.make(x.device(), false, stream);
-        return molora_route_mlp(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, r.get(stream), logits, ws.p, ws.n, status, stream);
+        return molora_route_mlp(x.data_ptr(), dt, m.rows, d, m.pitch, w1, b1, H, w2, b2, C, r.get(stream), logits, ws.p, ws.n, status, stream.p);
     });
     return wrap(r.t);
 }
@@ -384,7 +392,7 @@ PyObject* tuple_of(std::initializer_list<at::Tensor> ts)
     return t;
 }
 
-// ---- (r, C, counts, offsets, perm, ws, dev_status, stream)
+// ---- (r, C, counts, offsets, perm, ws, dev_status, stream.p)
 PyObject* group(PyObject* const* a)
 {
     const at::Tensor& r = i32_dev(a[0], "r");
@@ -393,11 +401,11 @@ PyObject* group(PyObject* const* a)
     Out counts(a[2], "counts", C, dev), offsets(a[3], "offsets", C + 1, dev), perm(a[4], "perm", std::max<int64_t>(N, 1), dev);
     Workspace ws(a[5], molora_group_workspace_bytes(N, (int32_t)C));
     uint32_t* status = status_word(a[6]);
-    void* stream = stream_of(a[7]);
+    const Stream stream(a[7]);
     call("molora_group", [&] {
         int32_t *c = counts.get(stream), *o = offsets.get(stream), *p = perm.get(stream);
         ws.make(dev, true, stream);
-        return molora_group(i32(r), N, (int32_t)C, c, o, p, ws.p, ws.n, status, stream);
+        return molora_group(i32(r), N, (int32_t)C, c, o, p, ws.p, ws.n, status, stream.p);
     });
     return tuple_of({counts.t, offsets.t, perm.t});
 }
@@ -410,10 +418,10 @@ PyObject* apply_batched(PyObject* const* a)
     Workspace ws(a[3], a[3] == Py_None ? pr.apply_bytes() : 0);
     const at::Device dev = ws.need > 0 ? tensor(a[1], "offsets").device() : at::Device(at::kCUDA);
     uint32_t* status = status_word(a[4]);
-    void* stream = stream_of(a[5]);
+    const Stream stream(a[5]);
     call("molora_apply_batched", [&] {
         ws.make(dev, true, stream);
-        return molora_apply_batched(pr.d, pr.P, pr.dt, pr.N, (int32_t)pr.C, offsets, perm, ws.p, ws.n, status, stream);
+        return molora_apply_batched(pr.d, pr.P, pr.dt, pr.N, (int32_t)pr.C, offsets, perm, ws.p, ws.n, status, stream.p);
     });
     Py_RETURN_NONE;
 }
@@ -429,11 +437,11 @@ PyObject* group_apply_batched(PyObject* const* a)
     Out counts(a[3], "counts", C, dev), offsets(a[4], "offsets", C + 1, dev), perm(a[5], "perm", std::max<int64_t>(pr.N, 1), dev);
     Workspace ws(a[6], a[6] == Py_None ? pr.apply_bytes() : 0);
     uint32_t* status = status_word(a[7]);
-    void* stream = stream_of(a[8]);
+    const Stream stream(a[8]);
     call("molora_group_apply_batched", [&] {
         int32_t *c = counts.get(stream), *o = offsets.get(stream), *p = perm.get(stream);
         ws.make(dev, true, stream);
-        return molora_group_apply_batched(i32(r), pr.N, (int32_t)C, c, o, p, pr.d, pr.P, pr.dt, ws.p, ws.n, status, stream);
+        return molora_group_apply_batched(i32(r), pr.N, (int32_t)C, c, o, p, pr.d, pr.P, pr.dt, ws.p, ws.n, status, stream.p);
     });
     return tuple_of({counts.t, offsets.t, perm.t});
 }
@@ -445,18 +453,18 @@ PyObject* topk_softmax(PyObject* const* a)
     if (z.scalar_type() != at::kFloat || z.dim() != 2 || !z.is_contiguous()) raise(PyExc_ValueError, "logits must be a dense fp32 [N, C] tensor");
     Ref kk(PyNumber_Long(a[1]));
     const int64_t k = integer(kk.p), N = z.size(0);
-    void* stream = stream_of(a[2]);
+    const Stream stream(a[2]);
     at::Tensor idx, w;
     call("molora_topk_softmax", [&] {
         idx = allocate(stream, [&] { return at::empty({k, N}, at::TensorOptions().dtype(at::kInt).device(z.device())); });
         w = allocate(stream, [&] { return at::empty({k, N}, at::TensorOptions().dtype(at::kFloat).device(z.device())); });
         return molora_topk_softmax(static_cast<const float*>(z.data_ptr()), N, (int32_t)z.size(1), (int32_t)k, i32(idx),
-                                   static_cast<float*>(w.data_ptr()), stream);
+                                   static_cast<float*>(w.data_ptr()), stream.p);
     });
     return tuple_of({idx, w});
 }
 
-// ---- (projs, idx, w, C, ws, dev_status, stream)
+// ---- (projs, idx, w, C, ws, dev_status, stream.p)
 PyObject* apply_topk(PyObject* const* a)
 {
     const Projs pr(a[0], Py_None);
@@ -468,7 +476,7 @@ PyObject* apply_topk(PyObject* const* a)
     const bool zero = pr.apply_bytes() > 0;
     Workspace ws(a[4], a[4] == Py_None ? molora_apply_topk_workspace_bytes(pr.d, pr.P, pr.N, (int32_t)C) + 256 : 0);
     uint32_t* status = status_word(a[5]);
-    void* stream = stream_of(a[6]);
+    const Stream stream(a[6]);
     at::Tensor idx, w;
     call("molora_apply_topk", [&] {
         idx = allocate(stream, [&] { return idx0.contiguous(); });
@@ -476,7 +484,7 @@ PyObject* apply_topk(PyObject* const* a)
         ws.make(idx.device(), zero, stream);        // (only the apply part has to start cleared, and only where a kernel keeps control words in it)
         const size_t off = std::min((size_t)(-(intptr_t)ws.p) % 256, ws.n);      // (a shorter workspace is refused as too small)
         return molora_apply_topk(pr.d, pr.P, pr.dt, pr.N, (int32_t)C, (int32_t)idx.size(0), i32(idx), static_cast<const float*>(w.data_ptr()),
-                                 static_cast<char*>(ws.p) + off, ws.n - off, status, stream);
+                                 static_cast<char*>(ws.p) + off, ws.n - off, status, stream.p);
     });
     Py_RETURN_NONE;
 }
