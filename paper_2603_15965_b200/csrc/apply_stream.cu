@@ -746,7 +746,7 @@ static cudaError_t stream_launch(StreamParams prm, [[maybe_unused]] const Stream
 
 // Estimated time of a launch (us, without its fixed part) and the CTAs per item that give it.  A launch lasts as long as its
 // busiest cluster: `tiles` items per projection (and slice), each of nks + ne chunk jobs spread over S CTAs, on sms / S clusters (a few
-// SMs are lost to S = 4 and 8: clusters do not straddle a GPC).  The exchange of t costs an item about 2.25 jobs.  A chunk job
+// SMs are lost to S = 4 and 8: clusters do not straddle a GPC).  The exchange of t costs an item about 3 jobs.  A chunk job
 // costs 1.30 us with 16 x 1024 and 1.19 us with 32 x 512 elements of x or y (rank 16), 1.17 / 1.72 us (rank 32, 512 columns),
 // 0.90 / 1.67 us (rank 64, 256 columns), fitted to one projection of 300 - 8000 tokens and layers of 8 - 1000 tokens; a third of it
 // does not depend on the chunk's width.  Against an estimate that knew neither slices nor partial chunks and counted half a tile
@@ -757,10 +757,13 @@ static double stream_estimate(const StreamParams& prm, int64_t rows, int& split)
 {
     using Cfg = FsCfg<R, SHORT, (SHORT && R >= 32 ? kFsCluster : kFsOne)>;
     const double job_us = R == 16 ? (SHORT ? 1.30 : 1.19) : R == 32 ? (SHORT ? 1.17 : 1.72) : (SHORT ? 0.90 : 1.67);
-    // tiles of segments of about equal size: one each while that is well below a tile's height, half a tile lost per segment from there on
-    // (of the adapter sets of top-k routing only those of different adapters are met; the others are there for callers that repeat one)
-    const int64_t met = prm.parts > 1 && prm.n_adapters >= prm.parts ? binom_small(prm.n_adapters, prm.parts) : prm.C;
-    const double segments = (double)std::min<int64_t>(met, rows), fill = (double)rows / segments / Cfg::ROWS;
+    // Tiles of segments of about equal size: one each while that is well below a tile's height, half a tile lost per segment from there
+    // on.  Of the segments as many are counted as three quarters of the rows, spread at random, meet: adapters are not equally popular
+    // (rank 64, 4096 wide, 20 tokens of 16 adapters by popularity: clusters of four 26 us, of two, as for all 16, 32).  Of the adapter
+    // sets of top-k routing only those of different adapters are met; the others are there for callers that repeat one.
+    const double met = (double)(prm.parts > 1 && prm.n_adapters >= prm.parts ? binom_small(prm.n_adapters, prm.parts) : prm.C);
+    const double segments = std::min((double)rows, std::max(1.0, met * (1.0 - std::pow(1.0 - 1.0 / met, 0.75 * (double)rows))));
+    const double fill = (double)rows / segments / Cfg::ROWS;
     const double tiles = segments * (fill <= 0.75 ? 1.0 : fill <= 1.0 ? 1.0 + 2.0 * (fill - 0.75) : fill + 0.5);
     auto jobs = [](int width) {            // jobs that `width` columns cost
         const int full = width / Cfg::CH, rest = width % Cfg::CH;
@@ -780,7 +783,7 @@ static double stream_estimate(const StreamParams& prm, int64_t rows, int& split)
             // (the CTAs of a cluster take whole chunks: the first one has the most)
             const int in = S == 1 ? prm.p[i].d_in : std::min(prm.p[i].d_in, ceil_div(ceil_div(prm.p[i].d_in, Cfg::CH), S) * Cfg::CH);
             const int out = std::min(prm.p[i].d_out, ceil_div(och[i], S) * Cfg::CH);
-            const double each = jobs(in) + jobs(out) + (S > 1 ? 2.25 : 0.0);
+            const double each = jobs(in) + jobs(out) + (S > 1 ? 3.0 : 0.0);
             sum += each * (ustart[i + 1] - ustart[i]);
             longest = std::max(longest, each);
         }
