@@ -5,7 +5,7 @@
 // for it as two chained MMAs whose intermediate never leaves the SM:
 //
 //   shrink   T[128, R]   = X[128, d_in] * A_c[d_in, R]      accumulator in TMEM, K streamed in chunks of 64
-//   split    T = T_hi + T_lo (two bf16 tiles in shared memory; keeps ~16 mantissa bits of the fp32 T)
+//   split    T = T_hi + T_lo (two bf16 operands, in TMEM; keeps ~16 mantissa bits of the fp32 T)
 //   expand   D[128, 64]  = T_hi * B_c[:, n0:n0+64] + T_lo * B_c[:, n0:n0+64]   per 64-column chunk of d_out
 //   epilogue y[rows, n0:n0+64] += D    (fp32 add, one rounding to bf16, written back at the original rows)
 //
@@ -25,6 +25,12 @@
 // all of them hold the same bits), and CTA q then expands into the q-th slice of d_out.  x, y, A_c and B_c
 // are still read exactly once per tile.  The exchange uses mbarriers with remote arrives (bounded waits);
 // the only hardware cluster barriers are one after set-up and one before exit, which every thread reaches.
+//
+// What bounds it: large calls the memory, then (per SM) the shared-memory port, which an expand chunk of rank 64 takes for ~700
+// cycles -- y in, read, added and written, read again for the copy-out, B_c twice -- and before that the instruction stream of
+// the MMA warp, see there.  MMAs issued by one lane of a divergent branch, T in shared memory and 128 arrivals per D buffer (before)
+// against an elected lane of a uniform loop, T in TMEM and four arrivals (after), us: whole step of a wide layer at 8192 tokens 417 ->
+// 384, of 16384 interleaved tokens 135 -> 132, one 4096-wide projection at 1000 tokens behind the MLP router 37.2 -> 34.8.
 //
 // Warp roles (448 threads): warps 0-3 gather X and Y chunks, warp 4 fetches the A_c / B_c chunks, warp 5 issues
 // the MMAs and owns TMEM, warps 6-9 and 10-13 are two epilogue groups that take alternate 64-column chunks.  X chunks and Y chunks travel
@@ -245,7 +251,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
         mbar_init(bar(&ctrl->t_ready), 2 * kTileM);      // both epilogue groups
         for (int b = 0; b < kDBufs; ++b) {
             mbar_init(bar(&ctrl->d_full[b]), 1);
-            mbar_init(bar(&ctrl->d_empty[b]), kTileM);
+            mbar_init(bar(&ctrl->d_empty[b]), 4);        // the warps of an epilogue group
         }
         mbar_init(bar(&ctrl->part_full), 1);         // the partials arrive as asynchronous stores that count their bytes here
         // one push (ranks 16, 32): unused.  Two pushes (rank 64): the finished rows of T arrive by bulk copies that
@@ -298,6 +304,8 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
     const uint32_t tmem = ctrl->tmem_base;
     const uint32_t tmem_T = tmem;                               // columns [0, R)
     auto tmem_D = [&](int b) { return tmem + 64u + 64u * (uint32_t)b; };
+    const uint32_t tmem_T16 = tmem + 64u + 64u * kDBufs;        // bf16 T, two values a column: hi in columns [0, R/2), lo behind it
+    static_assert(64 + 64 * kDBufs + R <= kTmemCols, "TMEM columns");
 
     if (warp < kProducerWarps) {
         // ============================================================ gather producer
@@ -369,61 +377,60 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
         __syncwarp();
     } else if (warp == kMmaWarp) {
         // ============================================================ MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t idesc_shrink = idesc_bf16_f32(kTileM, rp, 0, 1);
-            // rows of an A chunk are r x 2 bytes: 128-, 64- or 32-byte swizzle
-            constexpr uint32_t wlayout = swizzle_layout_type(rp == 64 ? Swizzle::B128 : rp == 32 ? Swizzle::B64 : Swizzle::B32);
-            constexpr uint32_t wrow = (uint32_t)rp * 2u;
-            constexpr uint32_t idesc_expand = idesc_bf16_f32(kTileM, kChunkCols, 0, 1);
-            constexpr uint32_t kL128 = swizzle_layout_type(Swizzle::B128);
-            for (int it = 0; it < KX; ++it) {
-                const int s = it % Cfg::kStages;
-                const uint32_t ph = (uint32_t)(it / Cfg::kStages) & 1u;
-                wait_bar(bar(&ctrl->full[s]), ph, abort_flag, prm.dev_status);
-                fence_proxy_async_smem();     // the gathered rows were written through the generic proxy
-                tc_fence_after();
-                if (!*abort_flag) {
-                    const uint32_t a0 = stage(s), w0 = a0 + kTileBytes;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {   // four K = 16 steps per 64-column chunk
-                        const uint64_t ad = smem_desc(a0 + j * 32, 16, 1024, kL128);
-#pragma unroll
-                        for (int pt = 0; pt < PARTS; ++pt) {          // part pt -> columns [pt r, (pt + 1) r) of T
-                            const uint64_t bd = smem_desc(w0 + (uint32_t)pt * kChunkCols * wrow + j * (16 * wrow), 0, 8 * wrow, wlayout);
-                            umma_bf16(tmem_T + (uint32_t)(pt * rp), ad, bd, idesc_shrink, it > 0 || j > 0);
-                        }
-                    }
-                    umma_commit(bar(&ctrl->empty[s]));          // arrives when the MMAs have read the stage ...
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) mbar_arrive(bar(&ctrl->empty[s]));   // ... and completes the count of four
-                }
-            }
-            if (!*abort_flag) umma_commit(bar(&ctrl->t_full));
-            wait_bar(bar(&ctrl->t_ready), 0, abort_flag, prm.dev_status);
+        // The whole warp walks the chunks and one elected lane issues: descriptors and addresses are then the same in every lane, which
+        // is what the instruction takes, and cost an addition each.  Issued from code of one lane, a chunk of the shrink took ~600
+        // cycles and one of the expand ~1200 at rank 64, more than its bytes do.
+        const bool leader = elect_one();
+        const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem, 0);
+        constexpr uint32_t idesc_shrink = idesc_bf16_f32(kTileM, rp, 0, 1);
+        // rows of an A chunk are r x 2 bytes: 128-, 64- or 32-byte swizzle
+        constexpr uint32_t wlayout = swizzle_layout_type(rp == 64 ? Swizzle::B128 : rp == 32 ? Swizzle::B64 : Swizzle::B32);
+        constexpr uint32_t wrow = (uint32_t)rp * 2u;
+        constexpr uint32_t idesc_expand = idesc_bf16_f32(kTileM, kChunkCols, 0, 1);
+        constexpr uint32_t kL128 = swizzle_layout_type(Swizzle::B128);
+        // of stage 0; the address field counts 16 bytes and does not overflow below 256 KB
+        const uint64_t x_desc = smem_desc(base, 16, 1024, kL128);
+        const uint64_t a_desc = smem_desc(base + kTileBytes, 0, 8 * wrow, wlayout);
+        const uint64_t b_desc = smem_desc(base + kTileBytes, 0, 1024, kL128);
+        bool live = true;                           // no wait has run out
+        int s = 0;
+        uint32_t ph = 0;
+        for (int it = 0; it < KX; ++it) {
+            live = wait_bar(bar(&ctrl->full[s]), ph, abort_flag, prm.dev_status) && live;
+            fence_proxy_async_smem();               // the gathered rows were written through the generic proxy
             tc_fence_after();
-            for (int nc = 0; nc < NY; ++nc) {
-                const int it = KX + nc;
-                const int s = it % Cfg::kStages;
-                const uint32_t ph = (uint32_t)(it / Cfg::kStages) & 1u;
-                const int b = nc % kDBufs;
-                wait_bar(bar(&ctrl->full[s]), ph, abort_flag, prm.dev_status);
-                wait_bar(bar(&ctrl->d_empty[b]), ((uint32_t)(nc / kDBufs) & 1u) ^ 1u, abort_flag, prm.dev_status);
-                tc_fence_after();
-                if (!*abort_flag) {
-                    const uint32_t w0 = stage(s) + kTileBytes;
+            if (leader && live) {
+                const uint64_t at = (uint64_t)(s * (Cfg::kStageBytes >> 4));
 #pragma unroll
-                    for (int hl = 0; hl < 2; ++hl) {
-                        const uint32_t tb = hl ? tlo : thi;
+                for (int j = 0; j < 4; ++j)         // four K = 16 steps per 64-column chunk
 #pragma unroll
-                        for (int j = 0; j < R / 16; ++j) {
-                            const uint64_t ad = smem_desc(tb + j * 32, 16, 8 * Cfg::kTRowBytes, Cfg::kWLayout);
-                            const uint64_t bd = smem_desc(w0 + j * 2048, 0, 1024, kL128);
-                            umma_bf16(tmem_D(b), ad, bd, idesc_expand, hl > 0 || j > 0);
-                        }
-                    }
-                    umma_commit(bar(&ctrl->d_full[b]));
-                }
+                    for (int pt = 0; pt < PARTS; ++pt)           // part pt -> columns [pt r, (pt + 1) r) of T
+                        umma_bf16(tm + (uint32_t)(pt * rp), x_desc + at + j * (32 >> 4),
+                                  a_desc + at + ((pt * kChunkCols * wrow + j * 16 * wrow) >> 4), idesc_shrink, it > 0 || j > 0);
+                umma_commit(bar(&ctrl->empty[s]));               // arrives when the MMAs have read the stage ...
+                mbar_arrive_n(bar(&ctrl->empty[s]), 3);          // ... and completes the count of four
             }
+            if (++s == Cfg::kStages) { s = 0; ph ^= 1u; }
+        }
+        if (leader && live) umma_commit(bar(&ctrl->t_full));
+        live = wait_bar(bar(&ctrl->t_ready), 0, abort_flag, prm.dev_status) && live;
+        tc_fence_after();
+        for (int nc = 0; nc < NY; ++nc) {
+            const int b = nc % kDBufs;
+            live = wait_bar(bar(&ctrl->full[s]), ph, abort_flag, prm.dev_status) && live;
+            live = wait_bar(bar(&ctrl->d_empty[b]), ((uint32_t)(nc / kDBufs) & 1u) ^ 1u, abort_flag, prm.dev_status) && live;
+            tc_fence_after();
+            if (leader && live) {
+                const uint64_t at = (uint64_t)(s * (Cfg::kStageBytes >> 4));
+                const uint32_t d = tm + 64u + 64u * (uint32_t)b, t16 = tm + 64u + 64u * kDBufs;
+#pragma unroll
+                for (int hl = 0; hl < 2; ++hl)
+#pragma unroll
+                    for (int j = 0; j < R / 16; ++j)
+                        umma_bf16_ts(d, t16 + (uint32_t)(hl * (R / 2) + j * 8), b_desc + at + j * (2048 >> 4), idesc_expand, hl > 0 || j > 0);
+                umma_commit(bar(&ctrl->d_full[b]));
+            }
+            if (++s == Cfg::kStages) { s = 0; ph ^= 1u; }
         }
         __syncwarp();
     } else {
@@ -458,24 +465,22 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
             for (int j = 0; j < kUmmaMaxParts; ++j)
                 tscale[j] = pj.scale * ((pj.row_scale != nullptr && my_tok >= 0 && j < parts)
                                             ? __ldg(pj.row_scale + (int64_t)j * prm.N + my_tok) : 1.f);
-            // my half row -> T_hi / T_lo of this CTA
-            auto publish_local = [&]() {
+            // my half row of T, scaled, as bf16 hi and lo words
+            uint32_t hw[RH / 2], lw[RH / 2];
+            auto split_row = [&]() {
 #pragma unroll
-                for (int c8 = 0; c8 < RH / 8; ++c8) {
-                    float hi[8], lo[8];
-                    const int tpart = (col0 + c8 * 8) / rp;       // (r is a multiple of 16: a block of 8 columns has one part)
+                for (int c2 = 0; c2 < RH / 2; ++c2) {
+                    const int tpart = (col0 + c2 * 2) / rp;       // (r is a multiple of 16: a pair of columns has one part)
                     const float ts = PARTS == 1 ? tscale[0] : tpart == 0 ? tscale[0] : tpart == 1 ? tscale[1] : tpart == 2 ? tscale[2] : tscale[3];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const float t = __uint_as_float(tv[c8 * 8 + e]) * ts;
-                        hi[e] = __bfloat162float(__float2bfloat16_rn(t));
-                        lo[e] = t - hi[e];
-                    }
-                    const uint32_t off = swizzle_offset((uint32_t)row * Cfg::kTRowBytes + (uint32_t)(col0 / 8 + c8) * 16, Cfg::kSwzBits);
-                    const uint4 h = pack<__nv_bfloat16>(hi), l = pack<__nv_bfloat16>(lo);
-                    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(thi + off), "r"(h.x), "r"(h.y), "r"(h.z), "r"(h.w) : "memory");
-                    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(tlo + off), "r"(l.x), "r"(l.y), "r"(l.z), "r"(l.w) : "memory");
+                    const float t0 = __uint_as_float(tv[2 * c2]) * ts, t1 = __uint_as_float(tv[2 * c2 + 1]) * ts;
+                    const float h0 = __bfloat162float(__float2bfloat16_rn(t0)), h1 = __bfloat162float(__float2bfloat16_rn(t1));
+                    hw[c2] = f32x2_to_bf16x2(h0, h1);
+                    lw[c2] = f32x2_to_bf16x2(t0 - h0, t1 - h1);
                 }
+            };
+            // where 8 columns of my row lie in the shared-memory tiles that travel between the CTAs of a cluster (rank 64)
+            auto trow_offset = [&](int c8) {
+                return swizzle_offset((uint32_t)row * Cfg::kTRowBytes + (uint32_t)(col0 / 8 + c8) * 16, Cfg::kSwzBits);
             };
             const float4* recv_p = reinterpret_cast<const float4*>(smem_raw + (recv - raw));
             if (Cfg::kOnePush && S > 1) {
@@ -497,7 +502,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
                 }
                 wait_bar_cluster(bar(&ctrl->part_full), 0, abort_flag, prm.dev_status);
                 sum_partials<RH>(tv, recv_p + (col0 / 4) * kTileM + row, kTileM, kTileM * R / 4, S, crank);
-                publish_local();                                // tv holds the full half row
+                split_row();                                    // tv holds the full half row
             } else if (S > 1) {
                 // Exchange of the partial T tiles in two pushes through distributed shared memory.  CTA o owns the
                 // tile rows [o*128/S, (o+1)*128/S): (1) every CTA sends its partial of a row to the row's owner;
@@ -528,7 +533,15 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
                 wait_bar_cluster(bar(&ctrl->part_full), 0, abort_flag, prm.dev_status);
                 if ((uint32_t)owner == crank) {
                     sum_partials<RH>(tv, recv_p + (col0 / 4) * rows_max + (row - own_lo), rows_max, rows_max * R / 4, S, crank);
-                    publish_local();
+                    split_row();
+#pragma unroll
+                    for (int c8 = 0; c8 < RH / 8; ++c8) {
+                        const uint32_t off = trow_offset(c8);
+                        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(thi + off), "r"(hw[4 * c8]), "r"(hw[4 * c8 + 1]),
+                                     "r"(hw[4 * c8 + 2]), "r"(hw[4 * c8 + 3]) : "memory");
+                        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(tlo + off), "r"(lw[4 * c8]), "r"(lw[4 * c8 + 1]),
+                                     "r"(lw[4 * c8 + 2]), "r"(lw[4 * c8 + 3]) : "memory");
+                    }
                 }
                 // (3) my rows are a contiguous piece of each T tile (the swizzle permutes inside a row): two bulk copies
                 // per peer carry them over and count their bytes on the peer's barrier
@@ -544,64 +557,78 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
                         bulk_copy_to_peer(map_to_cta(thi + out_off, (uint32_t)lane), thi + out_off, out_bytes, pb);
                         bulk_copy_to_peer(map_to_cta(tlo + out_off, (uint32_t)lane), tlo + out_off, out_bytes, pb);
                     }
-                    wait_bar_cluster(bar(&ctrl->part_free), 0, abort_flag, prm.dev_status);   // all 128 rows of T are here
+                }
+                wait_bar_cluster(bar(&ctrl->part_free), 0, abort_flag, prm.dev_status);       // all 128 rows of T are here
+                if (group == 0) {
                     // tell every peer that its rows have arrived: it must not retire while the copy engine still reads them
                     if (warp == kEpiWarp0 && (uint32_t)lane < S && (uint32_t)lane != crank)
                         mbar_arrive_remote(map_to_cta(bar(&ctrl->peers_done), (uint32_t)lane));
                 }
+#pragma unroll
+                for (int c8 = 0; c8 < RH / 8; ++c8) {
+                    const uint32_t off = trow_offset(c8);
+                    const uint4 h = *reinterpret_cast<const uint4*>(smem_raw + (thi + off - raw));
+                    const uint4 l = *reinterpret_cast<const uint4*>(smem_raw + (tlo + off - raw));
+                    hw[4 * c8] = h.x, hw[4 * c8 + 1] = h.y, hw[4 * c8 + 2] = h.z, hw[4 * c8 + 3] = h.w;
+                    lw[4 * c8] = l.x, lw[4 * c8 + 1] = l.y, lw[4 * c8 + 2] = l.z, lw[4 * c8 + 3] = l.w;
+                }
             } else {
-                publish_local();
+                split_row();
             }
-            fence_proxy_async_smem();
+            // the operand of the expand stays in TMEM: its MMAs read it once per 64 columns of y, 2 x 128 x R x 2 bytes that would
+            // otherwise come through the shared-memory port the epilogue needs
+            __syncwarp();
+            tmem_st<RH / 2>(tmem_T16 + lane_addr + (uint32_t)(col0 / 2), hw);
+            tmem_st<RH / 2>(tmem_T16 + lane_addr + (uint32_t)(R / 2 + col0 / 2), lw);
+            tmem_wait_st();
             tc_fence_before();
             mbar_arrive(bar(&ctrl->t_ready));
         }
 
         // Copy-out mapping: a warp finishes and stores its OWN 32 rows (the TMEM lanes it reads), so the four warps of a
-        // group never wait for one another inside a chunk: piece (lane & 7) of rows q*32 + (lane >> 3) + 4 i.
-        const int piece = lane & 7;
-        int otok[8];
+        // group never wait for one another inside a chunk: piece (lane & 7) of rows q*32 + (lane >> 3) + 4 i, or, with 256-bit
+        // stores, pieces 2 (lane & 3) and the next of rows q*32 + (lane >> 2) + 8 i.
+        const bool wide = pj.wide_store != 0;
+        __nv_bfloat16* orow[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) otok[i] = ctrl->rows[q * 32 + (lane >> 3) + 4 * i];
-        int wtok[4];                                    // 256-bit variant: rows q*32 + (lane >> 2) + 8 i
-#pragma unroll
-        for (int i = 0; i < 4; ++i) wtok[i] = ctrl->rows[q * 32 + (lane >> 2) + 8 * i];
+        for (int i = 0; i < 8; ++i) {
+            const int r = wide ? (lane >> 2) + 8 * (i & 3) : (lane >> 3) + 4 * i;
+            const int tok = ctrl->rows[q * 32 + r];
+            orow[i] = tok < 0 ? nullptr : pj.y + (int64_t)tok * pj.ldy + ny0 * kChunkCols + (wide ? (lane & 3) * 16 : (lane & 7) * 8);
+        }
+        int s = (KX + group) % Cfg::kStages;
+        uint32_t ph = (uint32_t)((KX + group) / Cfg::kStages) & 1u;
         for (int nc = group; nc < NY; nc += kEpiGroups) {
-            const int it = KX + nc;
-            const int s = it % Cfg::kStages;
-            const uint32_t ph = (uint32_t)(it / Cfg::kStages) & 1u;
             const int b = nc % kDBufs;
+            uint8_t* ytile = smem_raw + (stage(s) - raw);
+            wait_bar(bar(&ctrl->full[s]), ph, abort_flag, prm.dev_status);   // the Y chunk of this stage has landed
+            uint4 yp[8];
+#pragma unroll
+            for (int c8 = 0; c8 < 8; ++c8)
+                yp[c8] = *reinterpret_cast<const uint4*>(ytile + swizzle_offset((uint32_t)row * 128u + c8 * 16, 3));
             wait_bar(bar(&ctrl->d_full[b]), (uint32_t)(nc / kDBufs) & 1u, abort_flag, prm.dev_status);
             tc_fence_after();
             uint32_t dv[64];
 #pragma unroll
             for (int c = 0; c < 4; ++c) tmem_ld_x16(tmem_D(b) + lane_addr + c * 16, dv + c * 16);
+            const bool dead = *abort_flag != 0;        // (every wait this chunk depends on is over)
             tmem_wait_ld();
             tc_fence_before();
-            mbar_arrive(bar(&ctrl->d_empty[b]));
-            wait_bar(bar(&ctrl->full[s]), ph, abort_flag, prm.dev_status);   // the Y chunk of this stage has landed
-            uint8_t* ytile = smem_raw + (stage(s) - raw);
-            {
-                uint4 yp[8];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(&ctrl->d_empty[b]));
 #pragma unroll
-                for (int c8 = 0; c8 < 8; ++c8)
-                    yp[c8] = *reinterpret_cast<const uint4*>(ytile + swizzle_offset((uint32_t)row * 128u + c8 * 16, 3));
+            for (int c8 = 0; c8 < 8; ++c8) {
+                float yv[8];
+                unpack<__nv_bfloat16>(yp[c8], yv);
 #pragma unroll
-                for (int c8 = 0; c8 < 8; ++c8) {
-                    float yv[8];
-                    unpack<__nv_bfloat16>(yp[c8], yv);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) yv[e] += __uint_as_float(dv[c8 * 8 + e]);
-                    *reinterpret_cast<uint4*>(ytile + swizzle_offset((uint32_t)row * 128u + c8 * 16, 3)) =
-                        pack<__nv_bfloat16>(yv);
-                }
+                for (int e = 0; e < 8; ++e) yv[e] += __uint_as_float(dv[c8 * 8 + e]);
+                *reinterpret_cast<uint4*>(ytile + swizzle_offset((uint32_t)row * 128u + c8 * 16, 3)) = pack<__nv_bfloat16>(yv);
             }
             __syncwarp();                              // my warp's 32 rows are finished in the stage
-            if (!*abort_flag) {
-                if (pj.wide_store) {
+            if (!dead) {
+                if (wide) {
                     // 32 bytes per lane: four lanes cover a 128-byte row segment, a warp instruction eight rows
                     const int p32 = lane & 3;
-                    __nv_bfloat16* dstc = pj.y + (ny0 + nc) * kChunkCols + p32 * 16;
                     uint4 lo4[4], hi4[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
@@ -611,9 +638,9 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
                     }
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        if (wtok[i] >= 0) stg256(dstc + (int64_t)wtok[i] * pj.ldy, lo4[i], hi4[i]);
+                        if (orow[i] != nullptr) stg256(orow[i] + nc * kChunkCols, lo4[i], hi4[i]);
                 } else {
-                    __nv_bfloat16* dstc = pj.y + (ny0 + nc) * kChunkCols + piece * 8;
+                    const int piece = lane & 7;
                     uint4 op[8];
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
@@ -621,11 +648,13 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
                             ytile + swizzle_offset((uint32_t)(q * 32 + (lane >> 3) + 4 * i) * 128u + piece * 16, 3));
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
-                        if (otok[i] >= 0) stg128(dstc + (int64_t)otok[i] * pj.ldy, op[i]);
+                        if (orow[i] != nullptr) stg128(orow[i] + nc * kChunkCols, op[i]);
                 }
             }
             __syncwarp();                              // every lane has read its pieces
             if (lane == 0) mbar_arrive(bar(&ctrl->empty[s]));   // one of four: the stage may be refilled when all warps are done
+            s += kEpiGroups;
+            if (s >= Cfg::kStages) { s -= Cfg::kStages; ph ^= 1u; }
         }
     }
 

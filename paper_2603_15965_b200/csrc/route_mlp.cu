@@ -149,28 +149,31 @@ __global__ void __launch_bounds__(kMlpThreads, 1) route_mlp_umma_kernel(const __
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16_f32(128, 192, 0, 0);              // both operands K-major
-            constexpr uint32_t kL128 = swizzle_layout_type(Swizzle::B128);
-            int s = 0;
-            uint32_t ph = 0;
-            for (int kc = kc0; kc < kc1; ++kc) {
-                wait_bar(bar(&ctrl->full[s]), ph, abort_flag, prm.dev_status);
-                tc_fence_after();
-                if (!*abort_flag) {
-                    const uint32_t a0 = stage(s), b0 = a0 + kMlpTileBytes;
+        // (the warp walks the chunks, one elected lane issues: see apply_umma.cu)
+        const bool leader = elect_one();
+        const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem, 0);
+        constexpr uint32_t idesc = idesc_bf16_f32(128, 192, 0, 0);              // both operands K-major
+        constexpr uint32_t kL128 = swizzle_layout_type(Swizzle::B128);
+        const uint64_t x_desc = smem_desc(base, 16, 1024, kL128), w_desc = smem_desc(base + kMlpTileBytes, 16, 1024, kL128);
+        bool live = true;
+        int s = 0;
+        uint32_t ph = 0;
+        for (int kc = kc0; kc < kc1; ++kc) {
+            live = wait_bar(bar(&ctrl->full[s]), ph, abort_flag, prm.dev_status) && live;
+            tc_fence_after();
+            if (leader && live) {
+                const uint64_t at = (uint64_t)(s * (STAGE >> 4));
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
+                for (int j = 0; j < 4; ++j)
 #pragma unroll
-                        for (int h2 = 0; h2 < NMMA; ++h2)
-                            umma_bf16(tmem + 192u * h2, smem_desc(a0 + j * 32, 16, 1024, kL128),
-                                      smem_desc(b0 + h2 * 192 * 128 + j * 32, 16, 1024, kL128), idesc, kc > kc0 || j > 0);
-                    umma_commit(bar(&ctrl->empty[s]));
-                }
-                if (++s == STAGES) { s = 0; ph ^= 1u; }
+                    for (int h2 = 0; h2 < NMMA; ++h2)
+                        umma_bf16(tm + 192u * h2, x_desc + at + j * (32 >> 4), w_desc + at + ((h2 * 192 * 128 + j * 32) >> 4), idesc,
+                                  kc > kc0 || j > 0);
+                umma_commit(bar(&ctrl->empty[s]));
             }
-            if (!*abort_flag) umma_commit(bar(&ctrl->done));
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
+        if (leader && live) umma_commit(bar(&ctrl->done));
         __syncwarp();
     } else {
         // ============================================================ epilogue: thread = token
