@@ -226,11 +226,24 @@ __global__ void __launch_bounds__(WARPS * 32) route_gate_mma_kernel(const __nv_b
 // launch.  Measured (us, before -> after): 93 tokens x 4096, C = 16: 34.4 -> 5.7; 777 x 2048, C = 8: 12.0 -> 4.7.
 // Every 16 tokens read the whole weight image (L2), and a second wave of CTAs costs as much as the first; gate_split_preferred says
 // which of the larger calls it still takes.
+// RAW: the weights come as they are (fp32 G [d, C]) and a warp splits its chunk's fragments in registers -- the values, and so
+// the results, of the image -- instead of reading an image that a launch before this one wrote.  Both launches -> this one, us:
+// 93 x 4096, C = 16 7.0 -> 5.2; 777 x 2048, C = 8 5.3 -> 4.3; 2048 x 2048 5.9 -> 5.7; 1000 x 4096, C = 16 9.2 -> 7.4.
 constexpr int kGateSplitWarps = 8;
-template <int NT, int KC>
+// two fp32 weights -> the three terms of both, packed
+__device__ __forceinline__ void gate_split_pair(float v0, float v1, uint32_t (&w)[3])
+{
+    const float h0 = __bfloat162float(__float2bfloat16_rn(v0)), h1 = __bfloat162float(__float2bfloat16_rn(v1));
+    const float r0 = v0 - h0, r1 = v1 - h1;
+    const float m0 = __bfloat162float(__float2bfloat16_rn(r0)), m1 = __bfloat162float(__float2bfloat16_rn(r1));
+    w[0] = f32x2_to_bf16x2(h0, h1);
+    w[1] = f32x2_to_bf16x2(m0, m1);
+    w[2] = f32x2_to_bf16x2(r0 - m0, r1 - m1);
+}
+template <int NT, int KC, bool RAW>
 __global__ void __launch_bounds__(kGateSplitWarps * 32, 2)
     route_gate_split_kernel(const __nv_bfloat16* __restrict__ x, int64_t N, int d, int64_t ldx,
-                            const __nv_bfloat16* __restrict__ img, const float* __restrict__ bias, int C,
+                            const void* __restrict__ weights, const float* __restrict__ bias, int C,
                             int32_t* __restrict__ r_out, float* __restrict__ logits_out)
 {
     using Img = GateImage<NT, KC>;
@@ -252,7 +265,6 @@ __global__ void __launch_bounds__(kGateSplitWarps * 32, 2)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[n][t][i] = 0.f;
     const int chunks = (d + KC - 1) / KC;
-    bool waited = false;
     for (int ch = crank * kGateSplitWarps + warp; ch < chunks; ch += S * kGateSplitWarps) {
         uint4 va[NB], vb[NB];
 #pragma unroll
@@ -262,27 +274,50 @@ __global__ void __launch_bounds__(kGateSplitWarps * 32, 2)
             va[b] = in ? ldg128_stream(xa + k) : make_uint4(0, 0, 0, 0);
             vb[b] = in ? ldg128_stream(xb + k) : make_uint4(0, 0, 0, 0);
         }
-        if (!waited) ptx::grid_dependency_sync();                     // the weight images come from gate_split_kernel
-        waited = true;
-        const __nv_bfloat16* gi = img + (int64_t)ch * Img::kElems + g * ROW + q * 4;
         constexpr int BB = NT == 1 ? 4 : NT == 2 ? 2 : 1;             // blocks whose weights are in flight at once
         static_assert(NB % BB == 0, "whole batches");
 #pragma unroll
         for (int b0 = 0; b0 < NB; b0 += BB) {
             uint32_t w[BB][2][NT][3][2];
-            // (volatile: the compiler must not move these above the wait for the kernel that writes the image)
+            if constexpr (RAW) {
+                // fragment slots 4 s + e of a 32-wide block are k = 8 q + 4 s + e, e = 0..3: eight rows of G per block and lane
+                float v[BB][NT][8];
 #pragma unroll
-            for (int b = 0; b < BB; ++b)
+                for (int b = 0; b < BB; ++b)
 #pragma unroll
-                for (int s = 0; s < 2; ++s)
+                    for (int n = 0; n < NT; ++n) {
+                        const int k = ch * KC + (b0 + b) * 32 + q * 8, c = n * 8 + g;
+                        const bool in = k < d && c < C;                  // (d is a multiple of 8)
+                        const float* Gk = static_cast<const float*>(weights) + (int64_t)k * C + c;
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) v[b][n][e] = in ? __ldg(Gk + e * C) : 0.f;
+                    }
+#pragma unroll
+                for (int b = 0; b < BB; ++b)
 #pragma unroll
                     for (int n = 0; n < NT; ++n)
 #pragma unroll
-                        for (int t = 0; t < 3; ++t)
-                            asm volatile("ld.global.v2.u32 {%0,%1}, [%2];"
-                                         : "=r"(w[b][s][n][t][0]), "=r"(w[b][s][n][t][1])
-                                         : "l"(gi + (t * CP + n * 8) * ROW + (b0 + b) * 32 + s * 16)
-                                         : "memory");
+                        for (int e = 0; e < 8; e += 2) {
+                            uint32_t terms[3];
+                            gate_split_pair(v[b][n][e], v[b][n][e + 1], terms);
+#pragma unroll
+                            for (int t = 0; t < 3; ++t) w[b][e >> 2][n][t][(e >> 1) & 1] = terms[t];
+                        }
+            } else {
+                const __nv_bfloat16* gi = static_cast<const __nv_bfloat16*>(weights) + (int64_t)ch * Img::kElems + g * ROW + q * 4;
+#pragma unroll
+                for (int b = 0; b < BB; ++b)
+#pragma unroll
+                    for (int s = 0; s < 2; ++s)
+#pragma unroll
+                        for (int n = 0; n < NT; ++n)
+#pragma unroll
+                            for (int t = 0; t < 3; ++t)
+                                asm volatile("ld.global.v2.u32 {%0,%1}, [%2];"
+                                             : "=r"(w[b][s][n][t][0]), "=r"(w[b][s][n][t][1])
+                                             : "l"(gi + (t * CP + n * 8) * ROW + (b0 + b) * 32 + s * 16)
+                                             : "memory");
+            }
 #pragma unroll
             for (int b = 0; b < BB; ++b)
 #pragma unroll
@@ -296,7 +331,6 @@ __global__ void __launch_bounds__(kGateSplitWarps * 32, 2)
                 }
         }
     }
-    if (!waited) ptx::grid_dependency_sync();
 #pragma unroll
     for (int n = 0; n < NT; ++n)
 #pragma unroll
@@ -374,6 +408,16 @@ static molora_status_t gate_mma_launch(const void* x, int64_t N, int d, int64_t 
     __nv_bfloat16* img = static_cast<__nv_bfloat16*>(ws);
     const int chunks = (d + KC - 1) / KC;
     const int64_t elems = (int64_t)chunks * KC * NT * 8;
+    if (image != kImageBuildOnly && gate_split_preferred(N, d, C)) {
+        const int S = gate_split_ctas(chunks);
+        const dim3 grid((unsigned)(ceil_div64(N, 16) * S)), block(kGateSplitWarps * 32);
+        const __nv_bfloat16* xt = static_cast<const __nv_bfloat16*>(x);
+        if (image == kImageBuildAndUse)            // no image for one use: the kernel splits what it needs
+            return cuda_ok(launch_kernel(route_gate_split_kernel<NT, KC, true>, grid, block, 0, s, (unsigned)S, false, xt, N, d, ldx, G,
+                                         bias, C, r_out, logits_out));
+        return cuda_ok(launch_kernel(route_gate_split_kernel<NT, KC, false>, grid, block, 0, s, (unsigned)S, false, xt, N, d, ldx, img,
+                                     bias, C, r_out, logits_out));
+    }
     if (image != kImageUseOnly) {
         if (cudaError_t e = launch_kernel(gate_split_kernel<NT, KC>,
                                           dim3((unsigned)std::min<int64_t>(ceil_div64(elems, 256), 148 * 4)), dim3(256), 0, s,
@@ -382,12 +426,6 @@ static molora_status_t gate_mma_launch(const void* x, int64_t N, int d, int64_t 
             return MOLORA_ERR_CUDA;
     }
     if (image == kImageBuildOnly) return MOLORA_OK;
-    if (gate_split_preferred(N, d, C)) {
-        const int S = gate_split_ctas(chunks);
-        return cuda_ok(launch_kernel(route_gate_split_kernel<NT, KC>, dim3((unsigned)(ceil_div64(N, 16) * S)), dim3(kGateSplitWarps * 32), 0,
-                                     s, (unsigned)S, image == kImageBuildAndUse, static_cast<const __nv_bfloat16*>(x), N, d, ldx, img, bias,
-                                     C, r_out, logits_out));
-    }
     const int64_t blocks = ceil_div64(N, 16 * WARPS);
     return cuda_ok(launch_kernel(route_gate_mma_kernel<NT, WARPS, KC>, dim3((unsigned)blocks), dim3(WARPS * 32), 0, s, 1,
                                  image == kImageBuildAndUse,
