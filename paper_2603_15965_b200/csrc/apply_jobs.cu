@@ -232,8 +232,9 @@ __global__ void __launch_bounds__(kJbThreads, 1) apply_jobs_kernel(const __grid_
     }
     asm volatile("" ::"r"(warm));
     if constexpr (GROUP) {
-        group_in_cta<kJbThreads, kJbMaxTokens>(prm.r, prm.N, prm.C, offs_s, tstart_s, perm_s, dsm, true, prm.counts_out,
-                                               prm.offsets_out, prm.perm_out, prm.dev_status);
+        group_in_cta<kJbThreads, kJbMaxTokens>(prm.r, prm.N, prm.C, offs_s, tstart_s, perm_s, dsm, 0, true, prm.counts_out,
+                                               prm.offsets_out, prm.dev_status);
+        group_write_perm(perm_s, offs_s[prm.C], prm.perm_out, tid, kJbThreads);
     } else {
         for (int i = tid; i <= prm.C; i += kJbThreads) offs_s[i] = __ldg(prm.offsets + i);
         for (int i = tid; i < prm.N; i += kJbThreads) perm_s[i] = __ldg(prm.perm + i);

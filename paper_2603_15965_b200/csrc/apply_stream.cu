@@ -135,6 +135,7 @@ struct FsCfg {
     static constexpr int SMEM = NSTAGE * STAGE + RECV + 1024;  // (the stages start at a 1024-byte boundary)
     static_assert(SMEM + 20992 <= 232448, "with the static tables a CTA fits an SM");
     static_assert(KW * TFLOATS * 4 <= STAGE, "the per-warp partials are summed through one stage");
+    static_assert(kGroupInCtaScratch<kFsThreads> <= NSTAGE * STAGE, "the grouping scratch is the ring");
 };
 template <int R, bool SHORT, int V>
 struct FsArgs : std::conditional_t<FsCfg<R, SHORT, V>::BOX, StreamMaps, NoMaps>, StreamParams {
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
     const int cid = (int)blockIdx.x / S, ncl = (int)gridDim.x / S;
     unsigned char* dsm = dsm_raw + ((1024u - (smem_u32(dsm_raw) & 1023u)) & 1023u);
     float* recv = reinterpret_cast<float*>(dsm + NS * Cfg::STAGE);         // [slot][rank][TFLOATS]
-    if (tid == 0) {
+    if (tid == kFsThreads - 32) {              // (not of the first warps: the tokens of a small call are theirs)
         for (int s = 0; s < NS; ++s) {
             mbar_init(smem_u32(&full_s[s]), kFsCopyWarps);
             mbar_init(smem_u32(&done_s[s]), kFsWarps);
@@ -248,8 +249,8 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
             reinterpret_cast<uint32_t*>(set_tab_s)[i] = __ldg(reinterpret_cast<const uint32_t*>(prm.set_table) + i);
     if constexpr (GROUP) {
         // the grouping itself, on this CTA, while the ring is idle (its memory is the scratch)
-        group_in_cta<kFsThreads, kFsPermCache>(prm.r, prm.N, prm.C, offs_s, tstart_s, perm_s, dsm, true, prm.counts_out,
-                                               prm.offsets_out, prm.perm_out, prm.dev_status);
+        group_in_cta<kFsThreads, kFsPermCache>(prm.r, prm.N, prm.C, offs_s, tstart_s, perm_s, dsm, Cfg::ROWS, true, prm.counts_out,
+                                               prm.offsets_out, prm.dev_status);
     } else {
         // segment table and (small calls) the permutation on chip in one memory round trip
         for (int i = tid; i <= prm.C; i += kFsThreads) offs_s[i] = __ldg(prm.offsets + i);
@@ -259,8 +260,11 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
     }
     // tiles of the segments before each segment (those with 1 <= rows < max_rows own tiles here), so that an item finds
     // its tile by bisection instead of a walk over all segments
-    if (warp == 0) tile_starts(offs_s, prm.C, Cfg::ROWS, 1, prm.max_rows, tstart_s);
-    __syncthreads();
+    // (the grouping variant has done that)
+    if constexpr (!GROUP) {
+        if (warp == 0) tile_starts(offs_s, prm.C, Cfg::ROWS, 1, prm.max_rows, tstart_s);
+        __syncthreads();
+    }
     const int T = tstart_s[prm.C];
     const int nitems = T * prm.ustart[prm.P];
     // Items of my cluster: one of every ncl consecutive ones, from the front and from the back in turn.  Items are numbered
@@ -406,6 +410,7 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
         const int g4 = lane >> 2, q = lane & 3;
         const int kw = warp % Cfg::KW, n0 = warp / Cfg::KW * (NT * 8);        // my share of the k blocks, my columns of t
         uint32_t g = 0;
+        if constexpr (GROUP) group_write_perm(perm_s, offs_s[prm.C], prm.perm_out, tid, kFsWarps * 32);
         auto slot_of = [&](int i, int rank) { return recv + ((i & 1) * S + rank) * Cfg::TFLOATS; };
         // LoRA scale x the token's routing weight (top-k in one pass: the weight of the part the column belongs to)
         auto scaled = [&](const FsItem& it, const molora_proj_desc_t& pd, int e4, float4 v) {

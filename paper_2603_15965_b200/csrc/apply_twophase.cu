@@ -125,8 +125,10 @@ __device__ __forceinline__ int tp_load_tables(const TwoPhaseParams& prm, int32_t
 {
     const int tid = threadIdx.x;
     if constexpr (GROUP) {
-        group_in_cta<kTpThreads, kTpPermCache>(prm.r, prm.N, prm.C, offs_s, tstart_s, perm_s, scratch, write_out, prm.counts_out,
-                                               prm.offsets_out, prm.perm_out, prm.dev_status);
+        group_in_cta<kTpThreads, kTpPermCache>(prm.r, prm.N, prm.C, offs_s, tstart_s, perm_s, scratch, kTpRows, write_out, prm.counts_out,
+                                               prm.offsets_out, prm.dev_status);
+        if (write_out) group_write_perm(perm_s, offs_s[prm.C], prm.perm_out, tid, kTpThreads);
+        return tstart_s[prm.C];
     } else {
         for (int i = tid; i <= prm.C; i += kTpThreads) offs_s[i] = __ldg(prm.offsets + i);
         if (prm.N <= kTpPermCache)
@@ -472,8 +474,7 @@ size_t decode_workspace_bytes(int64_t N, int32_t d_in, int32_t rank)
 template <int R, bool GROUP>
 static cudaError_t twophase_launch(const TwoPhaseParams& prm, int64_t N, cudaStream_t s)
 {
-    static_assert(kGroupInCtaTableMaxC * kTpThreads * 4 + 4 * kGroupInCtaTableMaxC <= TpCfg<R>::SHRINK_SMEM &&
-                      kGroupInCtaTableMaxC * kTpThreads * 4 + 4 * kGroupInCtaTableMaxC <= TpCfg<R>::EXPAND_SMEM,
+    static_assert(kGroupInCtaScratch<kTpThreads> <= TpCfg<R>::SHRINK_SMEM && kGroupInCtaScratch<kTpThreads> <= TpCfg<R>::EXPAND_SMEM,
                   "the grouping scratch fits the staging areas");
     using Cfg = TpCfg<R>;
     // resident CTAs of each kernel on this device: the size of a wave

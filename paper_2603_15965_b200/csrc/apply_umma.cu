@@ -231,9 +231,8 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
     int32_t* perm_s = reinterpret_cast<int32_t*>(smem_raw + (base - raw));
     int32_t* gtmp_s = perm_s + kUmmaGroupMaxN;
     unsigned char* gscratch = reinterpret_cast<unsigned char*>(gtmp_s + MOLORA_MAX_ADAPTERS);
-    static_assert(kUmmaGroupMaxN * 4 + MOLORA_MAX_ADAPTERS * 4 + kGroupInCtaTableMaxC * kUmmaThreads * 4 + 4 * kGroupInCtaTableMaxC <=
-                      Cfg::kStages * Cfg::kStageBytes, "the grouping scratch must fit the ring");
-    static_assert(kUmmaThreads / 32 * MOLORA_MAX_ADAPTERS * 4 <= kGroupInCtaTableMaxC * kUmmaThreads * 4, "ballot-path scratch");
+    static_assert(kUmmaGroupMaxN * 4 + MOLORA_MAX_ADAPTERS * 4 + kGroupInCtaScratch<kUmmaThreads> <= Cfg::kStages * Cfg::kStageBytes,
+                  "the grouping scratch must fit the ring");
     int32_t offs_v[(MOLORA_MAX_ADAPTERS + kUmmaThreads) / kUmmaThreads];
 #pragma unroll
     for (int j = 0; j < (MOLORA_MAX_ADAPTERS + kUmmaThreads) / kUmmaThreads; ++j) {
@@ -267,8 +266,9 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
     }
     // which tile is mine: the segment table goes on chip (or is built there), then the tile is looked up there
     if (grouping) {
-        group_in_cta<kUmmaThreads, kUmmaGroupMaxN>(prm.r, prm.N, prm.C, offs_s, gtmp_s, perm_s, gscratch, blockIdx.y == 0,
-                                                   prm.counts_out, prm.offsets_out, prm.perm_out, prm.dev_status);
+        group_in_cta<kUmmaThreads, kUmmaGroupMaxN>(prm.r, prm.N, prm.C, offs_s, gtmp_s, perm_s, gscratch, 0, blockIdx.y == 0,
+                                                   prm.counts_out, prm.offsets_out, prm.dev_status);
+        if (blockIdx.y == 0) group_write_perm(perm_s, offs_s[prm.C], prm.perm_out, tid, kUmmaThreads);
     } else {
 #pragma unroll
         for (int j = 0; j < (MOLORA_MAX_ADAPTERS + kUmmaThreads) / kUmmaThreads; ++j) {
@@ -354,6 +354,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
     } else if (warp == kWeightWarp) {
         // ============================================================ weight-chunk producer (TMA)
         if (lane == 0) {
+            if (grouping) fence_proxy_async_smem();          // the ring was the grouping's scratch
             int s = 0;
             uint32_t ph = 1;
             for (int it = 0; it < total; ++it) {

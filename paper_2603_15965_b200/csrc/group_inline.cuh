@@ -1,26 +1,86 @@
 // Section 3.3 steps 1-3 (histogram, exclusive scan, stable permutation) done by ONE CTA in its own shared memory, for
 // kernels that start from the routing decisions r instead of offsets / perm: every CTA of such a kernel runs this
 // before its first copy request, which replaces the table load and saves the grouping launch.  At most MAXN tokens.
-// Results: offs_s[0..C], perm_s[0..offs_s[C]); with write_out the CTAs also write counts, offsets and perm to global
-// memory (CTA 0 the two small arrays, every CTA a slice of perm), bit-equal to what molora_group writes.
-//   scratch   shared memory that is idle at this point: max(kGroupInCtaTableMaxC * NT * 4 + 4 * kGroupInCtaTableMaxC,
-//             NT / 32 * MOLORA_MAX_ADAPTERS * 4) bytes
-//   tstart_s  MOLORA_MAX_ADAPTERS ints of temporary storage (the caller's tile prefix, filled afterwards)
+// Results: offs_s[0..C], perm_s[0..offs_s[C]) and, with tile_rows > 0, tstart_s[0..C] (tiles of tile_rows rows before each segment);
+// with write_out CTA 0 also writes counts and offsets to global memory and the CTAs are to write perm with group_write_perm, a slice
+// each, whenever it suits them -- bit-equal to what molora_group writes.
+//   scratch   shared memory that is idle at this point: kGroupInCtaScratch<NT> bytes
+//   tstart_s  MOLORA_MAX_ADAPTERS + 1 ints (temporary storage where no tiles are asked for)
 // Ends with a block-wide barrier.  All NT threads of the CTA must call it.
 #pragma once
 #include "common.cuh"
 
 namespace molora {
 
-constexpr int kGroupInCtaTableMaxC = 32;       // adapters handled by the per-thread count table (ballots / match above)
+constexpr int kGroupInCtaTableMaxC = 32;       // adapters handled by lanes and by the per-thread count table (ballots / match above)
+template <int NT>
+constexpr int kGroupInCtaScratch = kGroupInCtaTableMaxC * NT * 4 + 4 * kGroupInCtaTableMaxC;      // (covers the histograms of the ballots)
 
 template <int NT, int MAXN>
 __device__ __forceinline__ void group_in_cta(const int32_t* __restrict__ r, int N_, int C_, int32_t* offs_s, int32_t* tstart_s,
-                                             int32_t* perm_s, unsigned char* scratch, bool write_out, int32_t* counts_out,
-                                             int32_t* offsets_out, int32_t* perm_out, uint32_t* dev_status)
+                                             int32_t* perm_s, unsigned char* scratch, int tile_rows, bool write_out, int32_t* counts_out,
+                                             int32_t* offsets_out, uint32_t* dev_status)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
         constexpr int NW = NT / 32;
+        static_assert(NW * MOLORA_MAX_ADAPTERS * 4 <= kGroupInCtaScratch<NT>, "histograms of the ballots");
+      if (C_ <= kGroupInCtaTableMaxC && N_ <= NT) {
+        // A token per thread, lane c counts adapter c: one ballot per bit of the adapter index, from which every lane takes the tokens
+        // of its adapter (for the count) and the tokens that share its own token's (for the rank); the warps meet once.  What bounds it
+        // is the code that a CTA meets for the first time, fetched at about ten cycles an instruction: the loops stay rolled.  With the
+        // table below a decode call of 8 tokens was grouped after 4900 cycles, so after 3500; with more steps a warp it is the slower one.
+        int* hist = reinterpret_cast<int*>(scratch);                               // [warp][32]
+        const int C = C_, N = N_;
+        const int raw = tid < N ? __ldg(r + tid) : -1;
+        const int v = raw < C ? raw : -1;
+        unsigned own = __ballot_sync(0xFFFFFFFFu, v >= 0), same = own;
+        const int bits = 32 - __clz(C - 1);
+#pragma unroll 1
+        for (int b = 0; b < bits; ++b) {
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, (v >> b) & 1);
+            own &= m ^ (((unsigned)lane >> b & 1u) - 1u);                          // (m where my bit is set, ~m where it is not)
+            same &= m ^ (((unsigned)v >> b & 1u) - 1u);
+        }
+        hist[warp * 32 + lane] = __popc(own);            // (lanes past C repeat others' counts and are never read)
+        __syncthreads();
+        int before = 0, total = 0;
+        const int warps = (N + 31) >> 5;
+#pragma unroll 4
+        for (int w = 0; w < warps; ++w) {
+            const int t = hist[w * 32 + lane];
+            if (w < warp) before += t;
+            total += t;
+        }
+        if (lane >= C) total = 0;
+        int incl = total, tiles = tile_rows > 0 ? (total + tile_rows - 1) / tile_rows : 0, tincl = tiles;
+#pragma unroll 1
+        for (int off = 1; off < 32; off <<= 1) {
+            const int up = __shfl_up_sync(0xFFFFFFFFu, incl, off), tup = __shfl_up_sync(0xFFFFFFFFu, tincl, off);
+            if (lane >= off) {
+                incl += up;
+                tincl += tup;
+            }
+        }
+        const int at = __shfl_sync(0xFFFFFFFFu, incl - total + before, v & 31) + __popc(same & ((1u << lane) - 1u));
+        if (v >= 0) perm_s[at] = tid;
+        if (warp == 0 && lane < C) {
+            offs_s[lane] = incl - total;
+            if (lane == C - 1) offs_s[C] = incl;
+            if (tile_rows > 0) {
+                tstart_s[lane] = tincl - tiles;
+                if (lane == C - 1) tstart_s[C] = tincl;
+            }
+            if (write_out && blockIdx.x == 0) {
+                counts_out[lane] = total;
+                offsets_out[lane] = incl - total;
+                if (lane == C - 1) offsets_out[C] = incl;
+            }
+        }
+        if ((write_out && blockIdx.x == 0) && dev_status != nullptr && __any_sync(0xFFFFFFFFu, raw < -1 || raw >= C) && lane == 0)
+            atomicOr(dev_status, MOLORA_DEV_BAD_ROUTE);
+        __syncthreads();
+        return;
+      }
       if (C_ <= kGroupInCtaTableMaxC) {
         // Up to 32 adapters: every thread owns a contiguous run of tokens and counts it into its own column of a
         // [adapter][thread] table in shared memory (consecutive threads hit consecutive banks); a warp
@@ -183,13 +243,19 @@ __device__ __forceinline__ void group_in_cta(const int32_t* __restrict__ r, int 
         }
         __syncthreads();
       }
-        if (write_out) {   // my slice of perm
-            const int C = C_;
-            const int total = offs_s[C];
-            const int per = (total + (int)gridDim.x - 1) / (int)gridDim.x;
-            const int lo = (int)blockIdx.x * per, hi = min(lo + per, total);
-            for (int i = lo + tid; i < hi; i += NT) perm_out[i] = perm_s[i];
+        if (tile_rows > 0) {
+            if (warp == 0) tile_starts(offs_s, C_, tile_rows, 1, INT32_MAX, tstart_s);
+            __syncthreads();
         }
+}
+
+// Writes the CTA's slice of perm out, with `threads` threads numbered from `tid`.
+__device__ __forceinline__ void group_write_perm(const int32_t* perm_s, int total, int32_t* perm_out, int tid, int threads)
+{
+    const int per = (total + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int lo = (int)blockIdx.x * per, hi = min(lo + per, total);
+#pragma unroll 1
+    for (int i = lo + tid; i < hi; i += threads) perm_out[i] = perm_s[i];
 }
 
 }  // namespace molora
