@@ -267,7 +267,8 @@ molora_status_t molora_apply_batched(const molora_proj_desc_t *projs, int32_t P,
  * (counts, offsets and perm are written, bit-equal to molora_group's), status bits and error behaviour of those two
  * calls; ws / ws_bytes as for molora_apply_batched.  When every projection of the call runs, with one rank, on the
  * single-launch streaming kernel, on the tcgen05 kernel (at most 64 adapters) or, where "small_path" asks for it, on the job-list
- * kernel (bf16, at most 4096 tokens; 1024 for the job-list kernel) the whole call is ONE launch: every CTA builds the grouping in its shared memory before its first copy
+ * kernel (bf16, at most 4096 tokens; 1024 for the job-list kernel), or on the CUDA-core kernel while its tiles fit one wave (fp32
+ * storage or rank 8, at most 2048 tokens), the whole call is ONE launch: every CTA builds the grouping in its shared memory before its first copy
  * request, which saves the grouping launch; the two-launch small-tile kernels do the same for at most 1024 tokens;
  * otherwise the grouping launch and the apply launches are enqueued in stream order. */
 molora_status_t molora_group_apply_batched(const int32_t *r, int64_t N, int32_t C, int32_t *counts, int32_t *offsets,

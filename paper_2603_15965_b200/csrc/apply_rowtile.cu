@@ -16,6 +16,7 @@
 // The intermediate t never leaves the chip.  Tiles are located on the device from `offsets`
 // (no host read of the histogram), so the grid is sized for the worst case and surplus CTAs exit.
 #include "common.cuh"
+#include "group_inline.cuh"
 #include "sm100_ptx.cuh"
 #include "warp_reduce.cuh"
 
@@ -28,11 +29,27 @@ struct ApplyBatchParams {
     int32_t P;
     int32_t C;
     int32_t max_rows;     // segments with at least this many rows belong to the tensor-core kernel
+    // grouping variant only: the routing decisions and where counts / offsets / perm are written (as by molora_group)
+    const int32_t* r;
+    int32_t* counts_out;
+    int32_t* offsets_out;
+    int32_t* perm_out;
+    uint32_t* dev_status;
+    int32_t N;
 };
 
 constexpr int kRowTileThreads = 256;
+constexpr int kRowTileGroupMaxN = 2048;
+// what group_in_cta needs, all of it static: offsets, temporary words, perm and its scratch
+struct RowTileGroup {
+    int32_t offs[MOLORA_MAX_ADAPTERS + 1], tmp[MOLORA_MAX_ADAPTERS + 1], perm[kRowTileGroupMaxN];
+    alignas(16) unsigned char scratch[kGroupInCtaScratch<kRowTileThreads>];
+};
 
-template <typename T, int R>
+// GROUP: the call starts from the routing decisions r (at most kRowTileGroupMaxN tokens); every CTA groups them on chip, which costs
+// it ~1 us against a grouping launch of 3.4 us and the gap behind it (256 fp32 tokens 512 wide, vocabulary routing included: 15.4 us
+// in three launches, 12.3 in two).
+template <typename T, int R, bool GROUP>
 __global__ void __launch_bounds__(kRowTileThreads, 1) apply_rowtile_kernel(const __grid_constant__ ApplyBatchParams prm)
 {
     constexpr int VEC = VecTraits<T>::kElems;
@@ -45,14 +62,27 @@ __global__ void __launch_bounds__(kRowTileThreads, 1) apply_rowtile_kernel(const
 
     ptx::grid_dependency_sync();             // offsets and perm come from the grouping kernel
     int seg, row0, rows;
-    if (!find_tile(prm.offsets, prm.C, TM, blockIdx.x, 1, prm.max_rows, seg, row0, rows)) return;
+    const int32_t* perm_s = nullptr;
+    if constexpr (GROUP) {
+        __shared__ RowTileGroup grp;
+        group_in_cta<kRowTileThreads, kRowTileGroupMaxN>(prm.r, prm.N, prm.C, grp.offs, grp.tmp, grp.perm, grp.scratch, 0, blockIdx.y == 0,
+                                                         prm.counts_out, prm.offsets_out, prm.dev_status);
+        if (blockIdx.y == 0) group_write_perm(grp.perm, grp.offs[prm.C], prm.perm_out, threadIdx.x, kRowTileThreads);
+        if (!find_tile_smem(grp.offs, prm.C, TM, blockIdx.x, 1, INT32_MAX, seg, row0, rows)) return;
+        perm_s = grp.perm;
+    } else {
+        if (!find_tile(prm.offsets, prm.C, TM, blockIdx.x, 1, prm.max_rows, seg, row0, rows)) return;
+    }
 
     __shared__ __align__(16) float partial[WARPS][128];
     __shared__ __align__(16) float t_s[128];   // [TM][R]
     __shared__ int32_t row_s[TM];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (tid < TM) row_s[tid] = __ldg(prm.perm + row0 + (tid < rows ? tid : rows - 1));   // pad with the last row
+    if (tid < TM) {
+        const int pos = row0 + (tid < rows ? tid : rows - 1);                              // pad with the last row
+        row_s[tid] = GROUP ? perm_s[pos] : __ldg(prm.perm + pos);
+    }
     __syncthreads();
 
     const int d_in = pd.d_in, d_out = pd.d_out;
@@ -141,7 +171,7 @@ __global__ void __launch_bounds__(kRowTileThreads, 1) apply_rowtile_kernel(const
     }
 }
 
-template <typename T, int R>
+template <typename T, int R, bool GROUP>
 static cudaError_t rowtile_launch(const ApplyBatchParams& prm, int64_t N, cudaStream_t s)
 {
     constexpr int TM = 128 / R;
@@ -149,10 +179,10 @@ static cudaError_t rowtile_launch(const ApplyBatchParams& prm, int64_t N, cudaSt
     const int64_t cap_rows = prm.max_rows == INT32_MAX ? N : (N < (int64_t)prm.C * prm.max_rows ? N : (int64_t)prm.C * prm.max_rows);
     const int64_t tiles = ceil_div64(cap_rows, TM) + prm.C;
     dim3 grid((unsigned)tiles, (unsigned)prm.P);
-    return launch_kernel(apply_rowtile_kernel<T, R>, grid, dim3(kRowTileThreads), 0, s, 1, false, prm);
+    return launch_kernel(apply_rowtile_kernel<T, R, GROUP>, grid, dim3(kRowTileThreads), 0, s, 1, false, prm);
 }
 
-template <typename T>
+template <typename T, bool GROUP>
 static cudaError_t rowtile_dispatch(const ApplyBatchParams& prm, int64_t N, cudaStream_t s)
 {
     bool has[4] = {false, false, false, false};
@@ -161,11 +191,21 @@ static cudaError_t rowtile_dispatch(const ApplyBatchParams& prm, int64_t N, cuda
         has[r == 8 ? 0 : r == 16 ? 1 : r == 32 ? 2 : 3] = true;
     }
     cudaError_t e = cudaSuccess;
-    if (has[0] && e == cudaSuccess) e = rowtile_launch<T, 8>(prm, N, s);
-    if (has[1] && e == cudaSuccess) e = rowtile_launch<T, 16>(prm, N, s);
-    if (has[2] && e == cudaSuccess) e = rowtile_launch<T, 32>(prm, N, s);
-    if (has[3] && e == cudaSuccess) e = rowtile_launch<T, 64>(prm, N, s);
+    if (has[0] && e == cudaSuccess) e = rowtile_launch<T, 8, GROUP>(prm, N, s);
+    if (has[1] && e == cudaSuccess) e = rowtile_launch<T, 16, GROUP>(prm, N, s);
+    if (has[2] && e == cudaSuccess) e = rowtile_launch<T, 32, GROUP>(prm, N, s);
+    if (has[3] && e == cudaSuccess) e = rowtile_launch<T, 64, GROUP>(prm, N, s);
     return e;
+}
+
+static ApplyBatchParams rowtile_params(const molora_proj_desc_t* projs, int32_t P, int32_t C, int32_t max_rows)
+{
+    ApplyBatchParams prm{};
+    for (int i = 0; i < P; ++i) prm.p[i] = projs[i];
+    prm.P = P;
+    prm.C = C;
+    prm.max_rows = max_rows;
+    return prm;
 }
 
 molora_status_t launch_apply_rowtile(const molora_proj_desc_t* projs, int32_t P, molora_dtype_t dt, int64_t N,
@@ -173,15 +213,35 @@ molora_status_t launch_apply_rowtile(const molora_proj_desc_t* projs, int32_t P,
                                      cudaStream_t s)
 {
     if (N == 0 || P == 0) return MOLORA_OK;
-    ApplyBatchParams prm;
-    for (int i = 0; i < P; ++i) prm.p[i] = projs[i];
-    for (int i = P; i < MOLORA_MAX_PROJECTIONS; ++i) prm.p[i] = molora_proj_desc_t{};
+    ApplyBatchParams prm = rowtile_params(projs, P, C, max_rows);
     prm.offsets = offsets;
     prm.perm = perm;
-    prm.P = P;
-    prm.C = C;
-    prm.max_rows = max_rows;
-    return cuda_ok(dt == MOLORA_BF16 ? rowtile_dispatch<__nv_bfloat16>(prm, N, s) : rowtile_dispatch<float>(prm, N, s));
+    return cuda_ok(dt == MOLORA_BF16 ? rowtile_dispatch<__nv_bfloat16, false>(prm, N, s) : rowtile_dispatch<float, false>(prm, N, s));
+}
+
+// Grouping and apply in one launch: calls that go to this kernel with one rank (fp32 storage, or rank 8) while every tile has an SM
+// of its own -- a second wave would group again.
+bool group_apply_rowtile_eligible(const molora_proj_desc_t* projs, int32_t P, molora_dtype_t dt, int64_t N, int32_t C)
+{
+    const int32_t rank = projs[0].rank;
+    if (N < 1 || N > kRowTileGroupMaxN || (dt != MOLORA_F32 && rank != 8)) return false;
+    for (int i = 0; i < P; ++i)
+        if (projs[i].rank != rank || decode_eligible(projs[i], dt)) return false;
+    return (ceil_div64(N, 128 / rank) + C) * P <= sm_count();
+}
+
+molora_status_t launch_group_apply_rowtile(const int32_t* r, const molora_proj_desc_t* projs, int32_t P, molora_dtype_t dt, int64_t N,
+                                           int32_t C, int32_t* counts, int32_t* offsets, int32_t* perm, uint32_t* dev_status,
+                                           cudaStream_t s)
+{
+    ApplyBatchParams prm = rowtile_params(projs, P, C, INT32_MAX);
+    prm.r = r;
+    prm.counts_out = counts;
+    prm.offsets_out = offsets;
+    prm.perm_out = perm;
+    prm.dev_status = dev_status;
+    prm.N = (int32_t)N;
+    return cuda_ok(dt == MOLORA_BF16 ? rowtile_dispatch<__nv_bfloat16, true>(prm, N, s) : rowtile_dispatch<float, true>(prm, N, s));
 }
 
 }  // namespace molora

@@ -281,6 +281,11 @@ molora_status_t launch_group(const int32_t* r, int64_t N, int32_t C, int32_t* co
 molora_status_t launch_apply_rowtile(const molora_proj_desc_t* projs, int32_t P, molora_dtype_t dt, int64_t N,
                                      int32_t C, const int32_t* offsets, const int32_t* perm, int32_t max_rows,
                                      cudaStream_t s);
+// ... with the grouping inside, one launch, for the calls that group_apply_rowtile_eligible names
+bool group_apply_rowtile_eligible(const molora_proj_desc_t* projs, int32_t P, molora_dtype_t dt, int64_t N, int32_t C);
+molora_status_t launch_group_apply_rowtile(const int32_t* r, const molora_proj_desc_t* projs, int32_t P, molora_dtype_t dt, int64_t N,
+                                           int32_t C, int32_t* counts, int32_t* offsets, int32_t* perm, uint32_t* dev_status,
+                                           cudaStream_t s);
 // tcgen05 path for the segments with at least min_rows rows (bf16, rank 16/32/64, d_in and d_out multiples of 64).
 bool umma_eligible(const molora_proj_desc_t& p, molora_dtype_t dt);
 // With r (routing decisions, at most 4096 tokens, one rank, min_rows 1) the kernel groups on chip: offsets / perm /
