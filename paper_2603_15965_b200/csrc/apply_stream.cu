@@ -694,7 +694,7 @@ bool stream_eligible(const molora_proj_desc_t& p, molora_dtype_t dt)
 }
 
 // Output slices: one item per (projection, tile) to start with; while `most` units (items per tile) allow it, the widest is split once
-// more (a second round of items costs more than the imbalance it removes).  Returns the number of units.
+// more.  Returns the number of units.
 static int slice_outputs(const StreamParams& prm, int CH, int64_t most, int32_t* och, int32_t* ustart)
 {
     int slices[MOLORA_MAX_PROJECTIONS], chunks[MOLORA_MAX_PROJECTIONS], total = prm.P;
@@ -717,8 +717,56 @@ static int slice_outputs(const StreamParams& prm, int CH, int64_t most, int32_t*
 // most tiles that `rows` rows in C segments can give (every segment that has rows adds at most one partial tile)
 static int64_t tiles_bound(int64_t rows, int64_t C, int tile_rows) { return std::min(rows, ceil_div64(rows, tile_rows) + std::min(C, rows)); }
 
+// Tiles that `rows` rows are expected to give.
+static double expected_tiles(const StreamParams& prm, int64_t rows, int tile_rows)
+{
+    // Tiles of segments of about equal size: one each while that is well below a tile's height, half a tile lost per segment from there
+    // on.  Of the segments as many are counted as three quarters of the rows, spread at random, meet: adapters are not equally popular
+    // (rank 64, 4096 wide, 20 tokens of 16 adapters by popularity: clusters of four 26 us, of two, as for all 16, 32).  Of the adapter
+    // sets of top-k routing only those of different adapters are met; the others are there for callers that repeat one.
+    const double met = (double)(prm.parts > 1 && prm.n_adapters >= prm.parts ? binom_small(prm.n_adapters, prm.parts) : prm.C);
+    const double segments = std::min((double)rows, std::max(1.0, met * (1.0 - std::pow(1.0 - 1.0 / met, 0.75 * (double)rows))));
+    const double fill = (double)rows / segments / tile_rows;
+    return segments * (fill <= 0.75 ? 1.0 : fill <= 1.0 ? 1.0 + 2.0 * (fill - 0.75) : fill + 0.5);
+}
+
+// Output slices of calls whose items no longer fit one wave (one CTA per item): the launch lasts as long as its busiest CTA, and a
+// gate or up projection in a layer is six expand jobs behind two shrinks while the average CTA has five jobs.  Cutting it in two costs
+// two more shrinks and evens that out.  The dealing of the items is followed for the tiles that are expected, with up to four cuts; a
+// shrink job counts 0.65, an expand job 1.0 (measured in place at rank 16: 1240 and 1900 cycles).  256 tokens of 8 adapters, sixteen layers
+// 2048 wide: 207 us without cuts, 186 with.  Returns the number of units.
+static int balanced_units(const StreamParams& prm, int CH, int clusters, int tiles, int32_t* och, int32_t* ustart)
+{
+    constexpr int kCuts = 4, kMaxClusters = 256;
+    int best_units = prm.P;
+    float best = 0.f;
+    for (int most = prm.P; most <= prm.P + kCuts; ++most) {
+        const int units = slice_outputs(prm, CH, most, och, ustart);
+        if (units < most) break;
+        float load[kMaxClusters] = {};
+        float longest = 0.f;
+        int item = 0;
+        for (int p = 0; p < prm.P; ++p)
+            for (int u = ustart[p]; u < ustart[p + 1]; ++u) {
+                const int ne = std::min(och[p], ceil_div(prm.p[p].d_out, CH) - (u - ustart[p]) * och[p]);
+                const float cost = 0.65f * (float)ceil_div(prm.p[p].d_in, CH) + 1.0f * (float)ne + 0.4f;
+                for (int t = 0; t < tiles; ++t, ++item) {
+                    const int round = item / clusters, c = item - round * clusters;
+                    float& l = load[(round & 1) ? clusters - 1 - c : c];
+                    l += cost;
+                    longest = std::max(longest, l);
+                }
+            }
+        if (most == prm.P || longest < 0.97f * best) {
+            best = longest;
+            best_units = units;
+        }
+    }
+    return slice_outputs(prm, CH, best_units, och, ustart);
+}
+
 template <int R, bool GROUP, bool SHORT, int V>
-static cudaError_t stream_launch(StreamParams prm, [[maybe_unused]] const StreamMaps& maps, int64_t tiles_max, int S, cudaStream_t s)
+static cudaError_t stream_launch(StreamParams prm, [[maybe_unused]] const StreamMaps& maps, int64_t rows, int S, cudaStream_t s)
 {
     using Cfg = FsCfg<R, SHORT, V>;
     static int clusters_dev[kMaxDevices][4] = {};  // resident clusters of 1, 2, 4, 8 CTAs per device: the size of a wave
@@ -741,7 +789,11 @@ static cudaError_t stream_launch(StreamParams prm, [[maybe_unused]] const Stream
         if (e != cudaSuccess) return e;
         clusters = std::max(1, n);
     }
-    prm.ustart[prm.P] = slice_outputs(prm, Cfg::CH, S == 1 ? clusters / tiles_max : 0, prm.och, prm.ustart);
+    const int64_t tiles_max = tiles_bound(rows, prm.C, Cfg::ROWS);
+    const int tiles = S == 1 && prm.P > 2 && tiles_max * prm.P > clusters && tiles_max * prm.P <= 3 * clusters && clusters <= 256
+                          ? (int)std::lround(expected_tiles(prm, rows, Cfg::ROWS)) : 0;
+    if (tiles > 0) prm.ustart[prm.P] = balanced_units(prm, Cfg::CH, clusters, tiles, prm.och, prm.ustart);
+    else prm.ustart[prm.P] = slice_outputs(prm, Cfg::CH, S == 1 ? clusters / tiles_max : 0, prm.och, prm.ustart);
     const unsigned grid = (unsigned)(std::max<int64_t>(1, std::min<int64_t>(tiles_max * prm.ustart[prm.P], clusters)) * S);
     FsArgs<R, SHORT, V> args;
     static_cast<StreamParams&>(args) = prm;
@@ -762,14 +814,7 @@ static double stream_estimate(const StreamParams& prm, int64_t rows, int& split)
 {
     using Cfg = FsCfg<R, SHORT, (SHORT && R >= 32 ? kFsCluster : kFsOne)>;
     const double job_us = R == 16 ? (SHORT ? 1.30 : 1.19) : R == 32 ? (SHORT ? 1.17 : 1.72) : (SHORT ? 0.90 : 1.67);
-    // Tiles of segments of about equal size: one each while that is well below a tile's height, half a tile lost per segment from there
-    // on.  Of the segments as many are counted as three quarters of the rows, spread at random, meet: adapters are not equally popular
-    // (rank 64, 4096 wide, 20 tokens of 16 adapters by popularity: clusters of four 26 us, of two, as for all 16, 32).  Of the adapter
-    // sets of top-k routing only those of different adapters are met; the others are there for callers that repeat one.
-    const double met = (double)(prm.parts > 1 && prm.n_adapters >= prm.parts ? binom_small(prm.n_adapters, prm.parts) : prm.C);
-    const double segments = std::min((double)rows, std::max(1.0, met * (1.0 - std::pow(1.0 - 1.0 / met, 0.75 * (double)rows))));
-    const double fill = (double)rows / segments / Cfg::ROWS;
-    const double tiles = segments * (fill <= 0.75 ? 1.0 : fill <= 1.0 ? 1.0 + 2.0 * (fill - 0.75) : fill + 0.5);
+    const double tiles = expected_tiles(prm, rows, Cfg::ROWS);
     auto jobs = [](int width) {            // jobs that `width` columns cost
         const int full = width / Cfg::CH, rest = width % Cfg::CH;
         return full + (rest > 0 ? 0.35 + 0.65 * rest / Cfg::CH : 0.0);
@@ -842,13 +887,11 @@ static cudaError_t stream_rank(const molora_proj_desc_t* projs, int32_t P, int64
                                          (uint32_t)pr, (uint32_t)(ch / bc), bc == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
             return cudaErrorInvalidValue;
     }
-    const int rows = small ? 16 : 32;
-    const int64_t tiles_max = tiles_bound(cap_rows, prm.C, rows);
     const int S = small ? split16 : split32;
     auto launch = [&](auto tile, auto variant) {
         constexpr bool SHORT = decltype(tile)::value;
         constexpr int V = decltype(variant)::value;
-        return group ? stream_launch<R, true, SHORT, V>(prm, maps, tiles_max, S, s) : stream_launch<R, false, SHORT, V>(prm, maps, tiles_max, S, s);
+        return group ? stream_launch<R, true, SHORT, V>(prm, maps, cap_rows, S, s) : stream_launch<R, false, SHORT, V>(prm, maps, cap_rows, S, s);
     };
     using One = std::integral_constant<int, kFsOne>;
     if (!small) return launch(std::false_type{}, One{});

@@ -90,3 +90,12 @@ def test_topk_passes_and_kernels(N, C, rank, k, width):
         bound += 2.0 ** -8 * np.abs(oracle.apply_topk(w.inputs["x"][rows], p.y[rows], p.A, p.B, np.ascontiguousarray(idx[:j, rows]),
                                                       np.ascontiguousarray(weight[:j, rows])))
     assert np.all(np.abs(to_f64(y)[rows] - ref) <= bound)
+
+
+@pytest.mark.parametrize("N,C,hidden,rank", [
+    # a layer whose items pass one wave: widths cut in two and not, one chunk and ragged ones, few tiles and many
+    (256, 8, 2048, 16), (257, 7, 2080, 16), (400, 3, 1056, 16), (150, 12, 1024, 16), (600, 2, 2048, 16), (330, 5, 960, 32),
+])
+def test_layers_of_more_items_than_a_wave(N, C, hidden, rank):
+    check(N, C, [(hidden, hidden), (hidden, 512), (hidden, 512), (hidden, hidden), (hidden, 3 * hidden), (hidden, 3 * hidden), (3 * hidden, hidden)],
+          rank, rows=60)
