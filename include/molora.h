@@ -371,9 +371,11 @@ molora_status_t molora_selftest_bounded_wait(uint32_t *dev_status, int64_t limit
 
 /* ---------------------------------------------------------------------------------------------
  * The whole path on HOST activations (one layer: route -> group -> apply for P projections), for callers
- * whose activations live in host memory.  Everything is enqueued on `stream` in this order: host-to-device
- * copies of the routing source and of every distinct x and every y into `arena`, the router, the grouping,
- * one batched apply (Eq. 2), device-to-host copies of every y back into y_host.  The call returns without
+ * whose activations live in host memory.  Enqueued in the order of `stream`: host-to-device copies of the routing
+ * source and of every distinct x and every y into `arena`, the router, the grouping, the apply (Eq. 2), device-to-host
+ * copies of every y back into y_host.  Calls of 8 MB and more go projection by projection, applied and copied back on a
+ * second stream of the call's own while the next ones come in; what is enqueued on `stream` afterwards follows all of
+ * it.  (In one piece on `stream` alone: calls under capture, and host buffers that overlap.)  The call returns without
  * waiting; x_host / y_host must stay valid (and should be pinned for the copies to be asynchronous) until the
  * stream has finished.  Adapter stacks, gate weights and vocabulary breaks are DEVICE pointers: weights stay
  * resident at fixed addresses (the hot-set idea of Definition 5.1), only activations travel.

@@ -755,6 +755,147 @@ bool plan_host(const molora_host_proj_t* projs, int32_t P, molora_dtype_t dt, in
     return true;
 }
 
+// Enqueues the copies and the apply of rows [lo, lo + n) of a host call.
+struct HostCall {
+    const HostPlan* pl;
+    const molora_host_proj_t* projs;
+    const molora_proj_desc_t* dev;       // the staged copies of all N rows
+    char* base;
+    int32_t P, C;
+    molora_dtype_t dt;
+    size_t e;                            // bytes per element
+    uint32_t* dev_status;
+
+    bool upload_x(int i, int64_t lo, int64_t n, cudaStream_t s) const
+    {
+        const size_t row = e * (size_t)projs[i].d_in;
+        return cudaMemcpyAsync(base + pl->x[i] + lo * row, static_cast<const char*>(projs[i].x_host) + lo * row, n * row,
+                               cudaMemcpyHostToDevice, s) == cudaSuccess;
+    }
+    bool upload_y(int i, int64_t lo, int64_t n, cudaStream_t s) const
+    {
+        const size_t row = e * (size_t)projs[i].d_out;
+        return cudaMemcpyAsync(base + pl->y[i] + lo * row, static_cast<const char*>(projs[i].y_host) + lo * row, n * row,
+                               cudaMemcpyHostToDevice, s) == cudaSuccess;
+    }
+    // y of projection i and its x, unless that has gone before with the projection it is shared with or with projection `there`
+    bool upload(int i, int64_t lo, int64_t n, int there, cudaStream_t s) const
+    {
+        const bool own = pl->x_owner[i] == i && !(there >= 0 && pl->x_owner[there] == i);
+        return (!own || upload_x(i, lo, n, s)) && upload_y(i, lo, n, s);
+    }
+    bool download(int i, int64_t lo, int64_t n, cudaStream_t s) const
+    {
+        const size_t row = e * (size_t)projs[i].d_out;
+        return cudaMemcpyAsync(static_cast<char*>(projs[i].y_host) + lo * row, base + pl->y[i] + lo * row, n * row,
+                               cudaMemcpyDeviceToHost, s) == cudaSuccess;
+    }
+    void* ws() const { return pl->apply_ws_bytes > 0 ? base + pl->apply_ws : nullptr; }
+    int32_t* ints(size_t at) const { return reinterpret_cast<int32_t*>(base + at); }
+    // grouping and apply of rows [lo, lo + n) of projections [first, first + count)
+    molora_status_t group_apply(int first, int count, int64_t lo, int64_t n, cudaStream_t s) const
+    {
+        molora_proj_desc_t rows[MOLORA_MAX_PROJECTIONS];
+        for (int i = 0; i < count; ++i) {
+            rows[i] = dev[first + i];
+            rows[i].x = static_cast<const char*>(rows[i].x) + lo * rows[i].ldx * e;
+            rows[i].y = static_cast<char*>(rows[i].y) + lo * rows[i].ldy * e;
+        }
+        return molora_group_apply_batched(ints(pl->r) + lo, n, C, ints(pl->counts), ints(pl->offsets), ints(pl->perm), rows, count, dt, ws(),
+                                          pl->apply_ws_bytes, dev_status, s);
+    }
+};
+
+// A second stream for the length of one call.  It lives until what was enqueued on it has run (the runtime keeps a destroyed stream
+// that long); an event is read when it is waited for, so one serves all hand-overs of its direction.
+struct SideStream {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t arrived = nullptr, done = nullptr;
+    bool open()
+    {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;          // (another thread may be capturing)
+        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
+        const bool ok = cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) == cudaSuccess &&
+                        cudaEventCreateWithFlags(&arrived, cudaEventDisableTiming) == cudaSuccess &&
+                        cudaEventCreateWithFlags(&done, cudaEventDisableTiming) == cudaSuccess;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        return ok;
+    }
+    bool follow(cudaStream_t s) { return cudaEventRecord(arrived, s) == cudaSuccess && cudaStreamWaitEvent(stream, arrived, 0) == cudaSuccess; }
+    bool join(cudaStream_t s) { return cudaEventRecord(done, stream) == cudaSuccess && cudaStreamWaitEvent(s, done, 0) == cudaSuccess; }
+    ~SideStream()
+    {
+        if (done != nullptr) cudaEventDestroy(done);
+        if (arrived != nullptr) cudaEventDestroy(arrived);
+        if (stream != nullptr) cudaStreamDestroy(stream);
+    }
+};
+
+// scratch that molora_group_apply_batched needs for n tokens of these projections
+size_t group_apply_workspace(const molora_proj_desc_t* projs, int32_t P, molora_dtype_t dt, int64_t n, int32_t C)
+{
+    size_t need = 0;
+    switch (group_apply_mode(projs, P, dt, n, C)) {
+        case 0: {
+            ApplyPlan pl;
+            plan_apply(projs, P, dt, n, C, nullptr, nullptr, false, nullptr, 0, pl);
+            return pl.ws_need;
+        }
+        case 2:
+            for (int i = 0; i < P; ++i) need += decode_workspace_bytes(n, projs[i].d_in, projs[i].rank);
+            return need;
+        case 3:
+            for (int i = 0; i < P; ++i) need += jobs_partial_bytes(n, C, projs[i].d_in, projs[i].rank);
+            return need + jobs_control_bytes();
+        default: return 0;
+    }
+}
+
+// Rows of a piece of the last projection of a host call whose projections go through one after the other; 0: everything goes in, runs
+// and comes back on the caller's stream.  The link carries both directions at once (49 GB/s each way against 55 one way), so results
+// return while later projections are on their way in; what cannot overlap is the last one's, which is cut where its pieces keep
+// 8 MB (a copy costs ~10 us besides its bytes: eight pieces of all tokens, copies of 1 MB, were no faster than one stream).  Calls that
+// move less than 8 MB stay in one piece: what they could hide is not much above what the second stream costs.  So do calls
+// on a stream that is being captured (the graph keeps its shape), calls whose host buffers overlap (results could replace what a later
+// projection has yet to send) and those whose parts would need more scratch than the arena holds.
+constexpr double kHostPieceBytes = 8e6;
+int64_t host_last_rows(const HostCall& c, int64_t N, const void* route_src, int gate, cudaStream_t s)
+{
+    struct Range {
+        const char *lo, *hi;
+        bool written;
+    } ranges[2 * MOLORA_MAX_PROJECTIONS + 1];
+    int n_ranges = 0;
+    double bytes = 0.0;
+    auto add = [&](const void* p, size_t n, bool written) {
+        ranges[n_ranges++] = {static_cast<const char*>(p), static_cast<const char*>(p) + n, written};
+        bytes += (double)n;
+    };
+    if (gate < 0) add(route_src, sizeof(int32_t) * (size_t)N, false);
+    for (int i = 0; i < c.P; ++i) {
+        if (c.pl->x_owner[i] == i) add(c.projs[i].x_host, c.e * (size_t)N * c.projs[i].d_in, false);
+        add(c.projs[i].y_host, c.e * (size_t)N * c.projs[i].d_out, true);
+    }
+    const int last = c.P - 1;
+    const bool own_x = c.pl->x_owner[last] == last && !(gate >= 0 && c.pl->x_owner[gate] == last);
+    const double last_bytes = (double)c.e * (double)N * ((own_x ? c.projs[last].d_in : 0) + (double)c.projs[last].d_out);
+    const int64_t pieces = std::max<int64_t>(1, std::min<int64_t>(4, (int64_t)(last_bytes / kHostPieceBytes)));
+    const int64_t rows = std::min(N, ceil_div64(ceil_div64(N, pieces), 64) * 64);
+    if (bytes < kHostPieceBytes || (c.P == 1 && rows == N)) return 0;
+    for (int i = 0; i < n_ranges; ++i)
+        for (int j = 0; j < i; ++j)
+            if ((ranges[i].written || ranges[j].written) && ranges[i].lo < ranges[j].hi && ranges[j].lo < ranges[i].hi) return 0;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return 0;
+    size_t need = std::max(group_apply_workspace(c.dev + last, 1, c.dt, rows, c.C), group_apply_workspace(c.dev + last, 1, c.dt, N % rows, c.C));
+    for (int i = 0; i < last; ++i) {
+        ApplyPlan pl;
+        plan_apply(c.dev + i, 1, c.dt, N, c.C, nullptr, nullptr, false, nullptr, 0, pl);
+        need = std::max(need, pl.ws_need);
+    }
+    return need <= c.pl->apply_ws_bytes ? rows : 0;
+}
+
 }  // namespace
 
 size_t molora_forward_host_arena_bytes(const molora_host_proj_t* projs, int32_t P, molora_dtype_t dt, int64_t N,
@@ -796,44 +937,63 @@ molora_status_t molora_forward_host(molora_router_t router, const int32_t* route
         if (st != MOLORA_OK) return st;
     }
     if (N == 0) return MOLORA_OK;
+    if (router == MOLORA_ROUTE_GATE && (dev[gate_proj].d_in % 8) != 0) return MOLORA_ERR_UNSUPPORTED;
+    HostCall call;
+    call.pl = &pl;
+    call.projs = projs;
+    call.dev = dev;
+    call.base = base;
+    call.P = P;
+    call.dt = dt;
+    call.C = C;
+    call.e = dt == MOLORA_BF16 ? 2 : 4;
+    call.dev_status = dev_status;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const size_t e = dt == MOLORA_BF16 ? 2 : 4;
     int32_t* r = reinterpret_cast<int32_t*>(base + pl.r);
     int32_t* ids = reinterpret_cast<int32_t*>(base + pl.ids);
-    // 1. activations and routing source: host -> device
-    if (router != MOLORA_ROUTE_GATE &&
-        cudaMemcpyAsync(router == MOLORA_ROUTE_VOCAB ? ids : r, route_src_host, sizeof(int32_t) * (size_t)N,
-                        cudaMemcpyHostToDevice, s) != cudaSuccess)
+    const int gate = router == MOLORA_ROUTE_GATE ? gate_proj : -1;
+    auto route = [&](cudaStream_t on) {
+        if (router == MOLORA_ROUTE_VOCAB) return launch_route_vocab(ids, N, breaks_dev, M, nullptr, 0, r, dev_status, on);
+        if (router != MOLORA_ROUTE_GATE) return MOLORA_OK;
+        return launch_route_gate(dev[gate].x, dt, N, dev[gate].d_in, dev[gate].ldx, G_dev, bias_dev, C, r, nullptr, base + pl.gate_ws,
+                                 dev_status, on);
+    };
+    // 1. what the router reads, whole: host -> device
+    if (gate < 0 && cudaMemcpyAsync(router == MOLORA_ROUTE_VOCAB ? ids : r, route_src_host, sizeof(int32_t) * (size_t)N,
+                                    cudaMemcpyHostToDevice, s) != cudaSuccess)
         return MOLORA_ERR_CUDA;
-    for (int i = 0; i < P; ++i) {
-        if (pl.x_owner[i] == i &&
-            cudaMemcpyAsync(base + pl.x[i], projs[i].x_host, e * (size_t)N * projs[i].d_in, cudaMemcpyHostToDevice, s) != cudaSuccess)
-            return MOLORA_ERR_CUDA;
-        if (cudaMemcpyAsync(base + pl.y[i], projs[i].y_host, e * (size_t)N * projs[i].d_out, cudaMemcpyHostToDevice, s) != cudaSuccess)
-            return MOLORA_ERR_CUDA;
+    if (gate >= 0 && !call.upload_x(gate, 0, N, s)) return MOLORA_ERR_CUDA;
+    const int64_t last_rows = host_last_rows(call, N, route_src_host, gate, s);
+    SideStream side;
+    if (last_rows == 0 || !side.open()) {
+        // on the caller's stream: the other activations, route, group and apply, results back
+        for (int i = 0; i < P; ++i)
+            if (!call.upload(i, 0, N, gate, s)) return MOLORA_ERR_CUDA;
+        molora_status_t st = route(s);
+        if (st == MOLORA_OK) st = call.group_apply(0, P, 0, N, s);
+        if (st != MOLORA_OK) return st;
+        for (int i = 0; i < P; ++i)
+            if (!call.download(i, 0, N, s)) return MOLORA_ERR_CUDA;
+        return MOLORA_OK;
     }
-    // 2. route
-    molora_status_t st = MOLORA_OK;
-    if (router == MOLORA_ROUTE_VOCAB) {
-        st = launch_route_vocab(ids, N, breaks_dev, M, nullptr, 0, r, dev_status, s);
-    } else if (router == MOLORA_ROUTE_GATE) {
-        const molora_proj_desc_t& gp = dev[gate_proj];
-        if ((gp.d_in % 8) != 0) return MOLORA_ERR_UNSUPPORTED;
-        st = launch_route_gate(gp.x, dt, N, gp.d_in, gp.ldx, G_dev, bias_dev, C, r, nullptr, base + pl.gate_ws, dev_status, s);
+    // 2. one projection after the other: the caller's stream uploads, the side stream routes and groups once, applies what has arrived and
+    // sends its results back while the next ones come in; the last projection goes in pieces of last_rows
+    molora_status_t st = side.follow(s) ? route(side.stream) : MOLORA_ERR_CUDA;
+    if (st == MOLORA_OK && P > 1)
+        st = molora_group(r, N, C, call.ints(pl.counts), call.ints(pl.offsets), call.ints(pl.perm), nullptr, 0, dev_status, side.stream);
+    for (int i = 0; i < P && st == MOLORA_OK; ++i) {
+        const int64_t piece = i == P - 1 ? last_rows : N;
+        for (int64_t lo = 0; lo < N && st == MOLORA_OK; lo += piece) {
+            const int64_t n = std::min(piece, N - lo);
+            if (!call.upload(i, lo, n, gate, s) || !side.follow(s)) st = MOLORA_ERR_CUDA;
+            if (st == MOLORA_OK)
+                st = i == P - 1 ? call.group_apply(i, 1, lo, n, side.stream)
+                                : molora_apply_batched(dev + i, 1, dt, N, C, call.ints(pl.offsets), call.ints(pl.perm), call.ws(), pl.apply_ws_bytes,
+                                                       dev_status, side.stream);
+            if (st == MOLORA_OK && !call.download(i, lo, n, side.stream)) st = MOLORA_ERR_CUDA;
+        }
     }
-    if (st != MOLORA_OK) return st;
-    // 3. group, 4. apply
-    int32_t* offsets = reinterpret_cast<int32_t*>(base + pl.offsets);
-    int32_t* perm = reinterpret_cast<int32_t*>(base + pl.perm);
-    st = molora_group_apply_batched(r, N, C, reinterpret_cast<int32_t*>(base + pl.counts), offsets, perm, dev, P, dt,
-                                    pl.apply_ws_bytes > 0 ? base + pl.apply_ws : nullptr, pl.apply_ws_bytes, dev_status,
-                                    stream);
-    if (st != MOLORA_OK) return st;
-    // 5. results: device -> host
-    for (int i = 0; i < P; ++i)
-        if (cudaMemcpyAsync(projs[i].y_host, base + pl.y[i], e * (size_t)N * projs[i].d_out, cudaMemcpyDeviceToHost, s) != cudaSuccess)
-            return MOLORA_ERR_CUDA;
-    return MOLORA_OK;
+    return side.join(s) ? st : MOLORA_ERR_CUDA;        // (whatever was enqueued there belongs to the caller's stream again)
 }
 
 }  // extern "C"
