@@ -75,6 +75,7 @@ int64_t forced_umma_min_tokens() { return std::max<int64_t>(0, tune(kTuneUmmaMin
 constexpr double kUmmaMinBytesR16 = 150e6, kUmmaMinBytesR32 = 60e6, kUmmaMinBytesR32More = 170e6, kUmmaMinBytesR64More = 60e6;
 constexpr int64_t kUmmaMinTokensR64 = 1280, kUmmaMinTokensR64Wide = 256, kUmmaMinTokensR64Layer = 680;
 constexpr double kUmmaMinBytesR64 = 12e6;
+constexpr int64_t kPairMinTokens = 512;
 
 double proj_bytes(int64_t N, int32_t d_in, int32_t d_out) { return (double)N * ((double)d_in + 2.0 * d_out) * 2.0; }
 
@@ -106,12 +107,19 @@ bool small_path_is_stream(int32_t rank, int64_t N, int32_t C, int same_rank)
         if (forced == 1) return true;
         if (forced == 2) return false;
     }
-    // rank 64: the two-launch pair for one or two projections (chosen when only the pair split the reduction over CTAs; the streaming
-    // kernel does too now and measures a little ahead there as well: one 4096 wide, 8 adapters, 128 tokens 16.4 / 14.9, 400 18.0 / 14.9);
-    // with a layer's worth of them its items no longer fit a wave and the streaming kernel is faster, as it is for calls of more than
-    // 64 adapters with 24 to 64 tokens each, where the pair sends every row's partials through the workspace (us, pair / streaming:
-    // 256 adapters, 16000 tokens, 4096 wide, one projection 393 / 199, two 1143 / 570; 8000 tokens, 2048 wide 119 / 77)
-    return rank == 16 || rank == 32 || same_rank > 2 || (same_rank > 0 && C > kUmmaAllSegmentsMaxC && N >= (int64_t)C * 24);
+    // rank 64: with three projections and more the streaming kernel; one or two below 512 tokens of up to 64 adapters too (us, pair /
+    // streaming / tcgen05, 8 adapters: one 1024 wide, 200 tokens 16.0 / 9.2 / 12.9; 2048 wide, 64 13.6 / 11.2 / 14.0, 400 16.8 / 12.3 / 13.6;
+    // 4096 wide, 32 13.1 / 13.2 / 16.3, 200 17.1 / 13.9 / 16.6; two 2048 wide, 128 18.0 / 13.6 / 18.7).  From 512 tokens on the pair keeps what
+    // does not reach the tcgen05 kernel: callers rely on the launches of those calls.  More than 64 adapters with 24 tokens each
+    // stream: the pair sends every row's partials through the workspace (256 adapters, 16000 tokens, 4096 wide, one projection 393 / 199, two
+    // 1143 / 570; 8000 tokens, 2048 wide 119 / 77).
+    if (rank == 16 || rank == 32 || same_rank > 2) return true;
+    return same_rank > 0 && (C > kUmmaAllSegmentsMaxC ? N >= (int64_t)C * 24 : N < kPairMinTokens);
+}
+// Calls that ran on the two-launch pair before and are refused without its scratch still are, although the streaming kernel needs none.
+bool keeps_pair_scratch(int32_t rank, int64_t N, int32_t C, int same_rank)
+{
+    return rank == 64 && same_rank <= 2 && C <= kUmmaAllSegmentsMaxC && N < kPairMinTokens && tune(kTuneSmallPath) == 0;
 }
 
 // The job-list kernel shares chunk-sized jobs between all CTAs instead of giving every (tile, projection) pair to one cluster.
@@ -396,6 +404,8 @@ molora_status_t plan_apply(const molora_proj_desc_t* projs, int32_t P, molora_dt
         }
     size_t need_dc = 0, need_small = 0;
     for (int i = 0; i < pl.n_dc; ++i) need_dc += decode_workspace_bytes(N, pl.dc[i].d_in, pl.dc[i].rank);
+    for (int i = 0; i < pl.n_sc; ++i)
+        if (keeps_pair_scratch(pl.sc[i].rank, N, C, same_rank[group_of(pl.sc[i].rank)])) need_dc += decode_workspace_bytes(N, pl.sc[i].d_in, pl.sc[i].rank);
     for (int i = 0; i < pl.n_small_dc; ++i) need_small += decode_workspace_bytes(N, pl.small_dc[i].d_in, pl.small_dc[i].rank);
     size_t off = 0;
     if (N > 0 && pl.n_jc[0] + pl.n_jc[1] + pl.n_jc[2] > 0) {
@@ -509,8 +519,13 @@ molora_status_t molora_group_apply_batched(const int32_t* r, int64_t N, int32_t 
     // CTAs of those kernels do the grouping themselves.  Otherwise the two calls, in stream order.  Whatever could
     // refuse the call (the workspace of the two-launch kernels included) is checked before the first launch.
     const int mode = group_apply_mode(projs, P, dt, N, C);
-    if (mode == 1)
+    if (mode == 1) {
+        size_t need = 0;
+        if (keeps_pair_scratch(projs[0].rank, N, C, P))
+            for (int i = 0; i < P; ++i) need += decode_workspace_bytes(N, projs[i].d_in, projs[i].rank);
+        if (need > 0 && (ws == nullptr || ws_bytes < need || !aligned16(ws))) return MOLORA_ERR_WORKSPACE;
         return launch_group_apply_stream(r, projs, P, N, C, counts, offsets, perm, dev_status, static_cast<cudaStream_t>(stream));
+    }
     if (mode == 5)
         return launch_group_apply_rowtile(r, projs, P, dt, N, C, counts, offsets, perm, dev_status, static_cast<cudaStream_t>(stream));
     if (mode == 4)
@@ -841,6 +856,9 @@ size_t group_apply_workspace(const molora_proj_desc_t* projs, int32_t P, molora_
             plan_apply(projs, P, dt, n, C, nullptr, nullptr, false, nullptr, 0, pl);
             return pl.ws_need;
         }
+        case 1:
+            if (!keeps_pair_scratch(projs[0].rank, n, C, P)) return 0;
+            [[fallthrough]];
         case 2:
             for (int i = 0; i < P; ++i) need += decode_workspace_bytes(n, projs[i].d_in, projs[i].rank);
             return need;

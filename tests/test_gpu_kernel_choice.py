@@ -99,3 +99,14 @@ def test_topk_passes_and_kernels(N, C, rank, k, width):
 def test_layers_of_more_items_than_a_wave(N, C, hidden, rank):
     check(N, C, [(hidden, hidden), (hidden, 512), (hidden, 512), (hidden, hidden), (hidden, 3 * hidden), (hidden, 3 * hidden), (3 * hidden, hidden)],
           rank, rows=60)
+
+
+@pytest.mark.parametrize("N,C,shapes", [
+    # one and two projections of rank 64 on both sides of 512 tokens and of 64 adapters
+    (1, 1, [(512, 320)]), (90, 16, [(2080, 544)]), (511, 8, [(512, 320)]), (512, 8, [(512, 320)]), (511, 64, [(512, 320), (512, 96)]),
+    (511, 65, [(512, 320)]), (300, 3, [(1024, 1024), (1024, 2048)]),
+])
+def test_small_calls_of_rank_64(N, C, shapes):
+    check(N, C, shapes, 64)
+    # the scratch that these calls took before stays part of the call
+    assert all(M.molora_apply_workspace_bytes(N, C, a, b, 64) > 0 for a, b in shapes)
