@@ -337,13 +337,13 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
                 if (it < KX) {
 #pragma unroll
                     for (int i = 0; i < kRowsPerThread; ++i) {
-                        if (valid[i]) cp_async_16(dst + soff[i], xsrc[i]);
+                        if (valid[i]) cp_async_16_ahead(dst + soff[i], xsrc[i]);
                         xsrc[i] += kChunkCols;
                     }
                 } else {
 #pragma unroll
                     for (int i = 0; i < kRowsPerThread; ++i) {
-                        if (valid[i]) cp_async_16(dst + soff[i], ysrc[i]);
+                        if (valid[i]) cp_async_16_ahead(dst + soff[i], ysrc[i]);
                         ysrc[i] += kChunkCols;
                     }
                 }

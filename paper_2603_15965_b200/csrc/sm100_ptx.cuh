@@ -184,6 +184,11 @@ __device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
+// ... that also asks for the rest of the 256 bytes around them to be brought into L2: for rows walked 128 bytes at a time
+__device__ __forceinline__ void cp_async_16_ahead(uint32_t dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
 // Arrive on an mbarrier once every cp.async this thread has issued so far has landed (the arrival is counted
 // in the barrier's initial count, hence "noinc").
 __device__ __forceinline__ void cp_async_arrive_noinc(uint32_t bar)
