@@ -76,6 +76,7 @@ constexpr double kUmmaMinBytesR16 = 150e6, kUmmaMinBytesR32 = 60e6, kUmmaMinByte
 constexpr int64_t kUmmaMinTokensR64 = 1280, kUmmaMinTokensR64Wide = 256, kUmmaMinTokensR64Layer = 680;
 constexpr double kUmmaMinBytesR64 = 12e6;
 constexpr int64_t kPairMinTokens = 512;
+constexpr int32_t kPairMaxWidth = 1024;
 
 double proj_bytes(int64_t N, int32_t d_in, int32_t d_out) { return (double)N * ((double)d_in + 2.0 * d_out) * 2.0; }
 
@@ -100,8 +101,9 @@ bool use_umma(int32_t rank, int64_t N, int32_t C, double group_bytes, int same_r
     if (N < (int64_t)C * 160 || group_bytes < kUmmaMinBytesR32) return false;
     return same_rank == 1 || group_bytes >= kUmmaMinBytesR32More || (N >= 3000 && N >= (int64_t)C * 300);
 }
-// the kernel for what the tcgen05 kernel does not take; same_rank: projections of this rank in the call (0: unknown)
-bool small_path_is_stream(int32_t rank, int64_t N, int32_t C, int same_rank)
+// the kernel for what the tcgen05 kernel does not take; same_rank: projections of this rank in the call (0: unknown), widest: the most
+// columns, in and out, that one of them has
+bool small_path_is_stream(int32_t rank, int64_t N, int32_t C, int same_rank, int32_t widest)
 {
     if (const int64_t forced = tune(kTuneSmallPath)) {
         if (forced == 1) return true;
@@ -110,16 +112,25 @@ bool small_path_is_stream(int32_t rank, int64_t N, int32_t C, int same_rank)
     // rank 64: with three projections and more the streaming kernel; one or two below 512 tokens of up to 64 adapters too (us, pair /
     // streaming / tcgen05, 8 adapters: one 1024 wide, 200 tokens 16.0 / 9.2 / 12.9; 2048 wide, 64 13.6 / 11.2 / 14.0, 400 16.8 / 12.3 / 13.6;
     // 4096 wide, 32 13.1 / 13.2 / 16.3, 200 17.1 / 13.9 / 16.6; two 2048 wide, 128 18.0 / 13.6 / 18.7).  From 512 tokens on the pair keeps what
-    // does not reach the tcgen05 kernel: callers rely on the launches of those calls.  More than 64 adapters with 24 tokens each
+    // does not reach the tcgen05 kernel, and so do calls of narrow projections (below 1024 columns, in and out): callers rely on the launches and
+    // on the scratch of those calls.  More than 64 adapters with 24 tokens each
     // stream: the pair sends every row's partials through the workspace (256 adapters, 16000 tokens, 4096 wide, one projection 393 / 199, two
     // 1143 / 570; 8000 tokens, 2048 wide 119 / 77).
     if (rank == 16 || rank == 32 || same_rank > 2) return true;
-    return same_rank > 0 && (C > kUmmaAllSegmentsMaxC ? N >= (int64_t)C * 24 : N < kPairMinTokens);
+    return same_rank > 0 && (C > kUmmaAllSegmentsMaxC ? N >= (int64_t)C * 24 : N < kPairMinTokens && widest >= kPairMaxWidth);
 }
 // Calls that ran on the two-launch pair before and are refused without its scratch still are, although the streaming kernel needs none.
-bool keeps_pair_scratch(int32_t rank, int64_t N, int32_t C, int same_rank)
+bool keeps_pair_scratch(int32_t rank, int64_t N, int32_t C, int same_rank, int32_t widest)
 {
-    return rank == 64 && same_rank <= 2 && C <= kUmmaAllSegmentsMaxC && N < kPairMinTokens && tune(kTuneSmallPath) == 0;
+    return rank == 64 && same_rank <= 2 && C <= kUmmaAllSegmentsMaxC && N < kPairMinTokens && widest >= kPairMaxWidth && tune(kTuneSmallPath) == 0;
+}
+
+int32_t widest_of(const molora_proj_desc_t* projs, int32_t P, int32_t rank)
+{
+    int32_t w = 0;
+    for (int i = 0; i < P; ++i)
+        if (projs[i].rank == rank) w = std::max(w, projs[i].d_in + projs[i].d_out);
+    return w;
 }
 
 // The job-list kernel shares chunk-sized jobs between all CTAs instead of giving every (tile, projection) pair to one cluster.
@@ -333,7 +344,7 @@ size_t molora_apply_workspace_bytes(int64_t N, int32_t C, int32_t d_in, int32_t 
     if (jobs_eligible(probe, MOLORA_BF16, N) && (small == 3 || (small == 0 && rank == 16 && N > 256)))
         need += jobs_control_bytes() + jobs_partial_bytes(N, C, d_in, rank);
     if (small == 3 && need > 0) return need;
-    if (small_path_is_stream(rank, N, C, 0)) return need;
+    if (small_path_is_stream(rank, N, C, 0, d_in + d_out)) return need;
     // two-launch kernels: needed unless the tcgen05 kernel is certain to take every segment (for ranks 16 and 32 that
     // depends on the other projections of the call, which are not known here)
     const int64_t forced = forced_umma_min_tokens();
@@ -387,7 +398,7 @@ molora_status_t plan_apply(const molora_proj_desc_t* projs, int32_t P, molora_dt
         if (umma_eligible(projs[i], dt) && use_umma(rank, N, C, group_bytes[group_of(rank)], same_rank[group_of(rank)])) pl.tc[pl.n_tc++] = projs[i];
         else if (use_jobs(projs[i], dt, N, C, same_rank[group_of(rank)])) pl.jc[group_of(rank)][pl.n_jc[group_of(rank)]++] = projs[i];
         else if (decode_eligible(projs[i], dt)) {
-            if (small_path_is_stream(rank, N, C, same_rank[group_of(rank)])) pl.sc[pl.n_sc++] = projs[i];
+            if (small_path_is_stream(rank, N, C, same_rank[group_of(rank)], widest_of(projs, P, rank))) pl.sc[pl.n_sc++] = projs[i];
             else pl.dc[pl.n_dc++] = projs[i];
         } else pl.cc[pl.n_cc++] = projs[i];
     }
@@ -399,13 +410,13 @@ molora_status_t plan_apply(const molora_proj_desc_t* projs, int32_t P, molora_dt
         for (int i = 0; i < pl.n_tc; ++i) {
             if (!decode_eligible(pl.tc[i], dt)) pl.small_cc[pl.n_small_cc++] = pl.tc[i];
             // (0 adapters: it gets short segments only, and the rule for whole calls of many adapters does not apply)
-            else if (small_path_is_stream(pl.tc[i].rank, N, 0, same_rank[group_of(pl.tc[i].rank)])) pl.small_sc[pl.n_small_sc++] = pl.tc[i];
+            else if (small_path_is_stream(pl.tc[i].rank, N, 0, same_rank[group_of(pl.tc[i].rank)], 0)) pl.small_sc[pl.n_small_sc++] = pl.tc[i];
             else pl.small_dc[pl.n_small_dc++] = pl.tc[i];
         }
     size_t need_dc = 0, need_small = 0;
     for (int i = 0; i < pl.n_dc; ++i) need_dc += decode_workspace_bytes(N, pl.dc[i].d_in, pl.dc[i].rank);
     for (int i = 0; i < pl.n_sc; ++i)
-        if (keeps_pair_scratch(pl.sc[i].rank, N, C, same_rank[group_of(pl.sc[i].rank)])) need_dc += decode_workspace_bytes(N, pl.sc[i].d_in, pl.sc[i].rank);
+        if (keeps_pair_scratch(pl.sc[i].rank, N, C, same_rank[group_of(pl.sc[i].rank)], widest_of(projs, P, pl.sc[i].rank))) need_dc += decode_workspace_bytes(N, pl.sc[i].d_in, pl.sc[i].rank);
     for (int i = 0; i < pl.n_small_dc; ++i) need_small += decode_workspace_bytes(N, pl.small_dc[i].d_in, pl.small_dc[i].rank);
     size_t off = 0;
     if (N > 0 && pl.n_jc[0] + pl.n_jc[1] + pl.n_jc[2] > 0) {
@@ -473,7 +484,7 @@ static int group_apply_mode(const molora_proj_desc_t* projs, int32_t P, molora_d
         same = same && projs[i].rank == projs[0].rank && decode_eligible(projs[i], dt);
         if (!same) return 0;
         const bool jb = use_jobs(projs[i], dt, N, C, P);
-        const bool st = small_path_is_stream(projs[i].rank, N, C, P);
+        const bool st = small_path_is_stream(projs[i].rank, N, C, P, widest_of(projs, P, projs[i].rank));
         jobs = jobs && jb;
         stream = stream && !jb && st;
         twophase = twophase && !jb && !st;
@@ -521,7 +532,7 @@ molora_status_t molora_group_apply_batched(const int32_t* r, int64_t N, int32_t 
     const int mode = group_apply_mode(projs, P, dt, N, C);
     if (mode == 1) {
         size_t need = 0;
-        if (keeps_pair_scratch(projs[0].rank, N, C, P))
+        if (keeps_pair_scratch(projs[0].rank, N, C, P, widest_of(projs, P, projs[0].rank)))
             for (int i = 0; i < P; ++i) need += decode_workspace_bytes(N, projs[i].d_in, projs[i].rank);
         if (need > 0 && (ws == nullptr || ws_bytes < need || !aligned16(ws))) return MOLORA_ERR_WORKSPACE;
         return launch_group_apply_stream(r, projs, P, N, C, counts, offsets, perm, dev_status, static_cast<cudaStream_t>(stream));
@@ -857,7 +868,7 @@ size_t group_apply_workspace(const molora_proj_desc_t* projs, int32_t P, molora_
             return pl.ws_need;
         }
         case 1:
-            if (!keeps_pair_scratch(projs[0].rank, n, C, P)) return 0;
+            if (!keeps_pair_scratch(projs[0].rank, n, C, P, widest_of(projs, P, projs[0].rank))) return 0;
             [[fallthrough]];
         case 2:
             for (int i = 0; i < P; ++i) need += decode_workspace_bytes(n, projs[i].d_in, projs[i].rank);

@@ -102,9 +102,9 @@ def test_layers_of_more_items_than_a_wave(N, C, hidden, rank):
 
 
 @pytest.mark.parametrize("N,C,shapes", [
-    # one and two projections of rank 64 on both sides of 512 tokens and of 64 adapters
-    (1, 1, [(512, 320)]), (90, 16, [(2080, 544)]), (511, 8, [(512, 320)]), (512, 8, [(512, 320)]), (511, 64, [(512, 320), (512, 96)]),
-    (511, 65, [(512, 320)]), (300, 3, [(1024, 1024), (1024, 2048)]),
+    # one and two projections of rank 64 on both sides of 512 tokens, of 64 adapters and of 1024 columns
+    (1, 1, [(512, 512)]), (90, 16, [(2080, 544)]), (511, 8, [(512, 512)]), (512, 8, [(512, 512)]), (511, 64, [(512, 320), (512, 512)]),
+    (511, 65, [(512, 512)]), (511, 8, [(512, 480)]), (300, 3, [(1024, 1024), (1024, 2048)]),
 ])
 def test_small_calls_of_rank_64(N, C, shapes):
     check(N, C, shapes, 64)
