@@ -519,8 +519,8 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
                 const int own_lo = owner * kTileM / (int)S;
                 cluster_wait();                                 // every peer is running, its barriers initialised
                 if (group == 0 && et == 0) {                    // what the peers will send me: their partials of my rows
-                    const int mine = (int)(crank + 1) * kTileM / (int)S - (int)crank * kTileM / (int)S;
-                    mbar_arrive_expect_tx(bar(&ctrl->part_full), (S - 1) * (uint32_t)(mine * R * 4));
+                    const int own = (int)(crank + 1) * kTileM / (int)S - (int)crank * kTileM / (int)S;
+                    mbar_arrive_expect_tx(bar(&ctrl->part_full), (S - 1) * (uint32_t)(own * R * 4));
                 }
                 if ((uint32_t)owner != crank) {
                     const uint32_t slot = crank < (uint32_t)owner ? crank : crank - 1;      // my slot at the owner
@@ -531,17 +531,72 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
                         st_async_cluster_u32x4(dst + (uint32_t)((col0 / 4 + c4) * rows_max + (row - own_lo)) * 16u, tv[4 * c4],
                                                tv[4 * c4 + 1], tv[4 * c4 + 2], tv[4 * c4 + 3], pb);
                 }
-                wait_bar_cluster(bar(&ctrl->part_full), 0, abort_flag, prm.dev_status);
-                if ((uint32_t)owner == crank) {
-                    sum_partials<RH>(tv, recv_p + (col0 / 4) * rows_max + (row - own_lo), rows_max, rows_max * R / 4, S, crank);
-                    split_row();
+                const int mine_lo = (int)crank * kTileM / (int)S, mine = (int)(crank + 1) * kTileM / (int)S - mine_lo;
+                if constexpr (WIDE) {
+                    // My rows' partial of my own waits in their place in the tiles (a row's 64 sums are 256 bytes, its two bf16 halves 128 each).
+                    auto own_piece = [&](int r, int c4) {
+                        return (c4 < 8 ? thi : tlo) + (uint32_t)r * 128u + (uint32_t)(((c4 & 7) ^ (r & 7)) * 16);
+                    };
+                    if ((uint32_t)owner == crank)
 #pragma unroll
-                    for (int c8 = 0; c8 < RH / 8; ++c8) {
-                        const uint32_t off = trow_offset(c8);
-                        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(thi + off), "r"(hw[4 * c8]), "r"(hw[4 * c8 + 1]),
-                                     "r"(hw[4 * c8 + 2]), "r"(hw[4 * c8 + 3]) : "memory");
-                        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(tlo + off), "r"(lw[4 * c8]), "r"(lw[4 * c8 + 1]),
-                                     "r"(lw[4 * c8 + 2]), "r"(lw[4 * c8 + 3]) : "memory");
+                        for (int c4 = 0; c4 < RH / 4; ++c4)
+                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(own_piece(row, col0 / 4 + c4)), "r"(tv[4 * c4]), "r"(tv[4 * c4 + 1]),
+                                         "r"(tv[4 * c4 + 2]), "r"(tv[4 * c4 + 3]) : "memory");
+                    wait_bar_cluster(bar(&ctrl->part_full), 0, abort_flag, prm.dev_status);
+                    asm volatile("bar.sync 3, 256;" ::: "memory");  // the eight epilogue warps
+                    // All of them sum: four columns of a row each, a few pieces a thread.  By the rows' own threads, sixteen in a cluster of
+                    // eight, this took most of the 9000 cycles from the last shrink MMA to the first expand MMA (one 4096-wide projection of 8
+                    // adapters, 600 / 1000 tokens 17.4 / 18.4 us, so 16.9 / 17.7); in clusters of two and three, where 64 and 43 rows have
+                    // threads of their own, they are the faster ones (4000 tokens 31.0 against 31.7).
+                    constexpr int kPieces = (kTileM / 4 * (R / 4) + 255) / 256;            // (of 32 rows: clusters of four and more)
+                    uint2 fh[kPieces], fl[kPieces];
+#pragma unroll
+                    for (int i = 0; i < kPieces; ++i) {
+                        const int at = group * 128 + et + i * 256, c4 = at / mine, r = mine_lo + at - c4 * mine;
+                        if (c4 < R / 4) {
+                            float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+                            for (uint32_t q2 = 0; q2 < S; ++q2) {   // rank order
+                                const float4 v = q2 == crank ? *reinterpret_cast<const float4*>(smem_raw + (own_piece(r, c4) - raw))
+                                                             : recv_p[((q2 < crank ? q2 : q2 - 1) * (R / 4) + c4) * rows_max + (r - mine_lo)];
+                                t.x += v.x;
+                                t.y += v.y;
+                                t.z += v.z;
+                                t.w += v.w;
+                            }
+                            const int tok = ctrl->rows[r], part = c4 * 4 / rp;
+                            const float ts = pj.scale * (pj.row_scale != nullptr && tok >= 0 ? __ldg(pj.row_scale + (int64_t)part * prm.N + tok) : 1.f);
+                            const float tt[4] = {t.x * ts, t.y * ts, t.z * ts, t.w * ts};
+                            float th[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) th[e] = __bfloat162float(__float2bfloat16_rn(tt[e]));
+                            fh[i] = make_uint2(f32x2_to_bf16x2(th[0], th[1]), f32x2_to_bf16x2(th[2], th[3]));
+                            fl[i] = make_uint2(f32x2_to_bf16x2(tt[0] - th[0], tt[1] - th[1]), f32x2_to_bf16x2(tt[2] - th[2], tt[3] - th[3]));
+                        }
+                    }
+                    asm volatile("bar.sync 3, 256;" ::: "memory");  // my own partials have been read
+#pragma unroll
+                    for (int i = 0; i < kPieces; ++i) {
+                        const int at = group * 128 + et + i * 256, c4 = at / mine, r = mine_lo + at - c4 * mine;
+                        if (c4 < R / 4) {
+                            const uint32_t off = swizzle_offset((uint32_t)r * Cfg::kTRowBytes + (uint32_t)(c4 >> 1) * 16, Cfg::kSwzBits) + (uint32_t)(c4 & 1) * 8;
+                            *reinterpret_cast<uint2*>(smem_raw + (thi + off - raw)) = fh[i];
+                            *reinterpret_cast<uint2*>(smem_raw + (tlo + off - raw)) = fl[i];
+                        }
+                    }
+                } else {
+                    wait_bar_cluster(bar(&ctrl->part_full), 0, abort_flag, prm.dev_status);
+                    if ((uint32_t)owner == crank) {
+                        sum_partials<RH>(tv, recv_p + (col0 / 4) * rows_max + (row - own_lo), rows_max, rows_max * R / 4, S, crank);
+                        split_row();
+#pragma unroll
+                        for (int c8 = 0; c8 < RH / 8; ++c8) {
+                            const uint32_t off = trow_offset(c8);
+                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(thi + off), "r"(hw[4 * c8]), "r"(hw[4 * c8 + 1]),
+                                         "r"(hw[4 * c8 + 2]), "r"(hw[4 * c8 + 3]) : "memory");
+                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(tlo + off), "r"(lw[4 * c8]), "r"(lw[4 * c8 + 1]),
+                                         "r"(lw[4 * c8 + 2]), "r"(lw[4 * c8 + 3]) : "memory");
+                        }
                     }
                 }
                 // (3) my rows are a contiguous piece of each T tile (the swizzle permutes inside a row): two bulk copies
@@ -549,9 +604,8 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
                 fence_proxy_async_smem();                       // my rows, written above, are read by the copy engine
                 asm volatile("bar.sync 3, 256;" ::: "memory");  // the eight epilogue warps
                 if (group == 0) {
-                    const int mine_lo = (int)crank * kTileM / (int)S, mine_hi = (int)(crank + 1) * kTileM / (int)S;
                     const uint32_t out_off = (uint32_t)mine_lo * Cfg::kTRowBytes;
-                    const uint32_t out_bytes = (uint32_t)(mine_hi - mine_lo) * Cfg::kTRowBytes;
+                    const uint32_t out_bytes = (uint32_t)mine * Cfg::kTRowBytes;
                     if (et == 0) mbar_arrive_expect_tx(bar(&ctrl->part_free), 2u * ((uint32_t)kTileM * Cfg::kTRowBytes - out_bytes));
                     if (warp == kEpiWarp0 && (uint32_t)lane < S && (uint32_t)lane != crank && !*abort_flag) {   // lane q2 serves CTA q2
                         const uint32_t pb = map_to_cta(bar(&ctrl->part_free), (uint32_t)lane);
