@@ -96,6 +96,7 @@ struct StreamParams {
     int32_t* counts_out;
     int32_t* offsets_out;
     int32_t* perm_out;
+    bool chained;                             // (host) launched under the kernel of the same call that made the tables or the sets
 };
 // adapter of part j of segment `seg`
 // (set_tab: the kernel's shared-memory copy of prm.set_table)
@@ -193,7 +194,7 @@ __device__ __forceinline__ FsItem fs_item(const StreamParams& prm, const int32_t
 }
 __device__ __forceinline__ int fs_token(const StreamParams& prm, const int32_t* perm_s, int pos)
 {
-    return prm.N <= kFsPermCache ? perm_s[pos] : __ldg(prm.perm + pos);
+    return prm.N <= kFsPermCache ? perm_s[pos] : ptx::ld_dependent(prm.perm + pos);
 }
 
 }  // namespace
@@ -244,18 +245,19 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
                 prefetch_tensormap(&args.tm_b[p]);
             }
     }
+    grid_dependency_sync();                    // tables, sets and weights may come from the kernel this one was launched under
     if (prm.parts > 1)                         // (visible after the block-wide barriers of the prologue below)
         for (int i = tid; i < prm.C; i += kFsThreads)
-            reinterpret_cast<uint32_t*>(set_tab_s)[i] = __ldg(reinterpret_cast<const uint32_t*>(prm.set_table) + i);
+            reinterpret_cast<uint32_t*>(set_tab_s)[i] = (uint32_t)ld_dependent(reinterpret_cast<const int32_t*>(prm.set_table) + i);
     if constexpr (GROUP) {
         // the grouping itself, on this CTA, while the ring is idle (its memory is the scratch)
         group_in_cta<kFsThreads, kFsPermCache>(prm.r, prm.N, prm.C, offs_s, tstart_s, perm_s, dsm, Cfg::ROWS, true, prm.counts_out,
                                                prm.offsets_out, prm.dev_status);
     } else {
         // segment table and (small calls) the permutation on chip in one memory round trip
-        for (int i = tid; i <= prm.C; i += kFsThreads) offs_s[i] = __ldg(prm.offsets + i);
+        for (int i = tid; i <= prm.C; i += kFsThreads) offs_s[i] = ld_dependent(prm.offsets + i);
         if (prm.N <= kFsPermCache)
-            for (int i = tid; i < prm.N; i += kFsThreads) perm_s[i] = __ldg(prm.perm + i);
+            for (int i = tid; i < prm.N; i += kFsThreads) perm_s[i] = ld_dependent(prm.perm + i);
         __syncthreads();
     }
     // tiles of the segments before each segment (those with 1 <= rows < max_rows own tiles here), so that an item finds
@@ -418,7 +420,7 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
             if (row >= it.rows) return make_float4(0.f, 0.f, 0.f, 0.f);       // rows past the tile hold stale shared memory
             float sc = pd.scale;
             if (pd.row_scale != nullptr)
-                sc *= __ldg(pd.row_scale + (int64_t)((e4 * 4 % R) / (R / prm.parts)) * prm.N + fs_token(prm, perm_s, it.row0 + row));
+                sc *= ld_dependent(pd.row_scale + (int64_t)((e4 * 4 % R) / (R / prm.parts)) * prm.N + fs_token(prm, perm_s, it.row0 + row));
             return make_float4(v.x * sc, v.y * sc, v.z * sc, v.w * sc);
         };
 
@@ -798,7 +800,7 @@ static cudaError_t stream_launch(StreamParams prm, [[maybe_unused]] const Stream
     FsArgs<R, SHORT, V> args;
     static_cast<StreamParams&>(args) = prm;
     if constexpr (Cfg::BOX) static_cast<StreamMaps&>(args) = maps;
-    return launch_kernel(apply_stream_kernel<R, GROUP, SHORT, V>, dim3(grid), dim3(kFsThreads), Cfg::SMEM, s, (unsigned)S, false, args);
+    return launch_kernel(apply_stream_kernel<R, GROUP, SHORT, V>, dim3(grid), dim3(kFsThreads), Cfg::SMEM, s, (unsigned)S, prm.chained, args);
 }
 
 // Estimated time of a launch (us, without its fixed part) and the CTAs per item that give it.  A launch lasts as long as its
@@ -891,7 +893,9 @@ static cudaError_t stream_rank(const molora_proj_desc_t* projs, int32_t P, int64
     auto launch = [&](auto tile, auto variant) {
         constexpr bool SHORT = decltype(tile)::value;
         constexpr int V = decltype(variant)::value;
-        return group ? stream_launch<R, true, SHORT, V>(prm, maps, cap_rows, S, s) : stream_launch<R, false, SHORT, V>(prm, maps, cap_rows, S, s);
+        const StreamParams now = prm;
+        prm.chained = false;                   // (what follows has another predecessor)
+        return group ? stream_launch<R, true, SHORT, V>(now, maps, cap_rows, S, s) : stream_launch<R, false, SHORT, V>(now, maps, cap_rows, S, s);
     };
     using One = std::integral_constant<int, kFsOne>;
     if (!small) return launch(std::false_type{}, One{});
@@ -917,7 +921,7 @@ static molora_status_t stream_enqueue(const molora_proj_desc_t* projs, int32_t P
 
 molora_status_t launch_apply_stream(const molora_proj_desc_t* projs, int32_t P, int64_t N, int32_t C,
                                     const int32_t* offsets, const int32_t* perm, int32_t max_rows, uint32_t* dev_status,
-                                    cudaStream_t s)
+                                    cudaStream_t s, bool after_group)
 {
     if (N == 0 || P == 0) return MOLORA_OK;
     StreamParams prm;
@@ -930,6 +934,7 @@ molora_status_t launch_apply_stream(const molora_proj_desc_t* projs, int32_t P, 
     prm.parts = 1;
     prm.n_adapters = C;
     prm.set_table = nullptr;
+    prm.chained = after_group;
     return stream_enqueue(projs, P, N, C, prm, false, s);
 }
 
@@ -950,6 +955,7 @@ molora_status_t launch_apply_stream_sets(const molora_proj_desc_t* projs, int32_
     prm.parts = parts;
     prm.n_adapters = n_adapters;
     prm.set_table = set_table;
+    prm.chained = true;
     return stream_enqueue(projs, P, N, n_sets, prm, false, s);
 }
 
@@ -972,6 +978,7 @@ molora_status_t launch_group_apply_stream_sets(const int32_t* sets, const molora
     prm.parts = parts;
     prm.n_adapters = n_adapters;
     prm.set_table = set_table;
+    prm.chained = true;
     return stream_enqueue(projs, P, N, n_sets, prm, true, s);
 }
 
@@ -993,6 +1000,7 @@ molora_status_t launch_group_apply_stream(const int32_t* r, const molora_proj_de
     prm.parts = 1;
     prm.n_adapters = C;
     prm.set_table = nullptr;
+    prm.chained = false;
     return stream_enqueue(projs, P, N, C, prm, true, s);
 }
 

@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
 #pragma unroll
     for (int j = 0; j < (MOLORA_MAX_ADAPTERS + kUmmaThreads) / kUmmaThreads; ++j) {
         const int i = tid + j * kUmmaThreads;
-        offs_v[j] = (!grouping && i <= prm.C) ? __ldg(prm.offsets + i) : 0;
+        offs_v[j] = (!grouping && i <= prm.C) ? ld_dependent(prm.offsets + i) : 0;
     }
     if (tid == 0) {
         prefetch_tensormap(&pj.tm_a);
@@ -289,14 +289,15 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
     constexpr int parts = PARTS, rp = R / PARTS;
     static_assert(rp >= 16 && rp * PARTS == R, "adapters of rank 16, 32 or 64");
     int adapter[kUmmaMaxParts];
+    uint32_t set_word = 0;
+    if constexpr (PARTS > 1) set_word = (uint32_t)ld_dependent(reinterpret_cast<const int32_t*>(prm.set_table) + seg);
 #pragma unroll
-    for (int j = 0; j < kUmmaMaxParts; ++j)
-        adapter[j] = PARTS == 1 ? seg : (j < PARTS ? (int)__ldg(prm.set_table + seg * 4 + j) : 0);
+    for (int j = 0; j < kUmmaMaxParts; ++j) adapter[j] = PARTS == 1 ? seg : (j < PARTS ? (int)(set_word >> (8 * j) & 255u) : 0);
     const int KXall = pj.d_in / kChunkCols, NYall = pj.d_out / kChunkCols;
     const int kx0 = (int)(crank * KXall / S), KX = (int)((crank + 1) * KXall / S) - kx0;   // my slice of d_in
     const int ny0 = (int)(crank * NYall / S), NY = (int)((crank + 1) * NYall / S) - ny0;   // my slice of d_out
     const int total = KX + NY;
-    if (tid < kTileM) ctrl->rows[tid] = tid < rows ? (grouping ? perm_s[row0 + tid] : __ldg(prm.perm + row0 + tid)) : -1;
+    if (tid < kTileM) ctrl->rows[tid] = tid < rows ? (grouping ? perm_s[row0 + tid] : ld_dependent(prm.perm + row0 + tid)) : -1;
     __syncthreads();                    // (the ring may be filled from here on: nobody reads perm_s any more)
     // "I am running and my barriers are initialised": the matching wait comes right before the first access to
     // a peer's shared memory (the T exchange), so the cluster barrier costs nothing here
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
 #pragma unroll
             for (int j = 0; j < kUmmaMaxParts; ++j)
                 tscale[j] = pj.scale * ((pj.row_scale != nullptr && my_tok >= 0 && j < parts)
-                                            ? __ldg(pj.row_scale + (int64_t)j * prm.N + my_tok) : 1.f);
+                                            ? ld_dependent(pj.row_scale + (int64_t)j * prm.N + my_tok) : 1.f);
             // my half row of T, scaled, as bf16 hi and lo words
             uint32_t hw[RH / 2], lw[RH / 2];
             auto split_row = [&]() {
@@ -565,7 +566,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
                                 t.w += v.w;
                             }
                             const int tok = ctrl->rows[r], part = c4 * 4 / rp;
-                            const float ts = pj.scale * (pj.row_scale != nullptr && tok >= 0 ? __ldg(pj.row_scale + (int64_t)part * prm.N + tok) : 1.f);
+                            const float ts = pj.scale * (pj.row_scale != nullptr && tok >= 0 ? ld_dependent(pj.row_scale + (int64_t)part * prm.N + tok) : 1.f);
                             const float tt[4] = {t.x * ts, t.y * ts, t.z * ts, t.w * ts};
                             float th[4];
 #pragma unroll
@@ -766,6 +767,7 @@ bool umma_eligible(const molora_proj_desc_t& p, molora_dtype_t dt)
 struct UmmaPlan {
     int split;       // CTAs per tile (cluster size)
     int tile_rows;   // positions per tile
+    bool chained = false;      // launched under the grouping kernel of the same call
 };
 
 template <int R, bool WIDE, int PARTS = 1>
@@ -800,8 +802,13 @@ static cudaError_t umma_launch_variant(UmmaParams prm, int64_t N, UmmaPlan plan,
     }
     const int64_t tiles = ceil_div64(N, prm.tile_rows) + prm.C;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     fill_launch_config<R, WIDE>(cfg, attr, tiles, prm.P, split, s);
+    if (plan.chained && chained_launch_enabled()) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+        ++cfg.numAttrs;
+    }
     note_launch();
     return cudaLaunchKernelEx(&cfg, apply_umma_kernel<R, WIDE, PARTS>, prm);
 }
@@ -934,7 +941,7 @@ bool group_apply_umma_eligible(int64_t N, int32_t C) { return N >= 1 && N <= kUm
 molora_status_t launch_apply_umma(const molora_proj_desc_t* projs, int32_t P, int64_t N, int32_t C,
                                   const int32_t* offsets, const int32_t* perm, uint32_t* dev_status, int32_t min_rows,
                                   cudaStream_t s, const int32_t* r, int32_t* counts_out, int32_t parts, int32_t cbase,
-                                  const uint8_t* set_table)
+                                  const uint8_t* set_table, bool after_group)
 {
     if (N == 0 || P == 0) return MOLORA_OK;
     if (parts < 1 || parts > kUmmaMaxParts) return MOLORA_ERR_INVALID_ARG;
@@ -1026,9 +1033,14 @@ molora_status_t launch_apply_umma(const molora_proj_desc_t* projs, int32_t P, in
     prm.min_rows = min_rows;
     prm.tile_rows = kTileM;
     cudaError_t e = cudaSuccess;
-    if (has[0] && e == cudaSuccess) e = umma_launch<16>(prm, N, choose_split_for_rank<16>(prm, N), s);
-    if (has[1] && e == cudaSuccess) e = umma_launch<32>(prm, N, choose_split_for_rank<32>(prm, N), s);
-    if (has[2] && e == cudaSuccess) e = umma_launch<64>(prm, N, choose_split_for_rank<64>(prm, N), s);
+    auto plan = [&](UmmaPlan pl) {               // (the first launch only: what follows it has another predecessor)
+        pl.chained = after_group;
+        after_group = false;
+        return pl;
+    };
+    if (has[0] && e == cudaSuccess) e = umma_launch<16>(prm, N, plan(choose_split_for_rank<16>(prm, N)), s);
+    if (has[1] && e == cudaSuccess) e = umma_launch<32>(prm, N, plan(choose_split_for_rank<32>(prm, N)), s);
+    if (has[2] && e == cudaSuccess) e = umma_launch<64>(prm, N, plan(choose_split_for_rank<64>(prm, N)), s);
     return cuda_ok(e);
 }
 

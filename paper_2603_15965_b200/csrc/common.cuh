@@ -294,7 +294,7 @@ bool group_apply_umma_eligible(int64_t N, int32_t C);
 molora_status_t launch_apply_umma(const molora_proj_desc_t* projs, int32_t P, int64_t N, int32_t C,
                                   const int32_t* offsets, const int32_t* perm, uint32_t* dev_status, int32_t min_rows,
                                   cudaStream_t s, const int32_t* r = nullptr, int32_t* counts_out = nullptr,
-                                  int32_t parts = 1, int32_t n_adapters = 0, const uint8_t* set_table = nullptr);
+                                  int32_t parts = 1, int32_t n_adapters = 0, const uint8_t* set_table = nullptr, bool after_group = false);
 // (parts > 1: top-k routing in one pass -- C counts adapter SETS of `parts` adapters out of `n_adapters`, set_table[4 * set +
 // j] names them, the projections carry the stacked rank parts x r and row_scale = the weights [parts][N]; adapters' rank
 // 16, 32 or 64)
@@ -306,7 +306,7 @@ bool decode_eligible(const molora_proj_desc_t& p, molora_dtype_t dt);
 // Single-launch streaming kernel for calls below the tcgen05 crossover (bf16, ranks 16 / 32 / 64, no workspace).
 molora_status_t launch_apply_stream(const molora_proj_desc_t* projs, int32_t P, int64_t N, int32_t C,
                                     const int32_t* offsets, const int32_t* perm, int32_t max_rows, uint32_t* dev_status,
-                                    cudaStream_t s);
+                                    cudaStream_t s, bool after_group = false);
 // The same kernel for top-k routing in one pass: segments are adapter sets (n_sets of them, set_table[4 * set + j] = the
 // j-th adapter of the set), the projections carry the stacked rank parts x r and row_scale = weights [parts][N].
 bool stream_eligible(const molora_proj_desc_t& p, molora_dtype_t dt);
@@ -357,8 +357,8 @@ constexpr int32_t kUmmaAllSegmentsMaxC = 64;   // up to this many adapters the t
 
 // Launch helper: a cluster of cluster_x CTAs along x when cluster_x > 1, and, when under_predecessor is set,
 // programmatic stream serialization: the kernel may start while the previous kernel of the stream still runs and
-// calls ptx::grid_dependency_wait() before it touches what that kernel writes.  Used only between the two
-// launches of one call (weight split -> tcgen05 gate, decode shrink -> expand), where the predecessor is known;
+// calls ptx::grid_dependency_wait() before it touches what that kernel writes.  Used only between two
+// launches of one call (weight split -> tcgen05 gate, decode shrink -> expand, grouping or adapter sets -> apply), where the predecessor is known;
 // across calls the kernels run in plain stream order (chaining them was measured: no gain on any workload).
 bool chained_launch_enabled();   // false when the "chained_launch_off" override is set (plain stream order everywhere)
 // Tuning overrides, for measurements and for tests that target one kernel: process-wide integers, 0 = the library's own

@@ -9,6 +9,7 @@
 // Ends with a block-wide barrier.  All NT threads of the CTA must call it.
 #pragma once
 #include "common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace molora {
 
@@ -31,7 +32,7 @@ __device__ __forceinline__ void group_in_cta(const int32_t* __restrict__ r, int 
         // table below a decode call of 8 tokens was grouped after 4900 cycles, so after 3500; with more steps a warp it is the slower one.
         int* hist = reinterpret_cast<int*>(scratch);                               // [warp][32]
         const int C = C_, N = N_;
-        const int raw = tid < N ? __ldg(r + tid) : -1;
+        const int raw = tid < N ? ptx::ld_dependent(r + tid) : -1;
         const int v = raw < C ? raw : -1;
         unsigned own = __ballot_sync(0xFFFFFFFFu, v >= 0), same = own;
         const int bits = 32 - __clz(C - 1);
@@ -97,7 +98,7 @@ __device__ __forceinline__ void group_in_cta(const int32_t* __restrict__ r, int 
         bool bad = false;
 #pragma unroll
         for (int j = 0; j < TPT; ++j) {
-            const int raw = b0 + j < e0 ? __ldg(r + b0 + j) : -1;
+            const int raw = b0 + j < e0 ? ptx::ld_dependent(r + b0 + j) : -1;
             bad |= (raw < -1) || (raw >= C);
             v[j] = (raw >= 0 && raw < C) ? raw : -1;
         }
@@ -166,7 +167,7 @@ __device__ __forceinline__ void group_in_cta(const int32_t* __restrict__ r, int 
 #pragma unroll
         for (int j = 0; j < STEPS; ++j) {
             const int i = begin + j * 32 + lane;
-            vreg[j] = i < end ? __ldg(r + i) : -1;
+            vreg[j] = i < end ? ptx::ld_dependent(r + i) : -1;
         }
         for (int c = lane; c < C; c += 32) hist[warp][c] = 0;
         __syncwarp();

@@ -328,6 +328,14 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, int a_mn_maj
 // predecessor has completed.  Both are no-ops in a kernel launched the ordinary way.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A word that the predecessor writes: unlike a load through the read-only path it cannot be moved above the wait.
+__device__ __forceinline__ int32_t ld_dependent(const int32_t* p)
+{
+    int32_t v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float ld_dependent(const float* p) { return __int_as_float(ld_dependent(reinterpret_cast<const int32_t*>(p))); }
 __device__ __forceinline__ void grid_dependency_sync()
 {
     grid_dependency_wait();

@@ -110,3 +110,34 @@ def test_small_calls_of_rank_64(N, C, shapes):
     check(N, C, shapes, 64)
     # the scratch that these calls took before stays part of the call
     assert all(M.molora_apply_workspace_bytes(N, C, a, b, 64) > 0 for a, b in shapes)
+
+
+@pytest.mark.parametrize("rank,kernel", [(16, {}), (64, {"umma_min_tokens": 1}), (32, {"umma_min_tokens": 1000000, "small_path": 1})])
+@pytest.mark.parametrize("top", [1, 2])
+def test_apply_started_under_the_launch_before_it(rank, kernel, top):
+    """More tokens than a CTA groups: the apply starts while the grouping (or the launch that forms the adapter sets) still runs.  Calls in a
+    row on the same buffers give what plain stream order gives, bit for bit."""
+    N, C, d = 4500, 6, 256
+    ws = [W.random_problem(rank + s, N, C, d, 320, rank, "bf16") for s in range(4)]
+    xs = [dev_tensor(w.inputs["x"], "bf16") for w in ws]
+    As, Bs = [dev_tensor(w.projections[0].A, "bf16") for w in ws], [dev_tensor(w.projections[0].B, "bf16") for w in ws]
+    rng = np.random.default_rng(rank)
+    idx = [dev_tensor(np.argsort(rng.random((C, N)), axis=0)[:top].astype(np.int32), "i") for _ in ws]
+    weight = dev_tensor((rng.random((top, N)) / top).astype(np.float32), "f32")
+    results = []
+    try:
+        for off in (1, 0):
+            for k, v in dict(kernel, chained_launch_off=off).items():
+                M.molora_debug_set(k, v)
+            ys = [dev_tensor(w.projections[0].y, "bf16") for w in ws]
+            for _ in range(5):
+                for x, y, A, B, i in zip(xs, ys, As, Bs, idx):
+                    if top == 1:
+                        M.molora_group_apply_batched(i[0], [M.ProjDesc(x, y, A, B)])
+                    else:
+                        M.molora_apply_topk([M.ProjDesc(x, y, A, B)], i, weight, C)
+            results.append([to_f64(y) for y in ys])
+    finally:
+        for k in M.TUNING_NAMES:
+            M.molora_debug_set(k, 0)
+    assert all(np.array_equal(a, b) for a, b in zip(*results))
