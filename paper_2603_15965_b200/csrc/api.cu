@@ -435,11 +435,8 @@ molora_status_t plan_apply(const molora_proj_desc_t* projs, int32_t P, molora_dt
 }
 
 molora_status_t enqueue_apply(const ApplyPlan& pl, molora_dtype_t dt, int64_t N, int32_t C, const int32_t* offsets,
-                              const int32_t* perm, void* ws, size_t ws_bytes, uint32_t* dev_status, cudaStream_t s,
-                              bool after_group = false)
+                              const int32_t* perm, void* ws, size_t ws_bytes, uint32_t* dev_status, cudaStream_t s)
 {
-    // (the launch that follows the grouping launch of the same call starts under it)
-    after_group = after_group && pl.n_jc[0] + pl.n_jc[1] + pl.n_jc[2] == 0;
     molora_status_t st = MOLORA_OK;
     char* base = static_cast<char*>(ws);
     void* dws = ws != nullptr ? base + pl.decode_off : nullptr;              // scratch of the two-launch kernels
@@ -449,12 +446,12 @@ molora_status_t enqueue_apply(const ApplyPlan& pl, molora_dtype_t dt, int64_t N,
             st = launch_apply_jobs(pl.jc[k], pl.n_jc[k], N, C, offsets, perm, base, base + pl.jobs_part_off[k], pl.jobs_part[k],
                                    dev_status, s);
     if (st == MOLORA_OK && pl.n_tc > 0) {
-        st = launch_apply_umma(pl.tc, pl.n_tc, N, C, offsets, perm, dev_status, pl.min_rows, s, nullptr, nullptr, 1, 0, nullptr, after_group);
+        st = launch_apply_umma(pl.tc, pl.n_tc, N, C, offsets, perm, dev_status, pl.min_rows, s);
         if (st == MOLORA_OK && pl.n_small_sc > 0) st = launch_apply_stream(pl.small_sc, pl.n_small_sc, N, C, offsets, perm, pl.min_rows, dev_status, s);
         if (st == MOLORA_OK && pl.n_small_dc > 0) st = launch_apply_decode(pl.small_dc, pl.n_small_dc, N, C, offsets, perm, pl.min_rows, dws, dws_bytes, dev_status, s);
         if (st == MOLORA_OK && pl.n_small_cc > 0) st = launch_apply_rowtile(pl.small_cc, pl.n_small_cc, dt, N, C, offsets, perm, pl.min_rows, s);
     }
-    if (st == MOLORA_OK && pl.n_sc > 0) st = launch_apply_stream(pl.sc, pl.n_sc, N, C, offsets, perm, INT32_MAX, dev_status, s, after_group && pl.n_tc == 0);
+    if (st == MOLORA_OK && pl.n_sc > 0) st = launch_apply_stream(pl.sc, pl.n_sc, N, C, offsets, perm, INT32_MAX, dev_status, s);
     if (st == MOLORA_OK && pl.n_dc > 0) st = launch_apply_decode(pl.dc, pl.n_dc, N, C, offsets, perm, INT32_MAX, dws, dws_bytes, dev_status, s);
     if (st == MOLORA_OK && pl.n_cc > 0) st = launch_apply_rowtile(pl.cc, pl.n_cc, dt, N, C, offsets, perm, INT32_MAX, s);
     return st;
@@ -564,7 +561,7 @@ molora_status_t molora_group_apply_batched(const int32_t* r, int64_t N, int32_t 
     if (st != MOLORA_OK) return st;
     st = molora_group(r, N, C, counts, offsets, perm, nullptr, 0, dev_status, stream);
     if (st != MOLORA_OK) return st;
-    return enqueue_apply(pl, dt, N, C, offsets, perm, ws, ws_bytes, dev_status, static_cast<cudaStream_t>(stream), N > 0);
+    return enqueue_apply(pl, dt, N, C, offsets, perm, ws, ws_bytes, dev_status, static_cast<cudaStream_t>(stream));
 }
 
 molora_status_t molora_apply(const void* x, int64_t ldx, void* y, int64_t ldy, molora_dtype_t dt, int64_t N,
@@ -704,10 +701,10 @@ molora_status_t molora_apply_topk(const molora_proj_desc_t* projs, int32_t P, mo
         if (st != MOLORA_OK) return st;
         if (one_pass == 2) {                         // tcgen05 kernel: one MMA per part in the shrink, stacked B in the expand
             if (group_apply_umma_eligible(N, n_sets))
-                return launch_apply_umma(pass, P, N, n_sets, offsets, perm, dev_status, 1, s, sets, counts, k, C, table, true);
+                return launch_apply_umma(pass, P, N, n_sets, offsets, perm, dev_status, 1, s, sets, counts, k, C, table);
             st = molora_group(sets, N, n_sets, counts, offsets, perm, nullptr, 0, dev_status, stream);
             if (st != MOLORA_OK) return st;
-            return launch_apply_umma(pass, P, N, n_sets, offsets, perm, dev_status, 1, s, nullptr, nullptr, k, C, table, true);
+            return launch_apply_umma(pass, P, N, n_sets, offsets, perm, dev_status, 1, s, nullptr, nullptr, k, C, table);
         }
         if (group_apply_stream_eligible(N))         // the CTAs of the apply group the sets themselves
             return launch_group_apply_stream_sets(sets, pass, P, N, n_sets, k, C, table, counts, offsets, perm, dev_status, s);

@@ -57,10 +57,10 @@ __global__ void __launch_bounds__(kRowTileThreads, 1) apply_rowtile_kernel(const
     constexpr int WARPS = kRowTileThreads / 32;
     constexpr int RV = R / VEC;              // 16-byte vectors per row of A_c
 
+    ptx::grid_dependency_sync();             // (launched under its predecessor, whatever that is)
     const molora_proj_desc_t& pd = prm.p[blockIdx.y];
     if (pd.rank != R) return;                // a launch of this instantiation serves the projections of rank R
 
-    ptx::grid_dependency_sync();             // offsets and perm come from the grouping kernel
     int seg, row0, rows;
     const int32_t* perm_s = nullptr;
     if constexpr (GROUP) {
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(kRowTileThreads, 1) apply_rowtile_kernel(const
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid < TM) {
         const int pos = row0 + (tid < rows ? tid : rows - 1);                              // pad with the last row
-        row_s[tid] = GROUP ? perm_s[pos] : __ldg(prm.perm + pos);
+        row_s[tid] = GROUP ? perm_s[pos] : ptx::ld_dependent(prm.perm + pos);
     }
     __syncthreads();
 
@@ -99,12 +99,12 @@ __global__ void __launch_bounds__(kRowTileThreads, 1) apply_rowtile_kernel(const
     for (int k0 = tid * VEC; k0 < d_in; k0 += kRowTileThreads * VEC) {
         uint4 xp[TM];
 #pragma unroll
-        for (int m = 0; m < TM; ++m) xp[m] = ldg128_stream(x + (int64_t)row_s[m] * pd.ldx + k0);
+        for (int m = 0; m < TM; ++m) xp[m] = ld128_rw_stream(x + (int64_t)row_s[m] * pd.ldx + k0);
 #pragma unroll
         for (int j = 0; j < VEC; ++j) {
             float af[R];
 #pragma unroll
-            for (int v = 0; v < RV; ++v) unpack<T>(ldg128(Ac + (int64_t)(k0 + j) * R + v * VEC), af + v * VEC);
+            for (int v = 0; v < RV; ++v) unpack<T>(ptx::ld_dependent(reinterpret_cast<const uint4*>(Ac + (int64_t)(k0 + j) * R + v * VEC)), af + v * VEC);
 #pragma unroll
             for (int m = 0; m < TM; ++m) {
                 float xv[VEC];
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kRowTileThreads, 1) apply_rowtile_kernel(const
 #pragma unroll
         for (int w = 0; w < WARPS; ++w) s += partial[w][tid];
         // fold the LoRA scale (and the token's routing weight, if given) into t once: t_s is [TM][R], row m = tid / R
-        const float rs = pd.row_scale != nullptr ? __ldg(pd.row_scale + row_s[tid / R]) : 1.f;
+        const float rs = pd.row_scale != nullptr ? ptx::ld_dependent(pd.row_scale + row_s[tid / R]) : 1.f;
         t_s[tid] = s * pd.scale * rs;
     }
     __syncthreads();
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kRowTileThreads, 1) apply_rowtile_kernel(const
         for (int n4 = 0; n4 < R; n4 += 4) {
             float bf[4][VEC];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) unpack<T>(ldg128(Bc + (int64_t)(n4 + q) * d_out + o0), bf[q]);
+            for (int q = 0; q < 4; ++q) unpack<T>(ptx::ld_dependent(reinterpret_cast<const uint4*>(Bc + (int64_t)(n4 + q) * d_out + o0)), bf[q]);
 #pragma unroll
             for (int m = 0; m < TM; ++m) {
                 const float4 tv = *reinterpret_cast<const float4*>(&t_s[m * R + n4]);
@@ -179,7 +179,7 @@ static cudaError_t rowtile_launch(const ApplyBatchParams& prm, int64_t N, cudaSt
     const int64_t cap_rows = prm.max_rows == INT32_MAX ? N : (N < (int64_t)prm.C * prm.max_rows ? N : (int64_t)prm.C * prm.max_rows);
     const int64_t tiles = ceil_div64(cap_rows, TM) + prm.C;
     dim3 grid((unsigned)tiles, (unsigned)prm.P);
-    return launch_kernel(apply_rowtile_kernel<T, R, GROUP>, grid, dim3(kRowTileThreads), 0, s, 1, false, prm);
+    return launch_kernel(apply_rowtile_kernel<T, R, GROUP>, grid, dim3(kRowTileThreads), 0, s, 1, true, prm);
 }
 
 template <typename T, bool GROUP>

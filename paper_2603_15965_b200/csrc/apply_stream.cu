@@ -96,7 +96,6 @@ struct StreamParams {
     int32_t* counts_out;
     int32_t* offsets_out;
     int32_t* perm_out;
-    bool chained;                             // (host) launched under the kernel of the same call that made the tables or the sets
 };
 // adapter of part j of segment `seg`
 // (set_tab: the kernel's shared-memory copy of prm.set_table)
@@ -245,7 +244,7 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
                 prefetch_tensormap(&args.tm_b[p]);
             }
     }
-    grid_dependency_sync();                    // tables, sets and weights may come from the kernel this one was launched under
+    grid_dependency_sync();                    // (launched under its predecessor, whatever that is)
     if (prm.parts > 1)                         // (visible after the block-wide barriers of the prologue below)
         for (int i = tid; i < prm.C; i += kFsThreads)
             reinterpret_cast<uint32_t*>(set_tab_s)[i] = (uint32_t)ld_dependent(reinterpret_cast<const int32_t*>(prm.set_table) + i);
@@ -800,7 +799,7 @@ static cudaError_t stream_launch(StreamParams prm, [[maybe_unused]] const Stream
     FsArgs<R, SHORT, V> args;
     static_cast<StreamParams&>(args) = prm;
     if constexpr (Cfg::BOX) static_cast<StreamMaps&>(args) = maps;
-    return launch_kernel(apply_stream_kernel<R, GROUP, SHORT, V>, dim3(grid), dim3(kFsThreads), Cfg::SMEM, s, (unsigned)S, prm.chained, args);
+    return launch_kernel(apply_stream_kernel<R, GROUP, SHORT, V>, dim3(grid), dim3(kFsThreads), Cfg::SMEM, s, (unsigned)S, true, args);
 }
 
 // Estimated time of a launch (us, without its fixed part) and the CTAs per item that give it.  A launch lasts as long as its
@@ -893,9 +892,7 @@ static cudaError_t stream_rank(const molora_proj_desc_t* projs, int32_t P, int64
     auto launch = [&](auto tile, auto variant) {
         constexpr bool SHORT = decltype(tile)::value;
         constexpr int V = decltype(variant)::value;
-        const StreamParams now = prm;
-        prm.chained = false;                   // (what follows has another predecessor)
-        return group ? stream_launch<R, true, SHORT, V>(now, maps, cap_rows, S, s) : stream_launch<R, false, SHORT, V>(now, maps, cap_rows, S, s);
+        return group ? stream_launch<R, true, SHORT, V>(prm, maps, cap_rows, S, s) : stream_launch<R, false, SHORT, V>(prm, maps, cap_rows, S, s);
     };
     using One = std::integral_constant<int, kFsOne>;
     if (!small) return launch(std::false_type{}, One{});
@@ -921,7 +918,7 @@ static molora_status_t stream_enqueue(const molora_proj_desc_t* projs, int32_t P
 
 molora_status_t launch_apply_stream(const molora_proj_desc_t* projs, int32_t P, int64_t N, int32_t C,
                                     const int32_t* offsets, const int32_t* perm, int32_t max_rows, uint32_t* dev_status,
-                                    cudaStream_t s, bool after_group)
+                                    cudaStream_t s)
 {
     if (N == 0 || P == 0) return MOLORA_OK;
     StreamParams prm;
@@ -934,7 +931,6 @@ molora_status_t launch_apply_stream(const molora_proj_desc_t* projs, int32_t P, 
     prm.parts = 1;
     prm.n_adapters = C;
     prm.set_table = nullptr;
-    prm.chained = after_group;
     return stream_enqueue(projs, P, N, C, prm, false, s);
 }
 
@@ -955,7 +951,6 @@ molora_status_t launch_apply_stream_sets(const molora_proj_desc_t* projs, int32_
     prm.parts = parts;
     prm.n_adapters = n_adapters;
     prm.set_table = set_table;
-    prm.chained = true;
     return stream_enqueue(projs, P, N, n_sets, prm, false, s);
 }
 
@@ -978,7 +973,6 @@ molora_status_t launch_group_apply_stream_sets(const int32_t* sets, const molora
     prm.parts = parts;
     prm.n_adapters = n_adapters;
     prm.set_table = set_table;
-    prm.chained = true;
     return stream_enqueue(projs, P, N, n_sets, prm, true, s);
 }
 
@@ -1000,7 +994,6 @@ molora_status_t launch_group_apply_stream(const int32_t* r, const molora_proj_de
     prm.parts = 1;
     prm.n_adapters = C;
     prm.set_table = nullptr;
-    prm.chained = false;
     return stream_enqueue(projs, P, N, C, prm, true, s);
 }
 

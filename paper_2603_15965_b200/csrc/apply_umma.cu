@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
 
     // ---------------------------------------------------------------- set-up
     // The segment table is requested first; barriers and TMEM are set up while it is on its way.
-    grid_dependency_sync();            // offsets and perm come from the grouping kernel; y from the base projection
+    grid_dependency_sync();            // (launched under its predecessor, whatever that is)
     __shared__ int32_t offs_s[MOLORA_MAX_ADAPTERS + 1];
     const bool grouping = prm.r != nullptr;
     // grouping: perm, a scratch table and 256 temporary words live in the ring stages, which are idle until the tile is known
@@ -767,7 +767,6 @@ bool umma_eligible(const molora_proj_desc_t& p, molora_dtype_t dt)
 struct UmmaPlan {
     int split;       // CTAs per tile (cluster size)
     int tile_rows;   // positions per tile
-    bool chained = false;      // launched under the grouping kernel of the same call
 };
 
 template <int R, bool WIDE, int PARTS = 1>
@@ -804,7 +803,7 @@ static cudaError_t umma_launch_variant(UmmaParams prm, int64_t N, UmmaPlan plan,
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     fill_launch_config<R, WIDE>(cfg, attr, tiles, prm.P, split, s);
-    if (plan.chained && chained_launch_enabled()) {
+    if (chained_launch_enabled()) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
         ++cfg.numAttrs;
@@ -941,7 +940,7 @@ bool group_apply_umma_eligible(int64_t N, int32_t C) { return N >= 1 && N <= kUm
 molora_status_t launch_apply_umma(const molora_proj_desc_t* projs, int32_t P, int64_t N, int32_t C,
                                   const int32_t* offsets, const int32_t* perm, uint32_t* dev_status, int32_t min_rows,
                                   cudaStream_t s, const int32_t* r, int32_t* counts_out, int32_t parts, int32_t cbase,
-                                  const uint8_t* set_table, bool after_group)
+                                  const uint8_t* set_table)
 {
     if (N == 0 || P == 0) return MOLORA_OK;
     if (parts < 1 || parts > kUmmaMaxParts) return MOLORA_ERR_INVALID_ARG;
@@ -1033,14 +1032,9 @@ molora_status_t launch_apply_umma(const molora_proj_desc_t* projs, int32_t P, in
     prm.min_rows = min_rows;
     prm.tile_rows = kTileM;
     cudaError_t e = cudaSuccess;
-    auto plan = [&](UmmaPlan pl) {               // (the first launch only: what follows it has another predecessor)
-        pl.chained = after_group;
-        after_group = false;
-        return pl;
-    };
-    if (has[0] && e == cudaSuccess) e = umma_launch<16>(prm, N, plan(choose_split_for_rank<16>(prm, N)), s);
-    if (has[1] && e == cudaSuccess) e = umma_launch<32>(prm, N, plan(choose_split_for_rank<32>(prm, N)), s);
-    if (has[2] && e == cudaSuccess) e = umma_launch<64>(prm, N, plan(choose_split_for_rank<64>(prm, N)), s);
+    if (has[0] && e == cudaSuccess) e = umma_launch<16>(prm, N, choose_split_for_rank<16>(prm, N), s);
+    if (has[1] && e == cudaSuccess) e = umma_launch<32>(prm, N, choose_split_for_rank<32>(prm, N), s);
+    if (has[2] && e == cudaSuccess) e = umma_launch<64>(prm, N, choose_split_for_rank<64>(prm, N), s);
     return cuda_ok(e);
 }
 

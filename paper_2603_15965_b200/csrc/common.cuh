@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "molora.h"
+#include "sm100_ptx.cuh"
 
 namespace molora {
 
@@ -117,9 +118,9 @@ __device__ __forceinline__ bool find_tile(const int32_t* __restrict__ offsets, i
                                           int min_rows, int max_rows, int& seg, int& row0, int& rows)
 {
     int base = 0;
-    int prev = __ldg(offsets);
+    int prev = ptx::ld_dependent(offsets);
     for (int c = 0; c < C; ++c) {
-        const int next = __ldg(offsets + c + 1);
+        const int next = ptx::ld_dependent(offsets + c + 1);
         const int n = next - prev;
         const int tiles = (n >= min_rows && n < max_rows) ? (n + tile_rows - 1) / tile_rows : 0;
         if (tile < base + tiles) {
@@ -294,7 +295,7 @@ bool group_apply_umma_eligible(int64_t N, int32_t C);
 molora_status_t launch_apply_umma(const molora_proj_desc_t* projs, int32_t P, int64_t N, int32_t C,
                                   const int32_t* offsets, const int32_t* perm, uint32_t* dev_status, int32_t min_rows,
                                   cudaStream_t s, const int32_t* r = nullptr, int32_t* counts_out = nullptr,
-                                  int32_t parts = 1, int32_t n_adapters = 0, const uint8_t* set_table = nullptr, bool after_group = false);
+                                  int32_t parts = 1, int32_t n_adapters = 0, const uint8_t* set_table = nullptr);
 // (parts > 1: top-k routing in one pass -- C counts adapter SETS of `parts` adapters out of `n_adapters`, set_table[4 * set +
 // j] names them, the projections carry the stacked rank parts x r and row_scale = the weights [parts][N]; adapters' rank
 // 16, 32 or 64)
@@ -306,7 +307,7 @@ bool decode_eligible(const molora_proj_desc_t& p, molora_dtype_t dt);
 // Single-launch streaming kernel for calls below the tcgen05 crossover (bf16, ranks 16 / 32 / 64, no workspace).
 molora_status_t launch_apply_stream(const molora_proj_desc_t* projs, int32_t P, int64_t N, int32_t C,
                                     const int32_t* offsets, const int32_t* perm, int32_t max_rows, uint32_t* dev_status,
-                                    cudaStream_t s, bool after_group = false);
+                                    cudaStream_t s);
 // The same kernel for top-k routing in one pass: segments are adapter sets (n_sets of them, set_table[4 * set + j] = the
 // j-th adapter of the set), the projections carry the stacked rank parts x r and row_scale = weights [parts][N].
 bool stream_eligible(const molora_proj_desc_t& p, molora_dtype_t dt);
@@ -356,10 +357,14 @@ constexpr int64_t kUmmaMinTokens = 1024;     // below this no projection uses th
 constexpr int32_t kUmmaAllSegmentsMaxC = 64;   // up to this many adapters the tensor-core kernel takes all segments
 
 // Launch helper: a cluster of cluster_x CTAs along x when cluster_x > 1, and, when under_predecessor is set,
-// programmatic stream serialization: the kernel may start while the previous kernel of the stream still runs and
-// calls ptx::grid_dependency_wait() before it touches what that kernel writes.  Used only between two
-// launches of one call (weight split -> tcgen05 gate, decode shrink -> expand, grouping or adapter sets -> apply), where the predecessor is known;
-// across calls the kernels run in plain stream order (chaining them was measured: no gain on any workload).
+// programmatic stream serialization: the kernel may start while the previous kernel of the stream still runs, if that one lets it, and
+// calls ptx::grid_dependency_sync() before it touches global memory at all -- whoever wrote what it reads, or still reads what
+// it writes.  (Two kernels know their predecessor, the preparation launch of the same call, and load activations before they wait.)
+// The apply kernels, the grouping, the vocabulary and top-k routers and the MLP router with prepared images are launched so: their
+// set-up and the launch itself run behind the end of what is before them.  Measured with and without (us, whole steps): mixed 777
+// tokens 33.6 / 30.7, MLP-routed 1000 32.8 / 27.8, 3001 composite 44.4 / 39.8, top-2 2048 88.4 / 84.3, decode layers from a graph 184.7 / 180.7.
+// Not the gates: started early, their small CTAs crowd onto the SMs that are free first (four decode layers with a gate each 172 as it is,
+// 209 with chained gates).
 bool chained_launch_enabled();   // false when the "chained_launch_off" override is set (plain stream order everywhere)
 // Tuning overrides, for measurements and for tests that target one kernel: process-wide integers, 0 = the library's own
 // choice.  Their start values come from the environment (MOLORA_UMMA_MIN_TOKENS, MOLORA_SMALL_PATH=stream|twophase|jobs,

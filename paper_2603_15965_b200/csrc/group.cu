@@ -51,14 +51,14 @@ __global__ void __launch_bounds__(kGroupThreads) group_cluster_kernel(const int3
     if (S > 1) cluster_arrive_relaxed();   // "I am running"; waited for before the first write to a peer
     for (int c = lane; c < C; c += 32) hist[warp][c] = 0;
     __syncwarp();
-    ptx::grid_dependency_sync();   // r is the router's output
+    ptx::grid_dependency_sync();   // (launched under its predecessor, as a rule the router)
 
     // the first kGroupCached steps of the warp's tokens stay in registers for both passes (all loads in flight at once)
     int vreg[kGroupCached];
 #pragma unroll
     for (int j = 0; j < kGroupCached; ++j) {
         const int64_t i = begin + j * 32 + lane;
-        vreg[j] = i < end ? __ldg(r + i) : -1;
+        vreg[j] = i < end ? ptx::ld_dependent(r + i) : -1;
     }
     auto route_of = [&](int64_t i0) {
         const int64_t j = (i0 - begin) >> 5;
@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(kGroupThreads) group_cluster_kernel(const int3
                 if (jj == j) v = vreg[jj];
         } else {
             const int64_t i = i0 + lane;
-            v = i < end ? __ldg(r + i) : -1;
+            v = i < end ? ptx::ld_dependent(r + i) : -1;
         }
         return v;
     };
@@ -182,7 +182,7 @@ molora_status_t launch_group(const int32_t* r, int64_t N, int32_t C, int32_t* co
     int split = 1;
     while (split < kGroupMaxCluster && (int64_t)split * 1024 < N) split *= 2;
     if (const int64_t forced = tune(kTuneGroupSplit)) split = (int)std::max<int64_t>(1, std::min<int64_t>(forced, kGroupMaxCluster));
-    return cuda_ok(launch_kernel(group_cluster_kernel, dim3((unsigned)split), dim3(kGroupThreads), 0, s, (unsigned)split, false,
+    return cuda_ok(launch_kernel(group_cluster_kernel, dim3((unsigned)split), dim3(kGroupThreads), 0, s, (unsigned)split, true,
                                   r, N, C, counts, offsets, perm, dev_status));
 }
 

@@ -27,12 +27,12 @@ __global__ void __launch_bounds__(256) route_vocab_kernel(const int32_t* __restr
 {
     __shared__ int32_t b[MOLORA_MAX_ADAPTERS + 1];
     ptx::grid_dependency_sync();
-    for (int i = threadIdx.x; i <= M; i += blockDim.x) b[i] = __ldg(breaks + i);
+    for (int i = threadIdx.x; i <= M; i += blockDim.x) b[i] = ptx::ld_dependent(breaks + i);
     __syncthreads();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     bool any_bad = false;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
-        const int32_t v = __ldg(ids + i);
+        const int32_t v = ptx::ld_dependent(ids + i);
         int32_t m;
         if (M <= 8) {
             m = 0;
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(256) route_vocab_kernel(const int32_t* __restr
         }
         bool inside = (v >= b[0]) && (v < b[M]);
         if (adapter != nullptr) {
-            int32_t a = __ldg(adapter + i);
+            int32_t a = ptx::ld_dependent(adapter + i);
             if (slot_of != nullptr)                // hot-set: adapter id -> slot through the slot table's inverse (may be
                 a = (a >= 0 && a < n_catalog) ? __ldcg(slot_of + a) : -1;      // rewritten by the maintenance stream)
             inside = inside && a >= 0 && a < n_adapters;
@@ -69,7 +69,7 @@ molora_status_t launch_route_vocab(const int32_t* ids, int64_t N, const int32_t*
     const int threads = 256;
     const int64_t want = ceil_div64(N, threads);
     const int blocks = (int)(want < 148 * 8 ? want : 148 * 8);
-    return cuda_ok(launch_kernel(route_vocab_kernel, dim3(blocks), dim3(threads), 0, s, 1, false, ids, N, breaks, M, adapter,
+    return cuda_ok(launch_kernel(route_vocab_kernel, dim3(blocks), dim3(threads), 0, s, 1, true, ids, N, breaks, M, adapter,
                                   n_adapters, slot_of, n_catalog, r_out, dev_status));
 }
 
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(256) topk_softmax_kernel(const float* __restri
     if (i >= N) return;
     float z[32];
 #pragma unroll
-    for (int c = 0; c < 32; ++c) z[c] = c < C ? __ldg(logits + i * C + c) : 0.f;
+    for (int c = 0; c < 32; ++c) z[c] = c < C ? ptx::ld_dependent(logits + i * C + c) : 0.f;
     uint32_t taken = 0;
     float zmax = 0.f, den = 0.f;
     float kept[32];
@@ -523,7 +523,7 @@ molora_status_t launch_topk_softmax(const float* logits, int64_t N, int32_t C, i
                                     cudaStream_t s)
 {
     if (N == 0) return MOLORA_OK;
-    return cuda_ok(launch_kernel(topk_softmax_kernel, dim3((unsigned)ceil_div64(N, 256)), dim3(256), 0, s, 1, false, logits, N,
+    return cuda_ok(launch_kernel(topk_softmax_kernel, dim3((unsigned)ceil_div64(N, 256)), dim3(256), 0, s, 1, true, logits, N,
                                  (int)C, (int)k, idx_out, w_out));
 }
 
@@ -557,8 +557,8 @@ __global__ void __launch_bounds__(256) topk_sets_kernel(const int32_t* __restric
     bool ok = true;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        a[j] = j < k ? __ldg(idx + (int64_t)j * N + i) : 0x7FFFFFFF;
-        f[j] = j < k ? __ldg(w + (int64_t)j * N + i) : 0.f;
+        a[j] = j < k ? ptx::ld_dependent(idx + (int64_t)j * N + i) : 0x7FFFFFFF;
+        f[j] = j < k ? ptx::ld_dependent(w + (int64_t)j * N + i) : 0.f;
         ok = ok && (j >= k || (a[j] >= 0 && a[j] < C));
     }
 #pragma unroll
@@ -583,7 +583,7 @@ molora_status_t launch_topk_sets(const int32_t* idx, const float* w, int64_t N, 
                                  float* w_out, uint8_t* table_out, cudaStream_t s)
 {
     if (N == 0) return MOLORA_OK;
-    return cuda_ok(launch_kernel(topk_sets_kernel, dim3((unsigned)ceil_div64(N, 256)), dim3(256), 0, s, 1, false, idx, w, N, (int)C,
+    return cuda_ok(launch_kernel(topk_sets_kernel, dim3((unsigned)ceil_div64(N, 256)), dim3(256), 0, s, 1, true, idx, w, N, (int)C,
                                  (int)k, set_out, w_out, table_out));
 }
 

@@ -246,6 +246,7 @@ __global__ void __launch_bounds__(kGateSplitWarps * 32, 2)
                             const void* __restrict__ weights, const float* __restrict__ bias, int C,
                             int32_t* __restrict__ r_out, float* __restrict__ logits_out)
 {
+    ptx::grid_dependency_sync();             // (what follows may set up meanwhile)
     using Img = GateImage<NT, KC>;
     constexpr int CP = Img::CP, ROW = Img::ROW, NB = KC / 32;
     __shared__ __align__(16) float part_s[kGateSplitWarps][16][CP + 4];

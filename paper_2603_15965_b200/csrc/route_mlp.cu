@@ -46,6 +46,7 @@ struct MlpParams {
     uint32_t* dev_status;
     int64_t N;
     int32_t d, H, C;
+    int32_t after_prepare;      // the previous launch made the weight images (and was an ordinary one): only they have to be waited for
 };
 
 struct MlpCtrl {
@@ -113,12 +114,13 @@ __global__ void __launch_bounds__(kMlpThreads, 1) route_mlp_umma_kernel(const __
         tmem_alloc(smem_u32(&ctrl->tmem_base), 512);
         tmem_relinquish();
     }
+    if (!prm.after_prepare) grid_dependency_sync();        // (launched under its predecessor, whatever that is)
     // second-layer weights and first-layer bias on chip (rows of hidden units that do not exist are zero)
     for (int e = tid; e < HP * prm.C; e += kMlpThreads) {
         const int j = e / prm.C, c = e - j * prm.C;
-        w2s[j * kMlpMaxC + c] = j < prm.H ? __ldg(prm.W2 + (int64_t)j * prm.C + c) : 0.f;
+        w2s[j * kMlpMaxC + c] = j < prm.H ? ld_dependent(prm.W2 + (int64_t)j * prm.C + c) : 0.f;
     }
-    for (int j = tid; j < HP; j += kMlpThreads) b1s[j] = (prm.b1 != nullptr && j < prm.H) ? __ldg(prm.b1 + j) : 0.f;
+    for (int j = tid; j < HP; j += kMlpThreads) b1s[j] = (prm.b1 != nullptr && j < prm.H) ? ld_dependent(prm.b1 + j) : 0.f;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -259,7 +261,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) route_mlp_umma_kernel(const __
                     for (int c = 0; c < prm.C; ++c) {
                         float v = 0.f;
                         for (int p2 = 0; p2 < parts; ++p2) v += zbuf[(p2 * RO + tl2) * kMlpMaxC + c];
-                        if (prm.b2 != nullptr) v += __ldg(prm.b2 + c);
+                        if (prm.b2 != nullptr) v += ld_dependent(prm.b2 + c);
                         if (prm.logits_out != nullptr) prm.logits_out[i * prm.C + c] = v;
                         if (c == 0 || v > best) { best = v; arg = c; }   // strict '>' keeps the lowest index on ties
                     }
@@ -294,7 +296,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) route_mlp_umma_kernel(const __
             for (int c = 0; c < kMlpMaxC; ++c) {
                 if (c < prm.C) {
                     float v = z[c];
-                    if (prm.b2 != nullptr) v += __ldg(prm.b2 + c);
+                    if (prm.b2 != nullptr) v += ld_dependent(prm.b2 + c);
                     if (prm.logits_out != nullptr) prm.logits_out[i * prm.C + c] = v;
                     if (c == 0 || v > best) { best = v; arg = c; }      // strict '>' keeps the lowest index on ties
                 }
@@ -410,8 +412,8 @@ static molora_status_t mlp_umma_launch(const void* x, int64_t N, int d, int64_t 
             return MOLORA_ERR_CUDA;
         if (image == kImageBuildOnly) return MOLORA_OK;
     }
-    const bool chained = image == kImageBuildAndUse;       // overlap with the tail of the preparation kernel
     MlpParams prm;
+    prm.after_prepare = image == kImageBuildAndUse;        // (overlaps with its tail)
     if (!make_tensor_map_bf16_2d(&prm.tm_x, x, (uint64_t)d, (uint64_t)N, (uint64_t)ldx, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_tensor_map_bf16_2d(&prm.tm_w, img, 64, (uint64_t)(d / 64) * NP, 64, 64, 192, CU_TENSOR_MAP_SWIZZLE_128B))
         return MOLORA_ERR_CUDA;
@@ -427,9 +429,9 @@ static molora_status_t mlp_umma_launch(const void* x, int64_t N, int d, int64_t 
     prm.C = C;
     if (split > 1)
         return cuda_ok(launch_kernel(route_mlp_umma_kernel<HP, true>, dim3((unsigned)tiles * split), dim3(kMlpThreads),
-                                     MlpCfg<HP, true>::SMEM, s, split, chained, prm));
+                                     MlpCfg<HP, true>::SMEM, s, split, true, prm));
     return cuda_ok(launch_kernel(route_mlp_umma_kernel<HP, false>, dim3((unsigned)tiles), dim3(kMlpThreads),
-                                 MlpCfg<HP, false>::SMEM, s, 1, chained, prm));
+                                 MlpCfg<HP, false>::SMEM, s, 1, true, prm));
 }
 
 template <typename T>

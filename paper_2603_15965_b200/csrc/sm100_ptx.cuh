@@ -335,6 +335,12 @@ __device__ __forceinline__ int32_t ld_dependent(const int32_t* p)
     asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ uint4 ld_dependent(const uint4* p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ float ld_dependent(const float* p) { return __int_as_float(ld_dependent(reinterpret_cast<const int32_t*>(p))); }
 __device__ __forceinline__ void grid_dependency_sync()
 {
