@@ -413,14 +413,19 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
         uint32_t g = 0;
         if constexpr (GROUP) group_write_perm(perm_s, offs_s[prm.C], prm.perm_out, tid, kFsWarps * 32);
         auto slot_of = [&](int i, int rank) { return recv + ((i & 1) * S + rank) * Cfg::TFLOATS; };
-        // LoRA scale x the token's routing weight (top-k in one pass: the weight of the part the column belongs to)
-        auto scaled = [&](const FsItem& it, const molora_proj_desc_t& pd, int e4, float4 v) {
+        // LoRA scale x the token's routing weight (top-k in one pass: the weight of the part the column belongs to) of the pieces of t
+        // that this thread finishes.  With one CTA per item it is asked for before the item's chunks: in front of the sum the two loads in a
+        // row cost every item of a top-2 call ~0.5 us (a layer of 2048 tokens 72.5 us, so 70.9).
+        constexpr int PIECES = (Cfg::TFLOATS / 4 + kFsWarps * 32 - 1) / (kFsWarps * 32);
+        auto scale_of = [&](const FsItem& it, const molora_proj_desc_t& pd, int e4) {
             const int row = e4 * 4 / R;
-            if (row >= it.rows) return make_float4(0.f, 0.f, 0.f, 0.f);       // rows past the tile hold stale shared memory
             float sc = pd.scale;
-            if (pd.row_scale != nullptr)
+            if (pd.row_scale != nullptr && row < it.rows)
                 sc *= ld_dependent(pd.row_scale + (int64_t)((e4 * 4 % R) / (R / prm.parts)) * prm.N + fs_token(prm, perm_s, it.row0 + row));
-            return make_float4(v.x * sc, v.y * sc, v.z * sc, v.w * sc);
+            return sc;
+        };
+        auto scaled = [&](float sc, bool live, float4 v) {          // rows past the tile hold stale shared memory
+            return live ? make_float4(v.x * sc, v.y * sc, v.z * sc, v.w * sc) : make_float4(0.f, 0.f, 0.f, 0.f);
         };
 
         // ---- shrink: this CTA's partial of t = x A_c, item i of the cluster
@@ -428,6 +433,11 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
             const molora_proj_desc_t& pd = prm.p[it.proj];
             const bool two = MT == 2 && it.rows > 16;   // the second 16-row MMA tile holds valid rows
             const int pr = R / prm.parts, wbytes = pr * 2;
+            [[maybe_unused]] float sc[PIECES];
+            if constexpr (Cfg::MAXS == 1) {
+#pragma unroll
+                for (int k = 0; k < PIECES; ++k) sc[k] = scale_of(it, pd, tid + k * kFsWarps * 32);
+            }
             float acc[MT][NT][4];
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt)
@@ -490,7 +500,10 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
                         }
                     fs_compute_sync();
                     float* out = slot_of(i, crank);
-                    for (int e4 = tid; e4 < Cfg::TFLOATS / 4; e4 += kFsWarps * 32) {
+#pragma unroll
+                    for (int k = 0; k < PIECES; ++k) {
+                        const int e4 = tid + k * kFsWarps * 32;
+                        if (e4 >= Cfg::TFLOATS / 4) break;
                         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                         for (int w = 0; w < Cfg::KW; ++w) {
@@ -500,7 +513,8 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
                             v.z += u.z;
                             v.w += u.w;
                         }
-                        *reinterpret_cast<float4*>(&out[e4 * 4]) = S == 1 ? scaled(it, pd, e4, v) : v;
+                        if constexpr (Cfg::MAXS == 1) v = scaled(sc[k], e4 * 4 / R < it.rows, v);
+                        *reinterpret_cast<float4*>(&out[e4 * 4]) = v;
                     }
                     fence_proxy_async_smem();          // my writes are ordered before the copies that refill the stage or read the slot
                     fs_compute_sync();                 // the partial is complete; the stage is free
@@ -535,7 +549,7 @@ __global__ void __launch_bounds__(kFsThreads, 1) apply_stream_kernel(const __gri
                         v.z += u.z;
                         v.w += u.w;
                     }
-                    *reinterpret_cast<float4*>(&tfin[e4 * 4]) = scaled(it, pd, e4, v);
+                    *reinterpret_cast<float4*>(&tfin[e4 * 4]) = scaled(scale_of(it, pd, e4), e4 * 4 / R < it.rows, v);
                 }
                 fs_compute_sync();
             }
