@@ -42,6 +42,7 @@
 #include <stdlib.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "group_inline.cuh"
@@ -121,7 +122,6 @@ struct UmmaCfg {
     static constexpr int kTRowBytes = R * 2;                          // one row of T_hi / T_lo
     static constexpr int kTBytes = kTileM * kTRowBytes;
     static constexpr int kSwzBits = R == 64 ? 3 : R == 32 ? 2 : 1;    // swizzle width of R*2-byte rows
-    static constexpr uint32_t kWLayout = swizzle_layout_type(static_cast<Swizzle>(kSwzBits));
     // partial T rows received from the cluster peers: (S - 1) * ceil(128 / S) rows of R fp32: 64, 86, 96 rows for
     // S = 2, 3, 4 and at most 114 (S = 7) up to S = 8.  Rank 64 stops at S = 3 (shared memory) unless WIDE.
     // Ranks 16 and 32 have room for the whole partial of every peer ((S - 1) * 128 rows): one push, every CTA sums
@@ -883,8 +883,18 @@ static UmmaPlan choose_split_for_rank(const UmmaParams& prm, int64_t N)
         min_kx = std::min(min_kx, prm.p[i].d_in / kChunkCols);
         chunks[nproj++] = (double)((prm.p[i].d_in + prm.p[i].d_out) / kChunkCols);
     }
-    // expected tiles per projection: every segment has at least one and ends in a partial one
-    auto tiles_for = [&](int rows) { return std::max<int64_t>(prm.C, ceil_div64(N, rows) + prm.C / 2); };
+    // Tiles per projection, as many as a balanced or a random load has: a segment ends in a partial tile, half a tile on
+    // average with a spread of sqrt(C / 12) over C random remainders; equal segments all round up together.  The estimate
+    // takes the larger of the two because the two errors do not cost the same: a tile more than the resident clusters
+    // makes a second wave, a cluster size one step too small costs 5 - 10 % (2300 tokens of 8 adapters, 2048 -> 2048, rank
+    // 64: 24 tiles, 27.9 us over clusters of 6 that N / 128 + C / 2 tiles would have fit, 16.9 us now; 4096 -> 4096 36.9 and
+    // 23.2, with 16 adapters 42.5 and 27.1.  Of 48 such calls with 4 - 16 adapters the worst is 10 % off the best size, not
+    // 67 %; what it costs: up to 4 % where the tile that was feared does not come, 4096 -> 4096, 1700 tokens of 16).
+    auto tiles_for = [&](int rows) {
+        const int64_t random = ceil_div64(N, rows) + (int64_t)(prm.C / 2.0 + std::sqrt(prm.C / 12.0));
+        const int64_t equal = (int64_t)prm.C * ceil_div64(ceil_div64(N, prm.C), rows);
+        return std::max<int64_t>(prm.C, std::max(random, equal));
+    };
     // Estimated time of the launch: the CTAs are dispatched heaviest projection first onto the resident clusters, so the
     // launch lasts as long as its heaviest tile or as the whole work spread over the cluster slots (plus a quarter of a
     // light tile of imbalance), whichever is longer; with equal tiles it is whole waves.
