@@ -60,7 +60,7 @@ namespace {
 //            (123 MB) 34.2 / 28.4, 16384 tokens 127 / 141; with 3000 tokens and 300 per adapter from 60 MB already, which is what
 //            narrow models reach: four projections 512 wide, 8000 tokens (74 MB) 25 / 36, 1024 wide, 5000 (92 MB) 29 / 37; a layer
 //            512 wide, 3500 tokens (100 MB) 24 / 35
-//   rank 64  one or two projections (the two-launch pair below): once they move ~12 MB with at least 256 tokens and segments
+//   rank 64  one or two projections (against the two-launch pair, which narrow ones and those of 512 tokens run on below): once they move ~12 MB with at least 256 tokens and segments
 //            of 32 rows on average (one 4096-wide projection: from 512 tokens, 21.0 against 24.3; two: 23.2 against 38.9 at
 //            512 tokens).  More: from 680 tokens with 60 per adapter: 600 tokens, 8 adapters 44.8 / 39.6, 777: 44.6 / 51.3;
 //            1000 tokens, 16 adapters 66.2 / 70.4; below that from 256 tokens where segments are long or the call is large: 120 per
