@@ -220,13 +220,18 @@ molora_status_t launch_apply_rowtile(const molora_proj_desc_t* projs, int32_t P,
 }
 
 // Grouping and apply in one launch: calls that go to this kernel with one rank (fp32 storage, or rank 8) while every tile has an SM
-// of its own -- a second wave would group again.
+// of its own -- a second wave would group again.  The launch-count queries ask this of descriptors that nobody has checked: what
+// molora_group_apply_batched refuses is no launch of this kernel.
 bool group_apply_rowtile_eligible(const molora_proj_desc_t* projs, int32_t P, molora_dtype_t dt, int64_t N, int32_t C)
 {
     const int32_t rank = projs[0].rank;
-    if (N < 1 || N > kRowTileGroupMaxN || (dt != MOLORA_F32 && rank != 8)) return false;
-    for (int i = 0; i < P; ++i)
-        if (projs[i].rank != rank || decode_eligible(projs[i], dt)) return false;
+    if (rank != 8 && rank != 16 && rank != 32 && rank != 64) return false;
+    if (dt != MOLORA_F32 && (dt != MOLORA_BF16 || rank != 8)) return false;
+    if (N < 1 || N > kRowTileGroupMaxN || C < 1 || C > MOLORA_MAX_ADAPTERS) return false;
+    for (int i = 0; i < P; ++i) {
+        const molora_proj_desc_t& p = projs[i];
+        if (p.rank != rank || p.d_in <= 0 || p.d_out <= 0 || (p.d_in % 8) != 0 || (p.d_out % 8) != 0 || decode_eligible(p, dt)) return false;
+    }
     return (ceil_div64(N, 128 / rank) + C) * P <= sm_count();
 }
 

@@ -195,3 +195,22 @@ def test_mixed_call_without_workspace_is_refused_before_any_launch(default_kerne
     arr64 = (_ProjDescC * 1)(_desc(512, 128, 64))
     assert lib.molora_group_apply_batched(fake, 300, 6, fake, fake, fake, arr64, 1, M.BF16, None, 0, None, None) == 3
     assert M.molora_launch_count() == before
+
+
+@pytest.mark.parametrize("dt,rank,width,C", [
+    (M.F32, 0, 64, 4), (M.F32, 24, 64, 4), (M.F32, 129, 64, 4), (M.F32, 256, 64, 4), (M.F32, -8, 64, 4), (M.BF16, 0, 64, 4), (M.BF16, 24, 64, 4),
+    (M.F32, 8, 60, 4), (M.F32, 8, 0, 4), (M.F32, 8, -64, 4), (M.F32, 8, 64, 257), (7, 8, 64, 4),
+])
+def test_launch_count_queries_of_descriptors_that_the_call_refuses(default_kernels, dt, rank, width, C):
+    """The queries answer 0 for them (one that divided by such a rank ended the process)."""
+    from paper_2603_15965_b200.binding import _ProjDescC
+    lib = M.load_library()
+    fake = ctypes.c_void_p(0x1000)
+    arr = (_ProjDescC * 1)(_desc(width, width, rank))
+    assert lib.molora_group_apply_is_one_launch(arr, 1, dt, 16, C) == 0
+    assert lib.molora_group_apply_skips_group_launch(arr, 1, dt, 16, C) == 0
+    before = M.molora_launch_count()
+    assert lib.molora_group_apply_batched(fake, 16, C, fake, fake, fake, arr, 1, dt, None, 0, None, None) != 0
+    assert M.molora_launch_count() == before
+    good = (_ProjDescC * 1)(_desc(64, 64, 8))                          # what it takes is still one launch
+    assert lib.molora_group_apply_is_one_launch(good, 1, M.F32, 16, 4) == 1
