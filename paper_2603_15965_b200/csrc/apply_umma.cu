@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
 
     // ---------------------------------------------------------------- set-up
     // The segment table is requested first; barriers and TMEM are set up while it is on its way.
-    grid_dependency_sync();            // (launched under its predecessor, whatever that is)
+    grid_dependency_wait();            // (launched under its predecessor, whatever that is)
     __shared__ int32_t offs_s[MOLORA_MAX_ADAPTERS + 1];
     const bool grouping = prm.r != nullptr;
     // grouping: perm, a scratch table and 256 temporary words live in the ring stages, which are idle until the tile is known
@@ -279,6 +279,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    grid_dependency_trigger();         // (not before TMEM is mine: see the launch helper)
     int seg, row0, rows;
     if (!find_tile_smem(offs_s, prm.C, prm.tile_rows, my_tile, prm.min_rows, INT32_MAX, seg, row0, rows)) {
         // past the last tile (the grid is sized from an upper bound); the whole cluster takes this exit together

@@ -359,7 +359,12 @@ constexpr int32_t kUmmaAllSegmentsMaxC = 64;   // up to this many adapters the t
 // Launch helper: a cluster of cluster_x CTAs along x when cluster_x > 1, and, when under_predecessor is set,
 // programmatic stream serialization: the kernel may start while the previous kernel of the stream still runs, if that one lets it, and
 // calls ptx::grid_dependency_sync() before it touches global memory at all -- whoever wrote what it reads, or still reads what
-// it writes.  (Two kernels know their predecessor, the preparation launch of the same call, and load activations before they wait.)
+// it writes.  Three kernels know their predecessor, an ordinary launch of the same call, and load before they wait what that one does not
+// write: the tensor-core routers behind the preparation of their weights (activations), the expand of the two-launch pair behind its shrink
+// (tables, y and B -- the shrink has to stay an ordinary launch for it).
+// A kernel that uses TMEM behind an unknown predecessor allocates it after the wait, and every one lets its successor start only
+// when its CTA has its columns: the allocation waits without a limit, and a CTA beside it on the SM that held the columns while it waits
+// for this kernel, or for one that has yet to allocate, would never give them back.
 // The apply kernels, the grouping, the vocabulary and top-k routers and the MLP router with prepared images are launched so: their
 // set-up and the launch itself run behind the end of what is before them.  Measured with and without (us, whole steps): mixed 777
 // tokens 33.6 / 30.7, MLP-routed 1000 32.8 / 27.8, 3001 composite 44.4 / 39.8, top-2 2048 88.4 / 84.3, decode layers from a graph 184.7 / 180.7.

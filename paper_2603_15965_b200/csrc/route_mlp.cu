@@ -110,11 +110,11 @@ __global__ void __launch_bounds__(kMlpThreads, 1) route_mlp_umma_kernel(const __
         ctrl->abort_flag = 0;
         fence_mbar_init();
     }
+    if (!prm.after_prepare) grid_dependency_wait();        // (launched under its predecessor, whatever that is)
     if (warp == 1) {
         tmem_alloc(smem_u32(&ctrl->tmem_base), 512);
         tmem_relinquish();
     }
-    if (!prm.after_prepare) grid_dependency_sync();        // (launched under its predecessor, whatever that is)
     // second-layer weights and first-layer bias on chip (rows of hidden units that do not exist are zero)
     for (int e = tid; e < HP * prm.C; e += kMlpThreads) {
         const int j = e / prm.C, c = e - j * prm.C;
@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) route_mlp_umma_kernel(const __
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (!prm.after_prepare) grid_dependency_trigger();     // (not before TMEM is mine: see the launch helper)
     // "I am running and my barriers are initialised": the matching wait comes right before the first store into a peer
     if (SPLIT) cluster_arrive_relaxed();
     const uint32_t tmem = ctrl->tmem_base;
