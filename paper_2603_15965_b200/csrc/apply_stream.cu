@@ -57,6 +57,7 @@
 #include "group_inline.cuh"
 #include "pipeline.cuh"
 #include "sm100_ptx.cuh"
+#include "stream_slices.cuh"
 #include "tensor_map.cuh"
 
 namespace molora {
@@ -708,25 +709,15 @@ bool stream_eligible(const molora_proj_desc_t& p, molora_dtype_t dt)
     return dt == MOLORA_BF16 && (p.rank == 16 || p.rank == 32 || p.rank == 64) && (p.d_in % 32) == 0 && (p.d_out % 32) == 0;
 }
 
-// Output slices: one item per (projection, tile) to start with; while `most` units (items per tile) allow it, the widest is split once
-// more.  Returns the number of units.
-static int slice_outputs(const StreamParams& prm, int CH, int64_t most, int32_t* och, int32_t* ustart)
+static SliceShapes slice_shapes(const StreamParams& prm, int CH)
 {
-    int slices[MOLORA_MAX_PROJECTIONS], chunks[MOLORA_MAX_PROJECTIONS], total = prm.P;
+    SliceShapes sh;
+    sh.P = prm.P;
     for (int i = 0; i < prm.P; ++i) {
-        och[i] = chunks[i] = ceil_div(prm.p[i].d_out, CH);
-        slices[i] = 1;
+        sh.in[i] = ceil_div(prm.p[i].d_in, CH);
+        sh.out[i] = ceil_div(prm.p[i].d_out, CH);
     }
-    for (; total + 1 <= most; ++total) {
-        int widest = 0;
-        for (int i = 1; i < prm.P; ++i)
-            if (och[i] > och[widest]) widest = i;
-        if (och[widest] <= 1) break;
-        och[widest] = ceil_div(chunks[widest], ++slices[widest]);
-    }
-    ustart[0] = 0;
-    for (int i = 0; i < prm.P; ++i) ustart[i + 1] = ustart[i] + ceil_div(chunks[i], och[i]);
-    return ustart[prm.P];
+    return sh;
 }
 
 // most tiles that `rows` rows in C segments can give (every segment that has rows adds at most one partial tile)
@@ -743,41 +734,6 @@ static double expected_tiles(const StreamParams& prm, int64_t rows, int tile_row
     const double segments = std::min((double)rows, std::max(1.0, met * (1.0 - std::pow(1.0 - 1.0 / met, 0.75 * (double)rows))));
     const double fill = (double)rows / segments / tile_rows;
     return segments * (fill <= 0.75 ? 1.0 : fill <= 1.0 ? 1.0 + 2.0 * (fill - 0.75) : fill + 0.5);
-}
-
-// Output slices of calls whose items no longer fit one wave (one CTA per item): the launch lasts as long as its busiest CTA, and a
-// gate or up projection in a layer is six expand jobs behind two shrinks while the average CTA has five jobs.  Cutting it in two costs
-// two more shrinks and evens that out.  The dealing of the items is followed for the tiles that are expected, with up to four cuts; a
-// shrink job counts 0.65, an expand job 1.0 (measured in place at rank 16: 1240 and 1900 cycles).  256 tokens of 8 adapters, sixteen layers
-// 2048 wide: 207 us without cuts, 186 with.  Returns the number of units.
-static int balanced_units(const StreamParams& prm, int CH, int clusters, int tiles, int32_t* och, int32_t* ustart)
-{
-    constexpr int kCuts = 4, kMaxClusters = 256;
-    int best_units = prm.P;
-    float best = 0.f;
-    for (int most = prm.P; most <= prm.P + kCuts; ++most) {
-        const int units = slice_outputs(prm, CH, most, och, ustart);
-        if (units < most) break;
-        float load[kMaxClusters] = {};
-        float longest = 0.f;
-        int item = 0;
-        for (int p = 0; p < prm.P; ++p)
-            for (int u = ustart[p]; u < ustart[p + 1]; ++u) {
-                const int ne = std::min(och[p], ceil_div(prm.p[p].d_out, CH) - (u - ustart[p]) * och[p]);
-                const float cost = 0.65f * (float)ceil_div(prm.p[p].d_in, CH) + 1.0f * (float)ne + 0.4f;
-                for (int t = 0; t < tiles; ++t, ++item) {
-                    const int round = item / clusters, c = item - round * clusters;
-                    float& l = load[(round & 1) ? clusters - 1 - c : c];
-                    l += cost;
-                    longest = std::max(longest, l);
-                }
-            }
-        if (most == prm.P || longest < 0.97f * best) {
-            best = longest;
-            best_units = units;
-        }
-    }
-    return slice_outputs(prm, CH, best_units, och, ustart);
 }
 
 template <int R, bool GROUP, bool SHORT, int V>
@@ -805,10 +761,11 @@ static cudaError_t stream_launch(StreamParams prm, [[maybe_unused]] const Stream
         clusters = std::max(1, n);
     }
     const int64_t tiles_max = tiles_bound(rows, prm.C, Cfg::ROWS);
-    const int tiles = S == 1 && prm.P > 2 && tiles_max * prm.P > clusters && tiles_max * prm.P <= 3 * clusters && clusters <= 256
+    const SliceShapes shapes = slice_shapes(prm, Cfg::CH);
+    const int tiles = S == 1 && prm.P > 2 && tiles_max * prm.P > clusters && tiles_max * prm.P <= 3 * clusters && clusters <= kSliceMaxClusters
                           ? (int)std::lround(expected_tiles(prm, rows, Cfg::ROWS)) : 0;
-    if (tiles > 0) prm.ustart[prm.P] = balanced_units(prm, Cfg::CH, clusters, tiles, prm.och, prm.ustart);
-    else prm.ustart[prm.P] = slice_outputs(prm, Cfg::CH, S == 1 ? clusters / tiles_max : 0, prm.och, prm.ustart);
+    if (tiles > 0) prm.ustart[prm.P] = balanced_units(shapes, clusters, tiles, prm.och, prm.ustart);
+    else prm.ustart[prm.P] = slice_outputs(shapes, S == 1 ? clusters / tiles_max : 0, prm.och, prm.ustart);
     const unsigned grid = (unsigned)(std::max<int64_t>(1, std::min<int64_t>(tiles_max * prm.ustart[prm.P], clusters)) * S);
     FsArgs<R, SHORT, V> args;
     static_cast<StreamParams&>(args) = prm;
@@ -838,11 +795,12 @@ static double stream_estimate(const StreamParams& prm, int64_t rows, int& split)
     for (int i = 0; i < prm.P; ++i) most = std::min(most, ceil_div(prm.p[i].d_in, Cfg::CH));      // every CTA shrinks something
     const int64_t forced = tune(kTuneStreamSplit);
     const int sms = sm_count();
+    const SliceShapes shapes = slice_shapes(prm, Cfg::CH);
     double best = 1e30;
     for (int S = 1; S <= most; S *= 2) {
         const double clusters = S <= 2 ? sms / S : S == 4 ? sms * 0.9 / 4 : sms * 0.86 / 8;
         int32_t och[MOLORA_MAX_PROJECTIONS], ustart[MOLORA_MAX_PROJECTIONS + 1];
-        const int units = slice_outputs(prm, Cfg::CH, S == 1 ? sms / tiles_bound(rows, prm.C, Cfg::ROWS) : 0, och, ustart);
+        const int units = slice_outputs(shapes, S == 1 ? sms / tiles_bound(rows, prm.C, Cfg::ROWS) : 0, och, ustart);
         double sum = 0.0, longest = 0.0;
         for (int i = 0; i < prm.P; ++i) {
             // (the CTAs of a cluster take whole chunks: the first one has the most)
