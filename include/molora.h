@@ -373,8 +373,8 @@ molora_status_t molora_selftest_bounded_wait(uint32_t *dev_status, int64_t limit
  * The whole path on HOST activations (one layer: route -> group -> apply for P projections), for callers
  * whose activations live in host memory.  Enqueued in the order of `stream`: host-to-device copies of the routing
  * source and of every distinct x and every y into `arena`, the router, the grouping, the apply (Eq. 2), device-to-host
- * copies of every y back into y_host.  Calls of 8 MB and more go projection by projection, applied and copied back on a
- * second stream of the call's own while the next ones come in; what is enqueued on `stream` afterwards follows all of
+ * copies of every y back into y_host.  Calls of 8 MB and more go projection by projection, applied and copied back on
+ * two streams of the call's own while the next ones come in; what is enqueued on `stream` afterwards follows all of
  * it.  (In one piece on `stream` alone: calls under capture, and host buffers that overlap.)  The call returns without
  * waiting; x_host / y_host must stay valid (and should be pinned for the copies to be asynchronous) until the
  * stream has finished.  Adapter stacks, gate weights and vocabulary breaks are DEVICE pointers: weights stay
@@ -389,7 +389,8 @@ molora_status_t molora_selftest_bounded_wait(uint32_t *dev_status, int64_t limit
  * arena        device scratch of at least molora_forward_host_arena_bytes(...) bytes, 256-byte aligned, zero-filled
  *              before its first use (it holds the apply workspace, see molora_apply)
  * dev_status   device uint32 or NULL (as for the individual calls)
- * Errors are detected before anything is enqueued, as for the individual calls. */
+ * Errors in the arguments are detected before anything is enqueued, as for the individual calls.  Copies into y_host are enqueued
+ * last: after MOLORA_ERR_CUDA from a copy to the device or from a launch every y_host is as it was. */
 typedef enum { MOLORA_ROUTE_VOCAB = 0, MOLORA_ROUTE_GATE = 1, MOLORA_ROUTE_GIVEN = 2 } molora_router_t;
 typedef struct {
     const void *x_host; /* [N, d_in]  dense (pitch d_in)                         */

@@ -832,28 +832,41 @@ struct HostCall {
     }
 };
 
-// A second stream for the length of one call.  It lives until what was enqueued on it has run (the runtime keeps a destroyed stream
-// that long); an event is read when it is waited for, so one serves all hand-overs of its direction.
-struct SideStream {
-    cudaStream_t stream = nullptr;
-    cudaEvent_t arrived = nullptr, done = nullptr;
-    bool open()
+// Two more streams for the length of one call, one that applies and one that copies results back.  They live until what was enqueued on
+// them has run (the runtime keeps a destroyed stream that long); an event is read when it is waited for, so one serves all hand-overs of
+// its direction -- but not the results: their copies are enqueued after all launches, each behind an event of its own.
+constexpr int kHostMaxPieces = 4;                                           // of the last projection
+struct SideStreams {
+    cudaStream_t apply = nullptr, back = nullptr;
+    cudaEvent_t arrived = nullptr, done = nullptr, applied[MOLORA_MAX_PROJECTIONS - 1 + kHostMaxPieces] = {};
+    bool open(int results)
     {
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;          // (another thread may be capturing)
         if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
-        const bool ok = cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) == cudaSuccess &&
-                        cudaEventCreateWithFlags(&arrived, cudaEventDisableTiming) == cudaSuccess &&
-                        cudaEventCreateWithFlags(&done, cudaEventDisableTiming) == cudaSuccess;
+        bool ok = cudaStreamCreateWithFlags(&apply, cudaStreamNonBlocking) == cudaSuccess &&
+                  cudaStreamCreateWithFlags(&back, cudaStreamNonBlocking) == cudaSuccess &&
+                  cudaEventCreateWithFlags(&arrived, cudaEventDisableTiming) == cudaSuccess &&
+                  cudaEventCreateWithFlags(&done, cudaEventDisableTiming) == cudaSuccess;
+        for (int i = 0; i < results && ok; ++i) ok = cudaEventCreateWithFlags(&applied[i], cudaEventDisableTiming) == cudaSuccess;
         cudaThreadExchangeStreamCaptureMode(&mode);
         return ok;
     }
-    bool follow(cudaStream_t s) { return cudaEventRecord(arrived, s) == cudaSuccess && cudaStreamWaitEvent(stream, arrived, 0) == cudaSuccess; }
-    bool join(cudaStream_t s) { return cudaEventRecord(done, stream) == cudaSuccess && cudaStreamWaitEvent(s, done, 0) == cudaSuccess; }
-    ~SideStream()
+    bool follow(cudaStream_t s) { return cudaEventRecord(arrived, s) == cudaSuccess && cudaStreamWaitEvent(apply, arrived, 0) == cudaSuccess; }
+    bool join(cudaStream_t s)
     {
+        bool ok = true;
+        for (cudaStream_t side : {apply, back})
+            ok = cudaEventRecord(done, side) == cudaSuccess && cudaStreamWaitEvent(s, done, 0) == cudaSuccess && ok;
+        return ok;
+    }
+    ~SideStreams()
+    {
+        for (cudaEvent_t e : applied)
+            if (e != nullptr) cudaEventDestroy(e);
         if (done != nullptr) cudaEventDestroy(done);
         if (arrived != nullptr) cudaEventDestroy(arrived);
-        if (stream != nullptr) cudaStreamDestroy(stream);
+        if (back != nullptr) cudaStreamDestroy(back);
+        if (apply != nullptr) cudaStreamDestroy(apply);
     }
 };
 
@@ -908,7 +921,7 @@ int64_t host_last_rows(const HostCall& c, int64_t N, const void* route_src, int 
     const int last = c.P - 1;
     const bool own_x = c.pl->x_owner[last] == last && !(gate >= 0 && c.pl->x_owner[gate] == last);
     const double last_bytes = (double)c.e * (double)N * ((own_x ? c.projs[last].d_in : 0) + (double)c.projs[last].d_out);
-    const int64_t pieces = std::max<int64_t>(1, std::min<int64_t>(4, (int64_t)(last_bytes / kHostPieceBytes)));
+    const int64_t pieces = std::max<int64_t>(1, std::min<int64_t>(kHostMaxPieces, (int64_t)(last_bytes / kHostPieceBytes)));
     const int64_t rows = std::min(N, ceil_div64(ceil_div64(N, pieces), 64) * 64);
     if (bytes < kHostPieceBytes || (c.P == 1 && rows == N)) return 0;
     for (int i = 0; i < n_ranges; ++i)
@@ -993,8 +1006,8 @@ molora_status_t molora_forward_host(molora_router_t router, const int32_t* route
         return MOLORA_ERR_CUDA;
     if (gate >= 0 && !call.upload_x(gate, 0, N, s)) return MOLORA_ERR_CUDA;
     const int64_t last_rows = host_last_rows(call, N, route_src_host, gate, s);
-    SideStream side;
-    if (last_rows == 0 || !side.open()) {
+    SideStreams side;
+    if (last_rows == 0 || !side.open(P - 1 + (int)ceil_div64(N, last_rows))) {
         // on the caller's stream: the other activations, route, group and apply, results back
         for (int i = 0; i < P; ++i)
             if (!call.upload(i, 0, N, gate, s)) return MOLORA_ERR_CUDA;
@@ -1005,21 +1018,36 @@ molora_status_t molora_forward_host(molora_router_t router, const int32_t* route
             if (!call.download(i, 0, N, s)) return MOLORA_ERR_CUDA;
         return MOLORA_OK;
     }
-    // 2. one projection after the other: the caller's stream uploads, the side stream routes and groups once, applies what has arrived and
-    // sends its results back while the next ones come in; the last projection goes in pieces of last_rows
-    molora_status_t st = side.follow(s) ? route(side.stream) : MOLORA_ERR_CUDA;
+    // 2. one projection after the other: the caller's stream uploads, a second one routes and groups once and applies what has arrived; the
+    // last projection goes in pieces of last_rows
+    molora_status_t st = side.follow(s) ? route(side.apply) : MOLORA_ERR_CUDA;
     if (st == MOLORA_OK && P > 1)
-        st = molora_group(r, N, C, call.ints(pl.counts), call.ints(pl.offsets), call.ints(pl.perm), nullptr, 0, dev_status, side.stream);
+        st = molora_group(r, N, C, call.ints(pl.counts), call.ints(pl.offsets), call.ints(pl.perm), nullptr, 0, dev_status, side.apply);
+    int results = 0;
     for (int i = 0; i < P && st == MOLORA_OK; ++i) {
         const int64_t piece = i == P - 1 ? last_rows : N;
         for (int64_t lo = 0; lo < N && st == MOLORA_OK; lo += piece) {
             const int64_t n = std::min(piece, N - lo);
             if (!call.upload(i, lo, n, gate, s) || !side.follow(s)) st = MOLORA_ERR_CUDA;
             if (st == MOLORA_OK)
-                st = i == P - 1 ? call.group_apply(i, 1, lo, n, side.stream)
+                st = i == P - 1 ? call.group_apply(i, 1, lo, n, side.apply)
                                 : molora_apply_batched(dev + i, 1, dt, N, C, call.ints(pl.offsets), call.ints(pl.perm), call.ws(), pl.apply_ws_bytes,
-                                                       dev_status, side.stream);
-            if (st == MOLORA_OK && !call.download(i, lo, n, side.stream)) st = MOLORA_ERR_CUDA;
+                                                       dev_status, side.apply);
+            if (st == MOLORA_OK && cudaEventRecord(side.applied[results++], side.apply) != cudaSuccess) st = MOLORA_ERR_CUDA;
+        }
+    }
+    // 3. all of it has been accepted (a call that is refused half-way leaves every y_host as it was): a third stream sends each result back
+    // as soon as it has been applied, while the next projections come in -- the host is here long before the first of them is there.  The
+    // last one follows its apply on that stream.
+    const int n_results = results;
+    results = 0;
+    for (int i = 0; i < P && st == MOLORA_OK; ++i) {
+        const int64_t piece = i == P - 1 ? last_rows : N;
+        for (int64_t lo = 0; lo < N && st == MOLORA_OK; lo += piece, ++results) {
+            const bool final = results == n_results - 1;
+            if ((!final && cudaStreamWaitEvent(side.back, side.applied[results], 0) != cudaSuccess) ||
+                !call.download(i, lo, std::min(piece, N - lo), final ? side.apply : side.back))
+                st = MOLORA_ERR_CUDA;
         }
     }
     return side.join(s) ? st : MOLORA_ERR_CUDA;        // (whatever was enqueued there belongs to the caller's stream again)
