@@ -723,17 +723,30 @@ static SliceShapes slice_shapes(const StreamParams& prm, int CH)
 // most tiles that `rows` rows in C segments can give (every segment that has rows adds at most one partial tile)
 static int64_t tiles_bound(int64_t rows, int64_t C, int tile_rows) { return std::min(rows, ceil_div64(rows, tile_rows) + std::min(C, rows)); }
 
+// Segments that may have rows: of the adapter sets of top-k routing only those of different adapters are met; the others are there for
+// callers that repeat one.
+static double segments_met(const StreamParams& prm)
+{
+    return (double)(prm.parts > 1 && prm.n_adapters >= prm.parts ? binom_small(prm.n_adapters, prm.parts) : prm.C);
+}
+
 // Tiles that `rows` rows are expected to give.
 static double expected_tiles(const StreamParams& prm, int64_t rows, int tile_rows)
 {
     // Tiles of segments of about equal size: one each while that is well below a tile's height, half a tile lost per segment from there
     // on.  Of the segments as many are counted as three quarters of the rows, spread at random, meet: adapters are not equally popular
-    // (rank 64, 4096 wide, 20 tokens of 16 adapters by popularity: clusters of four 26 us, of two, as for all 16, 32).  Of the adapter
-    // sets of top-k routing only those of different adapters are met; the others are there for callers that repeat one.
-    const double met = (double)(prm.parts > 1 && prm.n_adapters >= prm.parts ? binom_small(prm.n_adapters, prm.parts) : prm.C);
+    // (rank 64, 4096 wide, 20 tokens of 16 adapters by popularity: clusters of four 26 us, of two, as for all 16, 32).
+    const double met = segments_met(prm);
     const double segments = std::min((double)rows, std::max(1.0, met * (1.0 - std::pow(1.0 - 1.0 / met, 0.75 * (double)rows))));
     const double fill = (double)rows / segments / tile_rows;
     return segments * (fill <= 0.75 ? 1.0 : fill <= 1.0 ? 1.0 + 2.0 * (fill - 0.75) : fill + 0.5);
+}
+
+// Tiles of as many rows spread evenly.
+static int equal_tiles(const StreamParams& prm, int64_t rows, int tile_rows)
+{
+    const int64_t segments = std::max<int64_t>(1, std::min(rows, (int64_t)segments_met(prm)));
+    return (int)(segments * ceil_div64(ceil_div64(rows, segments), tile_rows));
 }
 
 template <int R, bool GROUP, bool SHORT, int V>
@@ -764,7 +777,7 @@ static cudaError_t stream_launch(StreamParams prm, [[maybe_unused]] const Stream
     const SliceShapes shapes = slice_shapes(prm, Cfg::CH);
     const int tiles = S == 1 && prm.P > 2 && tiles_max * prm.P > clusters && tiles_max * prm.P <= 3 * clusters && clusters <= kSliceMaxClusters
                           ? (int)std::lround(expected_tiles(prm, rows, Cfg::ROWS)) : 0;
-    if (tiles > 0) prm.ustart[prm.P] = balanced_units(shapes, clusters, tiles, prm.och, prm.ustart);
+    if (tiles > 0) prm.ustart[prm.P] = balanced_units(shapes, clusters, tiles, equal_tiles(prm, rows, Cfg::ROWS), prm.och, prm.ustart);
     else prm.ustart[prm.P] = slice_outputs(shapes, S == 1 ? clusters / tiles_max : 0, prm.och, prm.ustart);
     const unsigned grid = (unsigned)(std::max<int64_t>(1, std::min<int64_t>(tiles_max * prm.ustart[prm.P], clusters)) * S);
     FsArgs<R, SHORT, V> args;

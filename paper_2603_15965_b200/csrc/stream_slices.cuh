@@ -67,18 +67,25 @@ inline int busiest_cluster(const SliceShapes& sh, const int32_t* och, const int3
 // gate or up projection in a layer is six expand jobs behind two shrinks while the average CTA has five jobs.  Cutting it in two costs
 // two more shrinks and evens that out.  The dealing of the items is followed for the tiles that are expected, with up to four cuts; a
 // shrink job counts 0.65 of an expand job (measured in place at rank 16: 1240 and 1900 cycles).  256 tokens of 8 adapters, sixteen layers
-// 2048 wide: 207 us without cuts, 186 with.  Returns the number of units.
-inline int balanced_units(const SliceShapes& sh, int clusters, int tiles, int32_t* och, int32_t* ustart)
+// 2048 wide: 207 us without cuts, 186 with.
+// How many tiles there are depends on the load, which the host does not know, so a cut must not lengthen the launch of an evenly spread one
+// (equal_tiles) either: of 32 adapters 40 tokens are expected to meet 20 and may meet all, and the cuts for 20 tiles made a layer 3072 wide
+// 23.3 us where none take 18.3 (36 tokens, 2560 wide 21.1 / 16.8; rank 64, 44 tokens, 512 wide 17.8 / 15.4).
+// The costs are those of rank 16; layers and attention projections of all ranks, 16 to 1200 tokens, us with cuts / without, where the
+// rule cuts: rank 16 0.87 to 1.0, rank 32 0.91 to 1.03, rank 64 0.90 to 1.0 of the time.  Returns the number of units.
+inline int balanced_units(const SliceShapes& sh, int clusters, int tiles, int equal_tiles, int32_t* och, int32_t* ustart)
 {
     constexpr int kCuts = 4;
-    int best_units = sh.P, best = 0;
+    int best_units = sh.P, best = 0, best_equal = 0;
     for (int most = sh.P; most <= sh.P + kCuts; ++most) {
         if (slice_outputs(sh, most, och, ustart) < most) break;
         const int longest = busiest_cluster(sh, och, ustart, clusters, tiles);
-        if (most == sh.P || (int64_t)longest * 100 < (int64_t)best * 97) {
-            best = longest;
-            best_units = most;
-        }
+        if (most > sh.P && (int64_t)longest * 100 >= (int64_t)best * 97) continue;
+        const int equal = equal_tiles == tiles ? longest : busiest_cluster(sh, och, ustart, clusters, equal_tiles);
+        if (most > sh.P && equal > best_equal) continue;
+        best = longest;
+        best_equal = equal;
+        best_units = most;
     }
     return slice_outputs(sh, best_units, och, ustart);
 }

@@ -25,9 +25,9 @@ extern "C" int busiest(int P, const int* in, const int* out, const int* och, con
 {
     return busiest_cluster(shapes(P, in, out), och, ustart, clusters, tiles);
 }
-extern "C" int balanced(int P, const int* in, const int* out, int clusters, int tiles, int* och, int* ustart)
+extern "C" int balanced(int P, const int* in, const int* out, int clusters, int tiles, int equal, int* och, int* ustart)
 {
-    return balanced_units(shapes(P, in, out), clusters, tiles, och, ustart);
+    return balanced_units(shapes(P, in, out), clusters, tiles, equal, och, ustart);
 }
 extern "C" double shortest_us(int P, const int* in, const int* out, int clusters, int tiles)
 {
@@ -36,7 +36,7 @@ extern "C" double shortest_us(int P, const int* in, const int* out, int clusters
     double best = 1e9;
     for (int i = 0; i < 2000; ++i) {
         const auto t0 = std::chrono::steady_clock::now();
-        sink = sink + balanced_units(shapes(P, in, out), clusters, tiles, och, ustart);
+        sink = sink + balanced_units(shapes(P, in, out), clusters, tiles, tiles + 4, och, ustart);
         best = std::min(best, std::chrono::duration<double, std::micro>(std::chrono::steady_clock::now() - t0).count());
     }
     return best;
@@ -84,6 +84,7 @@ def test_busiest_cluster_and_choice(lib, clusters):
         P = int(rng.integers(1, 9))
         ins, outs = [int(v) for v in rng.integers(1, 13, P)], [int(v) for v in rng.integers(1, 25, P)]
         tiles = int(rng.choice([1, 2, clusters - 1, clusters, clusters + 1, int(rng.integers(1, 3 * clusters + 2))])) or 1
+        equal = int(rng.choice([tiles, max(1, tiles // 2), int(rng.integers(1, 3 * clusters + 2))]))
         och, ustart = (ctypes.c_int * 8)(), (ctypes.c_int * 9)()
         best, best_units, slices_of = None, None, {}
         for most in range(P, P + 5):
@@ -92,9 +93,10 @@ def test_busiest_cluster_and_choice(lib, clusters):
             slices_of[most] = list(och[:P])
             longest = walk(ins, outs, och, ustart, clusters, tiles)
             assert lib.busiest(P, ints(ins), ints(outs), och, ustart, clusters, tiles) == longest
-            if best is None or longest * 100 < best * 97:
-                best, best_units = longest, most
-        assert lib.balanced(P, ints(ins), ints(outs), clusters, tiles, och, ustart) == best_units
+            evenly = walk(ins, outs, och, ustart, clusters, equal)
+            if best is None or (longest * 100 < best[0] * 97 and evenly <= best[1]):
+                best, best_units = (longest, evenly), most
+        assert lib.balanced(P, ints(ins), ints(outs), clusters, tiles, equal, och, ustart) == best_units
         assert list(och[:P]) == slices_of[best_units]
 
 
@@ -104,3 +106,15 @@ def test_cost_does_not_grow_with_the_tiles(lib):
     few, many = (min(lib.shortest_us(7, ins, outs, 148, t) for _ in range(3)) for t in (14, 112))
     print(few, many)
     assert many < 3 * few
+
+
+@pytest.mark.parametrize("hidden,chunk,tiles,equal", [(3072, 1024, 20, 32), (2560, 1024, 18, 32), (512, 256, 21, 32)])
+def test_no_cut_that_lengthens_an_evenly_spread_load(lib, hidden, chunk, tiles, equal):
+    """Layers of few tokens of 32 adapters: a cut that pays for the tiles that are expected would cost the tiles of an even load more."""
+    kv, inter = hidden // 4 // 64 * 64, 3 * hidden
+    widths = [(hidden, inter), (hidden, inter), (inter, hidden), (hidden, hidden), (hidden, hidden), (hidden, kv), (hidden, kv)]
+    ins, outs = ([-(-w[i] // chunk) for w in widths] for i in (0, 1))
+    och, ustart = (ctypes.c_int * 8)(), (ctypes.c_int * 9)()
+    units = lib.balanced(7, ints(ins), ints(outs), 148, tiles, equal, och, ustart)
+    assert walk(ins, outs, och, ustart, 148, equal) <= walk(ins, outs, outs, list(range(8)), 148, equal)
+    assert units == 7 and lib.balanced(7, ints(ins), ints(outs), 148, tiles, tiles, och, ustart) > 7
