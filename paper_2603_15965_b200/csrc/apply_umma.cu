@@ -42,13 +42,13 @@
 #include <stdlib.h>
 
 #include <algorithm>
-#include <cmath>
 
 #include "common.cuh"
 #include "group_inline.cuh"
 #include "pipeline.cuh"
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
+#include "umma_split.cuh"
 
 namespace molora {
 
@@ -765,11 +765,6 @@ bool umma_eligible(const molora_proj_desc_t& p, molora_dtype_t dt)
            (p.d_out % kChunkCols) == 0;
 }
 
-struct UmmaPlan {
-    int split;       // CTAs per tile (cluster size)
-    int tile_rows;   // positions per tile
-};
-
 template <int R, bool WIDE, int PARTS = 1>
 static void fill_launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int64_t tiles, int P, int split,
                                cudaStream_t s)
@@ -868,12 +863,6 @@ static int max_active_clusters(int split)
 template <int R>
 constexpr int max_split_for_rank() { return R == 64 ? kMaxWideSplit : UmmaCfg<R>::kMaxSplitR; }
 
-// CTAs per tile.  Tiles are 128 rows, so small calls have too few of them for 148 SMs; a tile can be split over a
-// cluster (up to 4 CTAs; up to 8 at rank 64).  Pick the split with the smallest estimated time, in microseconds, from a
-// model fitted to one-projection 4096 -> 4096 calls at rank 64 (64 ... 4096 tokens, every split, graph replay): a wave of
-// resident clusters costs a fixed 9 us (launch, tile look-up, first arrival, last stores), 3 us more for the exchange
-// of the partial T tiles, and 0.40 us per 64-column chunk a CTA walks (shrink chunks + expand chunks divided by the
-// split); shorter tiles make a chunk only a little cheaper (the gathers are bound by requests in flight, not bytes).
 template <int R>
 static UmmaPlan choose_split_for_rank(const UmmaParams& prm, int64_t N)
 {
@@ -884,64 +873,11 @@ static UmmaPlan choose_split_for_rank(const UmmaParams& prm, int64_t N)
         min_kx = std::min(min_kx, prm.p[i].d_in / kChunkCols);
         chunks[nproj++] = (double)((prm.p[i].d_in + prm.p[i].d_out) / kChunkCols);
     }
-    // Tiles per projection, as many as a balanced or a random load has: a segment ends in a partial tile, half a tile on
-    // average with a spread of sqrt(C / 12) over C random remainders; equal segments all round up together.  The estimate
-    // takes the larger of the two because the two errors do not cost the same: a tile more than the resident clusters
-    // makes a second wave, a cluster size one step too small costs 5 - 10 % (2300 tokens of 8 adapters, 2048 -> 2048, rank
-    // 64: 24 tiles, 27.9 us over clusters of 6 that N / 128 + C / 2 tiles would have fit, 16.9 us now; 4096 -> 4096 36.9 and
-    // 23.2, with 16 adapters 42.5 and 27.1.  Of 48 such calls with 4 - 16 adapters the worst is 10 % off the best size, not
-    // 67 %; what it costs: up to 4 % where the tile that was feared does not come, 4096 -> 4096, 1700 tokens of 16).
-    auto tiles_for = [&](int rows) {
-        const int64_t random = ceil_div64(N, rows) + (int64_t)(prm.C / 2.0 + std::sqrt(prm.C / 12.0));
-        const int64_t equal = (int64_t)prm.C * ceil_div64(ceil_div64(N, prm.C), rows);
-        return std::max<int64_t>(prm.C, std::max(random, equal));
-    };
-    // Estimated time of the launch: the CTAs are dispatched heaviest projection first onto the resident clusters, so the
-    // launch lasts as long as its heaviest tile or as the whole work spread over the cluster slots (plus a quarter of a
-    // light tile of imbalance), whichever is longer; with equal tiles it is whole waves.
-    auto cost_for = [&](int rows, int split, bool& one_wave) {
-        const int resident = max_active_clusters<R>(split);
-        const int64_t tiles = tiles_for(rows);
-        // (a chunk costs up to 1.4 times as much once every SM streams: 35 GB/s per SM instead of ~50)
-        const double load = std::min(1.0, (double)(tiles * nproj * split) / 148.0);
-        const double fixed = 9.0 + (split > 1 ? 3.0 : 0.0);
-        const double per_chunk = 0.40 * (1.0 + 0.4 * load * load) * (0.7 + 0.3 * rows / 128.0) / split;
-        double cmax = 0.0, cmin = 1e30, total = 0.0;
-        for (int i = 0; i < nproj; ++i) {
-            const double c = fixed + per_chunk * chunks[i];
-            cmax = std::max(cmax, c);
-            cmin = std::min(cmin, c);
-            total += c * (double)tiles;
-        }
-        one_wave = tiles * nproj * 1.1 <= resident;         // (margin: the tile count is an estimate)
-        if (one_wave) return cmax;
-        if (cmax - cmin < 1e-9) return cmax * (double)((tiles * nproj + resident - 1) / resident);
-        return std::max(cmax, total / resident + 0.25 * cmin);
-    };
-    UmmaPlan best = {1, kTileM};
     const int64_t fsplit = tune(kTuneUmmaSplit), frows = tune(kTuneUmmaTileRows);          // tuning overrides
-    if (fsplit > 0 || frows > 0) {
-        if (fsplit > 0) best.split = (int)std::max<int64_t>(1, std::min<int64_t>(fsplit, max_split_for_rank<R>()));
-        if (frows > 0) best.tile_rows = (int)std::max<int64_t>(32, std::min<int64_t>(frows, kTileM));
-    } else if (nproj > 0) {
-        double best_cost = 1e30;
-        bool best_one_wave = false;
-        for (int split = 1; split <= max_split_for_rank<R>(); ++split) {    // cluster sizes need not be powers of two
-            bool one_wave;
-            const double cost = cost_for(kTileM, split, one_wave);
-            if (cost < best_cost - 1e-9) { best_cost = cost; best_one_wave = one_wave; best = {split, kTileM}; }
-        }
-        // A call that does not even fill one wave can use shorter tiles (the MMA tile keeps 128 lanes, the extra
-        // lanes idle) to put more SMs to work, as long as everything still fits in one wave.
-        if (best_one_wave && tiles_for(kTileM) * nproj * best.split < 0.85 * 148) {
-            for (int rows = 96; rows >= 64; rows -= 32)
-                for (int split = 1; split <= max_split_for_rank<R>(); ++split) {
-                    bool one_wave;
-                    const double cost = cost_for(rows, split, one_wave);
-                    if (one_wave && cost < best_cost - 1e-9) { best_cost = cost; best = {split, rows}; }
-                }
-        }
-    }
+    if (fsplit <= 0 && frows <= 0) return choose_umma_split(chunks, nproj, min_kx, N, prm.C, max_split_for_rank<R>(), 148, max_active_clusters<R>);
+    UmmaPlan best = {1, kTileM};
+    if (fsplit > 0) best.split = (int)std::max<int64_t>(1, std::min<int64_t>(fsplit, max_split_for_rank<R>()));
+    if (frows > 0) best.tile_rows = (int)std::max<int64_t>(32, std::min<int64_t>(frows, kTileM));
     while (best.split > 1 && min_kx / best.split < 4) --best.split;   // keep at least four chunks of d_in per CTA
     return best;
 }
