@@ -839,12 +839,14 @@ constexpr int kHostMaxPieces = 4;                                           // o
 struct SideStreams {
     cudaStream_t apply = nullptr, back = nullptr;
     cudaEvent_t arrived = nullptr, done = nullptr, applied[MOLORA_MAX_PROJECTIONS - 1 + kHostMaxPieces] = {};
-    bool open(int results)
+    bool open(int results, cudaStream_t s)
     {
+        int priority = 0;                                                   // the kernels keep that of the caller's stream
+        if (cudaStreamGetPriority(s, &priority) != cudaSuccess) return false;
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;          // (another thread may be capturing)
         if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
-        bool ok = cudaStreamCreateWithFlags(&apply, cudaStreamNonBlocking) == cudaSuccess &&
-                  cudaStreamCreateWithFlags(&back, cudaStreamNonBlocking) == cudaSuccess &&
+        bool ok = cudaStreamCreateWithPriority(&apply, cudaStreamNonBlocking, priority) == cudaSuccess &&
+                  cudaStreamCreateWithPriority(&back, cudaStreamNonBlocking, priority) == cudaSuccess &&
                   cudaEventCreateWithFlags(&arrived, cudaEventDisableTiming) == cudaSuccess &&
                   cudaEventCreateWithFlags(&done, cudaEventDisableTiming) == cudaSuccess;
         for (int i = 0; i < results && ok; ++i) ok = cudaEventCreateWithFlags(&applied[i], cudaEventDisableTiming) == cudaSuccess;
@@ -1007,7 +1009,7 @@ molora_status_t molora_forward_host(molora_router_t router, const int32_t* route
     if (gate >= 0 && !call.upload_x(gate, 0, N, s)) return MOLORA_ERR_CUDA;
     const int64_t last_rows = host_last_rows(call, N, route_src_host, gate, s);
     SideStreams side;
-    if (last_rows == 0 || !side.open(P - 1 + (int)ceil_div64(N, last_rows))) {
+    if (last_rows == 0 || !side.open(P - 1 + (int)ceil_div64(N, last_rows), s)) {
         // on the caller's stream: the other activations, route, group and apply, results back
         for (int i = 0; i < P; ++i)
             if (!call.upload(i, 0, N, gate, s)) return MOLORA_ERR_CUDA;

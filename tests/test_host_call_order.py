@@ -107,3 +107,10 @@ def test_a_call_that_is_refused_half_way_returns_no_results(fake, N, shapes):
             ran, at_end = before(log)
             if name != "record":
                 assert at_end == frozenset(ran)
+
+
+@pytest.mark.parametrize("priority", [0, -3])
+def test_streams_of_a_call_have_the_priority_of_the_callers(fake, priority):
+    _, log = call(fake, 2048, 8, ATTENTION, priority=priority)
+    made = [a[1] for n, a in log if n == "stream"]
+    assert len(made) == 2 and set(made) == {priority}
