@@ -926,6 +926,8 @@ int64_t host_last_rows(const HostCall& c, int64_t N, const void* route_src, int 
     const int64_t pieces = std::max<int64_t>(1, std::min<int64_t>(kHostMaxPieces, (int64_t)(last_bytes / kHostPieceBytes)));
     const int64_t rows = std::min(N, ceil_div64(ceil_div64(N, pieces), 64) * 64);
     if (bytes < kHostPieceBytes || (c.P == 1 && rows == N)) return 0;
+    // (the job-list kernel, which runs where a measurement asks for it, keeps control words where the scratch of another projection's call begins)
+    if (tune(kTuneSmallPath) == 3) return 0;
     for (int i = 0; i < n_ranges; ++i)
         for (int j = 0; j < i; ++j)
             if ((ranges[i].written || ranges[j].written) && ranges[i].lo < ranges[j].hi && ranges[j].lo < ranges[i].hi) return 0;

@@ -114,3 +114,16 @@ def test_streams_of_a_call_have_the_priority_of_the_callers(fake, priority):
     _, log = call(fake, 2048, 8, ATTENTION, priority=priority)
     made = [a[1] for n, a in log if n == "stream"]
     assert len(made) == 2 and set(made) == {priority}
+
+
+def test_scratch_of_one_projection_spares_the_control_words_of_another(fake):
+    """1100 tokens, "small_path" 3: the rank-64 projection on the pair, whose scratch begins where the workspace does when it is applied by
+    itself; the rank-16 one in pieces would be small enough for the job-list kernel, whose control words are there."""
+    fake.molora_debug_set(b"small_path", 3)
+    try:
+        st, log = call(fake, 1100, 32, [(1024, 1024, 64), (1024, 8192, 16)])
+    finally:
+        fake.molora_debug_set(b"small_path", 0)
+    assert st == 0
+    pair, jobs = ([a[2] for n, a in log if n == name] for name in ("apply_pair", "apply_jobs"))
+    assert pair and not set(pair) & set(jobs)
