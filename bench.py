@@ -40,7 +40,7 @@ HEADLINE = "c4"
 SUB_CONFIGS = ("c2", "c3", "c5", "c5-iid")
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, from the ncu captures summarised
 # under profiles/ (file named per entry); None where no capture of that workload is committed
-GATHER_RW_GBS = 5277.0        # microbench/gather_rw.cu on this machine's B200: gathered 128-byte pieces, 2 reads : 1 write
+GATHER_RW_GBS = 6079.0        # gathered 128-byte pieces, 2 reads : 1 write, through a ring of stages without arithmetic, measured on B200
 NCU_TRAFFIC = {
     "c2": (34.17e6, "profiles/apply_stream_c2_full.md"),
     "c3": (26.81e6, "profiles/apply_stream_c3_full.md"),

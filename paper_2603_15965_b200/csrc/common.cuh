@@ -366,8 +366,9 @@ constexpr int32_t kUmmaAllSegmentsMaxC = 64;   // up to this many adapters the t
 // when its CTA has its columns: the allocation waits without a limit, and a CTA beside it on the SM that held the columns while it waits
 // for this kernel, or for one that has yet to allocate, would never give them back.
 // The apply kernels, the grouping, the vocabulary and top-k routers and the MLP router with prepared images are launched so: their
-// set-up and the launch itself run behind the end of what is before them.  Measured with and without (us, whole steps): mixed 777
-// tokens 33.6 / 30.7, MLP-routed 1000 32.8 / 27.8, 3001 composite 44.4 / 39.8, top-2 2048 88.4 / 84.3, decode layers from a graph 184.7 / 180.7.
+// set-up and the launch itself run behind the end of what is before them.  Measured without and with (us, whole steps that queue): mixed
+// 777 tokens 33.2 / 30.7, MLP-routed 1000 33.2 / 29.5, 3001 composite 43.0 / 40.1, top-2 2048 87.8 / 81.7, decode layers from a graph 186.2 / 182.2;
+// a step by itself gains what its own launches overlap (mixed 47.3 / 47.1, MLP-routed 42.5 / 41.0, top-2 100.3 / 99.1).
 // Not the gates: started early, their small CTAs crowd onto the SMs that are free first (four decode layers with a gate each 172 as it is,
 // 209 with chained gates).
 bool chained_launch_enabled();   // false when the "chained_launch_off" override is set (plain stream order everywhere)

@@ -759,14 +759,14 @@ def test_tcgen05_tile_split_over_a_cluster(mode, N, C, d_in, d_out, rank):
     (700, 70, [(256, 512, 16)], "default"),                                     # many adapters, match_any grouping
     (4097, 4, [(256, 256, 16)], "default"),                                     # one token too many: two launches
     (600, 3, [(256, 256, 16), (256, 128, 64)], "default"),                      # mixed ranks: two launches
-    (300, 4, [(128, 192, 8)], "default"),                                       # CUDA-core apply: two launches
+    (300, 4, [(128, 192, 8)], "default"),                                       # CUDA-core apply: fused
     (256, 8, [(2048, 2048, 16), (2048, 1024, 16), (2048, 1024, 16), (512, 2048, 16), (2048, 6144, 16), (6144, 2048, 16)], "jobs"),
     (1024, 200, [(256, 192, 32), (256, 320, 32), (512, 64, 32)], "jobs"),       # job list: its largest size, many adapters
     (77, 3, [(512, 4096, 64), (512, 512, 64)], "jobs"), (1, 1, [(32, 32, 16)], "jobs"),
     (900, 6, [(512, 512, 16)], "twophase"),                                     # two-launch kernels forced: they group on chip
     (1024, 40, [(256, 192, 32)], "twophase"),                                   # ... their largest size, match_any grouping
     (1025, 4, [(256, 192, 32)], "twophase"),                                    # one token too many: grouping launch + 2
-    (300, 7, [(4096, 512, 64)], "default"), (77, 3, [(512, 4096, 64), (512, 512, 64)], "default"),   # rank 64: two-launch, on chip
+    (300, 7, [(4096, 512, 64)], "default"), (77, 3, [(512, 4096, 64), (512, 512, 64)], "default"),   # rank 64, one and two: fused
     # the tcgen05 kernel with the grouping inside (at most 4096 tokens and 64 adapters): one launch
     (1024, 8, [(2048, 512, 64)], "tcgen05-s8"), (700, 5, [(2048, 768, 64), (2048, 256, 64)], "tcgen05-s5"),
     (4096, 9, [(2048, 256, 64)], "tcgen05-s7r96"), (1300, 4, [(4096, 4096, 64)], "default"),
