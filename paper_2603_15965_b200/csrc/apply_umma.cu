@@ -120,14 +120,14 @@ struct UmmaCfg {
     static constexpr int kStageBytes = kTileBytes + kWBytes;
     static constexpr int kStages = R == 64 ? (WIDE ? 6 : 7) : 8;
     static constexpr int kTRowBytes = R * 2;                          // one row of T_hi / T_lo
-    static constexpr int kTBytes = kTileM * kTRowBytes;
+    static constexpr bool kOnePush = R != 64;
+    static constexpr int kTBytes = kOnePush ? 0 : kTileM * kTRowBytes;      // (only finished rows that travel to the peers pass through)
     static constexpr int kSwzBits = R == 64 ? 3 : R == 32 ? 2 : 1;    // swizzle width of R*2-byte rows
     // partial T rows received from the cluster peers: (S - 1) * ceil(128 / S) rows of R fp32: 64, 86, 96 rows for
     // S = 2, 3, 4 and at most 114 (S = 7) up to S = 8.  Rank 64 stops at S = 3 (shared memory) unless WIDE.
     // Ranks 16 and 32 have room for the whole partial of every peer ((S - 1) * 128 rows): one push, every CTA sums
     // for itself.
     static constexpr int kMaxSplitR = R == 64 ? (WIDE ? kMaxWideSplit : 3) : kMaxSplit;
-    static constexpr bool kOnePush = R != 64;
     static constexpr int kRecvBytes = kOnePush ? (kMaxSplit - 1) * kTileM * R * 4 : (WIDE ? 114 : 86) * R * 4;
     static constexpr int kCtrlBytes = 768;
     static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + 2 * kTBytes + kRecvBytes + kCtrlBytes;
@@ -445,10 +445,11 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) apply_umma_kernel(const __gri
         const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
 
         {
-            // T -> scaled bf16 hi/lo pair in shared memory, K-major, swizzled like a TMA tile of R*2-byte rows.  Both
-            // epilogue groups take part, group g with the columns [g R/2, (g+1) R/2) of every row: a lone warp runs the
-            // few hundred dependent instructions of a row at one every four cycles, and its stores into a peer's shared
-            // memory at one every ~0.14 us, so the work per thread is what this step costs.
+            // T -> scaled bf16 hi/lo pair in TMEM, the A operand of the expand (rank 64 in a cluster: by way of shared memory, K-major and
+            // swizzled, where the finished rows go from CTA to CTA).  Both epilogue groups take part, group g with the columns
+            // [g R/2, (g+1) R/2) of every row: a lone warp runs the few hundred dependent instructions of a row at one every
+            // four cycles, and its stores into a peer's shared memory at one every ~0.14 us, so the work per thread is
+            // what this step costs.
             constexpr int RH = R / 2;
             const int col0 = group * RH;
             wait_bar(bar(&ctrl->t_full), 0, abort_flag, prm.dev_status);
