@@ -32,11 +32,11 @@ inline UmmaTiles umma_tiles(int64_t N, int32_t C, int rows)
 // chunks + expand chunks divided by the split); shorter tiles make a chunk only a little cheaper (the gathers are bound by requests in
 // flight, not bytes).
 // Which load there is the host does not know, and the errors do not cost the same: a tile more than the resident clusters makes a second
-// wave.  So a split is charged what it takes under both, the worse one in full and half of their mean on top.  Of 864 calls (rank 64;
-// one, two and four projections 1024 - 4096 wide, 600 - 6000 tokens, 2 - 16 adapters, three loads), every split measured, the choice
-// is 0.9 % above the best split in the mean and 34 % at worst; charged for the larger number of tiles alone 1.1 % and 34 %, and five
-// calls were slower than before that (1700 tokens of 16 adapters, four projections 2048 wide: one CTA a tile 31.8 us, two
-// 25.0); for N / 128 + C / 2 tiles 2.0 % and 70 % (2300 tokens of 16, 2048 -> 2048).
+// wave.  So a split is charged what it takes under both, the worse one in full and half of their mean on top.  Of 2160 calls (ranks 32 and
+// 64; one, two, four and seven projections 1024 - 4096 wide, 600 - 8000 tokens, 2 - 16 adapters, three loads) 29 shapes choose another
+// split than for the larger number of tiles alone, from 16 % faster to 4 % slower, 3 % faster in the mean; none is slower than with
+// N / 128 + C / 2 tiles, which the kernel before had (1700 tokens of 16 adapters, four projections 2048 wide: one CTA a tile 32.7 us,
+// two 25.3; 3000 of 16, 1024 -> 1024: four 20.3, three 17.3; the worst of it: 1300 of 4, four 4096 wide: two 33.4, three 34.3).
 //   chunks    64-column chunks that a tile of each of the nproj projections walks (d_in + d_out); min_kx: least of d_in
 //   resident  clusters of that many CTAs that are resident at once
 template <typename Resident>
@@ -58,11 +58,10 @@ UmmaPlan choose_umma_split(const double* chunks, int nproj, int min_kx, int64_t 
             cmin = std::min(cmin, c);
             total += c * (double)tiles;
         }
-        // (margins: the tile count is an estimate, and the last clusters of a full wave start late: 25 tiles on the 26 clusters of
-        // five that fit 21.5 us, on clusters of four 18.3)
-        if (tiles * nproj * 1.1 <= slots) return cmax;
+        if (tiles * nproj * 1.1 <= slots) return cmax;       // (margin: the tile count is an estimate)
         one_wave = false;
-        if (cmax - cmin < 1e-9) return cmax * std::ceil(1.05 * (double)(tiles * nproj) / slots);
+        // (a wave that is almost full takes longer: 25 tiles on the 26 clusters of five that fit 21.5 us, on clusters of four 18.3)
+        if (cmax - cmin < 1e-9) return cmax * (1.08 * (double)((tiles * nproj + slots - 1) / slots));
         return std::max(cmax, total / slots + 0.25 * cmin);
     };
     auto cost_for = [&](int rows, int split, bool& one_wave) {
