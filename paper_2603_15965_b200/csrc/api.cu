@@ -832,24 +832,33 @@ struct HostCall {
     }
 };
 
-// Two more streams for the length of one call, one that applies and one that copies results back.  They live until what was enqueued on
-// them has run (the runtime keeps a destroyed stream that long); an event is read when it is waited for, so one serves all hand-overs of
-// its direction -- but not the results: their copies are enqueued after all launches, each behind an event of its own.
+// Two more streams for a host call, one that applies and one that copies results back.  A thread keeps one pair (for the device and the
+// priority it used last; given back when the thread ends): made for every call they cost the host 110 us each, and lone calls of 8 to
+// 15 MB took up to 14 % longer than on the caller's stream alone.  Calls of one thread on several streams meet in them in the order
+// they were made, which is that of their uploads; whoever waits follows what was enqueued before, so there is no circle.  An event is read
+// when it is waited for, so one serves all hand-overs of its direction, call after call -- but not the results: their copies are
+// enqueued after all launches, each behind an event of its own.
 constexpr int kHostMaxPieces = 4;                                           // of the last projection
 struct SideStreams {
+    int device = -1, priority = 0;
     cudaStream_t apply = nullptr, back = nullptr;
     cudaEvent_t arrived = nullptr, done = nullptr, applied[MOLORA_MAX_PROJECTIONS - 1 + kHostMaxPieces] = {};
     bool open(int results, cudaStream_t s)
     {
-        int priority = 0;                                                   // the kernels keep that of the caller's stream
-        if (cudaStreamGetPriority(s, &priority) != cudaSuccess) return false;
+        int dev = 0, prio = 0;                                              // the kernels keep the priority of the caller's stream
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaStreamGetPriority(s, &prio) != cudaSuccess) return false;
+        if (dev != device || prio != priority) close();
+        device = dev;
+        priority = prio;
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;          // (another thread may be capturing)
         if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
-        bool ok = cudaStreamCreateWithPriority(&apply, cudaStreamNonBlocking, priority) == cudaSuccess &&
-                  cudaStreamCreateWithPriority(&back, cudaStreamNonBlocking, priority) == cudaSuccess &&
-                  cudaEventCreateWithFlags(&arrived, cudaEventDisableTiming) == cudaSuccess &&
-                  cudaEventCreateWithFlags(&done, cudaEventDisableTiming) == cudaSuccess;
-        for (int i = 0; i < results && ok; ++i) ok = cudaEventCreateWithFlags(&applied[i], cudaEventDisableTiming) == cudaSuccess;
+        bool ok = true;
+        for (cudaStream_t* side : {&apply, &back})
+            ok = ok && (*side != nullptr || cudaStreamCreateWithPriority(side, cudaStreamNonBlocking, priority) == cudaSuccess);
+        auto make = [&](cudaEvent_t& e) { ok = ok && (e != nullptr || cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess); };
+        make(arrived);
+        make(done);
+        for (int i = 0; i < results; ++i) make(applied[i]);
         cudaThreadExchangeStreamCaptureMode(&mode);
         return ok;
     }
@@ -861,15 +870,19 @@ struct SideStreams {
             ok = cudaEventRecord(done, side) == cudaSuccess && cudaStreamWaitEvent(s, done, 0) == cudaSuccess && ok;
         return ok;
     }
-    ~SideStreams()
+    // (what is enqueued there still runs: the runtime keeps a destroyed stream that long)
+    void close()
     {
-        for (cudaEvent_t e : applied)
-            if (e != nullptr) cudaEventDestroy(e);
+        for (cudaEvent_t& e : applied)
+            if (e != nullptr) cudaEventDestroy(e), e = nullptr;
         if (done != nullptr) cudaEventDestroy(done);
         if (arrived != nullptr) cudaEventDestroy(arrived);
         if (back != nullptr) cudaStreamDestroy(back);
         if (apply != nullptr) cudaStreamDestroy(apply);
+        done = arrived = nullptr;
+        back = apply = nullptr;
     }
+    ~SideStreams() { close(); }
 };
 
 // scratch that molora_group_apply_batched needs for n tokens of these projections
@@ -899,7 +912,9 @@ size_t group_apply_workspace(const molora_proj_desc_t* projs, int32_t P, molora_
 // and comes back on the caller's stream.  The link carries both directions at once (49 GB/s each way against 55 one way), so results
 // return while later projections are on their way in; what cannot overlap is the last one's, which is cut where its pieces keep
 // 8 MB (a copy costs ~10 us besides its bytes: eight pieces of all tokens, copies of 1 MB, were no faster than one stream).  Calls that
-// move less than 8 MB stay in one piece: what they could hide is not much above what the second stream costs.  So do calls
+// move less than 8 MB stay in one piece: what they could hide is not above what the streams and events cost (attention projections 2048 wide, us on
+// one stream / three, queued and by itself: 384 tokens, 7.9 MB, 291 / 287 and 314 / 314; 448, 9.2 MB, 328 / 283 and 356 / 317; 768, 15.7 MB,
+// 519 / 440 and 546 / 470; 2048, 42 MB, 1280 / 1032 and 1308 / 1058).  So do calls
 // on a stream that is being captured (the graph keeps its shape), calls whose host buffers overlap (results could replace what a later
 // projection has yet to send) and those whose parts would need more scratch than the arena holds.
 constexpr double kHostPieceBytes = 8e6;
@@ -1010,7 +1025,7 @@ molora_status_t molora_forward_host(molora_router_t router, const int32_t* route
         return MOLORA_ERR_CUDA;
     if (gate >= 0 && !call.upload_x(gate, 0, N, s)) return MOLORA_ERR_CUDA;
     const int64_t last_rows = host_last_rows(call, N, route_src_host, gate, s);
-    SideStreams side;
+    thread_local SideStreams side;
     if (last_rows == 0 || !side.open(P - 1 + (int)ceil_div64(N, last_rows), s)) {
         // on the caller's stream: the other activations, route, group and apply, results back
         for (int i = 0; i < P; ++i)

@@ -3,6 +3,7 @@ a fake runtime and fake launchers (fake_runtime.cpp) that log every call; nothin
 import ctypes
 import os
 import subprocess
+import threading
 
 import pytest
 
@@ -31,14 +32,14 @@ def fake(tmp_path_factory):
     return lib
 
 
-def call(lib, N, C, shapes, fail=("", -1), priority=0, shared_x=True):
+def call(lib, N, C, shapes, fail=("", -1), priority=0, shared_x=True, stream=STREAM):
     """(status, log) of a gate-routed call; the host buffers lie 1 GB apart."""
     projs = (_HostProjC * len(shapes))(*[_HostProjC((X if shared_x else X + (100 + i << 30)), X + (i + 1 << 30), 0x2000, 0x3000, a, b, r, 1.0)
                                          for i, (a, b, r) in enumerate(shapes)])
     need = lib.molora_forward_host_arena_bytes(projs, len(shapes), M.BF16, N, C, M.ROUTE_GATE, 0)
     assert need > 0
     lib.fake_reset(fail[0].encode(), fail[1], priority)
-    st = lib.molora_forward_host(M.ROUTE_GATE, None, None, 0, G, None, 0, projs, len(shapes), M.BF16, N, C, 1 << 45, need, None, STREAM)
+    st = lib.molora_forward_host(M.ROUTE_GATE, None, None, 0, G, None, 0, projs, len(shapes), M.BF16, N, C, 1 << 45, need, None, stream)
     return st, [(w[0], [int(v) for v in w[1:]]) for w in (line.split() for line in lib.fake_log().decode().splitlines())]
 
 
@@ -48,7 +49,7 @@ CALLS = [(2048, ATTENTION), (5000, ATTENTION), (2048, [(2048, 512, 32), (2048, 8
 LAUNCHES = ("route", "group", "apply", "apply_pair", "apply_jobs")
 
 
-def before(log):
+def before(log, stream=STREAM):
     """For every entry the set of entries that have run when it runs, from stream order, events and waits; and those the caller's stream
     follows at the end."""
     last, event, sets = {}, {}, {}
@@ -60,7 +61,7 @@ def before(log):
         elif name in ("upload", "download") + LAUNCHES:
             sets[i] = last.get(a[0], frozenset())
             last[a[0]] = sets[i] | {i}
-    return sets, last.get(STREAM, frozenset())
+    return sets, last.get(stream, frozenset())
 
 
 @pytest.mark.parametrize("N,shapes", CALLS)
@@ -88,9 +89,6 @@ def test_every_step_follows_what_it_reads_and_the_stream_follows_all(fake, N, sh
             launch, = [(j, rows * cols * 2) for j, rows, projs in applies for at, cols in zip(projs[2::4], projs[3::4]) if at == a[2]]
             assert launch[0] in ran[i] and launch[1] == a[3]  # ... after the one launch that finishes it
     assert back == sum(N * b * 2 for _, b, _ in shapes)
-    for kind in ("stream", "event"):
-        made = [a[0] for n, a in log if n == kind]
-        assert sorted(made) == sorted(a[0] for n, a in log if n == "destroy_" + kind)
 
 
 @pytest.mark.parametrize("N,shapes", CALLS)
@@ -109,11 +107,39 @@ def test_a_call_that_is_refused_half_way_returns_no_results(fake, N, shapes):
                 assert at_end == frozenset(ran)
 
 
-@pytest.mark.parametrize("priority", [0, -3])
-def test_streams_of_a_call_have_the_priority_of_the_callers(fake, priority):
-    _, log = call(fake, 2048, 8, ATTENTION, priority=priority)
-    made = [a[1] for n, a in log if n == "stream"]
-    assert len(made) == 2 and set(made) == {priority}
+def test_a_thread_keeps_one_pair_of_streams(fake):
+    """Made by its first call, with the priority of the caller's stream, made again for another priority, given back when the thread ends."""
+    def names(log, kind):
+        return [a[0] for n, a in log if n == kind]
+    logs = []
+    def work():
+        for priority in (0, 0, -3, -3):
+            for N, shapes in ((2048, ATTENTION), (5000, ATTENTION), (4100, [(4096, 2048, 16)])):
+                logs.append((priority, call(fake, N, 8, shapes, priority=priority)[1]))
+        fake.fake_reset(b"", -1, 0)
+    thread = threading.Thread(target=work)
+    thread.start()
+    thread.join()
+    made = [[(a[1], p) for n, a in log if n == "stream"] for p, log in logs]
+    assert [len(m) for m in made] == [2] + [0] * 5 + [2] + [0] * 5 and all(q == p for m in made for q, p in m)
+    assert sum(len(names(log, "event")) for _, log in logs) <= 2 * (2 + 7 + 4)
+    end = [(w[0], [int(v) for v in w[1:]]) for w in (line.split() for line in fake.fake_log().decode().splitlines())]
+    for kind in ("stream", "event"):
+        assert sorted(sum((names(log, kind) for _, log in logs), [])) == sorted(sum((names(log, "destroy_" + kind) for _, log in logs), names(end, "destroy_" + kind)))
+
+
+def test_calls_of_one_thread_on_two_streams_follow_what_they_read(fake):
+    """The second call's work meets the first one's on the kept streams: each caller's stream still follows all of its own."""
+    both = []
+    for stream in (STREAM, STREAM + 1):
+        st, log = call(fake, 2048, 8, ATTENTION, stream=stream)
+        assert st == 0
+        both += [(n, a, stream) for n, a in log]
+    ran, _ = before([(n, a) for n, a, _ in both])
+    for stream in (STREAM, STREAM + 1):
+        own = {i for i in ran if both[i][2] == stream}
+        _, at_end = before([(n, a) for n, a, _ in both], stream)
+        assert own <= at_end
 
 
 def test_scratch_of_one_projection_spares_the_control_words_of_another(fake):
