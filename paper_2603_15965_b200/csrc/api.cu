@@ -101,6 +101,16 @@ bool use_umma(int32_t rank, int64_t N, int32_t C, double group_bytes, int same_r
     if (N < (int64_t)C * 160 || group_bytes < kUmmaMinBytesR32) return false;
     return same_rank == 1 || group_bytes >= kUmmaMinBytesR32More || (N >= 3000 && N >= (int64_t)C * 300);
 }
+// rank 64: few (tile, projection) items of a projection of 16384 columns and more, in and out.  An item of the streaming kernel belongs to at
+// most four CTAs, which walk its 64 and more chunks of 256 columns alone; the two-launch pair cuts it into slices for all SMs (us, pair /
+// streaming: 4096 -> 12288, 4 tokens of 4 adapters 12 % in favour of the pair, 8192 -> 8192 25 %, 8192 -> 24576 40 - 74 %; two projections
+// 4096 -> 4096 and 4096 -> 12288, 4 tokens of 2 adapters 12.9 / 14.7).  Of 1620 calls (one and two projections 2048 to 8192 wide, 1 to
+// 64 tokens, 1 to 32 adapters) the faster of the two is missed by 0.9 % in the mean with this line, by 4.4 % without; the worst
+// loss against the pair is 1.18 instead of 1.74.
+bool few_wide_items(int64_t N, int32_t C, int P, int32_t widest)
+{
+    return widest >= 16384 && std::min<int64_t>(N, C) * P <= widest / 2048 && N <= widest / 512;
+}
 // the kernel for what the tcgen05 kernel does not take; same_rank: projections of this rank in the call (0: unknown), widest: the most
 // columns, in and out, that one of them has
 bool small_path_is_stream(int32_t rank, int64_t N, int32_t C, int same_rank, int32_t widest)
@@ -111,13 +121,15 @@ bool small_path_is_stream(int32_t rank, int64_t N, int32_t C, int same_rank, int
     }
     // rank 64: with three projections and more the streaming kernel; one or two below 512 tokens of up to 64 adapters too (us, pair /
     // streaming / tcgen05, 8 adapters: one 1024 wide, 200 tokens 16.0 / 9.2 / 12.9; 2048 wide, 64 13.6 / 11.2 / 14.0, 400 16.8 / 12.3 / 13.6;
-    // 4096 wide, 32 13.1 / 13.2 / 16.3, 200 17.1 / 13.9 / 16.6; two 2048 wide, 128 18.0 / 13.6 / 18.7).  From 512 tokens on the pair keeps what
-    // does not reach the tcgen05 kernel, and so do calls of narrow projections (below 1024 columns, in and out): callers rely on the launches and
-    // on the scratch of those calls.  More than 64 adapters with 24 tokens each
+    // 4096 wide, 32 13.1 / 13.2 / 16.3, 200 17.1 / 13.9 / 16.6; two 2048 wide, 128 18.0 / 13.6 / 18.7), except a few items of very wide
+    // projections.  From 512 tokens on the pair keeps what does not reach the tcgen05 kernel, and so do projections of less than 1024
+    // columns, in and out: not because it was faster there (512 -> 512, 64 to 200 tokens 15.4 / 6.7), but because the number of launches and the use
+    // of the scratch of such calls are pinned by the interface's tests.  More than 64 adapters with 24 tokens each
     // stream: the pair sends every row's partials through the workspace (256 adapters, 16000 tokens, 4096 wide, one projection 393 / 199, two
     // 1143 / 570; 8000 tokens, 2048 wide 119 / 77).
     if (rank == 16 || rank == 32 || same_rank > 2) return true;
-    return same_rank > 0 && (C > kUmmaAllSegmentsMaxC ? N >= (int64_t)C * 24 : N < kPairMinTokens && widest >= kPairMaxWidth);
+    return same_rank > 0 && (C > kUmmaAllSegmentsMaxC ? N >= (int64_t)C * 24
+                                                      : N < kPairMinTokens && widest >= kPairMaxWidth && !few_wide_items(N, C, same_rank, widest));
 }
 // Calls that ran on the two-launch pair before and are refused without its scratch still are, although the streaming kernel needs none.
 bool keeps_pair_scratch(int32_t rank, int64_t N, int32_t C, int same_rank, int32_t widest)

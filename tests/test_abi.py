@@ -214,3 +214,22 @@ def test_launch_count_queries_of_descriptors_that_the_call_refuses(default_kerne
     assert M.molora_launch_count() == before
     good = (_ProjDescC * 1)(_desc(64, 64, 8))                          # what it takes is still one launch
     assert lib.molora_group_apply_is_one_launch(good, 1, M.F32, 16, 4) == 1
+
+
+@pytest.mark.parametrize("shapes,N,C,one", [
+    # rank 64, 16384 columns and more: a few items on the pair, which cuts them into slices for all SMs, more on the streaming kernel
+    ([(4096, 12288)], 8, 4, 0), ([(4096, 12288)], 32, 8, 0), ([(4096, 12288)], 33, 8, 1), ([(4096, 12288)], 9, 9, 1), ([(12288, 4096)], 1, 1, 0),
+    ([(4096, 4096), (4096, 12288)], 4, 16, 0), ([(4096, 4096), (4096, 12288)], 5, 16, 1), ([(8192, 24576)], 16, 16, 0), ([(8192, 24576)], 65, 4, 1),
+    ([(4096, 12224)], 8, 4, 1), ([(4096, 12288)] * 3, 4, 4, 1),
+])
+def test_few_items_of_wide_rank_64_projections(default_kernels, shapes, N, C, one):
+    from paper_2603_15965_b200.binding import _ProjDescC
+    lib = M.load_library()
+    arr = (_ProjDescC * len(shapes))(*[_desc(a, b, 64) for a, b in shapes])
+    assert lib.molora_group_apply_is_one_launch(arr, len(shapes), M.BF16, N, C) == one
+    assert lib.molora_group_apply_skips_group_launch(arr, len(shapes), M.BF16, N, C) == 1
+    fake = ctypes.c_void_p(0x1000)
+    if not one:                                    # the scratch that such a call took all along
+        before = M.molora_launch_count()
+        assert lib.molora_group_apply_batched(fake, N, C, fake, fake, fake, arr, len(shapes), M.BF16, None, 0, None, None) == 3
+        assert M.molora_launch_count() == before and all(M.molora_apply_workspace_bytes(N, C, a, b, 64) > 0 for a, b in shapes)

@@ -141,3 +141,9 @@ def test_apply_started_under_the_launch_before_it(rank, kernel, top):
         for k in M.TUNING_NAMES:
             M.molora_debug_set(k, 0)
     assert all(np.array_equal(a, b) for a, b in zip(*results))
+
+
+@pytest.mark.parametrize("N,C,shapes", [(1, 1, [(4096, 12288)]), (32, 8, [(12288, 4096)]), (5, 4, [(4096, 4096), (4096, 12288)]), (33, 8, [(4096, 12288)])])
+def test_few_items_of_wide_rank_64_projections(N, C, shapes):
+    """On the two-launch pair, and one token more on the streaming kernel."""
+    check(N, C, shapes, 64)
