@@ -8,6 +8,8 @@
 #include <cstring>
 #include <mutex>
 
+#include <unistd.h>
+
 using namespace molora;
 
 namespace molora {
@@ -853,6 +855,7 @@ struct HostCall {
 constexpr int kHostMaxPieces = 4;                                           // of the last projection
 struct SideStreams {
     int device = -1, priority = 0;
+    pid_t owner = 0;                                                        // (a forked child ends without touching its parent's)
     cudaStream_t apply = nullptr, back = nullptr;
     cudaEvent_t arrived = nullptr, done = nullptr, applied[MOLORA_MAX_PROJECTIONS - 1 + kHostMaxPieces] = {};
     bool open(int results, cudaStream_t s)
@@ -862,6 +865,7 @@ struct SideStreams {
         if (dev != device || prio != priority) close();
         device = dev;
         priority = prio;
+        owner = getpid();
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;          // (another thread may be capturing)
         if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
         bool ok = true;
@@ -894,7 +898,10 @@ struct SideStreams {
         done = arrived = nullptr;
         back = apply = nullptr;
     }
-    ~SideStreams() { close(); }
+    ~SideStreams()
+    {
+        if (owner == getpid()) close();
+    }
 };
 
 // scratch that molora_group_apply_batched needs for n tokens of these projections

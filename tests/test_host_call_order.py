@@ -3,6 +3,7 @@ a fake runtime and fake launchers (fake_runtime.cpp) that log every call; nothin
 import ctypes
 import os
 import subprocess
+import sys
 import threading
 
 import pytest
@@ -126,6 +127,31 @@ def test_a_thread_keeps_one_pair_of_streams(fake):
     end = [(w[0], [int(v) for v in w[1:]]) for w in (line.split() for line in fake.fake_log().decode().splitlines())]
     for kind in ("stream", "event"):
         assert sorted(sum((names(log, kind) for _, log in logs), [])) == sorted(sum((names(log, "destroy_" + kind) for _, log in logs), names(end, "destroy_" + kind)))
+
+
+FORKED = """
+import ctypes, os, sys
+lib = ctypes.CDLL(sys.argv[1])
+lib.molora_forward_host_arena_bytes.restype = ctypes.c_size_t
+class P(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_void_p) for n in ("x", "y", "A", "B")] + [(n, ctypes.c_int32) for n in ("d_in", "d_out", "rank")] + [("scale", ctypes.c_float)]
+projs = (P * 2)(*[P(0x10000000, 0x10000000 + (i + 1 << 30), 0x2000, 0x3000, 2048, 2048, 16, 1.0) for i in range(2)])
+v, n = ctypes.c_void_p, ctypes.c_int64
+need = lib.molora_forward_host_arena_bytes(projs, 2, 1, n(2048), 8, 1, 0)
+assert lib.molora_forward_host(1, None, None, 0, v(0x1000), None, 0, projs, 2, 1, n(2048), 8, v(1 << 45), ctypes.c_size_t(need), None, v(0x11)) == 0
+lib.fake_report_at_exit()
+if os.fork() == 0:
+    ctypes.CDLL(None).exit(0)
+os.wait()
+print("parent", flush=True)
+"""
+
+
+def test_a_forked_child_ends_without_touching_its_parents_streams(fake):
+    res = subprocess.run([sys.executable, "-c", FORKED, fake._name], capture_output=True, text=True)
+    assert res.returncode == 0, res.stderr
+    child, parent = res.stdout.split("parent")
+    assert "end" in child and "destroy_stream" not in child and parent.count("destroy_stream") == 2
 
 
 def test_calls_of_one_thread_on_two_streams_follow_what_they_read(fake):
